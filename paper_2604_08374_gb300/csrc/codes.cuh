@@ -1,0 +1,317 @@
+// codes.cuh -- bit-plane codes of the registers, the form in which the grouped
+// union gathers them from the second pass on.
+//
+// No register j of any node ever exceeds G[j], the largest rho inserted with
+// index j (kept from Alg. 1's initialisation).  A pass therefore needs only
+// the top of each register's range:
+//   K = 4  code = max(0, R - B[j]) with B[j] = max(0, G[j] - 15): 4 bits, exact
+//          for every value above B[j];
+//   K = 1  one bit, R == G[j] (the register has reached its final value).
+// A register whose gathered code is 0 while its own value lies below B[j]
+// (K = 4) or G[j] (K = 1) is left open: its (node, slice) pair is marked in the
+// need masks and recomputed from the bytes, so every result is exact.
+//
+// Why: the union is bound by the L2 bytes of its row gathers.  A K = 4 row
+// holds twice the registers of a byte row and a K = 1 row eight times.  After
+// pass 1 practically no register lies 15 below G (measured on the city and
+// medium graphs); after pass 2, 82-99 % of the registers equal G, and after
+// pass 3 all but 1e-5 of the city's.
+//
+// Measured (GB300): the city graph's pass 2 takes four launches of 128-byte
+// K = 4 rows at 3.6 ms and pass 3 one of K = 1 rows at 2.8 ms, where the byte
+// union takes eight at 2.8 ms each; the d = 3 analysis 54.8 -> 29.7 ms, the
+// unlimited p = 12 one 342 -> 116 ms, medium d = 3 3.2 -> 2.2 ms.
+//
+// Layout: a 16-byte unit holds 32 registers as four bit planes (K = 4; word k =
+// bit k of the codes, bit i = register i) or 128 registers as one plane
+// (K = 1).  In planes the maximum of 32 codes takes 8 three-input logic
+// operations (a borrow chain, then a select), 2.5 times fewer per register
+// than byte maxima on 16-bit lanes, and the maximum of one-bit codes is OR.
+#pragma once
+
+#include "hb_device.cuh"
+
+namespace vga {
+namespace {
+
+// Registers per 16-byte unit.
+template <int K>
+constexpr int kUnitRegs = K == 4 ? 32 : 128;
+
+// Lane-wise maximum of two units.
+template <int K>
+__device__ __forceinline__ uint4 code_max(uint4 a, uint4 b) {
+    if (K == 1) return make_uint4(a.x | b.x, a.y | b.y, a.z | b.z, a.w | b.w);
+    uint32_t t = a.x & ~b.x;                 // a > b on bit 0, then up the planes
+    t = (a.y & ~b.y) | (t & (a.y | ~b.y));
+    t = (a.z & ~b.z) | (t & (a.z | ~b.z));
+    t = (a.w & ~b.w) | (t & (a.w | ~b.w));
+    return make_uint4((a.x & t) | (b.x & ~t), (a.y & t) | (b.y & ~t), (a.z & t) | (b.z & ~t),
+                      (a.w & t) | (b.w & ~t));
+}
+
+// Bit 0 of a word's 4 bytes (or 8 nibbles) gathered into its low bits, and back.
+__device__ __forceinline__ uint32_t gather_bytes(uint32_t w) { return ((w & 0x01010101u) * 0x01020408u) >> 24; }
+__device__ __forceinline__ uint32_t spread_bytes(uint32_t b) { return (b * 0x00204081u) & 0x01010101u; }
+__device__ __forceinline__ uint32_t gather_nibbles(uint32_t w) {
+    w &= 0x11111111u;
+    w = (w | w >> 3) & 0x03030303u;
+    w = (w | w >> 6) & 0x000F000Fu;
+    return (w | w >> 12) & 0xFFu;
+}
+__device__ __forceinline__ uint32_t spread_nibbles(uint32_t b) {
+    b = (b | b << 12) & 0x000F000Fu;
+    b = (b | b << 6) & 0x03030303u;
+    return (b | b << 3) & 0x11111111u;
+}
+
+// The register window of a run, one word array each in the registers' own
+// format (bytes, or nibbles): top[j] = G[j] and low[j] = B[j].
+struct CodeWindow {
+    const uint32_t *top, *low;
+};
+
+// Address of byte `byte` of node v's registers (slice-major, slices of
+// 2^s_log2 bytes).
+__device__ __forceinline__ uint64_t reg_at(uint32_t n, int s_log2, uint32_t v, uint32_t byte) {
+    return (((uint64_t)(byte >> s_log2) * n + v) << s_log2) + (byte & ((1u << s_log2) - 1u));
+}
+
+// Codes of unit u of node v, from its registers.
+template <int K, bool NIB>
+__device__ __forceinline__ uint4 code_pack(const uint8_t *__restrict__ cur, uint32_t n, int s_log2, uint32_t v,
+                                           uint32_t u, const CodeWindow &win) {
+    constexpr int F = NIB ? 8 : 4;                  // registers per word
+    constexpr int BYTES = kUnitRegs<K> * 4 / F;     // register bytes of a unit
+    uint32_t p[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int h = 0; h < BYTES / 16; h++) {
+        const uint32_t byte = u * BYTES + 16u * h;
+        const uint4 x = __ldg(reinterpret_cast<const uint4 *>(cur + reg_at(n, s_log2, v, byte)));
+        const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const int r = (4 * h + i) * F;          // first register of the word, within the unit
+            if (K == 4) {
+                const uint32_t c = NIB ? w[i] : __vsubus4(w[i], __ldg(win.low + byte / 4u + i));
+#pragma unroll
+                for (int k = 0; k < 4; k++)
+                    p[k] |= (NIB ? gather_nibbles(c >> k) : gather_bytes(c >> k)) << r;
+            } else {
+                const uint32_t e = equal_bits<NIB>(w[i], __ldg(win.top + byte / 4u + i));
+                p[r / 32] |= (NIB ? gather_nibbles(e) : gather_bytes(e)) << (r % 32);
+            }
+        }
+    }
+    return make_uint4(p[0], p[1], p[2], p[3]);
+}
+
+// next[v] for the registers of unit u, from the unit's gathered codes and the
+// node's own registers; returns whether a register changed (bit 0) per 16
+// register bytes h in `chg16` and left open in `open16` (bit h each).
+template <int K, bool NIB>
+__device__ __forceinline__ void code_store(uint4 code, const uint8_t *__restrict__ cur, uint8_t *__restrict__ nxt,
+                                           uint32_t n, int s_log2, uint32_t v, uint32_t u, const CodeWindow &win,
+                                           uint32_t &chg16, uint32_t &open16) {
+    constexpr int F = NIB ? 8 : 4;
+    constexpr int BYTES = kUnitRegs<K> * 4 / F;
+    const uint32_t p[4] = {code.x, code.y, code.z, code.w};
+    chg16 = open16 = 0;
+#pragma unroll
+    for (int h = 0; h < BYTES / 16; h++) {
+        const uint32_t byte = u * BYTES + 16u * h;
+        const uint64_t at = reg_at(n, s_log2, v, byte);
+        const uint4 x = __ldg(reinterpret_cast<const uint4 *>(cur + at));
+        const uint32_t own[4] = {x.x, x.y, x.z, x.w};
+        uint32_t res[4], diff = 0, open = 0;
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const int r = (4 * h + i) * F;
+            if (K == 4) {
+                uint32_t c = 0;
+#pragma unroll
+                for (int k = 0; k < 4; k++) {
+                    const uint32_t b = (p[k] >> r) & (NIB ? 0xFFu : 0xFu);
+                    c |= (NIB ? spread_nibbles(b) : spread_bytes(b)) << k;
+                }
+                if (NIB) {
+                    res[i] = RegFmt<NIB>::max_word(own[i], c);
+                } else {
+                    const uint32_t low = __ldg(win.low + byte / 4u + i);
+                    const uint32_t zero = __vcmpeq4(c, 0u);       // 0xFF where the code is 0
+                    res[i] = __vmaxu4(own[i], (c + low) & ~zero);  // c + low <= 15 + B: no carry between bytes
+                    open |= zero & __vcmpltu4(own[i], low);
+                }
+            } else {
+                const uint32_t b = (p[r / 32] >> (r % 32)) & (NIB ? 0xFFu : 0xFu);
+                const uint32_t set = (NIB ? spread_nibbles(b) * 0xFu : spread_bytes(b) * 0xFFu);
+                const uint32_t top = __ldg(win.top + byte / 4u + i);
+                res[i] = (own[i] & ~set) | (top & set);
+                open |= res[i] ^ top;
+            }
+            diff |= res[i] ^ own[i];
+        }
+        *reinterpret_cast<uint4 *>(nxt + at) = make_uint4(res[0], res[1], res[2], res[3]);
+        chg16 |= diff ? 1u << h : 0u;
+        open16 |= open ? 1u << h : 0u;
+    }
+}
+
+// Fold the code rows of entries buf[lo .. hi) of a staged chunk into acc: the
+// lane mapping and the steps of lean_fold.
+template <int S, int K>
+__device__ __forceinline__ void code_fold(const uint8_t *__restrict__ base, const uint32_t *buf, int lo, int hi, int g,
+                                          uint4 (&acc)[LeanShape<S>::V4]) {
+    using Sh = LeanShape<S>;
+    constexpr int STEP = Sh::P * Sh::U;
+    auto step = [&](int kb, bool check) {
+        uint32_t r[Sh::U];
+        if constexpr (Sh::U == 4) {
+            const uint4 t = *reinterpret_cast<const uint4 *>(buf + kb);
+            r[0] = t.x;
+            r[1] = t.y;
+            r[2] = t.z;
+            r[3] = t.w;
+        } else {
+            const uint2 t = *reinterpret_cast<const uint2 *>(buf + kb);
+            r[0] = t.x;
+            r[1] = t.y;
+        }
+        uint4 x[Sh::U][Sh::V4];
+#pragma unroll
+        for (int u = 0; u < Sh::U; u++) {
+            if (!check || (kb + u >= lo && kb + u < hi)) {
+                load_row_chunk<Sh::V4>(base + (uint64_t)r[u] * S, x[u]);
+            } else {
+#pragma unroll
+                for (int q = 0; q < Sh::V4; q++) x[u][q] = make_uint4(0, 0, 0, 0);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < Sh::V4; q++) {
+            uint4 t = code_max<K>(x[0][q], x[1][q]);
+            if constexpr (Sh::U == 4) t = code_max<K>(t, code_max<K>(x[2][q], x[3][q]));
+            acc[q] = code_max<K>(acc[q], t);
+        }
+    };
+    int k0 = lo & ~(Sh::U - 1);
+    if (k0 < lo) {
+        const int kb = k0 + g * Sh::U;
+        if (kb < hi) step(kb, true);
+        k0 += STEP;
+    }
+    for (; k0 + STEP <= hi; k0 += STEP) step(k0 + g * Sh::U, false);
+    if (k0 < hi) {
+        const int kb = k0 + g * Sh::U;
+        if (kb < hi) step(kb, true);
+    }
+}
+
+// Fold the warp's P lane groups together (every lane ends with the maximum of
+// its part of the row).
+template <int S, int K>
+__device__ __forceinline__ void code_finish(uint4 (&acc)[LeanShape<S>::V4]) {
+    using Sh = LeanShape<S>;
+#pragma unroll
+    for (int o = Sh::G; o < 32; o <<= 1)
+#pragma unroll
+        for (int q = 0; q < Sh::V4; q++) {
+            uint4 y;
+            y.x = __shfl_xor_sync(0xffffffffu, acc[q].x, o);
+            y.y = __shfl_xor_sync(0xffffffffu, acc[q].y, o);
+            y.z = __shfl_xor_sync(0xffffffffu, acc[q].z, o);
+            y.w = __shfl_xor_sync(0xffffffffu, acc[q].w, o);
+            acc[q] = code_max<K>(acc[q], y);
+        }
+}
+
+// The code maxima of one group's nodes (union_group's walk over its distinct
+// rows, class by class) into part[NODES][S / 16].
+template <int S, int K, int NODES>
+__device__ __forceinline__ void code_group(const GroupItem &gi, const uint32_t *__restrict__ rows,
+                                           const uint2 *__restrict__ cls, const uint8_t *__restrict__ tab, uint4 *part,
+                                           LkStage &st, uint32_t &phase, int lane, int *err) {
+    using Sh = LeanShape<S>;
+    constexpr int W16 = S / 16;
+    const uint32_t cnt = gi.cnt, nc = gi.nc;
+    const uint64_t cls0 = gi.cls;
+    uint4 acc[Sh::V4] = {};
+    const int g = lane / Sh::G, sub = lane % Sh::G;
+    const uint8_t *base = tab + sub * Sh::CH;
+    if (cnt == 0) return;
+    uint32_t ci = 0;
+    uint2 cd = cls[cls0];
+    uint32_t cend = cd.y;
+    const StageStream ss(rows, gi.b, gi.b + cnt);
+    ss.start(st, lane);
+    for (uint32_t c = 0; c < ss.chunks; c++) {
+        const uint32_t *buf = ss.acquire(st, c, phase, err, lane);
+        const uint32_t s0 = c * kLkChunk;
+        uint32_t lo = s0;
+        const uint32_t hi = min(cnt, s0 + (uint32_t)kLkChunk);
+        while (lo < hi) {  // warp-uniform: split the chunk at class ends
+            const uint32_t seg = min(hi, cend);
+            if (seg > lo) code_fold<S, K>(base, buf, (int)(lo - s0), (int)(seg - s0), g, acc);
+            lo = seg;
+            if (lo == cend) {  // the class is complete
+                code_finish<S, K>(acc);
+                if (g == 0) {
+#pragma unroll
+                    for (int j = 0; j < NODES; j++)
+                        if ((cd.x >> j) & 1u)
+#pragma unroll
+                            for (int q = 0; q < Sh::V4; q++) {
+                                uint4 &pp = part[j * W16 + sub * Sh::V4 + q];
+                                pp = code_max<K>(pp, acc[q]);
+                            }
+                }
+#pragma unroll
+                for (int q = 0; q < Sh::V4; q++) acc[q] = make_uint4(0, 0, 0, 0);
+                if (++ci < nc) {
+                    cd = cls[cls0 + ci];
+                    cend += cd.y;
+                } else {
+                    cend = 0xffffffffu;
+                }
+            }
+        }
+        ss.release(st, c, lane);
+    }
+}
+
+// Rows [r0, r0 + B) of a code slice's table region (units c0 .. c0 + S / 16 of
+// every node) straight from the registers: the rows and their halo are packed
+// into `buf` once, then each thread folds the window of one output unit, as in
+// table_item.  All threads of the CTA take part.
+template <int S, int K, bool NIB>
+__device__ void code_table_item(const uint8_t *__restrict__ cur, uint8_t *__restrict__ tab, uint32_t n, int s_log2,
+                                uint32_t c0, uint32_t r0, uint8_t *buf, int scheme, const CodeWindow &win) {
+    using T = TableShape<S>;
+    uint4 *b4 = reinterpret_cast<uint4 *>(buf);
+    const uint32_t avail = (n - r0 < (uint32_t)T::R) ? n - r0 : (uint32_t)T::R;
+    for (int x = threadIdx.x; x < T::R * T::C16; x += blockDim.x) {
+        const uint32_t row = x / T::C16, c = x % T::C16;
+        b4[x] = row < avail ? code_pack<K, NIB>(cur, n, s_log2, r0 + row, c0 + c, win) : make_uint4(0, 0, 0, 0);
+    }
+    __syncthreads();
+    for (int x = threadIdx.x; x < T::B * T::C16; x += blockDim.x) {
+        const uint32_t row = x / T::C16, c = x % T::C16;
+        const uint64_t i = (uint64_t)r0 + row;
+        uint4 acc = b4[x];
+        if (i < n) reinterpret_cast<uint4 *>(tab + i * S)[c] = acc;
+#pragma unroll
+        for (int j = 1; j < 16; j++) {
+            acc = code_max<K>(acc, b4[x + j * T::C16]);
+            if ((j & (j + 1)) == 0) {
+                const int k = 31 - __clz(j + 1);
+                const bool kept = scheme == 0 || (k & 1) == 0;
+                const int slot = scheme == 0 ? k : k / 2;
+                if (kept && i + (1u << k) <= n)
+                    reinterpret_cast<uint4 *>(tab + ((uint64_t)slot * n + i) * S)[c] = acc;
+            }
+        }
+    }
+}
+
+}  // namespace
+}  // namespace vga

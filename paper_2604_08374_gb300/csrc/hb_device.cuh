@@ -92,6 +92,16 @@ struct RegFmt {
     }
 };
 
+// Bit 0 of every register of the word set where the registers of a and b agree.
+template <bool NIB>
+__device__ __forceinline__ uint32_t equal_bits(uint32_t a, uint32_t b) {
+    if (!NIB) return __vcmpeq4(a, b) & 0x01010101u;
+    uint32_t e = a ^ b;
+    e |= e >> 1;
+    e |= e >> 2;
+    return ~e & 0x11111111u;
+}
+
 // Fold the S-byte rows row(ids[0..cnt)) into acc (4 * V4 words per lane, split
 // form).  Loads for U rows per lane are issued before any is folded.
 template <int S, bool NIB, class Row>
@@ -868,14 +878,18 @@ __device__ __forceinline__ double u128_to_double(uint64_t hi, uint64_t lo) {
 // [b0, b1) of node v (slice-major storage whose slice 0 holds byte b0 ... of
 // every node): lo/hi accumulate sum of 2^(K - M) over the registers M >= 1,
 // zeros counts M = 0 (K = 65 - p).  Warp-cooperative; every lane ends with the
-// warp's totals.
+// warp's totals.  With top given (the node's register words of a window's
+// top), *at_top gets the number of registers equal to it.
 __device__ __forceinline__ void harmonic_partial(const uint8_t *__restrict__ regs, uint32_t n, int p, int S,
                                                  uint32_t b0, uint32_t b1, uint32_t v, int lane, bool nib,
-                                                 uint64_t &lo, uint64_t &hi, uint32_t &zeros) {
+                                                 uint64_t &lo, uint64_t &hi, uint32_t &zeros,
+                                                 const uint32_t *__restrict__ top = nullptr,
+                                                 uint32_t *at_top = nullptr) {
     const int K = 65 - p;
     lo = 0;
     hi = 0;
     zeros = 0;
+    uint32_t full = 0;
     const int fields = nib ? 8 : 4;  // registers per 32-bit word
     const int width = nib ? 4 : 8;
     const uint32_t fmask = nib ? 0xFu : 0xFFu;
@@ -884,6 +898,13 @@ __device__ __forceinline__ void harmonic_partial(const uint8_t *__restrict__ reg
         const uint32_t s = rel / (uint32_t)S, o = rel % (uint32_t)S;
         const uint4 x = *reinterpret_cast<const uint4 *>(regs + ((uint64_t)s * n + v) * (uint64_t)S + o);
         const uint32_t wv[4] = {x.x, x.y, x.z, x.w};
+        if (top) {  // registers equal to the window's top (codes.cuh)
+            const uint4 g = __ldg(reinterpret_cast<const uint4 *>(top) + r0 / 16u);
+            const uint32_t gv[4] = {g.x, g.y, g.z, g.w};
+#pragma unroll
+            for (int i = 0; i < 4; i++)
+                full += __popc(nib ? equal_bits<true>(wv[i], gv[i]) : equal_bits<false>(wv[i], gv[i]));
+        }
         // A lane adds at most m / 32 terms of at most 2^(K-1) = 2^(64-p) each in
         // this loop, so its sum stays below 2^59: no carry into hi here.
 #pragma unroll
@@ -903,6 +924,7 @@ __device__ __forceinline__ void harmonic_partial(const uint8_t *__restrict__ reg
         lo += olo;
         hi += ohi + (lo < olo);
     }
+    if (top) *at_top = __reduce_add_sync(0xffffffffu, full);
 }
 
 // HLL estimator (Sec. 2.3, Sec. 3.3) from the exact harmonic sum, then
@@ -911,7 +933,8 @@ __device__ __forceinline__ void harmonic_partial(const uint8_t *__restrict__ reg
 // harmonic_partial) and rounded once, so the result does not depend on
 // summation order.  E = alpha_m m^2 / Z; c = lc[V] = m ln(m/V) if E <= 2.5m
 // and V > 0, else E.  For t >= 1: sum_d += t * (c - c_prev), and inc_flag
-// records max_v(c - c_prev) > 0.5 (the paper's convergence test).
+// records max_v(c - c_prev) > 0.5 (the paper's convergence test); t = 0 clears
+// sum_d.
 __device__ __forceinline__ void estimate_finish(uint64_t lo, uint64_t hi, uint32_t zeros, int p, int t,
                                                 double alpha_mm, const double *__restrict__ lc,
                                                 const double *__restrict__ c_prev, double *__restrict__ c_cur,
@@ -932,6 +955,8 @@ __device__ __forceinline__ void estimate_finish(uint64_t lo, uint64_t hi, uint32
         const double diff = __dsub_rn(c, c_prev[v]);
         sum_d[v] = __dadd_rn(sum_d[v], __dmul_rn((double)t, diff));
         if (diff > 0.5 && *reinterpret_cast<volatile uint32_t *>(inc_flag) == 0u) atomicOr(inc_flag, 1u);
+    } else {
+        sum_d[v] = 0.0;
     }
     c_cur[v] = c;
 }
@@ -942,11 +967,12 @@ __device__ __forceinline__ void estimate_node(const uint8_t *__restrict__ regs, 
                                               double alpha_mm, const double *__restrict__ lc,
                                               const double *__restrict__ c_prev, double *__restrict__ c_cur,
                                               double *__restrict__ sum_d, uint32_t *__restrict__ inc_flag, uint32_t v,
-                                              int lane, bool nib = false) {
+                                              int lane, bool nib = false, const uint32_t *__restrict__ top = nullptr,
+                                              uint32_t *at_top = nullptr) {
     const uint32_t node_bytes = nib ? (1u << p) / 2u : (1u << p);  // 4-bit registers: two per byte
     uint64_t lo, hi;
     uint32_t zeros;
-    harmonic_partial(regs, n, p, S, 0u, node_bytes, v, lane, nib, lo, hi, zeros);
+    harmonic_partial(regs, n, p, S, 0u, node_bytes, v, lane, nib, lo, hi, zeros, top, at_top);
     if (lane != 0) return;
     estimate_finish(lo, hi, zeros, p, t, alpha_mm, lc, c_prev, c_cur, sum_d, inc_flag, v);
 }

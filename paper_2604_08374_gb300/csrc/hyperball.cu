@@ -51,14 +51,20 @@ const std::vector<double> &lc_table(int p) {
 namespace {
 
 // Alg. 1 initialisation; with `keys` given, each node's key for the first
-// pass's scatter as well (KeyFmt: 16-bit for p <= kKey16MaxP, else 32-bit).
+// pass's scatter as well (KeyFmt: 16-bit for p <= kKey16MaxP, else 32-bit);
+// with `gmax` given (zeroed), the largest rho inserted per register index.
 __global__ void hb_init_kernel(uint8_t *__restrict__ regs, uint32_t n, int p, int S, uint64_t seed, int nib,
-                               uint32_t s0, uint32_t s1, void *__restrict__ keys) {
+                               uint32_t s0, uint32_t s1, void *__restrict__ keys, uint32_t *gmax = nullptr) {
     const uint64_t v = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= n) return;
     init_node(regs, n, p, S, seed, (uint32_t)v, nib != 0, s0, s1);
+    const uint32_t key = node_key((uint32_t)v, p, seed, nib != 0);
+    if (gmax) {
+        uint32_t *g = gmax + (key >> 8);
+        const uint32_t rho = key & 0xffu;
+        if (*reinterpret_cast<volatile uint32_t *>(g) < rho) atomicMax(g, rho);
+    }
     if (keys) {
-        const uint32_t key = node_key((uint32_t)v, p, seed, nib != 0);
         if (p <= kKey16MaxP)
             static_cast<uint16_t *>(keys)[v] = KeyFmt<uint16_t>::pack(key);
         else
@@ -173,14 +179,15 @@ __global__ void __maxnreg__(VGA_UNION_MAXNREG) hb_union_runs_kernel(
 // with its own registers and stored (lean_store).  The maximum over each
 // node's rows is that over its own lookup list, so the registers equal those
 // of hb_union_runs_kernel bit for bit.  With need given, a group none of whose
-// nodes needs slice `s` keeps its registers; otherwise all its nodes are
-// recomputed (a node that needed nothing gets its own registers back).
+// nodes needs slice `s` keeps its registers (keep != 0) or is left alone (its
+// next[] was settled by a code pass); otherwise all its nodes are recomputed
+// (a node that needed nothing gets its registers again).
 // Shared memory per warp: an LkStage, then NODES rows of S bytes.
 template <int S, bool NIB, int NODES>
 __global__ void __maxnreg__(VGA_UNION_MAXNREG) hb_union_groups_kernel(
     const GroupItem *__restrict__ items, uint64_t n_items, const uint32_t *__restrict__ rows,
     const uint2 *__restrict__ cls, const uint8_t *__restrict__ cur, const uint8_t *__restrict__ tab,
-    uint8_t *__restrict__ nxt, uint32_t *__restrict__ flags, const uint32_t *__restrict__ need, int s,
+    uint8_t *__restrict__ nxt, uint32_t *__restrict__ flags, const uint32_t *__restrict__ need, int s, int keep,
     uint8_t *__restrict__ chg) {
     constexpr int W16 = S / 16;  // uint4 words of a slice row
     extern __shared__ __align__(128) unsigned char s_dyn[];
@@ -201,6 +208,7 @@ __global__ void __maxnreg__(VGA_UNION_MAXNREG) hb_union_groups_kernel(
             any |= v != 0xffffffffu && ((need[v] >> s) & 1u);
         }
         if (!any) {
+            if (!keep) return;
 #pragma unroll
             for (int j = 0; j < NODES; j++) {
                 const uint32_t v = gi.node[j];
@@ -322,7 +330,9 @@ __global__ void __launch_bounds__(256) hb_need_csr_kernel(const uint64_t *__rest
 // per CTA of 256 threads, in one launch.
 template <int S, bool NIB>
 __global__ void __launch_bounds__(256) hb_table_kernel(const uint8_t *__restrict__ cur, uint8_t *__restrict__ tab,
-                                                       uint32_t n, int scheme) {
+                                                       uint32_t n, int scheme, const uint32_t *__restrict__ open,
+                                                       int s) {
+    if (open && !((*open >> s) & 1u)) return;  // a code pass left nothing open in this slice
     __shared__ __align__(16) uint8_t buf[TableShape<S>::R * S];
     table_item<S, NIB>(cur, tab, n, blockIdx.x * (uint32_t)TableShape<S>::B, buf, scheme);
 }
@@ -406,15 +416,33 @@ __global__ void __launch_bounds__(512) stream_bench_kernel(const uint4 *__restri
 }
 
 // HLL estimate of every node, then Eq. sumD (estimate_node); flags[1]
-// records the paper's convergence test max_v(c_t - c_{t-1}) > 0.5.
+// records the paper's convergence test max_v(c_t - c_{t-1}) > 0.5.  With top
+// given (the window of a run that unions codes), full[v] records the nodes
+// whose registers all equal it, and the 64-bit count at flags[6] adds up the
+// registers that do.
 __global__ void hb_estimate_kernel(const uint8_t *__restrict__ regs, uint32_t n, int p, int S, int t,
                                    double alpha_mm, const double *__restrict__ lc, const double *__restrict__ c_prev,
                                    double *__restrict__ c_cur, double *__restrict__ sum_d,
-                                   uint32_t *__restrict__ flags, int nib) {
+                                   uint32_t *__restrict__ flags, int nib, const uint32_t *__restrict__ top,
+                                   uint8_t *__restrict__ full) {
+    __shared__ uint32_t s_top[32];
     const int lane = threadIdx.x & 31;
     const uint64_t warp = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (warp >= n) return;
-    estimate_node(regs, n, p, S, t, alpha_mm, lc, c_prev, c_cur, sum_d, flags + 1, (uint32_t)warp, lane, nib != 0);
+    uint32_t at_top = 0;
+    if (warp < n)
+        estimate_node(regs, n, p, S, t, alpha_mm, lc, c_prev, c_cur, sum_d, flags + 1, (uint32_t)warp, lane, nib != 0,
+                      top, &at_top);
+    if (!top) return;
+    if (lane == 0) {
+        if (warp < n) full[warp] = at_top == (1u << p) ? 1u : 0u;
+        s_top[threadIdx.x >> 5] = at_top;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned long long sum = 0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); w++) sum += s_top[w];
+        if (sum) atomicAdd(reinterpret_cast<unsigned long long *>(flags + 6), sum);
+    }
 }
 
 // Register-range shard: node v's exact partial harmonic sum over the shard's
@@ -493,10 +521,11 @@ struct Plan {
     GroupList groups;      // runs mode with group > 0: the grouped lookup lists for `hub`
     bool first_scatter = false;  // pass 1 by the scatter of the nodes' keys (kept at off_tab)
     int track = 0;               // runs mode, slices <= 32: change tracking (0 off, 1 automatic, 2 every pass)
+    bool codes = false;          // passes from the second on gather register codes (codes.cuh)
     uint64_t n = 0;
     // workspace layout (byte offsets, 256-aligned)
     uint64_t off_cur = 0, off_next = 0, off_c0 = 0, off_c1 = 0, off_sum = 0, off_lc = 0, off_flags = 0, off_tab = 0,
-             off_chg = 0, off_need = 0, off_ortab = 0, chg_bytes = 0, total = 0;
+             off_chg = 0, off_need = 0, off_ortab = 0, off_win = 0, off_full = 0, chg_bytes = 0, total = 0;
 };
 
 static uint64_t align256(uint64_t x) { return (x + 255) & ~255ull; }
@@ -511,6 +540,11 @@ constexpr int kTrackMaxSlices = 32;
 // this share of the (node, slice) pairs: after a pass that changed more,
 // nearly every node has a changed neighbour in every slice.
 constexpr double kTrackBelow = 0.01;
+// A pass gathers one-bit codes once this share of the registers has reached
+// its maximum, and goes back to four bits after a one-bit pass that left more
+// than kOpenShare of the (group, slice) pairs to the byte union.
+constexpr double kTopShare = 0.75;
+constexpr double kOpenShare = 0.4;
 
 
 // Hub threshold of the run-aware union (lookups per work item).
@@ -571,6 +605,7 @@ static int make_plan(const vga_graph *g, int p, const vga_tuning *tune, Plan *P)
     // rows of counters the union reads per slice: the slice, or in runs mode its table region
     const uint64_t rows_per_node = P->mode == kModeRuns ? (uint64_t)table_rows(P->scheme) : 1;
     int S = tune ? tune->slice_bytes : 0;
+    bool auto_S = S == 0;
     if (S != 0) {
         if (S < 16 || S > 1024 || (S & (S - 1)) || (uint32_t)S > P->node_bytes) {
             set_error("slice_bytes = %d must be a power of two in [16, min(register bytes per node, 1024)]", S);
@@ -582,6 +617,7 @@ static int make_plan(const vga_graph *g, int p, const vga_tuning *tune, Plan *P)
         const uint64_t l2_bytes = (uint64_t)(l2 > 0 ? l2 : (64 << 20));
         // a tabled width is an upper bound; the slice must still fit the whole L2
         const bool tabled_S = tabled && te.slice_bytes > 0 && !(tune && tune->l2_budget_mb > 0);
+        auto_S = !tabled_S;
         uint64_t budget = (tune && tune->l2_budget_mb > 0) ? (uint64_t)tune->l2_budget_mb << 20
                           : tabled_S                       ? l2_bytes
                           : P->mode == kModeRuns && P->group ? grouped_l2_budget(g->device)
@@ -628,7 +664,6 @@ static int make_plan(const vga_graph *g, int p, const vga_tuning *tune, Plan *P)
     P->off_c1 = o;    o = align256(o + 8 * P->n);
     P->off_sum = o;   o = align256(o + 8 * P->n);
     P->off_lc = o;    o = align256(o + 8 * ((uint64_t)P->m + 1));
-    P->off_flags = o; o = align256(o + 64);
     // the table region; pass 1's scatter keeps the nodes' keys there (mode 1 has
     // no table region otherwise)
     P->off_tab = o;
@@ -645,12 +680,31 @@ static int make_plan(const vga_graph *g, int p, const vga_tuning *tune, Plan *P)
         return VGA_EINVAL;
     }
     P->track = !track_ok || track == 1 ? 0 : track == 2 ? 2 : 1;
+    // Codes: the grouped union with an automatic slice width (an explicit or
+    // tuned width asks for byte slices of that width, forced tracking for the
+    // need masks of its own rule), at least 32 registers, whole 32-register
+    // units in a register slice, and one need bit per slice.
+    P->codes = P->mode == kModeRuns && P->group == kCodeNodes && auto_S && P->track != 2 && P->m >= 32 &&
+               P->slices <= kTrackMaxSlices && S >= (P->nib ? 16 : 32);
+    // flags, change bytes and need masks side by side, so that a pass clears
+    // what it uses of them at once
+    P->off_flags = o; o = align256(o + 64);
     if (P->track) {
         P->chg_bytes = align256((uint64_t)P->slices * P->n);
         P->off_chg = o;   o = align256(o + P->chg_bytes);
+    }
+    if (P->track || P->codes) {
         P->off_need = o;  o = align256(o + 4 * P->n);
+    }
+    if (P->track) {
         P->off_ortab = o;  // range-OR table (mode 2), or the per-node change masks (mode 1)
         o = align256(o + 4ull * (P->mode == kModeRuns ? table_rows(P->scheme) : 1) * P->n);
+    }
+    if (P->codes) {
+        P->off_win = o;  // gmax (u32 per register), then the window's top and low words
+        o = align256(o + 4ull * P->m + 2ull * P->node_bytes);
+        P->off_full = o;
+        o = align256(o + P->n);
     }
     P->total = o;
     return VGA_OK;
@@ -718,17 +772,20 @@ struct PendingTiming {
     int S, mode, rows;
     bool first;    // the first pass's scatter (hb_first_pass_kernel), not a union slice
     bool tracked;  // a union slice of a change-tracked pass (its work depends on the changes)
+    bool partial;  // the byte union of the pairs a code pass left open
 };
 
 template <int SS, bool NIB>
 static void launch_union_slice(const Plan &P, const vga_graph *g, const uint8_t *c, uint8_t *x, uint8_t *tab,
-                               uint32_t *flags, cudaStream_t stream, const uint32_t *need, int s, uint8_t *chg) {
+                               uint32_t *flags, cudaStream_t stream, const uint32_t *need, int s, int keep,
+                               uint8_t *chg) {
     const unsigned blocks = (unsigned)((P.n + P.warps - 1) / P.warps);
     const size_t smem = (size_t)P.warps * 32 * sizeof(uint32_t);
     if (P.mode == kModeRuns) {
         const unsigned item_blocks = (unsigned)((P.items.count + P.warps - 1) / P.warps);
         const unsigned table_blocks = (unsigned)((P.n + TableShape<SS>::B - 1) / TableShape<SS>::B);
-        hb_table_kernel<SS, NIB><<<table_blocks, 256, 0, stream>>>(c, tab, (uint32_t)P.n, P.scheme);
+        hb_table_kernel<SS, NIB><<<table_blocks, 256, 0, stream>>>(c, tab, (uint32_t)P.n, P.scheme,
+                                                                   keep ? nullptr : flags + 8, s);
         count_launch();
         if (!P.group) {
             hb_union_runs_kernel<SS, NIB><<<item_blocks, P.warps * 32, (size_t)P.warps * sizeof(LkStage), stream>>>(
@@ -748,7 +805,7 @@ static void launch_union_slice(const Plan &P, const vga_graph *g, const uint8_t 
                 if (smem > (48u << 10))
                     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
                 kernel<<<group_blocks, P.warps * 32, smem, stream>>>(P.groups.items, P.groups.count, P.groups.rows,
-                                                                     P.groups.cls, c, tab, x, flags, need, s, chg);
+                                                                     P.groups.cls, c, tab, x, flags, need, s, keep, chg);
             };
             if (group_blocks) {
                 if (P.group == 2) launch_groups(hb_union_groups_kernel<SS, NIB, 2>);
@@ -764,12 +821,17 @@ static void launch_union_slice(const Plan &P, const vga_graph *g, const uint8_t 
 }
 
 // One pass of the union over every slice.  need (a change-tracked pass) and
-// chg (change bytes to record, [slice][N]) may be null.
+// chg (change bytes to record, [slice][N]) may be null.  After a code pass
+// (left_open: the slices with open pairs, marked in need) only those slices
+// run, and pairs that need nothing are left alone.
 static int launch_union(const Plan &P, const vga_graph *g, const uint8_t *cur, uint8_t *nxt, uint8_t *tab,
                         uint32_t *flags, cudaStream_t stream, std::vector<PendingTiming> *timings,
-                        const uint32_t *need = nullptr, uint8_t *chg = nullptr) {
+                        const uint32_t *need = nullptr, uint8_t *chg = nullptr, const uint32_t *left_open = nullptr,
+                        bool tracked = false) {
     const uint64_t slice_bytes = (uint64_t)P.n * P.S;
+    const int keep = left_open ? 0 : 1;
     for (int s = 0; s < P.slices; s++) {
+        if (left_open && !((*left_open >> s) & 1u)) continue;
         const uint8_t *c = cur + (uint64_t)s * slice_bytes;
         uint8_t *x = nxt + (uint64_t)s * slice_bytes;
         uint8_t *cs = chg ? chg + (uint64_t)s * P.n : nullptr;
@@ -780,20 +842,20 @@ static int launch_union(const Plan &P, const vga_graph *g, const uint8_t *cur, u
             VGA_CHECK_CUDA(cudaEventRecord(pt.start, stream));
         }
         switch (P.S) {
-            case 16: P.nib ? launch_union_slice<16, true>(P, g, c, x, tab, flags, stream, need, s, cs)
-                             : launch_union_slice<16, false>(P, g, c, x, tab, flags, stream, need, s, cs); break;
-            case 32: P.nib ? launch_union_slice<32, true>(P, g, c, x, tab, flags, stream, need, s, cs)
-                             : launch_union_slice<32, false>(P, g, c, x, tab, flags, stream, need, s, cs); break;
-            case 64: P.nib ? launch_union_slice<64, true>(P, g, c, x, tab, flags, stream, need, s, cs)
-                             : launch_union_slice<64, false>(P, g, c, x, tab, flags, stream, need, s, cs); break;
-            case 128: P.nib ? launch_union_slice<128, true>(P, g, c, x, tab, flags, stream, need, s, cs)
-                             : launch_union_slice<128, false>(P, g, c, x, tab, flags, stream, need, s, cs); break;
-            case 256: P.nib ? launch_union_slice<256, true>(P, g, c, x, tab, flags, stream, need, s, cs)
-                             : launch_union_slice<256, false>(P, g, c, x, tab, flags, stream, need, s, cs); break;
-            case 512: P.nib ? launch_union_slice<512, true>(P, g, c, x, tab, flags, stream, need, s, cs)
-                             : launch_union_slice<512, false>(P, g, c, x, tab, flags, stream, need, s, cs); break;
-            case 1024: P.nib ? launch_union_slice<1024, true>(P, g, c, x, tab, flags, stream, need, s, cs)
-                             : launch_union_slice<1024, false>(P, g, c, x, tab, flags, stream, need, s, cs); break;
+            case 16: P.nib ? launch_union_slice<16, true>(P, g, c, x, tab, flags, stream, need, s, keep, cs)
+                             : launch_union_slice<16, false>(P, g, c, x, tab, flags, stream, need, s, keep, cs); break;
+            case 32: P.nib ? launch_union_slice<32, true>(P, g, c, x, tab, flags, stream, need, s, keep, cs)
+                             : launch_union_slice<32, false>(P, g, c, x, tab, flags, stream, need, s, keep, cs); break;
+            case 64: P.nib ? launch_union_slice<64, true>(P, g, c, x, tab, flags, stream, need, s, keep, cs)
+                             : launch_union_slice<64, false>(P, g, c, x, tab, flags, stream, need, s, keep, cs); break;
+            case 128: P.nib ? launch_union_slice<128, true>(P, g, c, x, tab, flags, stream, need, s, keep, cs)
+                             : launch_union_slice<128, false>(P, g, c, x, tab, flags, stream, need, s, keep, cs); break;
+            case 256: P.nib ? launch_union_slice<256, true>(P, g, c, x, tab, flags, stream, need, s, keep, cs)
+                             : launch_union_slice<256, false>(P, g, c, x, tab, flags, stream, need, s, keep, cs); break;
+            case 512: P.nib ? launch_union_slice<512, true>(P, g, c, x, tab, flags, stream, need, s, keep, cs)
+                             : launch_union_slice<512, false>(P, g, c, x, tab, flags, stream, need, s, keep, cs); break;
+            case 1024: P.nib ? launch_union_slice<1024, true>(P, g, c, x, tab, flags, stream, need, s, keep, cs)
+                             : launch_union_slice<1024, false>(P, g, c, x, tab, flags, stream, need, s, keep, cs); break;
             default:
                 set_error("internal: slice width %d", P.S);
                 return VGA_EINVAL;
@@ -816,11 +878,71 @@ static int launch_union(const Plan &P, const vga_graph *g, const uint8_t *cur, u
             pt.S = P.S;
             pt.mode = P.mode;
             pt.rows = P.mode == kModeRuns ? table_rows(P.scheme) : 1;
-            pt.tracked = need != nullptr;
+            pt.tracked = left_open ? tracked : need != nullptr;
+            pt.partial = left_open != nullptr;
             timings->push_back(pt);
         }
     }
     VGA_CHECK_CUDA(cudaGetLastError());
+    return VGA_OK;
+}
+
+// One pass of the union over register codes of K bits, then over the bytes of
+// the pairs it left open.
+static int launch_codes(const Plan &P, const vga_graph *g, int K, uint8_t *base, const uint8_t *cur, uint8_t *nxt,
+                        uint32_t *flags, cudaStream_t stream, std::vector<PendingTiming> *timings, bool tracked,
+                        uint8_t *chg) {
+    CodePass C;
+    C.groups = &P.groups;
+    C.cur = cur;
+    C.nxt = nxt;
+    C.tab = base + P.off_tab;
+    C.n = (uint32_t)P.n;
+    C.s_log2 = __builtin_ctz((unsigned)P.S);
+    C.scheme = P.scheme;
+    C.warps = std::min(P.warps, 4);
+    C.nib = P.nib != 0;
+    C.K = K;
+    const int node_codes = (int)(P.m * (uint32_t)K / 8u);
+    C.S = std::min(P.S, node_codes);
+    const uint32_t *gmax = reinterpret_cast<const uint32_t *>(base + P.off_win);
+    C.top = gmax + P.m;
+    C.low = C.top + P.node_bytes / 4;
+    C.flags = flags;
+    C.full = base + P.off_full;
+    C.need = reinterpret_cast<uint32_t *>(base + P.off_need);
+    C.chg = chg;
+    C.stream = stream;
+    for (int s = 0; s < node_codes / C.S; s++) {
+        PendingTiming pt{};
+        if (timings) {
+            VGA_CHECK_CUDA(cudaEventCreate(&pt.start));
+            VGA_CHECK_CUDA(cudaEventCreate(&pt.stop));
+            VGA_CHECK_CUDA(cudaEventRecord(pt.start, stream));
+        }
+        VGA_TRY(launch_code_slice(C, s));
+        if (timings) {
+            VGA_CHECK_CUDA(cudaEventRecord(pt.stop, stream));
+            pt.edges = g->n_edges;
+            pt.gather_bytes = P.groups.rows_used * (uint64_t)C.S;
+            pt.hbm_bytes = 4 * P.groups.rows_used + 64 * P.groups.count +
+                           2 * P.n * (uint64_t)P.node_bytes * C.S / node_codes;
+            pt.S = C.S;
+            pt.mode = P.mode;
+            pt.rows = table_rows(P.scheme);
+            pt.tracked = tracked;
+            timings->push_back(pt);
+        }
+    }
+    // the byte union of the slices with open pairs: asked for with a wait when
+    // there are many slices, else launched for all (the kernels then return at
+    // once; a wait costs about 12 us, an idle pair of launches 4)
+    uint32_t open = P.slices >= 32 ? 0xffffffffu : (1u << P.slices) - 1u;
+    if (P.slices > 2) {
+        VGA_CHECK_CUDA(cudaMemcpyAsync(&open, flags + 8, 4, cudaMemcpyDeviceToHost, stream));
+        VGA_CHECK_CUDA(cudaStreamSynchronize(stream));
+    }
+    if (open) VGA_TRY(launch_union(P, g, cur, nxt, C.tab, flags, stream, timings, C.need, chg, &open, tracked));
     return VGA_OK;
 }
 
@@ -957,6 +1079,8 @@ static void settle_timings(std::vector<PendingTiming> &timings, bool to_profile,
         } else if (to_profile && ok && pt.tracked) {
             ps.acc.tracked_launches++;
             ps.acc.tracked_ms += ms;
+        } else if (to_profile && ok && pt.partial) {
+            ps.acc.union_ms += ms;
         } else if (to_profile && ok) {
             ps.acc.union_launches++;
             ps.acc.union_ms += ms;
@@ -974,12 +1098,13 @@ static void settle_timings(std::vector<PendingTiming> &timings, bool to_profile,
 }
 
 static int launch_estimate(const Plan &P, const uint8_t *regs, int t, const double *lc, const double *c_prev,
-                           double *c_cur, double *sum_d, uint32_t *flags, cudaStream_t stream) {
+                           double *c_cur, double *sum_d, uint32_t *flags, cudaStream_t stream,
+                           const uint32_t *top = nullptr, uint8_t *full = nullptr) {
     const int warps = 8;
     const unsigned blocks = (unsigned)((P.n + warps - 1) / warps);
     const double alpha_mm = hll_alpha_host(P.p) * (double)P.m * (double)P.m;
     hb_estimate_kernel<<<blocks, warps * 32, 0, stream>>>(regs, (uint32_t)P.n, P.p, P.S, t, alpha_mm, lc, c_prev,
-                                                          c_cur, sum_d, flags, P.nib);
+                                                          c_cur, sum_d, flags, P.nib, top, full);
     count_launch();
     VGA_CHECK_CUDA(cudaGetLastError());
     return VGA_OK;
@@ -1052,6 +1177,7 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
         P.hub = hub_threshold(g, P.scheme, P.hub_req);
         VGA_TRY(ensure_run_items(g, P.scheme, P.hub, stream, &P.items));
         if (P.group) VGA_TRY(ensure_group_list(g, P.scheme, P.hub, P.group, stream, &P.groups));
+        if (P.items.hubs) P.codes = false;  // split hubs merge bytes
     }
 
     bool profiling;
@@ -1075,17 +1201,23 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
         VGA_CHECK_CUDA(cudaMemsetAsync(cur, 0, P.n * P.node_bytes, stream));
         // split hubs merge into next[v] by atomic max: it must start below the result
         if (P.items.hubs) VGA_CHECK_CUDA(cudaMemsetAsync(nxt, 0, P.n * P.node_bytes, stream));
-        VGA_CHECK_CUDA(cudaMemsetAsync(sum_d, 0, 8 * P.n, stream));
         void *keys = P.first_scatter ? tab : nullptr;  // tab is unused in pass 1
+        uint32_t *gmax = P.codes ? reinterpret_cast<uint32_t *>(base + P.off_win) : nullptr;
+        uint32_t *top = P.codes ? gmax + P.m : nullptr;
+        uint8_t *full = P.codes ? base + P.off_full : nullptr;
+        if (gmax) VGA_CHECK_CUDA(cudaMemsetAsync(gmax, 0, 4ull * P.m, stream));
         hb_init_kernel<<<(unsigned)((P.n + 255) / 256), 256, 0, stream>>>(cur, (uint32_t)P.n, p, P.S, seed, P.nib, 0u,
-                                                                          (uint32_t)P.slices, keys);
+                                                                          (uint32_t)P.slices, keys, gmax);
         count_launch();
         VGA_CHECK_CUDA(cudaGetLastError());
+        if (gmax) VGA_TRY(launch_code_window(gmax, P.node_bytes / 4, P.nib, top, top + P.node_bytes / 4, stream));
         VGA_TRY(launch_estimate(P, cur, 0, lc, nullptr, c_prev, sum_d, flags, stream));  // c_0
         if (max_trace >= 0) VGA_TRY(copy_trace(P, cur, c_prev, 0, trace_regs, trace_c, stream));
         struct {
             uint32_t f[4];        // changed, estimate increase, bounded wait gave up, unused
             uint64_t n_changed;   // (node, slice) pairs changed by the pass (change tracking)
+            uint64_t n_top;       // registers at the window's top (codes)
+            uint32_t open[2];     // slices with pairs a code pass left open, and their number
         } h{};
         VGA_CHECK_CUDA(cudaMemsetAsync(flags, 0, sizeof(h), stream));
         L2Window window;
@@ -1100,23 +1232,32 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
         uint32_t *need = P.track ? reinterpret_cast<uint32_t *>(base + P.off_need) : nullptr;
         uint32_t *ortab = P.track ? reinterpret_cast<uint32_t *>(base + P.off_ortab) : nullptr;
         uint64_t changed_prev = ~0ull;
+        bool too_open = false;  // the last one-bit pass left too many pairs open
         for (t = 1;; t++) {
-            VGA_CHECK_CUDA(cudaMemsetAsync(flags, 0, 8, stream));
             const bool tracked = chg && t >= 2 &&
                                  (P.track == 2 || (double)changed_prev < kTrackBelow * (double)P.n * P.slices);
-            if (tracked) VGA_TRY(launch_need(P, g, chg, ortab, need, stream, timed ? &timings : nullptr));
-            if (chg) {
-                VGA_CHECK_CUDA(cudaMemsetAsync(chg, 0, P.chg_bytes, stream));
-                VGA_CHECK_CUDA(cudaMemsetAsync(flags + 4, 0, 8, stream));
+            // Codes, from the second pass on: one bit a register once most have
+            // reached G, else four (or, after a pass that changed little, the
+            // change-tracked byte union, which then has less to recompute).
+            int K = 0;
+            if (P.codes && t >= 2) {
+                const bool most = (double)h.n_top >= kTopShare * (double)P.n * P.m;
+                K = most && !too_open && P.m >= 128 ? 1 : tracked ? 0 : 4;
             }
-            if (t == 1 && keys)
+            if (tracked && !K) VGA_TRY(launch_need(P, g, chg, ortab, need, stream, timed ? &timings : nullptr));
+            const uint64_t clear = K ? P.off_need + 4 * P.n - P.off_flags
+                                     : chg ? P.off_chg + P.chg_bytes - P.off_flags : sizeof(h);
+            VGA_CHECK_CUDA(cudaMemsetAsync(flags, 0, clear, stream));
+            if (K) {
+                VGA_TRY(launch_codes(P, g, K, base, cur, nxt, flags, stream, timed ? &timings : nullptr, tracked, chg));
+            } else if (t == 1 && keys)
                 VGA_TRY(launch_first_pass(P, g, keys, nxt, 0u, (uint32_t)P.slices, flags, stream,
                                           timed ? &timings : nullptr, chg));
             else
                 VGA_TRY(launch_union(P, g, cur, nxt, tab, flags, stream, timed ? &timings : nullptr,
                                      tracked ? need : nullptr, chg));
             if (chg) VGA_TRY(launch_count(P, chg, flags, stream));
-            VGA_TRY(launch_estimate(P, nxt, t, lc, c_prev, c_cur, sum_d, flags, stream));
+            VGA_TRY(launch_estimate(P, nxt, t, lc, c_prev, c_cur, sum_d, flags, stream, top, full));
             if (t <= max_trace) VGA_TRY(copy_trace(P, nxt, c_cur, t, trace_regs, trace_c, stream));
             VGA_CHECK_CUDA(cudaMemcpyAsync(&h, flags, sizeof(h), cudaMemcpyDeviceToHost, stream));
             VGA_CHECK_CUDA(cudaStreamSynchronize(stream));
@@ -1125,6 +1266,7 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
                 return VGA_ETIMEOUT;
             }
             changed_prev = h.n_changed;
+            if (K == 1) too_open = (double)h.open[1] > kOpenShare * (double)P.groups.count * P.slices;
             std::swap(cur, nxt);
             std::swap(c_prev, c_cur);
             const bool stop = (conv_mode == 1) ? (h.f[1] == 0) : (h.f[0] == 0);

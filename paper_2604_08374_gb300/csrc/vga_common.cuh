@@ -232,6 +232,28 @@ struct GroupList {
 int ensure_group_list(const vga_graph *g, int scheme, uint32_t hub_lookups, int nodes, cudaStream_t stream,
                       GroupList *out);
 
+// One pass of the grouped union over register codes (codes.cu): table and
+// union of one code slice of S bytes a node at a time.
+constexpr int kCodeNodes = 4;  // nodes per group of the code kernels
+struct CodePass {
+    const GroupList *groups = nullptr;
+    const uint8_t *cur = nullptr;      // the node's registers, slice-major with slices of 2^s_log2 bytes
+    uint8_t *nxt = nullptr, *tab = nullptr;
+    uint32_t n = 0;
+    int s_log2 = 0, scheme = 0, warps = 4;
+    bool nib = false;
+    int K = 4, S = 16;                 // bits per code, bytes of a code slice's row
+    const uint32_t *top = nullptr, *low = nullptr;  // the window, in register words
+    uint32_t *flags = nullptr;
+    const uint8_t *full = nullptr;     // K = 1: nodes whose registers all equal G, or nullptr
+    uint32_t *need = nullptr;          // (node, slice) pairs left open, one bit per register slice
+    uint8_t *chg = nullptr;            // change bytes, or nullptr
+    cudaStream_t stream = nullptr;
+};
+int launch_code_slice(const CodePass &C, int slice);
+int launch_code_window(const uint32_t *gmax, uint32_t words, int nib, uint32_t *top, uint32_t *low,
+                       cudaStream_t stream);
+
 // Automatic hub threshold (lookups per work item): half of one warp's even
 // share of a slice's lookups when every SM holds 64 warps, and at least 2048,
 // so only nodes that would outlast the rest of a launch are split.  The

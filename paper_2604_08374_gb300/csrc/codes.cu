@@ -1,6 +1,8 @@
 // codes.cu -- the grouped union over register codes (codes.cuh): per code
 // slice, the table of range maxima packed straight from the registers, then
 // one warp per group gathering the group's distinct rows.
+#include <algorithm>
+
 #include "codes.cuh"
 
 namespace vga {
@@ -14,30 +16,39 @@ __global__ void __launch_bounds__(256) hb_code_table_kernel(const uint8_t *__res
     code_table_item<S, K, NIB>(cur, tab, n, s_log2, c0, blockIdx.x * (uint32_t)TableShape<S>::B, buf, scheme, win);
 }
 
-// One warp per group of kCodeNodes nodes: the code maxima of its nodes over
-// one code slice (code_group), then next[v] for the slice's registers
-// (code_store), all lanes on the group's (node, unit) pairs.  A group whose
-// nodes have all their registers at G (full[v], K = 1) has nothing to gather.
-// Open pairs go to the need masks; flags: [0] a register changed, [2] a
-// bounded wait ran out, [8] slices with open pairs, [9] open (group, slice)
-// pairs.
+// The code union of one slice: `split` warps per group of kCodeNodes nodes
+// (CTAs of `split` warps, or of several one-warp groups) gather the code
+// maxima of its nodes (code_group), then all their lanes settle next[v] for
+// the slice's registers, unit by unit (code_store).  A group whose nodes have
+// all their registers at G (full[v], K = 1) has nothing to gather.  Open
+// 16-byte register pieces go to the list (the first list_cap of them) and, by
+// register slice, to the need masks; flags: [0] a register changed, [2] a
+// bounded wait ran out, [8] slices with open pieces, [9] open pieces.
+// Bound: the L2 bytes of the rows (K = 1: 2.8 ms a city launch, 18 TB/s) and
+// the ALU pipe (K = 4: 3.1 ms, 8 logic operations a 16-byte unit).  One warp
+// per group until the groups fill the GPU twice; below that several, which
+// took 42,680 cells from 2.19 to 1.85 ms and 4,997 cells at p = 12 from 0.86 to
+// 0.74 ms an analysis.  56 registers: measured 25.4 ms on the city against 25.9
+// (40 or 64) and 27.7 (48).
 template <int S, int K, bool NIB>
-__global__ void __launch_bounds__(128) hb_code_groups_kernel(
+__global__ void __maxnreg__(56) hb_code_groups_kernel(
     const GroupItem *__restrict__ items, uint64_t n_items, const uint32_t *__restrict__ rows,
     const uint2 *__restrict__ cls, const uint8_t *__restrict__ cur, const uint8_t *__restrict__ tab,
     uint8_t *__restrict__ nxt, uint32_t n, int s_log2, uint32_t c0, CodeWindow win, uint32_t *__restrict__ flags,
-    const uint8_t *__restrict__ full, uint32_t *__restrict__ need, uint8_t *__restrict__ chg) {
+    const uint8_t *__restrict__ full, uint32_t *__restrict__ need, uint8_t *__restrict__ chg,
+    uint2 *__restrict__ list, uint32_t list_cap, uint32_t split, uint32_t len) {
     constexpr int W16 = S / 16;
     constexpr int UNIT_BYTES = kUnitRegs<K> / (NIB ? 2 : 1);
     extern __shared__ __align__(128) unsigned char s_dyn[];
-    const int nw = blockDim.x >> 5;
+    const uint32_t nw = blockDim.x >> 5;
     const int lane = threadIdx.x & 31;
-    const int wib = threadIdx.x >> 5;
+    const uint32_t wib = threadIdx.x >> 5;
     LkStage &st = reinterpret_cast<LkStage *>(s_dyn)[wib];
-    uint4 *part = reinterpret_cast<uint4 *>(s_dyn + (size_t)nw * sizeof(LkStage)) + (size_t)wib * kCodeNodes * W16;
-    const uint64_t warp = (uint64_t)blockIdx.x * nw + wib;
-    if (warp >= n_items) return;
-    const GroupItem &gi = items[warp];
+    uint4 *parts = reinterpret_cast<uint4 *>(s_dyn + (size_t)nw * sizeof(LkStage));
+    uint4 *part = parts + (size_t)wib * kCodeNodes * W16;
+    const uint64_t item = split > 1u ? blockIdx.x : (uint64_t)blockIdx.x * nw + wib;
+    if (item >= n_items) return;  // whole CTAs only when split > 1
+    const GroupItem &gi = items[item];
     for (int q = lane; q < kCodeNodes * W16; q += 32) part[q] = make_uint4(0, 0, 0, 0);
     bool gather = true;
     if (K == 1 && full) {
@@ -52,18 +63,25 @@ __global__ void __launch_bounds__(128) hb_code_groups_kernel(
     __syncwarp();
     if (gather) {
         lk_stage_init(st, lane);
-        uint32_t phase = 0;
-        code_group<S, K, kCodeNodes>(gi, rows, cls, tab, part, st, phase, lane, reinterpret_cast<int *>(flags + 2));
-        __syncwarp();
+        code_group<S, K, kCodeNodes>(gi, rows, cls, tab, part, st, lane, reinterpret_cast<int *>(flags + 2),
+                                     split > 1u ? wib : 0u, split, len);
     }
+    if (split > 1u) __syncthreads();
+    else __syncwarp();
     bool changed = false;
     uint32_t open_slices = 0;
-    for (int q = lane; q < kCodeNodes * W16; q += 32) {
+    const uint32_t q0 = split > 1u ? threadIdx.x : lane, dq = split > 1u ? blockDim.x : 32u;
+    for (uint32_t q = q0; q < (uint32_t)kCodeNodes * W16; q += dq) {
         const uint32_t v = gi.node[q / W16];
         if (v == 0xffffffffu) continue;
-        const uint32_t u = c0 + (uint32_t)(q % W16);
+        const uint32_t u = c0 + q % W16;
+        uint4 code = part[q];
+        if (split > 1u) {
+            code = parts[q];
+            for (uint32_t w = 1; w < split; w++) code = code_max<K>(code, parts[(size_t)w * kCodeNodes * W16 + q]);
+        }
         uint32_t chg16, open16;
-        code_store<K, NIB>(part[q], cur, nxt, n, s_log2, v, u, win, chg16, open16);
+        code_store<K, NIB>(code, cur, nxt, n, s_log2, v, u, win, chg16, open16);
         changed |= chg16 != 0u;
         uint32_t mine = 0;
 #pragma unroll
@@ -72,17 +90,78 @@ __global__ void __launch_bounds__(128) hb_code_groups_kernel(
             if (chg && ((chg16 >> h) & 1u)) chg[(uint64_t)s * n + v] = 1u;
             mine |= ((open16 >> h) & 1u) << s;
         }
-        if (mine) atomicOr(need + v, mine);
+        if (mine) {
+            atomicOr(need + v, mine);
+            uint32_t at = atomicAdd(flags + 9, (uint32_t)__popc(open16));
+            for (uint32_t b = open16; b && at < list_cap; b &= b - 1u)
+                list[at++] = make_uint2(v, u * (UNIT_BYTES / 16) + (uint32_t)__ffs(b) - 1u);
+        }
         open_slices |= mine;
     }
     if (__any_sync(0xffffffffu, changed) && lane == 0) {
         if (*reinterpret_cast<volatile uint32_t *>(flags) == 0u) atomicOr(flags, 1u);
     }
     open_slices = __reduce_or_sync(0xffffffffu, open_slices);
-    if (open_slices && lane == 0) {
-        if ((*reinterpret_cast<volatile uint32_t *>(flags + 8) & open_slices) != open_slices)
-            atomicOr(flags + 8, open_slices);
-        atomicAdd(flags + 9, (uint32_t)__popc(open_slices));
+    if (open_slices && lane == 0 &&
+        (*reinterpret_cast<volatile uint32_t *>(flags + 8) & open_slices) != open_slices)
+        atomicOr(flags + 8, open_slices);
+}
+
+// The open pieces of a pass (node, 16-byte register piece), when there are at
+// most list_cap: one CTA per piece takes the maximum over the node's
+// neighbours straight from their registers, a thread per range lookup.
+// Reading deg(v) pieces costs a 32-byte sector each, far more per register
+// than the table's rows, but a handful of open pieces in every slice would
+// otherwise cost each slice a table and the whole walk of their groups'
+// rows by single warps (city pass 3: 2.4 ms for 0.28 % of the pairs, now 0.1).
+template <bool NIB>
+__global__ void __launch_bounds__(256) hb_code_open_kernel(const uint2 *__restrict__ list, uint32_t list_cap,
+                                                           const uint64_t *__restrict__ lk_off,
+                                                           const uint32_t *__restrict__ lk,
+                                                           const uint8_t *__restrict__ cur, uint8_t *__restrict__ nxt,
+                                                           uint32_t n, int s_log2, int scheme,
+                                                           uint32_t *__restrict__ flags, uint8_t *__restrict__ chg) {
+    __shared__ uint4 s_max[8];
+    const uint32_t count = flags[9];
+    if (count > list_cap) return;
+    const int rows = table_rows(scheme);
+    for (uint32_t e = blockIdx.x; e < count; e += gridDim.x) {
+        const uint32_t v = list[e].x, byte = 16u * list[e].y;
+        const uint8_t *base = cur + ((uint64_t)(byte >> s_log2) * n << s_log2) + (byte & ((1u << s_log2) - 1u));
+        uint4 acc = make_uint4(0, 0, 0, 0);
+        const uint64_t e1 = lk_off[v + 1];
+        for (uint64_t k = lk_off[v] + threadIdx.x; k < e1; k += blockDim.x) {
+            const uint32_t r = __ldg(lk + k);
+            uint32_t slot = 0;
+            for (int s = 1; s < rows; s++) slot += r >= (uint32_t)s * n ? 1u : 0u;
+            const uint32_t i = r - slot * n, w = 1u << (scheme == 0 ? slot : 2u * slot);
+#pragma unroll 4
+            for (uint32_t j = 0; j < w; j++)
+                acc = RegFmt<NIB>::max4(acc, __ldg(reinterpret_cast<const uint4 *>(base + ((uint64_t)(i + j) << s_log2))));
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            uint4 y;
+            y.x = __shfl_xor_sync(0xffffffffu, acc.x, o);
+            y.y = __shfl_xor_sync(0xffffffffu, acc.y, o);
+            y.z = __shfl_xor_sync(0xffffffffu, acc.z, o);
+            y.w = __shfl_xor_sync(0xffffffffu, acc.w, o);
+            acc = RegFmt<NIB>::max4(acc, y);
+        }
+        if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = acc;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < 8; w++) acc = RegFmt<NIB>::max4(acc, s_max[w]);
+            const uint64_t at = reg_at(n, s_log2, v, byte);
+            const uint4 own = *reinterpret_cast<const uint4 *>(cur + at);
+            acc = RegFmt<NIB>::max4(acc, own);
+            *reinterpret_cast<uint4 *>(nxt + at) = acc;
+            if ((acc.x ^ own.x) | (acc.y ^ own.y) | (acc.z ^ own.z) | (acc.w ^ own.w)) {
+                if (*reinterpret_cast<volatile uint32_t *>(flags) == 0u) atomicOr(flags, 1u);
+                if (chg) chg[(uint64_t)(byte >> s_log2) * n + v] = 1u;
+            }
+        }
+        __syncthreads();
     }
 }
 
@@ -110,13 +189,13 @@ int launch_slice(const CodePass &C, int slice) {
     const unsigned table_blocks = (unsigned)(((uint64_t)C.n + TableShape<S>::B - 1) / TableShape<S>::B);
     hb_code_table_kernel<S, K, NIB><<<table_blocks, 256, 0, C.stream>>>(C.cur, C.tab, C.n, C.s_log2, c0, C.scheme, win);
     count_launch();
-    const size_t smem = (size_t)C.warps * (sizeof(LkStage) + (size_t)kCodeNodes * S);
-    auto kernel = hb_code_groups_kernel<S, K, NIB>;
-    const unsigned blocks = (unsigned)((C.groups->count + C.warps - 1) / C.warps);
+    const int warps = C.split > 1 ? C.split : C.warps;
+    const size_t smem = (size_t)warps * (sizeof(LkStage) + (size_t)kCodeNodes * S);
+    const unsigned blocks = (unsigned)(C.split > 1 ? C.groups->count : (C.groups->count + warps - 1) / warps);
     if (blocks) {
-        kernel<<<blocks, C.warps * 32, smem, C.stream>>>(C.groups->items, C.groups->count, C.groups->rows,
-                                                         C.groups->cls, C.cur, C.tab, C.nxt, C.n, C.s_log2, c0, win,
-                                                         C.flags, C.full, C.need, C.chg);
+        hb_code_groups_kernel<S, K, NIB><<<blocks, warps * 32, smem, C.stream>>>(
+            C.groups->items, C.groups->count, C.groups->rows, C.groups->cls, C.cur, C.tab, C.nxt, C.n, C.s_log2, c0,
+            win, C.flags, C.full, C.need, C.chg, C.list, C.list_cap, (uint32_t)C.split, (uint32_t)C.len);
         count_launch();
     }
     VGA_CHECK_CUDA(cudaGetLastError());
@@ -136,6 +215,19 @@ int launch_code_slice(const CodePass &C, int slice) {
     }
     set_error("internal: code slice width %d", C.S);
     return VGA_EINVAL;
+}
+
+int launch_code_open(const CodePass &C, const uint64_t *lk_off, const uint32_t *lk, int sms) {
+    const unsigned blocks = (unsigned)std::min<uint32_t>(std::max<uint32_t>(C.list_cap, 1u), (uint32_t)sms * 8u);
+    if (C.nib)
+        hb_code_open_kernel<true><<<blocks, 256, 0, C.stream>>>(C.list, C.list_cap, lk_off, lk, C.cur, C.nxt, C.n,
+                                                               C.s_log2, C.scheme, C.flags, C.chg);
+    else
+        hb_code_open_kernel<false><<<blocks, 256, 0, C.stream>>>(C.list, C.list_cap, lk_off, lk, C.cur, C.nxt, C.n,
+                                                                C.s_log2, C.scheme, C.flags, C.chg);
+    count_launch();
+    VGA_CHECK_CUDA(cudaGetLastError());
+    return VGA_OK;
 }
 
 int launch_code_window(const uint32_t *gmax, uint32_t words, int nib, uint32_t *top, uint32_t *low,

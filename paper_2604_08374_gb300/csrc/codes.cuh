@@ -18,9 +18,9 @@
 // pass 3 all but 1e-5 of the city's.
 //
 // Measured (GB300): the city graph's pass 2 takes four launches of 128-byte
-// K = 4 rows at 3.6 ms and pass 3 one of K = 1 rows at 2.8 ms, where the byte
-// union takes eight at 2.8 ms each; the d = 3 analysis 54.8 -> 29.7 ms, the
-// unlimited p = 12 one 342 -> 116 ms, medium d = 3 3.2 -> 2.2 ms.
+// K = 4 rows at 3.1 ms and pass 3 one of K = 1 rows at 2.8 ms, where the byte
+// union takes eight at 2.8 ms each; the d = 3 analysis 54.8 -> 25.4 ms, the
+// unlimited one 85.8 -> 27.0 ms, medium d = 3 3.2 -> 1.85 ms.
 //
 // Layout: a 16-byte unit holds 32 registers as four bit planes (K = 4; word k =
 // bit k of the codes, bit i = register i) or 128 registers as one plane
@@ -225,57 +225,83 @@ __device__ __forceinline__ void code_finish(uint4 (&acc)[LeanShape<S>::V4]) {
         }
 }
 
-// The code maxima of one group's nodes (union_group's walk over its distinct
-// rows, class by class) into part[NODES][S / 16].
+// One warp's share of the code maxima of a group's nodes, into part[NODES][S /
+// 16]: the group's distinct rows in pieces of `len` entries (a multiple of 4,
+// at most kLkChunk) through the warp's TMA stage, this warp taking pieces w, w
+// + split, ...  Within a piece the rows of a class fold into one accumulator,
+// merged into the class's nodes when the class or the piece ends.
 template <int S, int K, int NODES>
 __device__ __forceinline__ void code_group(const GroupItem &gi, const uint32_t *__restrict__ rows,
                                            const uint2 *__restrict__ cls, const uint8_t *__restrict__ tab, uint4 *part,
-                                           LkStage &st, uint32_t &phase, int lane, int *err) {
+                                           LkStage &st, int lane, int *err, uint32_t w, uint32_t split,
+                                           uint32_t len) {
     using Sh = LeanShape<S>;
     constexpr int W16 = S / 16;
-    const uint32_t cnt = gi.cnt, nc = gi.nc;
-    const uint64_t cls0 = gi.cls;
+    const uint32_t cnt = gi.cnt;
+    const uint32_t pieces = (cnt + len - 1) / len;
+    if (w >= pieces) return;
+    const uint32_t *src = rows + gi.b;  // 16-byte aligned; readable up to a multiple of 4 entries
+    auto load = [&](uint32_t k) {
+        const uint32_t s0 = (w + k * split) * len;
+        if (s0 < cnt) lk_bulk_load(st, (int)(k & 1u), src + s0, ((min(cnt - s0, len) + 3u) & ~3u) * 4u);
+    };
+    if (lane == 0) {
+        load(0);
+        load(1);
+    }
     uint4 acc[Sh::V4] = {};
     const int g = lane / Sh::G, sub = lane % Sh::G;
     const uint8_t *base = tab + sub * Sh::CH;
-    if (cnt == 0) return;
-    uint32_t ci = 0;
-    uint2 cd = cls[cls0];
-    uint32_t cend = cd.y;
-    const StageStream ss(rows, gi.b, gi.b + cnt);
-    ss.start(st, lane);
-    for (uint32_t c = 0; c < ss.chunks; c++) {
-        const uint32_t *buf = ss.acquire(st, c, phase, err, lane);
-        const uint32_t s0 = c * kLkChunk;
+    const uint2 *cp = cls + gi.cls;
+    uint2 cd = *cp;         // {node mask, rows} of the current class
+    uint32_t cend = cd.y;   // group entry where the current class ends
+    uint32_t phase = 0;
+    auto merge = [&]() {
+        code_finish<S, K>(acc);
+        if (g == 0) {
+#pragma unroll
+            for (int j = 0; j < NODES; j++)
+                if ((cd.x >> j) & 1u)
+#pragma unroll
+                    for (int q = 0; q < Sh::V4; q++) {
+                        uint4 &pp = part[j * W16 + sub * Sh::V4 + q];
+                        pp = code_max<K>(pp, acc[q]);
+                    }
+        }
+#pragma unroll
+        for (int q = 0; q < Sh::V4; q++) acc[q] = make_uint4(0, 0, 0, 0);
+    };
+    for (uint32_t k = 0;; k++) {
+        const uint32_t s0 = (w + k * split) * len;
+        if (s0 >= cnt) break;
+        const int slot = (int)(k & 1u);
+        if (!__all_sync(0xffffffffu, lk_wait(st, slot, (phase >> slot) & 1u))) {
+            if (lane == 0) atomicExch(err, 1);
+            lk_wait(st, slot, (phase >> slot) & 1u);  // give an in-flight copy a last chance
+        }
+        phase ^= 1u << slot;
+        const uint32_t *buf = st.buf[slot];
         uint32_t lo = s0;
-        const uint32_t hi = min(cnt, s0 + (uint32_t)kLkChunk);
-        while (lo < hi) {  // warp-uniform: split the chunk at class ends
+        const uint32_t hi = min(cnt, s0 + len);
+        while (cend <= lo) {  // the piece starts in a later class
+            cd = *++cp;
+            cend += cd.y;
+        }
+        while (lo < hi) {  // warp-uniform: split the piece at class ends
             const uint32_t seg = min(hi, cend);
-            if (seg > lo) code_fold<S, K>(base, buf, (int)(lo - s0), (int)(seg - s0), g, acc);
+            code_fold<S, K>(base, buf, (int)(lo - s0), (int)(seg - s0), g, acc);
             lo = seg;
-            if (lo == cend) {  // the class is complete
-                code_finish<S, K>(acc);
-                if (g == 0) {
-#pragma unroll
-                    for (int j = 0; j < NODES; j++)
-                        if ((cd.x >> j) & 1u)
-#pragma unroll
-                            for (int q = 0; q < Sh::V4; q++) {
-                                uint4 &pp = part[j * W16 + sub * Sh::V4 + q];
-                                pp = code_max<K>(pp, acc[q]);
-                            }
-                }
-#pragma unroll
-                for (int q = 0; q < Sh::V4; q++) acc[q] = make_uint4(0, 0, 0, 0);
-                if (++ci < nc) {
-                    cd = cls[cls0 + ci];
+            if (lo == cend) {
+                merge();
+                if (lo < cnt) {
+                    cd = *++cp;
                     cend += cd.y;
-                } else {
-                    cend = 0xffffffffu;
                 }
             }
         }
-        ss.release(st, c, lane);
+        if (split > 1u && hi < cend) merge();  // the class goes on in another warp's piece
+        __syncwarp();
+        if (lane == 0) load(k + 2u);
     }
 }
 

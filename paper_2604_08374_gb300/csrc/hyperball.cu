@@ -179,16 +179,16 @@ __global__ void __maxnreg__(VGA_UNION_MAXNREG) hb_union_runs_kernel(
 // with its own registers and stored (lean_store).  The maximum over each
 // node's rows is that over its own lookup list, so the registers equal those
 // of hb_union_runs_kernel bit for bit.  With need given, a group none of whose
-// nodes needs slice `s` keeps its registers (keep != 0) or is left alone (its
-// next[] was settled by a code pass); otherwise all its nodes are recomputed
-// (a node that needed nothing gets its registers again).
+// nodes needs slice `s` keeps its registers, or (list_cap >= 0, after a code
+// pass) is left alone; otherwise all its nodes are recomputed (a node that
+// needed nothing gets its registers again).
 // Shared memory per warp: an LkStage, then NODES rows of S bytes.
 template <int S, bool NIB, int NODES>
 __global__ void __maxnreg__(VGA_UNION_MAXNREG) hb_union_groups_kernel(
     const GroupItem *__restrict__ items, uint64_t n_items, const uint32_t *__restrict__ rows,
     const uint2 *__restrict__ cls, const uint8_t *__restrict__ cur, const uint8_t *__restrict__ tab,
-    uint8_t *__restrict__ nxt, uint32_t *__restrict__ flags, const uint32_t *__restrict__ need, int s, int keep,
-    uint8_t *__restrict__ chg) {
+    uint8_t *__restrict__ nxt, uint32_t *__restrict__ flags, const uint32_t *__restrict__ need, int s,
+    int64_t list_cap, uint8_t *__restrict__ chg) {
     constexpr int W16 = S / 16;  // uint4 words of a slice row
     extern __shared__ __align__(128) unsigned char s_dyn[];
     const int nw = blockDim.x >> 5;
@@ -200,6 +200,7 @@ __global__ void __maxnreg__(VGA_UNION_MAXNREG) hb_union_groups_kernel(
     if (warp >= n_items) return;
     const GroupItem &gi = items[warp];  // node ids are read again where needed, not held in registers
     int *err = reinterpret_cast<int *>(flags + 2);
+    if (list_cap >= 0 && flags[9] <= (uint64_t)list_cap) return;
     if (need) {
         bool any = false;
 #pragma unroll
@@ -208,7 +209,7 @@ __global__ void __maxnreg__(VGA_UNION_MAXNREG) hb_union_groups_kernel(
             any |= v != 0xffffffffu && ((need[v] >> s) & 1u);
         }
         if (!any) {
-            if (!keep) return;
+            if (list_cap >= 0) return;
 #pragma unroll
             for (int j = 0; j < NODES; j++) {
                 const uint32_t v = gi.node[j];
@@ -331,8 +332,9 @@ __global__ void __launch_bounds__(256) hb_need_csr_kernel(const uint64_t *__rest
 template <int S, bool NIB>
 __global__ void __launch_bounds__(256) hb_table_kernel(const uint8_t *__restrict__ cur, uint8_t *__restrict__ tab,
                                                        uint32_t n, int scheme, const uint32_t *__restrict__ open,
-                                                       int s) {
-    if (open && !((*open >> s) & 1u)) return;  // a code pass left nothing open in this slice
+                                                       uint32_t list_cap, int s) {
+    // after a code pass: nothing open in this slice, or all of it settled piece by piece
+    if (open && (!((open[0] >> s) & 1u) || open[1] <= list_cap)) return;
     __shared__ __align__(16) uint8_t buf[TableShape<S>::R * S];
     table_item<S, NIB>(cur, tab, n, blockIdx.x * (uint32_t)TableShape<S>::B, buf, scheme);
 }
@@ -525,7 +527,7 @@ struct Plan {
     uint64_t n = 0;
     // workspace layout (byte offsets, 256-aligned)
     uint64_t off_cur = 0, off_next = 0, off_c0 = 0, off_c1 = 0, off_sum = 0, off_lc = 0, off_flags = 0, off_tab = 0,
-             off_chg = 0, off_need = 0, off_ortab = 0, off_win = 0, off_full = 0, chg_bytes = 0, total = 0;
+             off_chg = 0, off_need = 0, off_ortab = 0, off_win = 0, off_full = 0, off_list = 0, chg_bytes = 0, total = 0;
 };
 
 static uint64_t align256(uint64_t x) { return (x + 255) & ~255ull; }
@@ -542,9 +544,9 @@ constexpr int kTrackMaxSlices = 32;
 constexpr double kTrackBelow = 0.01;
 // A pass gathers one-bit codes once this share of the registers has reached
 // its maximum, and goes back to four bits after a one-bit pass that left more
-// than kOpenShare of the (group, slice) pairs to the byte union.
+// than kOpenShare of the 16-byte register pieces open.
 constexpr double kTopShare = 0.75;
-constexpr double kOpenShare = 0.4;
+constexpr double kOpenShare = 0.2;
 
 
 // Hub threshold of the run-aware union (lookups per work item).
@@ -683,9 +685,11 @@ static int make_plan(const vga_graph *g, int p, const vga_tuning *tune, Plan *P)
     // Codes: the grouped union with an automatic slice width (an explicit or
     // tuned width asks for byte slices of that width, forced tracking for the
     // need masks of its own rule), at least 32 registers, whole 32-register
-    // units in a register slice, and one need bit per slice.
+    // units in a register slice, one need bit per slice, and a 32-bit count of
+    // open pieces.
     P->codes = P->mode == kModeRuns && P->group == kCodeNodes && auto_S && P->track != 2 && P->m >= 32 &&
-               P->slices <= kTrackMaxSlices && S >= (P->nib ? 16 : 32);
+               P->slices <= kTrackMaxSlices && S >= (P->nib ? 16 : 32) &&
+               P->n * P->node_bytes / 16 < (1ull << 32);
     // flags, change bytes and need masks side by side, so that a pass clears
     // what it uses of them at once
     P->off_flags = o; o = align256(o + 64);
@@ -705,6 +709,8 @@ static int make_plan(const vga_graph *g, int p, const vga_tuning *tune, Plan *P)
         o = align256(o + 4ull * P->m + 2ull * P->node_bytes);
         P->off_full = o;
         o = align256(o + P->n);
+        P->off_list = o;  // {node, 16-byte piece} of up to N open pieces
+        o = align256(o + 8 * P->n);
     }
     P->total = o;
     return VGA_OK;
@@ -777,7 +783,7 @@ struct PendingTiming {
 
 template <int SS, bool NIB>
 static void launch_union_slice(const Plan &P, const vga_graph *g, const uint8_t *c, uint8_t *x, uint8_t *tab,
-                               uint32_t *flags, cudaStream_t stream, const uint32_t *need, int s, int keep,
+                               uint32_t *flags, cudaStream_t stream, const uint32_t *need, int s, int64_t list_cap,
                                uint8_t *chg) {
     const unsigned blocks = (unsigned)((P.n + P.warps - 1) / P.warps);
     const size_t smem = (size_t)P.warps * 32 * sizeof(uint32_t);
@@ -785,7 +791,8 @@ static void launch_union_slice(const Plan &P, const vga_graph *g, const uint8_t 
         const unsigned item_blocks = (unsigned)((P.items.count + P.warps - 1) / P.warps);
         const unsigned table_blocks = (unsigned)((P.n + TableShape<SS>::B - 1) / TableShape<SS>::B);
         hb_table_kernel<SS, NIB><<<table_blocks, 256, 0, stream>>>(c, tab, (uint32_t)P.n, P.scheme,
-                                                                   keep ? nullptr : flags + 8, s);
+                                                                   list_cap < 0 ? nullptr : flags + 8,
+                                                                   (uint32_t)list_cap, s);
         count_launch();
         if (!P.group) {
             hb_union_runs_kernel<SS, NIB><<<item_blocks, P.warps * 32, (size_t)P.warps * sizeof(LkStage), stream>>>(
@@ -805,7 +812,7 @@ static void launch_union_slice(const Plan &P, const vga_graph *g, const uint8_t 
                 if (smem > (48u << 10))
                     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
                 kernel<<<group_blocks, P.warps * 32, smem, stream>>>(P.groups.items, P.groups.count, P.groups.rows,
-                                                                     P.groups.cls, c, tab, x, flags, need, s, keep, chg);
+                                                                     P.groups.cls, c, tab, x, flags, need, s, list_cap, chg);
             };
             if (group_blocks) {
                 if (P.group == 2) launch_groups(hb_union_groups_kernel<SS, NIB, 2>);
@@ -823,13 +830,13 @@ static void launch_union_slice(const Plan &P, const vga_graph *g, const uint8_t 
 // One pass of the union over every slice.  need (a change-tracked pass) and
 // chg (change bytes to record, [slice][N]) may be null.  After a code pass
 // (left_open: the slices with open pairs, marked in need) only those slices
-// run, and pairs that need nothing are left alone.
+// run, pairs that need nothing are left alone, and nothing is done when the
+// pass left at most list_cap pieces open (launch_code_open settled them).
 static int launch_union(const Plan &P, const vga_graph *g, const uint8_t *cur, uint8_t *nxt, uint8_t *tab,
                         uint32_t *flags, cudaStream_t stream, std::vector<PendingTiming> *timings,
                         const uint32_t *need = nullptr, uint8_t *chg = nullptr, const uint32_t *left_open = nullptr,
-                        bool tracked = false) {
+                        int64_t list_cap = -1, bool tracked = false) {
     const uint64_t slice_bytes = (uint64_t)P.n * P.S;
-    const int keep = left_open ? 0 : 1;
     for (int s = 0; s < P.slices; s++) {
         if (left_open && !((*left_open >> s) & 1u)) continue;
         const uint8_t *c = cur + (uint64_t)s * slice_bytes;
@@ -842,20 +849,20 @@ static int launch_union(const Plan &P, const vga_graph *g, const uint8_t *cur, u
             VGA_CHECK_CUDA(cudaEventRecord(pt.start, stream));
         }
         switch (P.S) {
-            case 16: P.nib ? launch_union_slice<16, true>(P, g, c, x, tab, flags, stream, need, s, keep, cs)
-                             : launch_union_slice<16, false>(P, g, c, x, tab, flags, stream, need, s, keep, cs); break;
-            case 32: P.nib ? launch_union_slice<32, true>(P, g, c, x, tab, flags, stream, need, s, keep, cs)
-                             : launch_union_slice<32, false>(P, g, c, x, tab, flags, stream, need, s, keep, cs); break;
-            case 64: P.nib ? launch_union_slice<64, true>(P, g, c, x, tab, flags, stream, need, s, keep, cs)
-                             : launch_union_slice<64, false>(P, g, c, x, tab, flags, stream, need, s, keep, cs); break;
-            case 128: P.nib ? launch_union_slice<128, true>(P, g, c, x, tab, flags, stream, need, s, keep, cs)
-                             : launch_union_slice<128, false>(P, g, c, x, tab, flags, stream, need, s, keep, cs); break;
-            case 256: P.nib ? launch_union_slice<256, true>(P, g, c, x, tab, flags, stream, need, s, keep, cs)
-                             : launch_union_slice<256, false>(P, g, c, x, tab, flags, stream, need, s, keep, cs); break;
-            case 512: P.nib ? launch_union_slice<512, true>(P, g, c, x, tab, flags, stream, need, s, keep, cs)
-                             : launch_union_slice<512, false>(P, g, c, x, tab, flags, stream, need, s, keep, cs); break;
-            case 1024: P.nib ? launch_union_slice<1024, true>(P, g, c, x, tab, flags, stream, need, s, keep, cs)
-                             : launch_union_slice<1024, false>(P, g, c, x, tab, flags, stream, need, s, keep, cs); break;
+            case 16: P.nib ? launch_union_slice<16, true>(P, g, c, x, tab, flags, stream, need, s, list_cap, cs)
+                             : launch_union_slice<16, false>(P, g, c, x, tab, flags, stream, need, s, list_cap, cs); break;
+            case 32: P.nib ? launch_union_slice<32, true>(P, g, c, x, tab, flags, stream, need, s, list_cap, cs)
+                             : launch_union_slice<32, false>(P, g, c, x, tab, flags, stream, need, s, list_cap, cs); break;
+            case 64: P.nib ? launch_union_slice<64, true>(P, g, c, x, tab, flags, stream, need, s, list_cap, cs)
+                             : launch_union_slice<64, false>(P, g, c, x, tab, flags, stream, need, s, list_cap, cs); break;
+            case 128: P.nib ? launch_union_slice<128, true>(P, g, c, x, tab, flags, stream, need, s, list_cap, cs)
+                             : launch_union_slice<128, false>(P, g, c, x, tab, flags, stream, need, s, list_cap, cs); break;
+            case 256: P.nib ? launch_union_slice<256, true>(P, g, c, x, tab, flags, stream, need, s, list_cap, cs)
+                             : launch_union_slice<256, false>(P, g, c, x, tab, flags, stream, need, s, list_cap, cs); break;
+            case 512: P.nib ? launch_union_slice<512, true>(P, g, c, x, tab, flags, stream, need, s, list_cap, cs)
+                             : launch_union_slice<512, false>(P, g, c, x, tab, flags, stream, need, s, list_cap, cs); break;
+            case 1024: P.nib ? launch_union_slice<1024, true>(P, g, c, x, tab, flags, stream, need, s, list_cap, cs)
+                             : launch_union_slice<1024, false>(P, g, c, x, tab, flags, stream, need, s, list_cap, cs); break;
             default:
                 set_error("internal: slice width %d", P.S);
                 return VGA_EINVAL;
@@ -911,6 +918,20 @@ static int launch_codes(const Plan &P, const vga_graph *g, int K, uint8_t *base,
     C.flags = flags;
     C.full = base + P.off_full;
     C.need = reinterpret_cast<uint32_t *>(base + P.off_need);
+    // Open pieces are settled one by one while their neighbours' 32-byte
+    // sectors stay below an eighth of the rows a whole byte union gathers.
+    C.list = reinterpret_cast<uint2 *>(base + P.off_list);
+    const double piece = 32.0 * (double)g->n_edges / (double)P.n;
+    C.list_cap = (uint32_t)std::min((double)P.n, (double)P.groups.rows_used * P.node_bytes / 8.0 / std::max(piece, 1.0));
+    // Warps per group: enough for twice the warps the GPU holds (about 40 an
+    // SM), no more than leaves each about 32 rows.
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const uint64_t rows_per_group = P.groups.rows_used / std::max<uint64_t>(P.groups.count, 1);
+    while (C.split < 8 && P.groups.count * C.split < (uint64_t)sms * 80 && rows_per_group / C.split > 32) C.split *= 2;
+    if (C.split > 1)  // equal pieces, one or more a warp
+        C.len = (int)std::min<uint64_t>(128, std::max<uint64_t>(16, (rows_per_group / C.split + 15) / 16 * 16));
     C.chg = chg;
     C.stream = stream;
     for (int s = 0; s < node_codes / C.S; s++) {
@@ -934,15 +955,18 @@ static int launch_codes(const Plan &P, const vga_graph *g, int K, uint8_t *base,
             timings->push_back(pt);
         }
     }
-    // the byte union of the slices with open pairs: asked for with a wait when
+    VGA_TRY(launch_code_open(C, g->lk[P.scheme].d_off, g->lk[P.scheme].d_lk, sms));
+    // more of them: the byte union of their slices, asked for with a wait when
     // there are many slices, else launched for all (the kernels then return at
     // once; a wait costs about 12 us, an idle pair of launches 4)
-    uint32_t open = P.slices >= 32 ? 0xffffffffu : (1u << P.slices) - 1u;
+    uint32_t open[2] = {P.slices >= 32 ? 0xffffffffu : (1u << P.slices) - 1u, 0xffffffffu};
     if (P.slices > 2) {
-        VGA_CHECK_CUDA(cudaMemcpyAsync(&open, flags + 8, 4, cudaMemcpyDeviceToHost, stream));
+        VGA_CHECK_CUDA(cudaMemcpyAsync(open, flags + 8, 8, cudaMemcpyDeviceToHost, stream));
         VGA_CHECK_CUDA(cudaStreamSynchronize(stream));
     }
-    if (open) VGA_TRY(launch_union(P, g, cur, nxt, C.tab, flags, stream, timings, C.need, chg, &open, tracked));
+    if (open[0] && open[1] > C.list_cap)
+        VGA_TRY(launch_union(P, g, cur, nxt, C.tab, flags, stream, timings, C.need, chg, &open[0], C.list_cap,
+                             tracked));
     return VGA_OK;
 }
 
@@ -1217,7 +1241,7 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
             uint32_t f[4];        // changed, estimate increase, bounded wait gave up, unused
             uint64_t n_changed;   // (node, slice) pairs changed by the pass (change tracking)
             uint64_t n_top;       // registers at the window's top (codes)
-            uint32_t open[2];     // slices with pairs a code pass left open, and their number
+            uint32_t open[2];     // slices where a code pass left pieces open, and the pieces
         } h{};
         VGA_CHECK_CUDA(cudaMemsetAsync(flags, 0, sizeof(h), stream));
         L2Window window;
@@ -1266,7 +1290,7 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
                 return VGA_ETIMEOUT;
             }
             changed_prev = h.n_changed;
-            if (K == 1) too_open = (double)h.open[1] > kOpenShare * (double)P.groups.count * P.slices;
+            if (K == 1) too_open = (double)h.open[1] > kOpenShare * (double)P.n * (P.node_bytes / 16.0);
             std::swap(cur, nxt);
             std::swap(c_prev, c_cur);
             const bool stop = (conv_mode == 1) ? (h.f[1] == 0) : (h.f[0] == 0);

@@ -247,10 +247,15 @@ struct CodePass {
     uint32_t *flags = nullptr;
     const uint8_t *full = nullptr;     // K = 1: nodes whose registers all equal G, or nullptr
     uint32_t *need = nullptr;          // (node, slice) pairs left open, one bit per register slice
+    uint2 *list = nullptr;             // the first list_cap open pieces {node, 16-byte piece}
+    uint32_t list_cap = 0;
+    int split = 1, len = 128;          // warps per group, row entries a warp takes at a time
     uint8_t *chg = nullptr;            // change bytes, or nullptr
     cudaStream_t stream = nullptr;
 };
 int launch_code_slice(const CodePass &C, int slice);
+// After the pass's slices: the open pieces, when they all fit the list.
+int launch_code_open(const CodePass &C, const uint64_t *lk_off, const uint32_t *lk, int sms);
 int launch_code_window(const uint32_t *gmax, uint32_t words, int nib, uint32_t *top, uint32_t *low,
                        cudaStream_t stream);
 

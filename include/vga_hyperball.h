@@ -166,11 +166,14 @@ int vga_graph_set_cells(vga_graph *g, int W, int H, const uint64_t *cell_of_node
  * each end open or closed) is kept; a target is visible iff its slope lies in
  * one of them (the diagonal target also needs the cell beside it, whose
  * corner its segment touches, free).  The result equals the pairwise rule
- * above for every pair.  Two passes (count, then write) produce the CSR.
+ * above for every pair.  The lists go to a stage and from there to the CSR.
  * Device scratch besides the CSR: obstacle bitmaps (2 x W x H bits with
  * margins), a W*H node-id table and 12 bytes a node; per CTA a node bitmap
  * (in shared memory up to ~800k nodes) and, for sources whose interval lists
- * outgrow shared memory, global lists of max(W, H) + 2 entries per warp.
+ * outgrow shared memory, global lists of max(W, H) + 2 entries per warp; and,
+ * while it is to be had, a stage of about the CSR's size (at most 256 MB, or a
+ * twentieth more than the sampled size), without which every source is swept
+ * twice.
  * Errors: VGA_EINVAL for bad sizes; VGA_ECORRUPT if the sweep's own checks
  * fail (a visible cell off the component, a list overflow past the proven
  * bound, a count/write mismatch).
@@ -178,9 +181,10 @@ int vga_graph_set_cells(vga_graph *g, int W, int H, const uint64_t *cell_of_node
 int vga_visibility_build(int W, int H, const uint8_t *obst, uint64_t *cell_of_node, vga_graph **out);
 
 /*
- * vga_set_visibility_sweep_limits -- test hook for the builder's two
+ * vga_set_visibility_sweep_limits -- test hook for the builder's
  * fallbacks: smem_list_cap (1..48, 0 = 48) caps the interval lists kept in
- * shared memory, so that more sources take the global-list retry;
+ * shared memory, so that more sources take the global-list retry, and (below
+ * 48) the stage at 64 bytes a node, so that some lists are swept twice;
  * smem_bitmap_nodes > 0 keeps the node bitmap in global memory for graphs
  * with more nodes than that (0 = whenever shared memory is too small).
  * Process-wide; both give the same graph as the defaults.

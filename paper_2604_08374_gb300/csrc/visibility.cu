@@ -10,10 +10,11 @@
 // tan-space [0, 1] loses the ranges obstacles cover), with the gaps' ends kept
 // as exact integer fractions so that the result equals the pairwise rule above
 // for every pair.  Pipeline: (host) main component and numbering, obstacle
-// bitmaps; (device) count pass: per source, the octants swept into a node
-// bitmap and the LEB128 bytes of its list counted; (host) prefix sum into
-// offsets; (device) write pass: the same sweep, the bytes written; then the
-// ordinary load path validates the stream and derives degrees.
+// bitmaps; (device) per source, the octants swept into a node bitmap and its
+// list's LEB128 bytes written to a stage in the order the sources finish;
+// (host) prefix sum of the lists' sizes into offsets; (device) the lists copied
+// to their places; then the ordinary load path validates the stream and derives
+// degrees.
 #include <algorithm>
 #include <utility>
 #include <vector>
@@ -116,7 +117,8 @@ constexpr int kPad = 64;                           // margin bits (obstacles) on
 constexpr uint32_t kNoSource = 0xffffffffu;
 
 // Test hooks: a smaller shared-memory list capacity sends more sources down
-// the global-list retry; a node limit moves the node bitmap to global memory.
+// the global-list retry (and makes the stage of the lists' bytes so small that
+// some are swept again); a node limit moves the node bitmap to global memory.
 int g_sweep_smem_cap = kSweepCap;
 uint32_t g_sweep_smem_bitmap_nodes = 0;   // 0: as many as shared memory allows
 
@@ -154,9 +156,12 @@ struct SweepArgs {
     const uint32_t *sources;       // the sources to sweep (nullptr: nodes 0 .. count - 1)
     uint32_t count;
     uint32_t *next;                // work counter, zero at launch
-    uint64_t *row_bytes;           // count pass: bytes of each source's list
-    const uint64_t *offsets;       // write pass: each list's first byte
-    uint8_t *out;
+    uint64_t *row_bytes;           // kSweepCount, kSweepStage: bytes of each source's list
+    const uint64_t *offsets;       // kSweepWrite: each list's first byte
+    uint8_t *out;                  // the lists (kSweepWrite) or the stage (kSweepStage)
+    unsigned long long *stage_used;    // kSweepStage: bytes of the stage given out, zero at launch
+    uint64_t stage_cap;
+    uint64_t *stage_at;            // kSweepStage: each list's first byte in the stage, or kNotStaged
     uint32_t *retry, *retry_count; // sources whose interval lists outgrew shared memory
     uint2 *glists;                 // global interval lists (cap glist_cap each, 2 per warp)
     int glist_cap;
@@ -358,13 +363,19 @@ __device__ bool sweep_octant(const SweepArgs &A, int oct, int sx, int sy, uint32
     return true;
 }
 
+// What becomes of a source's list: its bytes are counted; or written at its
+// place in the CSR (which the counts of all lists before it fix); or counted
+// and written to the next free bytes of a stage, in the order the sources
+// finish, from where stage_gather_kernel brings every list to its place.
+enum SweepMode { kSweepCount, kSweepWrite, kSweepStage };
+constexpr uint64_t kNotStaged = ~0ull;
+
 // Persistent CTAs of 8 warps take sources from a counter; each warp sweeps
 // one octant into the CTA's node bitmap, then the warps encode the bitmap's
-// set bits as the source's LEB128 delta list (WRITE = false: count the bytes
-// only).  GLOBAL_LISTS: interval lists in global memory with room for the
+// set bits as the source's LEB128 delta list (MODE).  GLOBAL_LISTS: interval lists in global memory with room for the
 // proven maximum (retried sources); otherwise kSweepCap entries in shared
 // memory, and a source whose list outgrows them is queued for the retry.
-template <bool WRITE, bool GLOBAL_LISTS, bool SMEM_BITMAP>
+template <SweepMode MODE, bool GLOBAL_LISTS, bool SMEM_BITMAP>
 __global__ void __launch_bounds__(kSweepThreads, 6) visibility_sweep_kernel(SweepArgs A) {
     extern __shared__ __align__(16) uint8_t smem[];
     __shared__ uint32_t s_src;
@@ -372,6 +383,7 @@ __global__ void __launch_bounds__(kSweepThreads, 6) visibility_sweep_kernel(Swee
     __shared__ int s_first[kSweepWarps], s_last[kSweepWarps];
     __shared__ uint32_t s_bytes[kSweepWarps];
     __shared__ int s_count[kSweepWarps];
+    __shared__ uint64_t s_at;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint8_t *p = smem;
     uint32_t *bm;
@@ -478,12 +490,27 @@ __global__ void __launch_bounds__(kSweepThreads, 6) visibility_sweep_kernel(Swee
                 total += bw;
                 if (s_last[w] > run) run = s_last[w];
             }
-            if (!WRITE) {
-                if (threadIdx.x == 0) A.row_bytes[u] = total;
-            } else {
+            if (MODE != kSweepWrite && threadIdx.x == 0) A.row_bytes[u] = total;
+            uint64_t list_at = 0, end = 0;
+            bool write = false;
+            if (MODE == kSweepWrite) {
+                list_at = A.offsets[u];
+                end = A.offsets[u + 1];
+                write = true;
+            } else if (MODE == kSweepStage) {
+                if (threadIdx.x == 0) {
+                    s_at = atomicAdd(A.stage_used, (unsigned long long)((total + 15) & ~15ull));
+                    if (s_at + total > A.stage_cap) s_at = kNotStaged;
+                    A.stage_at[u] = s_at;
+                }
+                __syncthreads();
+                list_at = s_at;
+                write = list_at != kNotStaged;
+                end = list_at + total;
+            }
+            if (write) {
                 // phase B: write the share's varints from its first byte on
-                uint64_t pos = A.offsets[u] + start;
-                const uint64_t end = A.offsets[u + 1];
+                uint64_t pos = list_at + start;
                 int run_prev = prev;
                 for (uint32_t c = mb; c < me; c += 32) {
                     const uint32_t wi = c + lane;
@@ -533,13 +560,14 @@ __global__ void __launch_bounds__(kSweepThreads, 6) visibility_sweep_kernel(Swee
                     if (cl > run_prev) run_prev = cl;
                 }
             }
-        } else if (!WRITE && threadIdx.x == 0) {
+        } else if (MODE != kSweepWrite && threadIdx.x == 0) {
             A.row_bytes[u] = 0;
+            if (MODE == kSweepStage) A.stage_at[u] = 0;
         }
         if (overflow && threadIdx.x == 0) {
             if (GLOBAL_LISTS) {
                 atomicOr(A.err, 2);
-            } else if (!WRITE) {
+            } else {
                 A.retry[atomicAdd(A.retry_count, 1u)] = u;
             }
         }
@@ -553,6 +581,38 @@ __global__ void __launch_bounds__(kSweepThreads, 6) visibility_sweep_kernel(Swee
                 else __stcg(bm + w, 0u);
             }
         __syncthreads();
+    }
+}
+
+// Brings the staged lists to their places in the CSR, one warp per list: the
+// stage's lists start on 16-byte boundaries, the CSR's anywhere, so each lane
+// builds aligned 16-byte words of the destination from five words of the
+// source (the stage is readable 16 bytes past its end).
+__global__ void __launch_bounds__(256) stage_gather_kernel(const uint8_t *__restrict__ stage,
+                                                           const uint64_t *__restrict__ stage_at,
+                                                           const uint64_t *__restrict__ offsets, uint32_t n,
+                                                           uint8_t *__restrict__ out) {
+    const int lane = threadIdx.x & 31;
+    const uint64_t v = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (v >= n || stage_at[v] == kNotStaged) return;
+    const uint64_t o0 = offsets[v], o1 = offsets[v + 1];
+    const uint8_t *src = stage + stage_at[v];
+    const uint64_t up = (o0 + 15) & ~15ull, down = o1 & ~15ull;
+    const uint64_t b0 = up < o1 ? up : o1, b1 = down > b0 ? down : b0;
+    if (o0 + lane < b0) out[o0 + lane] = src[lane];
+    if (b1 + lane < o1) out[b1 + lane] = src[b1 - o0 + lane];
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(src + ((b0 - o0) & ~3ull));
+    const uint32_t shift = 8u * (uint32_t)((b0 - o0) & 3u);
+    for (uint64_t q = lane; q < (b1 - b0) / 16; q += 32) {
+        uint32_t x[5];
+#pragma unroll
+        for (int i = 0; i < 5; i++) x[i] = __ldcs(w + 4 * q + i);
+        uint4 y;
+        y.x = __funnelshift_r(x[0], x[1], shift);
+        y.y = __funnelshift_r(x[1], x[2], shift);
+        y.z = __funnelshift_r(x[2], x[3], shift);
+        y.w = __funnelshift_r(x[3], x[4], shift);
+        *reinterpret_cast<uint4 *>(out + b0 + 16 * q) = y;
     }
 }
 
@@ -628,7 +688,7 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
     VGA_TRY(d_noc.alloc(node_of_cell.size() * 4));
     VGA_TRY(d_cells.alloc((size_t)std::max<uint32_t>(n, 1) * 4));
     VGA_TRY(d_rowbytes.alloc((size_t)std::max<uint32_t>(n, 1) * 8));
-    VGA_TRY(d_counter.alloc(4 * sizeof(uint32_t)));
+    VGA_TRY(d_counter.alloc(6 * sizeof(uint32_t)));
     VGA_TRY(d_retry.alloc((size_t)std::max<uint32_t>(n, 1) * 4));
     VGA_TRY(d_err.alloc(sizeof(int)));
     cudaStream_t stream = 0;
@@ -637,7 +697,7 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
     VGA_CHECK_CUDA(cudaMemcpyAsync(d_noc.ptr, node_of_cell.data(), node_of_cell.size() * 4, cudaMemcpyHostToDevice,
                                    stream));
     if (n) VGA_CHECK_CUDA(cudaMemcpyAsync(d_cells.ptr, cells.data(), (size_t)n * 4, cudaMemcpyHostToDevice, stream));
-    VGA_CHECK_CUDA(cudaMemsetAsync(d_counter.ptr, 0, 4 * sizeof(uint32_t), stream));
+    VGA_CHECK_CUDA(cudaMemsetAsync(d_counter.ptr, 0, 6 * sizeof(uint32_t), stream));
     VGA_CHECK_CUDA(cudaMemsetAsync(d_err.ptr, 0, sizeof(int), stream));
 
     SweepArgs sa{};
@@ -661,18 +721,20 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
 
     // one launch of the sweep over `count` sources (sources == nullptr: all
     // nodes), interval lists in shared memory or (retries) in global memory
-    auto launch = [&](bool write, bool global_lists, const uint32_t *sources, uint32_t count,
+    auto launch = [&](SweepMode mode, bool global_lists, const uint32_t *sources, uint32_t count,
                       uint32_t *counter) -> int {
         if (!count) return VGA_OK;
         const size_t smem = (smem_bitmap ? bitmap_smem : 0) + (global_lists ? 0 : list_smem) + mask_smem;
         void (*fn)(SweepArgs);
-        if (write) {
-            if (global_lists) fn = smem_bitmap ? visibility_sweep_kernel<true, true, true> : visibility_sweep_kernel<true, true, false>;
-            else fn = smem_bitmap ? visibility_sweep_kernel<true, false, true> : visibility_sweep_kernel<true, false, false>;
-        } else {
-            if (global_lists) fn = smem_bitmap ? visibility_sweep_kernel<false, true, true> : visibility_sweep_kernel<false, true, false>;
-            else fn = smem_bitmap ? visibility_sweep_kernel<false, false, true> : visibility_sweep_kernel<false, false, false>;
-        }
+#define VGA_SW(M)                                                                                   \
+    if (global_lists)                                                                               \
+        fn = smem_bitmap ? visibility_sweep_kernel<M, true, true> : visibility_sweep_kernel<M, true, false>;   \
+    else                                                                                            \
+        fn = smem_bitmap ? visibility_sweep_kernel<M, false, true> : visibility_sweep_kernel<M, false, false>
+        if (mode == kSweepWrite) VGA_SW(kSweepWrite);
+        else if (mode == kSweepStage) VGA_SW(kSweepStage);
+        else VGA_SW(kSweepCount);
+#undef VGA_SW
         VGA_CHECK_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         int per_sm = 0;
         VGA_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kSweepThreads, smem));
@@ -702,15 +764,19 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
         return VGA_OK;
     };
 
+    // The lists are swept once, into a stage of the size they are expected to
+    // take: the bound of n - 1 varints a list (one more byte for every 128 ids
+    // that a delta skips) while that is small, else what every kSampleStep-th
+    // source's list takes, and a twentieth on top.  What a full stage leaves
+    // out, and everything when the stage cannot be had, is swept again straight
+    // to its place in the CSR.
     std::vector<uint64_t> offsets((size_t)n + 1, 0);
+    std::vector<uint32_t> again;   // sources to be swept again
     uint32_t n_retry = 0;
-    if (n) {
-        // count pass; the sources whose lists outgrew shared memory are counted again
-        VGA_TRY(launch(false, false, nullptr, n, d_counter.as<uint32_t>()));
-        VGA_CHECK_CUDA(cudaMemcpyAsync(&n_retry, sa.retry_count, 4, cudaMemcpyDeviceToHost, stream));
-        VGA_CHECK_CUDA(cudaStreamSynchronize(stream));
-        VGA_TRY(launch(false, true, d_retry.as<uint32_t>(), n_retry, d_counter.as<uint32_t>() + 1));
-        std::vector<uint64_t> rb(n);
+    DeviceBuffer d_stage, d_stage_at;
+    uint32_t *retry_list = d_retry.as<uint32_t>();
+    auto read_row_bytes = [&](std::vector<uint64_t> &rb) -> int {
+        rb.resize(n);
         int err = 0;
         VGA_CHECK_CUDA(cudaMemcpyAsync(rb.data(), d_rowbytes.ptr, (size_t)n * 8, cudaMemcpyDeviceToHost, stream));
         VGA_CHECK_CUDA(cudaMemcpyAsync(&err, d_err.ptr, sizeof(int), cudaMemcpyDeviceToHost, stream));
@@ -719,21 +785,92 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
             set_error("visibility sweep failed its own checks (code %d)", err);
             return VGA_ECORRUPT;
         }
+        return VGA_OK;
+    };
+    // counters: [0], [1] sources taken, [2] retries, [4..5] stage bytes given out
+    auto sweep = [&](SweepMode mode, const uint32_t *sources, uint32_t count) -> int {
+        VGA_CHECK_CUDA(cudaMemsetAsync(d_counter.ptr, 0, 3 * sizeof(uint32_t), stream));
+        VGA_TRY(launch(mode, false, sources, count, d_counter.as<uint32_t>()));
+        VGA_CHECK_CUDA(cudaMemcpyAsync(&n_retry, sa.retry_count, 4, cudaMemcpyDeviceToHost, stream));
+        VGA_CHECK_CUDA(cudaStreamSynchronize(stream));
+        return launch(mode, true, retry_list, n_retry, d_counter.as<uint32_t>() + 1);
+    };
+    if (n) {
+        constexpr uint64_t kStageSmall = 256ull << 20;
+        constexpr uint32_t kSampleStep = 128;
+        std::vector<uint64_t> rb;
+        uint64_t cap = (uint64_t)n * ((uint64_t)n + n / 64 + 32);
+        if (cap > kStageSmall) {
+            std::vector<uint32_t> sample;
+            for (uint32_t v = kSampleStep / 2; v < n; v += kSampleStep) sample.push_back(v);
+            DeviceBuffer d_sample;
+            VGA_TRY(d_sample.alloc(sample.size() * 4));
+            VGA_CHECK_CUDA(cudaMemcpyAsync(d_sample.ptr, sample.data(), sample.size() * 4, cudaMemcpyHostToDevice,
+                                           stream));
+            VGA_TRY(sweep(kSweepCount, d_sample.as<uint32_t>(), (uint32_t)sample.size()));
+            VGA_TRY(read_row_bytes(rb));
+            uint64_t sum = 0;
+            for (uint32_t v : sample) sum += rb[v];
+            cap = std::min<uint64_t>(cap, (uint64_t)((double)sum / sample.size() * n * 1.05) + 32ull * n);
+        }
+        if (sa.smem_cap < kSweepCap) cap = std::min<uint64_t>(cap, 64ull * n);   // the test hook fills the stage, too
+        SweepMode mode = kSweepStage;
+        if (cudaMalloc(&d_stage.ptr, cap + 16) != cudaSuccess) {
+            cudaGetLastError();
+            d_stage.ptr = nullptr;
+            mode = kSweepCount;
+        }
+        VGA_TRY(d_stage_at.alloc((size_t)n * 8));
+        sa.out = d_stage.as<uint8_t>();
+        sa.stage_used = reinterpret_cast<unsigned long long *>(d_counter.as<uint32_t>() + 4);
+        sa.stage_cap = cap;
+        sa.stage_at = d_stage_at.as<uint64_t>();
+        VGA_TRY(sweep(mode, nullptr, n));
+        unsigned long long used = ~0ull;
+        if (mode == kSweepStage)
+            VGA_CHECK_CUDA(cudaMemcpyAsync(&used, sa.stage_used, 8, cudaMemcpyDeviceToHost, stream));
+        VGA_TRY(read_row_bytes(rb));
         for (uint32_t v = 0; v < n; v++) offsets[v + 1] = offsets[v] + rb[v];
+        if (mode == kSweepCount) {
+            again.resize(n);
+            for (uint32_t v = 0; v < n; v++) again[v] = v;
+        } else if (used > cap) {
+            std::vector<uint64_t> at(n);
+            VGA_CHECK_CUDA(cudaMemcpy(at.data(), d_stage_at.ptr, (size_t)n * 8, cudaMemcpyDeviceToHost));
+            for (uint32_t v = 0; v < n; v++)
+                if (at[v] == kNotStaged) again.push_back(v);
+        }
     }
     const uint64_t n_bytes = offsets[n];
     DeviceBuffer d_off, d_bytes;
     VGA_TRY(d_off.alloc(((size_t)n + 1) * 8));
-    VGA_TRY(d_bytes.alloc(n_bytes + kBytePad));
+    if (d_bytes.alloc(n_bytes + kBytePad) != VGA_OK) {
+        if (!d_stage.ptr) return VGA_ENOMEM;
+        // no room beside the stage: every list is swept again
+        cudaGetLastError();
+        clear_error();
+        d_stage.reset();
+        again.resize(n);
+        for (uint32_t v = 0; v < n; v++) again[v] = v;
+        VGA_TRY(d_bytes.alloc(n_bytes + kBytePad));
+    }
     VGA_CHECK_CUDA(cudaMemcpyAsync(d_off.ptr, offsets.data(), ((size_t)n + 1) * 8, cudaMemcpyHostToDevice, stream));
     VGA_CHECK_CUDA(cudaMemsetAsync(d_bytes.as<uint8_t>() + n_bytes, 0, kBytePad, stream));
-    if (n) {
-        // write pass: the same split between shared-memory and global lists
-        VGA_CHECK_CUDA(cudaMemsetAsync(d_counter.ptr, 0, 2 * sizeof(uint32_t), stream));
+    if (n && d_stage.ptr) {
+        stage_gather_kernel<<<(n + 7) / 8, 256, 0, stream>>>(d_stage.as<uint8_t>(), d_stage_at.as<uint64_t>(),
+                                                            d_off.as<uint64_t>(), n, d_bytes.as<uint8_t>());
+        count_launch();
+        VGA_CHECK_CUDA(cudaGetLastError());
+    }
+    if (!again.empty()) {
+        DeviceBuffer d_again, d_again_retry;
+        VGA_TRY(d_again.alloc(again.size() * 4));
+        VGA_TRY(d_again_retry.alloc(again.size() * 4));
+        VGA_CHECK_CUDA(cudaMemcpyAsync(d_again.ptr, again.data(), again.size() * 4, cudaMemcpyHostToDevice, stream));
         sa.offsets = d_off.as<uint64_t>();
         sa.out = d_bytes.as<uint8_t>();
-        VGA_TRY(launch(true, false, nullptr, n, d_counter.as<uint32_t>()));
-        VGA_TRY(launch(true, true, d_retry.as<uint32_t>(), n_retry, d_counter.as<uint32_t>() + 1));
+        sa.retry = retry_list = d_again_retry.as<uint32_t>();
+        VGA_TRY(sweep(kSweepWrite, d_again.as<uint32_t>(), (uint32_t)again.size()));
         int err = 0;
         VGA_CHECK_CUDA(cudaMemcpyAsync(&err, d_err.ptr, sizeof(int), cudaMemcpyDeviceToHost, stream));
         VGA_CHECK_CUDA(cudaStreamSynchronize(stream));
@@ -743,6 +880,7 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
         }
     }
     VGA_CHECK_CUDA(cudaStreamSynchronize(stream));
+    d_stage.reset();
     uint64_t *po = d_off.as<uint64_t>();
     uint8_t *pb = d_bytes.as<uint8_t>();
     d_off.release();

@@ -18,9 +18,10 @@
 // pass 3 all but 1e-5 of the city's.
 //
 // Measured (GB300): the city graph's pass 2 takes four launches of 128-byte
-// K = 4 rows at 3.1 ms and pass 3 one of K = 1 rows at 2.8 ms, where the byte
-// union takes eight at 2.8 ms each; the d = 3 analysis 54.8 -> 25.4 ms, the
-// unlimited one 85.8 -> 27.0 ms, medium d = 3 3.2 -> 1.85 ms.
+// K = 4 rows at 3.1 ms and pass 3 one of K = 1 rows at 0.5 ms (2.8 ms before
+// a class was cut short once all its bits were set, code_group), where the byte
+// union takes eight at 2.8 ms each; the d = 3 analysis 57.4 -> 24.3 ms, the
+// unlimited one at p = 12 342 -> 88 ms, medium d = 3 3.10 -> 1.94 ms.
 //
 // Layout: a 16-byte unit holds 32 registers as four bit planes (K = 4; word k =
 // bit k of the codes, bit i = register i) or 128 registers as one plane
@@ -225,11 +226,28 @@ __device__ __forceinline__ void code_finish(uint4 (&acc)[LeanShape<S>::V4]) {
         }
 }
 
+// Whether every one-bit code of this lane's accumulator is set.
+template <int V4>
+__device__ __forceinline__ bool code_all_set(const uint4 (&acc)[V4]) {
+    uint32_t all = 0xffffffffu;
+#pragma unroll
+    for (int q = 0; q < V4; q++) all &= acc[q].x & acc[q].y & acc[q].z & acc[q].w;
+    return all == 0xffffffffu;
+}
+
 // One warp's share of the code maxima of a group's nodes, into part[NODES][S /
 // 16]: the group's distinct rows in pieces of `len` entries (a multiple of 4,
 // at most kLkChunk) through the warp's TMA stage, this warp taking pieces w, w
 // + split, ...  Within a piece the rows of a class fold into one accumulator,
 // merged into the class's nodes when the class or the piece ends.
+//
+// K = 1: once every bit of a class's accumulator is set, its other rows change
+// nothing.  Every kCheck rows the warp looks; a class that is there is cut
+// short, one whose nodes are all there is passed over, and the walk ends once
+// all nodes are.  The classes come in decreasing mask order, so the rows that
+// all nodes share are first.  (K = 4 does not look: after pass 2 only 4 % of
+// the city's 256-register rows are at the top throughout, and looking cost
+// more than that.)
 template <int S, int K, int NODES>
 __device__ __forceinline__ void code_group(const GroupItem &gi, const uint32_t *__restrict__ rows,
                                            const uint2 *__restrict__ cls, const uint8_t *__restrict__ tab, uint4 *part,
@@ -237,6 +255,8 @@ __device__ __forceinline__ void code_group(const GroupItem &gi, const uint32_t *
                                            uint32_t len) {
     using Sh = LeanShape<S>;
     constexpr int W16 = S / 16;
+    constexpr int STEP = Sh::P * Sh::U;
+    constexpr uint32_t kCheck = STEP > 32 ? STEP : 32;  // rows between two looks at the accumulator
     const uint32_t cnt = gi.cnt;
     const uint32_t pieces = (cnt + len - 1) / len;
     if (w >= pieces) return;
@@ -256,52 +276,70 @@ __device__ __forceinline__ void code_group(const GroupItem &gi, const uint32_t *
     uint2 cd = *cp;         // {node mask, rows} of the current class
     uint32_t cend = cd.y;   // group entry where the current class ends
     uint32_t phase = 0;
+    uint32_t left = 0;      // nodes of the group not yet at the top (bit j: node j)
+#pragma unroll
+    for (int j = 0; j < NODES; j++) left |= gi.node[j] != 0xffffffffu ? 1u << j : 0u;
+    bool at_top = false;    // K = 1: every bit of the current class's accumulator is set
     auto merge = [&]() {
-        code_finish<S, K>(acc);
-        if (g == 0) {
+        if (K != 1 || (cd.x & left)) {
+            code_finish<S, K>(acc);
 #pragma unroll
             for (int j = 0; j < NODES; j++)
-                if ((cd.x >> j) & 1u)
+                if ((cd.x >> j) & 1u) {
+                    if (g == 0) {
 #pragma unroll
-                    for (int q = 0; q < Sh::V4; q++) {
-                        uint4 &pp = part[j * W16 + sub * Sh::V4 + q];
-                        pp = code_max<K>(pp, acc[q]);
+                        for (int q = 0; q < Sh::V4; q++) {
+                            uint4 &pp = part[j * W16 + sub * Sh::V4 + q];
+                            pp = code_max<K>(pp, acc[q]);
+                        }
                     }
+                }
+            if (K == 1 && at_top) left &= ~cd.x;
         }
 #pragma unroll
         for (int q = 0; q < Sh::V4; q++) acc[q] = make_uint4(0, 0, 0, 0);
     };
-    for (uint32_t k = 0;; k++) {
-        const uint32_t s0 = (w + k * split) * len;
-        if (s0 >= cnt) break;
+    auto wait = [&](uint32_t k) {
         const int slot = (int)(k & 1u);
         if (!__all_sync(0xffffffffu, lk_wait(st, slot, (phase >> slot) & 1u))) {
             if (lane == 0) atomicExch(err, 1);
             lk_wait(st, slot, (phase >> slot) & 1u);  // give an in-flight copy a last chance
         }
         phase ^= 1u << slot;
-        const uint32_t *buf = st.buf[slot];
+    };
+    for (uint32_t k = 0;; k++) {
+        const uint32_t s0 = (w + k * split) * len;
+        if (s0 >= cnt) break;
+        wait(k);
+        if (K == 1 && !left) break;  // the copy of this piece was the last one in flight
+        const uint32_t *buf = st.buf[k & 1u];
         uint32_t lo = s0;
         const uint32_t hi = min(cnt, s0 + len);
         while (cend <= lo) {  // the piece starts in a later class
             cd = *++cp;
             cend += cd.y;
+            at_top = false;
         }
         while (lo < hi) {  // warp-uniform: split the piece at class ends
-            const uint32_t seg = min(hi, cend);
-            code_fold<S, K>(base, buf, (int)(lo - s0), (int)(seg - s0), g, acc);
+            uint32_t seg = min(hi, cend);
+            if (K != 1 || (!at_top && (cd.x & left))) {
+                if (K == 1) seg = min(seg, s0 + ((lo - s0) & ~(Sh::U - 1u)) + kCheck);
+                code_fold<S, K>(base, buf, (int)(lo - s0), (int)(seg - s0), g, acc);
+                if (K == 1) at_top = __all_sync(0xffffffffu, code_all_set<Sh::V4>(acc));
+            }
             lo = seg;
             if (lo == cend) {
                 merge();
+                at_top = false;
                 if (lo < cnt) {
                     cd = *++cp;
                     cend += cd.y;
                 }
             }
         }
-        if (split > 1u && hi < cend) merge();  // the class goes on in another warp's piece
+        if (hi < cend && (split > 1u || at_top)) merge();  // goes on in another warp's piece, or is all set
         __syncwarp();
-        if (lane == 0) load(k + 2u);
+        if (left && lane == 0) load(k + 2u);
     }
 }
 

@@ -86,8 +86,8 @@ __device__ __forceinline__ uint32_t key_lower_bound(const uint32_t *__restrict__
 // sampled evenly from the group's longest list, and every lane merges its own
 // key range serially.  Without WRITE: count the group's entries of every class
 // into cc[group << NODES | class].  With WRITE: from those counts, write the
-// group's class descriptors (classes in increasing mask order, empty ones left
-// out) and its rows, sorted by class (within a class by key), at rows[b ...].
+// group's class descriptors (classes in decreasing mask order: the rows of all
+// nodes first, which the code passes cut short; empty ones left out) and its rows, sorted by class (within a class by key), at rows[b ...].
 // Shared memory: 2^NODES counters or write cursors per lane.
 template <int NODES, bool WRITE>
 __global__ void group_merge_kernel(const GroupItem *__restrict__ items, uint64_t n_groups,
@@ -167,11 +167,11 @@ __global__ void group_merge_kernel(const GroupItem *__restrict__ items, uint64_t
         load_windows();
     }
     if (WRITE) {
-        // this lane's cursor in class k: the class's base (classes in mask
-        // order) plus the counts of the lower lanes
+        // this lane's cursor in class k: the class's base (classes in decreasing
+        // mask order) plus the counts of the lower lanes
         uint32_t base = 0;
         uint64_t ci = it.cls;
-        for (uint32_t k = 1; k < C; k++) {
+        for (uint32_t k = C - 1; k > 0; k--) {
             const uint32_t total = mine[k];
             if (total == 0) continue;  // warp-uniform
             uint32_t mycount = c[k * 32], excl = mycount;

@@ -63,7 +63,8 @@ __global__ void __maxnreg__(56) hb_code_groups_kernel(
     __syncwarp();
     if (gather) {
         lk_stage_init(st, lane);
-        code_group<S, K, kCodeNodes>(gi, rows, cls, tab, part, st, lane, reinterpret_cast<int *>(flags + 2),
+        uint32_t phase = 0;
+        code_group<S, K, kCodeNodes>(gi, rows, cls, tab, part, st, phase, lane, reinterpret_cast<int *>(flags + 2),
                                      split > 1u ? wib : 0u, split, len);
     }
     if (split > 1u) __syncthreads();
@@ -92,9 +93,7 @@ __global__ void __maxnreg__(56) hb_code_groups_kernel(
         }
         if (mine) {
             atomicOr(need + v, mine);
-            uint32_t at = atomicAdd(flags + 9, (uint32_t)__popc(open16));
-            for (uint32_t b = open16; b && at < list_cap; b &= b - 1u)
-                list[at++] = make_uint2(v, u * (UNIT_BYTES / 16) + (uint32_t)__ffs(b) - 1u);
+            code_push_open<K, NIB>(open16, v, u, list, list_cap, flags + 9);
         }
         open_slices |= mine;
     }
@@ -124,44 +123,12 @@ __global__ void __launch_bounds__(256) hb_code_open_kernel(const uint2 *__restri
     __shared__ uint4 s_max[8];
     const uint32_t count = flags[9];
     if (count > list_cap) return;
-    const int rows = table_rows(scheme);
     for (uint32_t e = blockIdx.x; e < count; e += gridDim.x) {
         const uint32_t v = list[e].x, byte = 16u * list[e].y;
-        const uint8_t *base = cur + ((uint64_t)(byte >> s_log2) * n << s_log2) + (byte & ((1u << s_log2) - 1u));
-        uint4 acc = make_uint4(0, 0, 0, 0);
-        const uint64_t e1 = lk_off[v + 1];
-        for (uint64_t k = lk_off[v] + threadIdx.x; k < e1; k += blockDim.x) {
-            const uint32_t r = __ldg(lk + k);
-            uint32_t slot = 0;
-            for (int s = 1; s < rows; s++) slot += r >= (uint32_t)s * n ? 1u : 0u;
-            const uint32_t i = r - slot * n, w = 1u << (scheme == 0 ? slot : 2u * slot);
-#pragma unroll 4
-            for (uint32_t j = 0; j < w; j++)
-                acc = RegFmt<NIB>::max4(acc, __ldg(reinterpret_cast<const uint4 *>(base + ((uint64_t)(i + j) << s_log2))));
+        if (code_open_piece<NIB>(v, byte, lk_off[v], lk_off[v + 1], lk, cur, nxt, n, s_log2, scheme, s_max)) {
+            if (*reinterpret_cast<volatile uint32_t *>(flags) == 0u) atomicOr(flags, 1u);
+            if (chg) chg[(uint64_t)(byte >> s_log2) * n + v] = 1u;
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            uint4 y;
-            y.x = __shfl_xor_sync(0xffffffffu, acc.x, o);
-            y.y = __shfl_xor_sync(0xffffffffu, acc.y, o);
-            y.z = __shfl_xor_sync(0xffffffffu, acc.z, o);
-            y.w = __shfl_xor_sync(0xffffffffu, acc.w, o);
-            acc = RegFmt<NIB>::max4(acc, y);
-        }
-        if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = acc;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int w = 1; w < 8; w++) acc = RegFmt<NIB>::max4(acc, s_max[w]);
-            const uint64_t at = reg_at(n, s_log2, v, byte);
-            const uint4 own = *reinterpret_cast<const uint4 *>(cur + at);
-            acc = RegFmt<NIB>::max4(acc, own);
-            *reinterpret_cast<uint4 *>(nxt + at) = acc;
-            if ((acc.x ^ own.x) | (acc.y ^ own.y) | (acc.z ^ own.z) | (acc.w ^ own.w)) {
-                if (*reinterpret_cast<volatile uint32_t *>(flags) == 0u) atomicOr(flags, 1u);
-                if (chg) chg[(uint64_t)(byte >> s_log2) * n + v] = 1u;
-            }
-        }
-        __syncthreads();
     }
 }
 
@@ -171,15 +138,7 @@ __global__ void hb_window_kernel(const uint32_t *__restrict__ gmax, uint32_t wor
                                  uint32_t *__restrict__ low) {
     const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= words) return;
-    const int f = nib ? 8 : 4, w = nib ? 4 : 8;
-    uint32_t t = 0, l = 0;
-    for (int i = 0; i < f; i++) {
-        const uint32_t g = gmax[k * f + i];
-        t |= g << (w * i);
-        l |= (g > 15u ? g - 15u : 0u) << (w * i);  // 0 with 4-bit registers
-    }
-    top[k] = t;
-    low[k] = l;
+    window_word(gmax, k, nib != 0, top, low);
 }
 
 template <int S, int K, bool NIB>

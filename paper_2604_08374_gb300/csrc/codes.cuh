@@ -158,6 +158,76 @@ __device__ __forceinline__ void code_store(uint4 code, const uint8_t *__restrict
     }
 }
 
+// Open pieces of unit u of node v (open16: bit per 16 register bytes) to the
+// list, as far as it holds them; *count counts them all.
+template <int K, bool NIB>
+__device__ __forceinline__ void code_push_open(uint32_t open16, uint32_t v, uint32_t u, uint2 *__restrict__ list,
+                                               uint32_t list_cap, uint32_t *count) {
+    constexpr uint32_t PIECES = kUnitRegs<K> / (NIB ? 2 : 1) / 16;
+    uint32_t at = atomicAdd(count, (uint32_t)__popc(open16));
+    for (uint32_t b = open16; b && at < list_cap; b &= b - 1u)
+        list[at++] = make_uint2(v, u * PIECES + (uint32_t)__ffs(b) - 1u);
+}
+
+// next[v] for the open register piece at `byte`, from the registers of node v's
+// neighbours: the range lookups lk[b .. e), a thread each (CTAs of 256); thread
+// 0 gets whether it changed.
+template <bool NIB>
+__device__ __forceinline__ bool code_open_piece(uint32_t v, uint32_t byte, uint64_t b, uint64_t e,
+                                                const uint32_t *__restrict__ lk, const uint8_t *__restrict__ cur,
+                                                uint8_t *__restrict__ nxt, uint32_t n, int s_log2, int scheme,
+                                                uint4 *s_max) {
+    const int rows = table_rows(scheme);
+    const uint8_t *base = cur + ((uint64_t)(byte >> s_log2) * n << s_log2) + (byte & ((1u << s_log2) - 1u));
+    uint4 acc = make_uint4(0, 0, 0, 0);
+    for (uint64_t k = b + threadIdx.x; k < e; k += blockDim.x) {
+        const uint32_t r = __ldg(lk + k);
+        uint32_t slot = 0;
+        for (int s = 1; s < rows; s++) slot += r >= (uint32_t)s * n ? 1u : 0u;
+        const uint32_t i = r - slot * n, w = 1u << (scheme == 0 ? slot : 2u * slot);
+#pragma unroll 4
+        for (uint32_t j = 0; j < w; j++)
+            acc = RegFmt<NIB>::max4(acc, __ldg(reinterpret_cast<const uint4 *>(base + ((uint64_t)(i + j) << s_log2))));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        uint4 y;
+        y.x = __shfl_xor_sync(0xffffffffu, acc.x, o);
+        y.y = __shfl_xor_sync(0xffffffffu, acc.y, o);
+        y.z = __shfl_xor_sync(0xffffffffu, acc.z, o);
+        y.w = __shfl_xor_sync(0xffffffffu, acc.w, o);
+        acc = RegFmt<NIB>::max4(acc, y);
+    }
+    if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    bool changed = false;
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; w++) acc = RegFmt<NIB>::max4(acc, s_max[w]);
+        const uint64_t at = reg_at(n, s_log2, v, byte);
+        const uint4 own = *reinterpret_cast<const uint4 *>(cur + at);
+        acc = RegFmt<NIB>::max4(acc, own);
+        *reinterpret_cast<uint4 *>(nxt + at) = acc;
+        changed = ((acc.x ^ own.x) | (acc.y ^ own.y) | (acc.z ^ own.z) | (acc.w ^ own.w)) != 0u;
+    }
+    __syncthreads();
+    return changed;
+}
+
+// Word k of the window of a run (CodeWindow) from the largest rho inserted per
+// register index.
+__device__ __forceinline__ void window_word(const uint32_t *__restrict__ gmax, uint32_t k, bool nib,
+                                            uint32_t *__restrict__ top, uint32_t *__restrict__ low) {
+    const int f = nib ? 8 : 4, w = nib ? 4 : 8;
+    uint32_t t = 0, l = 0;
+    for (int i = 0; i < f; i++) {
+        const uint32_t g = gmax[k * f + i];
+        t |= g << (w * i);
+        l |= (g > 15u ? g - 15u : 0u) << (w * i);  // 0 with 4-bit registers
+    }
+    top[k] = t;
+    low[k] = l;
+}
+
 // Fold the code rows of entries buf[lo .. hi) of a staged chunk into acc: the
 // lane mapping and the steps of lean_fold.
 template <int S, int K>
@@ -239,7 +309,8 @@ __device__ __forceinline__ bool code_all_set(const uint4 (&acc)[V4]) {
 // 16]: the group's distinct rows in pieces of `len` entries (a multiple of 4,
 // at most kLkChunk) through the warp's TMA stage, this warp taking pieces w, w
 // + split, ...  Within a piece the rows of a class fold into one accumulator,
-// merged into the class's nodes when the class or the piece ends.
+// merged into the class's nodes when the class or the piece ends.  `phase`: the
+// stage's barrier phases, kept from one group of the warp to the next.
 //
 // K = 1: once every bit of a class's accumulator is set, its other rows change
 // nothing.  Every kCheck rows the warp looks; a class that is there is cut
@@ -251,8 +322,8 @@ __device__ __forceinline__ bool code_all_set(const uint4 (&acc)[V4]) {
 template <int S, int K, int NODES>
 __device__ __forceinline__ void code_group(const GroupItem &gi, const uint32_t *__restrict__ rows,
                                            const uint2 *__restrict__ cls, const uint8_t *__restrict__ tab, uint4 *part,
-                                           LkStage &st, int lane, int *err, uint32_t w, uint32_t split,
-                                           uint32_t len) {
+                                           LkStage &st, uint32_t &phase, int lane, int *err, uint32_t w,
+                                           uint32_t split, uint32_t len) {
     using Sh = LeanShape<S>;
     constexpr int W16 = S / 16;
     constexpr int STEP = Sh::P * Sh::U;
@@ -275,7 +346,6 @@ __device__ __forceinline__ void code_group(const GroupItem &gi, const uint32_t *
     const uint2 *cp = cls + gi.cls;
     uint2 cd = *cp;         // {node mask, rows} of the current class
     uint32_t cend = cd.y;   // group entry where the current class ends
-    uint32_t phase = 0;
     uint32_t left = 0;      // nodes of the group not yet at the top (bit j: node j)
 #pragma unroll
     for (int j = 0; j < NODES; j++) left |= gi.node[j] != 0xffffffffu ? 1u << j : 0u;

@@ -7,6 +7,9 @@
 //             the GPU; items run in job-major, slice-major order, so the
 //             counters being gathered are one job's slice at a time and stay
 //             in L2;
+//   codes     from the second pass on, jobs without split hubs gather register
+//             codes instead (codes.cuh): the same queue over code slices, then
+//             the pieces left open;
 //   estimate  one warp per node of every running job (estimator + Eq. sumD);
 //   step      one thread per job: pass count, stop rule, flags;
 //   finalize  mean depth and ball sizes of the jobs that just stopped.
@@ -21,8 +24,8 @@
 #include <mutex>
 #include <vector>
 
+#include "codes.cuh"
 #include "engine.cuh"
-#include "hb_device.cuh"
 
 namespace vga {
 
@@ -53,12 +56,25 @@ __global__ void batch_init_kernel(JobDev *jobs, const uint64_t *__restrict__ nod
         init_node(J.regs[0], J.n, J.p, J.S, J.seed, v);
         if (J.first) {
             const uint32_t key = node_key(v, J.p, J.seed, false);
+            if (J.codes) {
+                uint32_t *g = J.win + (key >> 8);
+                if (*reinterpret_cast<volatile uint32_t *>(g) < (key & 0xffu)) atomicMax(g, key & 0xffu);
+            }
             if (J.p <= kKey16MaxP)
                 reinterpret_cast<uint16_t *>(J.tab)[v] = KeyFmt<uint16_t>::pack(key);
             else
                 reinterpret_cast<uint32_t *>(J.tab)[v] = KeyFmt<uint32_t>::pack(key);
         }
     }
+}
+
+// The windows of the jobs that gather codes, one CTA per job.
+__global__ void batch_window_kernel(JobDev *jobs) {
+    const JobDev &J = jobs[blockIdx.x];
+    if (!J.codes) return;
+    const uint32_t m = 1u << J.p;
+    for (uint32_t k = threadIdx.x; k < m / 4u; k += blockDim.x)
+        window_word(J.win, k, false, J.win + m, J.win + m + m / 4u);
 }
 
 // Pass 1 of the jobs in fjobs[0 .. n) (all of precision p, all fresh) as the
@@ -91,6 +107,12 @@ __global__ void __launch_bounds__(kFirstPassWarps * 32) batch_first_pass_kernel(
     }
 }
 
+// The one-bit pass just run left too much open: it is done again in 4 bits.
+__device__ __forceinline__ bool pass_again(const JobDev &J) { return J.K == 1 && J.open > J.open_cap; }
+
+// Nodes that stand for all when the registers at the window's top are counted.
+constexpr uint32_t kTopSample = 8;
+
 // initial != 0: c_0 of every job; otherwise pass t = job.t + 1 of running jobs.
 __global__ void batch_estimate_kernel(JobDev *jobs, const uint64_t *__restrict__ node_start, int n_jobs,
                                       uint64_t total_nodes, int initial) {
@@ -100,10 +122,18 @@ __global__ void batch_estimate_kernel(JobDev *jobs, const uint64_t *__restrict__
         const int j = find_job(node_start, n_jobs, x);
         JobDev &J = jobs[j];
         if (!initial && J.state != 0) continue;
+        if (!initial && pass_again(J)) continue;
         const int t = initial ? 0 : J.t + 1;
         const double *c_prev = t ? J.c[(t - 1) & 1] : nullptr;
-        estimate_node(J.regs[t & 1], J.n, J.p, J.S, t, J.alpha_mm, J.lc, c_prev, J.c[t & 1], J.sum_d, &J.inc,
-                      (uint32_t)(x - node_start[j]), lane);
+        const uint32_t v = (uint32_t)(x - node_start[j]);
+        const uint32_t *top = J.codes && !initial ? J.win + (1u << J.p) : nullptr;
+        uint32_t at_top = 0;
+        estimate_node(J.regs[t & 1], J.n, J.p, J.S, t, J.alpha_mm, J.lc, c_prev, J.c[t & 1], J.sum_d, &J.inc, v, lane,
+                      false, top, &at_top);
+        if (top && lane == 0) {
+            J.full[v] = at_top == (1u << J.p) ? 1u : 0u;
+            if (v % kTopSample == 0) atomicAdd(&J.n_top, (unsigned long long)at_top);
+        }
     }
 }
 
@@ -193,8 +223,7 @@ __global__ void __launch_bounds__(kEngineWarps * 32) batch_union_kernel(JobDev *
             }
             q -= J.tblocks;
             if (threadIdx.x == 0) {
-                // every pass builds the slice's tables, but a scattered pass 1
-                s_ok = wait_tables(J.tab_done + s, (uint32_t)(t - J.first) * (uint32_t)J.tblocks);
+                s_ok = wait_tables(J.tab_done + s, (uint32_t)J.tblocks);
                 if (!s_ok) atomicExch(error, 1);
             }
             __syncthreads();
@@ -222,8 +251,142 @@ __global__ void __launch_bounds__(kEngineWarps * 32) batch_union_kernel(JobDev *
     }
 }
 
-// One thread per job: close the pass, apply the stop rule, reset the flags and
-// the union's item counter; report whether any job still runs.
+// Dynamic shared memory of a code union CTA: as engine_runs_smem.
+template <int S>
+constexpr size_t engine_code_smem() {
+    return engine_runs_smem<S>();
+}
+
+// Code union of the running jobs whose pass gathers K-bit codes, in code slices
+// of S bytes a node: the queue and the waits of batch_union_kernel (table items
+// of a code slice, then blocks of kEngineBlock groups), with the tables packed
+// from the registers (code_table_item) and each group gathered and settled by
+// one warp (code_group, code_store).  A CTA that meets a job whose pass is of
+// another kind moves the queue past all of that job's items.  64 registers (4
+// CTAs of 8 warps an SM) as in the single-graph kernel's measurement.
+template <int S, int K>
+__global__ void __launch_bounds__(kEngineWarps * 32, 4) batch_code_kernel(JobDev *jobs,
+                                                                         const uint32_t *__restrict__ gjobs,
+                                                                         const uint64_t *__restrict__ item_start,
+                                                                         int n_jobs, uint64_t total_items,
+                                                                         unsigned long long *counter, int *error) {
+    constexpr int W16 = S / 16;
+    constexpr uint32_t B = (uint32_t)TableShape<S>::B;
+    extern __shared__ __align__(128) unsigned char s_dyn[];
+    __shared__ unsigned long long s_item;
+    __shared__ uint32_t s_next;
+    __shared__ int s_ok;
+    const int lane = threadIdx.x & 31;
+    const int wib = threadIdx.x >> 5;
+    LkStage &st = reinterpret_cast<LkStage *>(s_dyn)[wib];
+    uint4 *part = reinterpret_cast<uint4 *>(s_dyn + (size_t)kEngineWarps * sizeof(LkStage)) +
+                  (size_t)wib * kEngineGroupNodes * W16;
+    uint8_t *s_tab = s_dyn + (size_t)kEngineWarps * sizeof(LkStage) + (size_t)kEngineWarps * kEngineGroupNodes * S;
+    uint32_t phase = 0;
+    lk_stage_init(st, lane);
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            s_item = atomicAdd(counter, 1ull);
+            s_next = 0;
+        }
+        __syncthreads();
+        const uint64_t item = s_item;
+        if (item >= total_items) break;
+        const int k = find_job(item_start, n_jobs, item);
+        JobDev &J = jobs[gjobs[k]];
+        if (J.state != 0 || J.K != K) {
+            if (threadIdx.x == 0) atomicMax(counter, (unsigned long long)item_start[k + 1]);
+            continue;
+        }
+        const uint32_t n = J.n;
+        const uint32_t tblocks = (n + B - 1u) / B;
+        const uint64_t per_slice = (uint64_t)((J.uunits + kEngineBlock - 1) / kEngineBlock) + tblocks;
+        const uint64_t r = item - item_start[k];
+        const uint32_t s = (uint32_t)(r / per_slice);
+        const uint64_t q = r % per_slice;
+        const uint32_t c0 = s * W16;
+        const int t = J.t + 1, s_log2 = __ffs(J.S) - 1;
+        const uint8_t *cur = J.regs[(t - 1) & 1];
+        uint8_t *nxt = J.regs[t & 1];
+        uint8_t *tab = J.tab + (uint64_t)s * table_rows(J.scheme) * n * S;
+        const uint32_t m = 1u << J.p;
+        const CodeWindow win{J.win + m, J.win + m + m / 4u};
+        if (q < tblocks) {
+            code_table_item<S, K, false>(cur, tab, n, s_log2, c0, (uint32_t)q * B, s_tab, J.scheme, win);
+            __threadfence();  // every writer publishes its table rows device-wide
+            __syncthreads();
+            if (threadIdx.x == 0) atomicAdd(J.tab_done + s, 1u);
+            continue;
+        }
+        if (threadIdx.x == 0) {
+            s_ok = wait_tables(J.tab_done + s, tblocks);
+            if (!s_ok) atomicExch(error, 1);
+        }
+        __syncthreads();
+        if (!s_ok) continue;
+        const uint32_t u0 = (uint32_t)(q - tblocks) * kEngineBlock;
+        const uint32_t u1 = min(u0 + kEngineBlock, J.uunits);
+        for (;;) {
+            uint32_t x = 0;
+            if (lane == 0) x = atomicAdd(&s_next, 1u);
+            x = u0 + __shfl_sync(0xffffffffu, x, 0);
+            if (x >= u1) break;
+            const GroupItem &gi = J.groups[x];
+            for (int w = lane; w < kEngineGroupNodes * W16; w += 32) part[w] = make_uint4(0, 0, 0, 0);
+            bool gather = true;
+            if (K == 1) {  // nothing to gather for a group whose registers are all at the top
+                gather = false;
+#pragma unroll
+                for (int j = 0; j < kEngineGroupNodes; j++) {
+                    const uint32_t v = gi.node[j];
+                    gather |= v != 0xffffffffu && !J.full[v];
+                }
+            }
+            __syncwarp();
+            if (gather)
+                code_group<S, K, kEngineGroupNodes>(gi, J.grows, J.gcls, tab, part, st, phase, lane, error, 0u, 1u,
+                                                    (uint32_t)kLkChunk);
+            __syncwarp();
+            bool changed = false;
+            for (int w = lane; w < kEngineGroupNodes * W16; w += 32) {
+                const uint32_t v = gi.node[w / W16];
+                if (v == 0xffffffffu) continue;
+                const uint32_t u = c0 + (uint32_t)(w % W16);
+                uint32_t chg16, open16;
+                code_store<K, false>(part[w], cur, nxt, n, s_log2, v, u, win, chg16, open16);
+                changed |= chg16 != 0u;
+                if (open16) code_push_open<K, false>(open16, v, u, J.list, J.list_cap, &J.open);
+            }
+            if (__any_sync(0xffffffffu, changed) && lane == 0) {
+                if (*reinterpret_cast<volatile uint32_t *>(&J.changed) == 0u) atomicOr(&J.changed, 1u);
+            }
+            __syncwarp();
+        }
+    }
+}
+
+// The pieces that this pass's code unions left open (code_open_piece),
+// kOpenCtas CTAs a job.
+constexpr unsigned kOpenCtas = 16;
+__global__ void __launch_bounds__(256) batch_open_kernel(JobDev *jobs) {
+    __shared__ uint4 s_max[8];
+    JobDev &J = jobs[blockIdx.x / kOpenCtas];
+    if (J.state != 0 || !J.K || pass_again(J)) return;
+    const int t = J.t + 1;
+    const uint32_t count = min(J.open, J.list_cap);
+    for (uint32_t e = blockIdx.x % kOpenCtas; e < count; e += kOpenCtas) {
+        const uint32_t v = J.list[e].x, byte = 16u * J.list[e].y;
+        const RunItem &it = J.items[v];  // no split hubs: one item per node, in id order
+        if (code_open_piece<false>(v, byte, it.b, it.b + it.cnt, J.lk, J.regs[(t - 1) & 1], J.regs[t & 1], J.n,
+                                   __ffs(J.S) - 1, J.scheme, s_max))
+            atomicOr(&J.changed, 1u);
+    }
+}
+
+// One thread per job: close the pass (or leave it to be done again), apply the
+// stop rule, choose the next pass's codes, reset the flags, the tables' counts
+// and the union's item counters; report whether any job still runs.
 __global__ void batch_step_kernel(JobDev *jobs, int n_jobs, unsigned long long *counters, int *any_running,
                                   cudaGraphConditionalHandle cond, int use_cond) {
     int running = 0;
@@ -231,13 +394,24 @@ __global__ void batch_step_kernel(JobDev *jobs, int n_jobs, unsigned long long *
         JobDev &J = jobs[j];
         if (J.state == 1) J.state = 2;
         if (J.state == 0) {
-            const int t = J.t + 1;
-            J.t = t;
-            bool stop = J.conv ? (J.inc == 0u) : (J.changed == 0u);
-            if (J.d > 0 && t >= J.d) stop = true;
-            if (stop) J.state = 1;
+            if (pass_again(J)) {
+                J.K = 4;
+                J.too_open = 1;
+            } else {
+                const int t = J.t + 1;
+                J.t = t;
+                bool stop = J.conv ? (J.inc == 0u) : (J.changed == 0u);
+                if (J.d > 0 && t >= J.d) stop = true;
+                if (stop) J.state = 1;
+                const double sampled = (double)((J.n + kTopSample - 1u) / kTopSample) * (double)(1u << J.p);
+                if (J.codes) J.K = (double)J.n_top >= kTopShare * sampled && !J.too_open ? 1 : 4;
+            }
             J.changed = 0u;
             J.inc = 0u;
+            J.open = 0u;
+            J.n_top = 0ull;
+            if (J.mode == 2)
+                for (int s = 0; s < J.slices; s++) J.tab_done[s] = 0u;
         }
         running |= (J.state == 0);
     }
@@ -304,6 +478,7 @@ int make_jobdev(const vga_graph *g, int p, int d, uint64_t seed, int conv, const
                 int group_nodes) {
     JobDev J{};
     const uint64_t n = g->n, m = 1ull << p;
+    uint64_t rows_used = 0;
     uint64_t o = 0;
     J.regs[0] = ws + o; o = align256(o + n * m);
     J.regs[1] = ws + o; o = align256(o + n * m);
@@ -331,6 +506,7 @@ int make_jobdev(const vga_graph *g, int p, int d, uint64_t seed, int conv, const
             J.gcls = groups.cls;
             J.hub_units = (uint32_t)list.hub_items;
             J.uunits = (uint32_t)(list.hub_items + groups.count);
+            rows_used = groups.rows_used;
         }
     } else {
         J.units = g->n;
@@ -338,6 +514,23 @@ int make_jobdev(const vga_graph *g, int p, int d, uint64_t seed, int conv, const
         if (p <= kFirstPassMaxP) J.tab = ws + o;  // the keys of pass 1's scatter (job_layout)
     }
     J.first = p <= kFirstPassMaxP ? 1 : 0;
+    if (L.mode == 2) {
+        // the code tables take at most half of the byte tables' region
+        const uint64_t tab_bytes = (uint64_t)table_rows(L.scheme) * n * m, pieces = n * m / 16;
+        uint64_t q = align256(tab_bytes / 2);
+        const uint64_t off_win = q;   q = align256(q + 6 * m);
+        const uint64_t off_full = q;  q = align256(q + n);
+        const uint64_t off_list = q;  q += 8 * pieces;
+        J.codes = J.first && J.hub_units == 0 && J.groups && m >= 128 && L.S >= 32 && q <= tab_bytes &&
+                  pieces < (1ull << 32);
+        if (J.codes) {
+            J.win = reinterpret_cast<uint32_t *>(J.tab + off_win);
+            J.full = J.tab + off_full;
+            J.list = reinterpret_cast<uint2 *>(J.tab + off_list);
+            J.list_cap = (uint32_t)pieces;
+            J.open_cap = (uint32_t)std::min((double)pieces, code_open_cap((double)rows_used, (uint32_t)m, g->n_edges, n));
+        }
+    }
     J.off = g->d_offsets;
     J.bytes = g->d_bytes;
     J.comp = g->d_comp;
@@ -379,7 +572,7 @@ int upload_lc_tables(uint8_t *dst, const bool *used, cudaStream_t stream) {
 
 uint64_t engine_arrays_bytes(int cap) {
     const uint64_t c = (uint64_t)std::max(cap, 1);
-    return align256(sizeof(JobDev) * c) + align256(8 * (c + 1)) + align256(4 * c) + align256(8 * (c + kGroups)) +
+    return align256(sizeof(JobDev) * c) + align256(8 * (c + 1)) + align256(8 * c) + align256(8 * (2 * c + kGroups)) +
            align256(8 * kGroups) + 256 + align256(4 * c) + align256(8 * (c + kGroups));
 }
 
@@ -389,8 +582,8 @@ EngineArrays engine_arrays_at(uint8_t *base, int cap) {
     uint64_t o = 0;
     A.jobs = reinterpret_cast<JobDev *>(base + o); o = align256(o + sizeof(JobDev) * c);
     A.node_start = reinterpret_cast<uint64_t *>(base + o); o = align256(o + 8 * (c + 1));
-    A.gjobs = reinterpret_cast<uint32_t *>(base + o); o = align256(o + 4 * c);
-    A.item_start = reinterpret_cast<uint64_t *>(base + o); o = align256(o + 8 * (c + kGroups));
+    A.gjobs = reinterpret_cast<uint32_t *>(base + o); o = align256(o + 8 * c);
+    A.item_start = reinterpret_cast<uint64_t *>(base + o); o = align256(o + 8 * (2 * c + kGroups));
     A.counters = reinterpret_cast<unsigned long long *>(base + o); o = align256(o + 8 * kGroups);
     A.any_running = reinterpret_cast<int *>(base + o);
     A.error = reinterpret_cast<int *>(base + o + 4);
@@ -401,7 +594,12 @@ EngineArrays engine_arrays_at(uint8_t *base, int cap) {
     return A;
 }
 
-int group_index(int mode, int S) { return (mode == 2 ? 7 : 0) + (31 - __builtin_clz((unsigned)S)) - 4; }
+int group_index(int mode, int S, int K) {
+    return (K == 1 ? 21 : K == 4 ? 14 : mode == 2 ? 7 : 0) + (31 - __builtin_clz((unsigned)S)) - 4;
+}
+
+// Bytes of a code slice's row in a job's K-bit passes, and its code slices.
+int code_slice_bytes(const JobDev &J, int K) { return std::min(J.S, (1 << J.p) * K / 8); }
 
 template <int S, bool RUNS>
 size_t union_smem() {
@@ -416,7 +614,13 @@ int union_smem_attrs() {
 #define VGA_A(SS)                                                                                                 \
     if (err == cudaSuccess)                                                                                       \
         err = cudaFuncSetAttribute(batch_union_kernel<SS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,    \
-                                   (int)engine_runs_smem<SS>());
+                                   (int)engine_runs_smem<SS>());                                                   \
+    if (err == cudaSuccess)                                                                                       \
+        err = cudaFuncSetAttribute(batch_code_kernel<SS, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,        \
+                                   (int)engine_code_smem<SS>());                                                  \
+    if (err == cudaSuccess)                                                                                       \
+        err = cudaFuncSetAttribute(batch_code_kernel<SS, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,        \
+                                   (int)engine_code_smem<SS>());
         VGA_A(16) VGA_A(32) VGA_A(64) VGA_A(128) VGA_A(256) VGA_A(512) VGA_A(1024)
 #undef VGA_A
     });
@@ -432,9 +636,18 @@ int union_grid(int sms) {
     return std::max(1, sms * std::max(1, per_sm));
 }
 
-int union_grid_for(int mode, int S, int sms) {
+template <int S, int K>
+int code_grid(int sms) {
+    int per_sm = 1;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_code_kernel<S, K>, kEngineWarps * 32,
+                                                  engine_code_smem<S>());
+    return std::max(1, sms * std::max(1, per_sm));
+}
+
+int union_grid_for(int mode, int S, int K, int sms) {
 #define VGA_G(SS)                                                                               \
     case SS:                                                                                    \
+        if (K) return K == 1 ? code_grid<SS, 1>(sms) : code_grid<SS, 4>(sms);                   \
         return mode == 2 ? union_grid<SS, true>(sms) : union_grid<SS, false>(sms);
     switch (S) {
         VGA_G(16) VGA_G(32) VGA_G(64) VGA_G(128) VGA_G(256) VGA_G(512) VGA_G(1024)
@@ -459,7 +672,15 @@ int engine_upload(const EngineArrays &A, const std::vector<JobDev> &jobs, Engine
     std::vector<uint64_t> ns(nj + 1, 0);
     for (int k = 0; k < nj; k++) ns[k + 1] = ns[k] + jobs[k].n;
     std::vector<std::vector<uint32_t>> members(kGroups);
-    for (int k = 0; k < nj; k++) members[group_index(jobs[k].mode, jobs[k].S)].push_back((uint32_t)k);
+    for (int k = 0; k < nj; k++) {
+        const JobDev &J = jobs[k];
+        if (J.codes) {  // pass 1 is the scatter, every later one gathers codes
+            members[group_index(2, code_slice_bytes(J, 4), 4)].push_back((uint32_t)k);
+            members[group_index(2, code_slice_bytes(J, 1), 1)].push_back((uint32_t)k);
+        } else {
+            members[group_index(J.mode, J.S, 0)].push_back((uint32_t)k);
+        }
+    }
     std::vector<uint32_t> gj;
     std::vector<uint64_t> is;
     E->groups.clear();
@@ -467,8 +688,9 @@ int engine_upload(const EngineArrays &A, const std::vector<JobDev> &jobs, Engine
         if (members[g].empty()) continue;
         EngineGroup G;
         G.index = g;
-        G.mode = jobs[members[g][0]].mode;
-        G.S = jobs[members[g][0]].S;
+        G.K = g >= 21 ? 1 : g >= 14 ? 4 : 0;
+        G.mode = g >= 7 ? 2 : 1;
+        G.S = 16 << (g % 7);
         G.n = (int)members[g].size();
         G.gjob_off = gj.size();
         G.item_off = is.size();
@@ -477,12 +699,17 @@ int engine_upload(const EngineArrays &A, const std::vector<JobDev> &jobs, Engine
             gj.push_back(k);
             is.push_back(items);
             const JobDev &J = jobs[k];
-            items += (uint64_t)J.slices * ((uint64_t)((J.uunits + kEngineBlock - 1) / kEngineBlock) +
-                                           (J.mode == 2 ? (uint64_t)J.tblocks : 0));
+            const uint64_t ublocks = (J.uunits + kEngineBlock - 1) / kEngineBlock;
+            if (G.K) {
+                const uint64_t B = G.S >= 1024 ? 16 : 32;  // rows of a table item (TableShape)
+                items += ((1ull << J.p) * G.K / 8 / G.S) * (ublocks + (J.n + B - 1) / B);
+            } else {
+                items += (uint64_t)J.slices * (ublocks + (J.mode == 2 ? (uint64_t)J.tblocks : 0));
+            }
         }
         is.push_back(items);
         G.total_items = items;
-        G.grid = (unsigned)union_grid_for(G.mode, G.S, sms);
+        G.grid = (unsigned)union_grid_for(G.mode, G.S, G.K, sms);
         E->groups.push_back(G);
     }
     if (nj) VGA_CHECK_CUDA(cudaMemcpyAsync(A.jobs, jobs.data(), sizeof(JobDev) * nj, cudaMemcpyHostToDevice, stream));
@@ -507,14 +734,16 @@ int engine_start(const EngineArrays &A, const std::vector<JobDev> &jobs, const E
     for (const JobDev &J : jobs) {
         VGA_CHECK_CUDA(cudaMemsetAsync(J.regs[0], 0, (uint64_t)J.n << J.p, stream));
         // split hubs merge into the pass's output by atomic max: it must start below the result
-        if (J.mode == 2) VGA_CHECK_CUDA(cudaMemsetAsync(J.regs[1], 0, (uint64_t)J.n << J.p, stream));
-        VGA_CHECK_CUDA(cudaMemsetAsync(J.sum_d, 0, 8ull * J.n, stream));
+        if (J.mode == 2 && !J.codes) VGA_CHECK_CUDA(cudaMemsetAsync(J.regs[1], 0, (uint64_t)J.n << J.p, stream));
+        if (J.codes) VGA_CHECK_CUDA(cudaMemsetAsync(J.win, 0, 4ull << J.p, stream));
         if (J.mode == 2) VGA_CHECK_CUDA(cudaMemsetAsync(J.tab_done, 0, 4ull * J.slices, stream));
     }
     if (!E.n_jobs) return VGA_OK;
     batch_init_kernel<<<E.grid_nodes, 256, 0, stream>>>(A.jobs, A.node_start, E.n_jobs, E.total_nodes);
     count_launch();
     batch_estimate_kernel<<<E.grid_warps, 256, 0, stream>>>(A.jobs, A.node_start, E.n_jobs, E.total_nodes, 1);
+    count_launch();
+    batch_window_kernel<<<E.n_jobs, 256, 0, stream>>>(A.jobs);
     count_launch();
     VGA_CHECK_CUDA(cudaGetLastError());
     // pass 1 of the run-aware jobs: the scatter, one launch per precision
@@ -590,6 +819,13 @@ void launch_group(const EngineArrays &A, const EngineGroup &G, cudaStream_t stre
                                                                          G.total_items, A.counters + G.index, A.error);
 }
 
+template <int S, int K>
+void launch_code_group(const EngineArrays &A, const EngineGroup &G, cudaStream_t stream, int grid_pct) {
+    const unsigned grid = (grid_pct > 0 && grid_pct < 100) ? std::max(1u, G.grid * (unsigned)grid_pct / 100u) : G.grid;
+    batch_code_kernel<S, K><<<grid, kEngineWarps * 32, engine_code_smem<S>(), stream>>>(
+        A.jobs, A.gjobs + G.gjob_off, A.item_start + G.item_off, G.n, G.total_items, A.counters + G.index, A.error);
+}
+
 EngineForks::~EngineForks() {
     for (cudaEvent_t e : events) cudaEventDestroy(e);
     for (cudaStream_t s : streams) cudaStreamDestroy(s);
@@ -625,7 +861,9 @@ int engine_pass(const EngineArrays &A, const EngineSet &E, cudaStream_t stream, 
         gi++;
 #define VGA_G(SS)                                                                         \
     case SS:                                                                              \
-        if (G.mode == 2) launch_group<SS, true>(A, G, gs, grid_pct);                      \
+        if (G.K == 4) launch_code_group<SS, 4>(A, G, gs, grid_pct);                       \
+        else if (G.K == 1) launch_code_group<SS, 1>(A, G, gs, grid_pct);                  \
+        else if (G.mode == 2) launch_group<SS, true>(A, G, gs, grid_pct);                 \
         else launch_group<SS, false>(A, G, gs, grid_pct);                                 \
         break;
         switch (G.S) {
@@ -637,6 +875,12 @@ int engine_pass(const EngineArrays &A, const EngineSet &E, cudaStream_t stream, 
     for (int k = 0; k < n_aux; k++) {
         VGA_CHECK_CUDA(cudaEventRecord(forks->events[1 + k], forks->streams[k]));
         VGA_CHECK_CUDA(cudaStreamWaitEvent(stream, forks->events[1 + k], 0));
+    }
+    bool codes = false;
+    for (const EngineGroup &G : E.groups) codes |= G.K != 0;
+    if (codes) {
+        batch_open_kernel<<<(unsigned)E.n_jobs * kOpenCtas, 256, 0, stream>>>(A.jobs);
+        count_launch();
     }
     batch_estimate_kernel<<<E.grid_warps, 256, 0, stream>>>(A.jobs, A.node_start, E.n_jobs, E.total_nodes, 0);
     count_launch();

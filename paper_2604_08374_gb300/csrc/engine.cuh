@@ -11,7 +11,9 @@ namespace vga {
 constexpr int kEngineWarps = 8;
 constexpr int kEngineGroupNodes = 4;  // nodes per group of the grouped union in the engine
 constexpr uint32_t kEngineBlock = 16;  // work units (hub chunks, node groups) per union block of the queue
-constexpr int kGroups = 14;  // union kernels: (per neighbour | per run) x slice width 16..1024
+// union kernels: (per neighbour | per run | 4-bit codes | 1-bit codes) x slice
+// width 16..1024
+constexpr int kGroups = 28;
 
 // One analysis as the batched kernels see it (device memory).
 struct JobDev {
@@ -21,7 +23,7 @@ struct JobDev {
     const uint32_t *lk;      // run-aware union: the graph's range lookups
     const RunItem *items;    // and its work list (nodes, split hubs' chunks)
     uint8_t *tab;            // table regions, slice s at tab + s * table_rows(scheme) * N * S
-    uint32_t *tab_done;      // per slice: table items finished, over all passes
+    uint32_t *tab_done;      // per slice: table items finished in this pass
     uint8_t *regs[2];   // slice-major [m/S][N][S]; pass t reads regs[(t-1)&1], writes regs[t&1]
     double *c[2];       // c_t lives in c[t&1]
     double *sum_d;
@@ -41,6 +43,18 @@ struct JobDev {
     int mode;               // 1 one gather per neighbour, 2 per run (sparse tables)
     int tblocks;            // table items per slice (mode 2), TableShape<S>::B rows each
     int scheme;             // table scheme of the lookups (mode 2)
+    // Codes (codes.cuh) from the second pass on, for run-aware jobs without split
+    // hubs.  Everything lies in the table region, whose lower half holds the
+    // code tables: win (gmax, then the window's top and low words), full, list.
+    int codes;
+    int K;                  // bits per code of the pass in progress (0: the scattered first pass)
+    int too_open;           // a one-bit pass left more than open_cap pieces open and was done again in 4 bits
+    uint32_t *win;
+    uint8_t *full;          // nodes whose registers have all reached the window's top
+    uint2 *list;            // open pieces of the pass {node, 16-byte piece}, list_cap = all there are
+    uint32_t list_cap, open_cap;
+    uint32_t open;          // pieces the pass left open
+    unsigned long long n_top;  // registers at the top, over every kTopSample-th node
     int first;              // 1: pass 1 is the scatter of the nodes' keys (engine_start; keys in tab)
     uint32_t changed, inc;  // flags of the pass in progress
     int t;                  // passes completed
@@ -58,8 +72,8 @@ struct JobLayout {
 struct EngineArrays {
     JobDev *jobs = nullptr;
     uint64_t *node_start = nullptr;         // cap + 1: prefix of nodes over all jobs
-    uint32_t *gjobs = nullptr;              // cap: job indices ordered by union group
-    uint64_t *item_start = nullptr;         // cap + kGroups: per group, prefix of items over its jobs
+    uint32_t *gjobs = nullptr;              // 2 cap: job indices ordered by union group
+    uint64_t *item_start = nullptr;         // 2 cap + kGroups: per group, prefix of items over its jobs
     unsigned long long *counters = nullptr; // kGroups: the groups' item queues
     int *any_running = nullptr;
     int *error = nullptr;                   // set when a bounded wait gave up
@@ -68,9 +82,10 @@ struct EngineArrays {
     int cap = 0;
 };
 
-// One union kernel launch: the jobs sharing a union variant and slice width.
+// One union kernel launch: the jobs sharing a union variant and slice width
+// (K > 0: the code passes of K bits; a job with codes is in both code groups).
 struct EngineGroup {
-    int mode = 1, S = 0, n = 0;
+    int mode = 1, S = 0, n = 0, K = 0;
     uint64_t gjob_off = 0, item_off = 0, total_items = 0;
     unsigned grid = 1;
     int index = 0;

@@ -542,10 +542,8 @@ constexpr int kTrackMaxSlices = 32;
 // this share of the (node, slice) pairs: after a pass that changed more,
 // nearly every node has a changed neighbour in every slice.
 constexpr double kTrackBelow = 0.01;
-// A pass gathers one-bit codes once this share of the registers has reached
-// its maximum, and goes back to four bits after a one-bit pass that left more
-// than kOpenShare of the 16-byte register pieces open.
-constexpr double kTopShare = 0.75;
+// A run goes back from one-bit codes (kTopShare) to four after a one-bit pass
+// that left more than this share of the 16-byte register pieces open.
 constexpr double kOpenShare = 0.2;
 
 
@@ -918,11 +916,8 @@ static int launch_codes(const Plan &P, const vga_graph *g, int K, uint8_t *base,
     C.flags = flags;
     C.full = base + P.off_full;
     C.need = reinterpret_cast<uint32_t *>(base + P.off_need);
-    // Open pieces are settled one by one while their neighbours' 32-byte
-    // sectors stay below an eighth of the rows a whole byte union gathers.
     C.list = reinterpret_cast<uint2 *>(base + P.off_list);
-    const double piece = 32.0 * (double)g->n_edges / (double)P.n;
-    C.list_cap = (uint32_t)std::min((double)P.n, (double)P.groups.rows_used * P.node_bytes / 8.0 / std::max(piece, 1.0));
+    C.list_cap = (uint32_t)std::min((double)P.n, code_open_cap((double)P.groups.rows_used, P.node_bytes, g->n_edges, P.n));
     // Warps per group: enough for twice the warps the GPU holds (about 40 an
     // SM), no more than leaves each about 32 rows.
     int dev = 0, sms = 1;

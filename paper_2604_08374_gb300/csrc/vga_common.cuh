@@ -235,6 +235,16 @@ int ensure_group_list(const vga_graph *g, int scheme, uint32_t hub_lookups, int 
 // One pass of the grouped union over register codes (codes.cu): table and
 // union of one code slice of S bytes a node at a time.
 constexpr int kCodeNodes = 4;  // nodes per group of the code kernels
+// A pass gathers one-bit codes once this share of the registers has reached its
+// maximum.
+constexpr double kTopShare = 0.75;
+// Open pieces of a code pass that are settled one by one: while their
+// neighbours' 32-byte sectors stay below an eighth of the bytes (node_bytes a
+// row) that a union of the groups' rows gathers.
+inline double code_open_cap(double rows_used, uint32_t node_bytes, uint64_t edges, uint64_t n) {
+    const double piece = 32.0 * (double)edges / (double)n;
+    return rows_used * node_bytes / 8.0 / (piece > 1.0 ? piece : 1.0);
+}
 struct CodePass {
     const GroupList *groups = nullptr;
     const uint8_t *cur = nullptr;      // the node's registers, slice-major with slices of 2^s_log2 bytes

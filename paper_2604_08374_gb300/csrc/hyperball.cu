@@ -524,10 +524,12 @@ struct Plan {
     bool first_scatter = false;  // pass 1 by the scatter of the nodes' keys (kept at off_tab)
     int track = 0;               // runs mode, slices <= 32: change tracking (0 off, 1 automatic, 2 every pass)
     bool codes = false;          // passes from the second on gather register codes (codes.cuh)
+    bool csr_codes = false;      // per-neighbour mode: the same, where the workspace has room past `total`
+    int code_bits = 4;           // widest code that has room
     uint64_t n = 0;
     // workspace layout (byte offsets, 256-aligned)
     uint64_t off_cur = 0, off_next = 0, off_c0 = 0, off_c1 = 0, off_sum = 0, off_lc = 0, off_flags = 0, off_tab = 0,
-             off_chg = 0, off_need = 0, off_ortab = 0, off_win = 0, off_full = 0, off_list = 0, chg_bytes = 0, total = 0;
+             off_chg = 0, off_need = 0, off_ortab = 0, off_win = 0, off_full = 0, off_list = 0, off_codes = 0, chg_bytes = 0, total = 0;
 };
 
 static uint64_t align256(uint64_t x) { return (x + 255) & ~255ull; }
@@ -711,7 +713,24 @@ static int make_plan(const vga_graph *g, int p, const vga_tuning *tune, Plan *P)
         o = align256(o + 8 * P->n);
     }
     P->total = o;
+    // Per-neighbour mode: codes where a workspace happens to hold them past the
+    // bytes that the mode asks for (plan_csr_codes).
+    P->csr_codes = P->mode == kModePerEdge && P->track != 2 && P->m >= 128 && P->slices <= kTrackMaxSlices &&
+                   S >= (P->nib ? 16 : 32) && P->n > 0 && P->n * P->node_bytes / 16 < (1ull << 32);
     return VGA_OK;
+}
+
+// Codes of the per-neighbour mode, in the bytes of a workspace past P->total:
+// 4-bit ones, or 1-bit ones only, or none.
+static void plan_csr_codes(Plan *P, uint64_t ws_bytes) {
+    if (!P->csr_codes) return;
+    uint64_t o = P->total;
+    P->off_win = o;   o = align256(o + 4ull * P->m + 2ull * P->node_bytes);
+    P->off_full = o;  o = align256(o + P->n);
+    P->off_list = o;  o = align256(o + 8 * P->n);
+    P->off_codes = o;
+    P->code_bits = o + P->n * P->m / 2 <= ws_bytes ? 4 : 1;
+    P->codes = o + P->n * P->m * P->code_bits / 8 <= ws_bytes;
 }
 
 
@@ -965,6 +984,56 @@ static int launch_codes(const Plan &P, const vga_graph *g, int K, uint8_t *base,
     return VGA_OK;
 }
 
+// One pass of the per-neighbour union over register codes of K bits.  One that
+// leaves more pieces open than are worth settling one by one is done again over
+// the bytes.
+static int launch_codes_csr(const Plan &P, const vga_graph *g, int K, uint8_t *base, const uint8_t *cur, uint8_t *nxt,
+                            uint32_t *flags, cudaStream_t stream, std::vector<PendingTiming> *timings, uint8_t *chg) {
+    CodePass C;
+    C.cur = cur;
+    C.nxt = nxt;
+    C.tab = base + P.off_codes;
+    C.n = (uint32_t)P.n;
+    C.s_log2 = __builtin_ctz((unsigned)P.S);
+    C.nib = P.nib != 0;
+    C.K = K;
+    C.S = (int)std::min<uint32_t>(P.m * (uint32_t)K / 8u, 1024u);
+    C.top = reinterpret_cast<const uint32_t *>(base + P.off_win) + P.m;
+    C.low = C.top + P.node_bytes / 4;
+    C.flags = flags;
+    C.full = base + P.off_full;
+    C.list = reinterpret_cast<uint2 *>(base + P.off_list);
+    C.list_cap = (uint32_t)std::min((double)P.n, code_open_cap((double)g->n_edges, P.node_bytes, g->n_edges, P.n));
+    C.chg = chg;
+    C.stream = stream;
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    PendingTiming pt{};
+    if (timings) {
+        VGA_CHECK_CUDA(cudaEventCreate(&pt.start));
+        VGA_CHECK_CUDA(cudaEventCreate(&pt.stop));
+        VGA_CHECK_CUDA(cudaEventRecord(pt.start, stream));
+    }
+    VGA_TRY(launch_code_csr(C, P.m, g->d_offsets, g->d_bytes, sms));
+    if (timings) {
+        VGA_CHECK_CUDA(cudaEventRecord(pt.stop, stream));
+        pt.edges = g->n_edges;
+        pt.gather_bytes = g->n_edges * (uint64_t)P.m * K / 8;
+        pt.hbm_bytes = g->n_bytes + 8 * (P.n + 1) + 2 * P.n * (uint64_t)P.node_bytes;
+        pt.S = C.S;
+        pt.mode = P.mode;
+        pt.rows = 1;
+        timings->push_back(pt);
+    }
+    uint32_t open = 0;
+    VGA_CHECK_CUDA(cudaMemcpyAsync(&open, flags + 9, 4, cudaMemcpyDeviceToHost, stream));
+    VGA_CHECK_CUDA(cudaStreamSynchronize(stream));
+    if (open > C.list_cap)
+        VGA_TRY(launch_union(P, g, cur, nxt, nullptr, flags, stream, timings, nullptr, chg));
+    return VGA_OK;
+}
+
 // First pass of a run (or of a register-range shard holding slices [s0, s1))
 // by the scatter of the nodes' keys; `keys` were written by hb_init_kernel.
 static int launch_first_pass(const Plan &P, const vga_graph *g, const void *keys, uint8_t *nxt, uint32_t s0,
@@ -1182,6 +1251,7 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
                   ws, (unsigned long long)P.total);
         return VGA_EINVAL;
     }
+    if (!own_ws.ptr) plan_csr_codes(&P, ws_bytes);
     uint8_t *base = static_cast<uint8_t *>(ws);
     uint8_t *cur = base + P.off_cur;
     uint8_t *nxt = base + P.off_next;
@@ -1261,13 +1331,15 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
             int K = 0;
             if (P.codes && t >= 2) {
                 const bool most = (double)h.n_top >= kTopShare * (double)P.n * P.m;
-                K = most && !too_open && P.m >= 128 ? 1 : tracked ? 0 : 4;
+                K = most && !too_open && P.m >= 128 ? 1 : tracked || P.code_bits < 4 ? 0 : 4;
             }
             if (tracked && !K) VGA_TRY(launch_need(P, g, chg, ortab, need, stream, timed ? &timings : nullptr));
-            const uint64_t clear = K ? P.off_need + 4 * P.n - P.off_flags
+            const uint64_t clear = K && P.mode == kModeRuns ? P.off_need + 4 * P.n - P.off_flags
                                      : chg ? P.off_chg + P.chg_bytes - P.off_flags : sizeof(h);
             VGA_CHECK_CUDA(cudaMemsetAsync(flags, 0, clear, stream));
-            if (K) {
+            if (K && P.mode == kModePerEdge) {
+                VGA_TRY(launch_codes_csr(P, g, K, base, cur, nxt, flags, stream, timed ? &timings : nullptr, chg));
+            } else if (K) {
                 VGA_TRY(launch_codes(P, g, K, base, cur, nxt, flags, stream, timed ? &timings : nullptr, tracked, chg));
             } else if (t == 1 && keys)
                 VGA_TRY(launch_first_pass(P, g, keys, nxt, 0u, (uint32_t)P.slices, flags, stream,

@@ -266,6 +266,9 @@ struct CodePass {
 int launch_code_slice(const CodePass &C, int slice);
 // After the pass's slices: the open pieces, when they all fit the list.
 int launch_code_open(const CodePass &C, const uint64_t *lk_off, const uint32_t *lk, int sms);
+// The same over neighbour lists instead of groups, for a caller without range
+// lookups: `tab` takes the codes of all slices (N * m * K / 8 bytes).
+int launch_code_csr(const CodePass &C, uint32_t m, const uint64_t *off, const uint8_t *bytes, int sms);
 int launch_code_window(const uint32_t *gmax, uint32_t words, int nib, uint32_t *top, uint32_t *low,
                        cudaStream_t stream);
 

@@ -26,6 +26,7 @@
 
 #include "codes.cuh"
 #include "engine.cuh"
+#include "first_pass.cuh"
 
 namespace vga {
 
@@ -60,7 +61,14 @@ __global__ void batch_init_kernel(JobDev *jobs, const uint64_t *__restrict__ nod
                 uint32_t *g = J.win + (key >> 8);
                 if (*reinterpret_cast<volatile uint32_t *>(g) < (key & 0xffu)) atomicMax(g, key & 0xffu);
             }
-            if (J.p <= kKey16MaxP)
+            if (J.group_scatter) {
+                const uint32_t rho = key & 0xffu, k = (key >> 8) << 4 | (min(rho, 16u) - 1u);
+                if (rho >= 16u) atomicOr(J.win + (1u << J.p) + (key >> 8), 1u << min(rho - 16u, 31u));
+                if (J.p <= kGroupKey16MaxP)
+                    reinterpret_cast<uint16_t *>(J.tab)[v] = (uint16_t)k;
+                else
+                    reinterpret_cast<uint32_t *>(J.tab)[v] = k;
+            } else if (J.p <= kKey16MaxP)
                 reinterpret_cast<uint16_t *>(J.tab)[v] = KeyFmt<uint16_t>::pack(key);
             else
                 reinterpret_cast<uint32_t *>(J.tab)[v] = KeyFmt<uint32_t>::pack(key);
@@ -74,7 +82,7 @@ __global__ void batch_window_kernel(JobDev *jobs) {
     if (!J.codes) return;
     const uint32_t m = 1u << J.p;
     for (uint32_t k = threadIdx.x; k < m / 4u; k += blockDim.x)
-        window_word(J.win, k, false, J.win + m, J.win + m + m / 4u);
+        window_word(J.win, k, false, J.win + 2 * m, J.win + 2 * m + m / 4u);
 }
 
 // Pass 1 of the jobs in fjobs[0 .. n) (all of precision p, all fresh) as the
@@ -107,6 +115,27 @@ __global__ void __launch_bounds__(kFirstPassWarps * 32) batch_first_pass_kernel(
     }
 }
 
+// The same for jobs whose pass 1 takes whole groups (first_pass_group), one CTA
+// per group of the concatenated group lists.
+template <class K>
+__global__ void __launch_bounds__(kGroupScatterWarps * 32) batch_first_groups_kernel(JobDev *jobs,
+                                                                                    const uint32_t *__restrict__ fjobs,
+                                                                                    const uint64_t *__restrict__ fstart,
+                                                                                    int n, int p) {
+    extern __shared__ __align__(16) uint32_t s_cells[];
+    __shared__ GroupScatterShared sh;
+    const uint64_t total = fstart[n];
+    const uint32_t m = 1u << p;
+    for (uint64_t x = blockIdx.x; x < total; x += gridDim.x) {
+        const int k = find_job(fstart, n, x);
+        JobDev &J = jobs[fjobs[k]];
+        first_pass_group<false, K>(J.groups[x - fstart[k]], J.grows, J.gcls, reinterpret_cast<const K *>(J.tab), J.n, p,
+                                   J.scheme, __ffs(J.S) - 1, J.win, J.win + m, J.seed, J.regs[1], &J.changed, nullptr,
+                                   s_cells, sh);
+        __syncthreads();  // the cells are read before the next group clears them
+    }
+}
+
 // The one-bit pass just run left too much open: it is done again in 4 bits.
 __device__ __forceinline__ bool pass_again(const JobDev &J) { return J.K == 1 && J.open > J.open_cap; }
 
@@ -126,7 +155,7 @@ __global__ void batch_estimate_kernel(JobDev *jobs, const uint64_t *__restrict__
         const int t = initial ? 0 : J.t + 1;
         const double *c_prev = t ? J.c[(t - 1) & 1] : nullptr;
         const uint32_t v = (uint32_t)(x - node_start[j]);
-        const uint32_t *top = J.codes && !initial ? J.win + (1u << J.p) : nullptr;
+        const uint32_t *top = J.codes && !initial ? J.win + (2u << J.p) : nullptr;
         uint32_t at_top = 0;
         estimate_node(J.regs[t & 1], J.n, J.p, J.S, t, J.alpha_mm, J.lc, c_prev, J.c[t & 1], J.sum_d, &J.inc, v, lane,
                       false, top, &at_top);
@@ -311,7 +340,7 @@ __global__ void __launch_bounds__(kEngineWarps * 32, 4) batch_code_kernel(JobDev
         uint8_t *nxt = J.regs[t & 1];
         uint8_t *tab = J.tab + (uint64_t)s * table_rows(J.scheme) * n * S;
         const uint32_t m = 1u << J.p;
-        const CodeWindow win{J.win + m, J.win + m + m / 4u};
+        const CodeWindow win{J.win + 2 * m, J.win + 2 * m + m / 4u};
         if (q < tblocks) {
             code_table_item<S, K, false>(cur, tab, n, s_log2, c0, (uint32_t)q * B, s_tab, J.scheme, win);
             __threadfence();  // every writer publishes its table rows device-wide
@@ -518,11 +547,13 @@ int make_jobdev(const vga_graph *g, int p, int d, uint64_t seed, int conv, const
         // the code tables take at most half of the byte tables' region
         const uint64_t tab_bytes = (uint64_t)table_rows(L.scheme) * n * m, pieces = n * m / 16;
         uint64_t q = align256(tab_bytes / 2);
-        const uint64_t off_win = q;   q = align256(q + 6 * m);
+        const uint64_t off_win = q;   q = align256(q + 10 * m);
         const uint64_t off_full = q;  q = align256(q + n);
         const uint64_t off_list = q;  q += 8 * pieces;
         J.codes = J.first && J.hub_units == 0 && J.groups && m >= 128 && L.S >= 32 && q <= tab_bytes &&
                   pieces < (1ull << 32);
+        // whole groups while few indices can have several rho above 16 (run_impl)
+        J.group_scatter = J.codes && n >> p <= kGroupScatterNodes;
         if (J.codes) {
             J.win = reinterpret_cast<uint32_t *>(J.tab + off_win);
             J.full = J.tab + off_full;
@@ -735,7 +766,7 @@ int engine_start(const EngineArrays &A, const std::vector<JobDev> &jobs, const E
         VGA_CHECK_CUDA(cudaMemsetAsync(J.regs[0], 0, (uint64_t)J.n << J.p, stream));
         // split hubs merge into the pass's output by atomic max: it must start below the result
         if (J.mode == 2 && !J.codes) VGA_CHECK_CUDA(cudaMemsetAsync(J.regs[1], 0, (uint64_t)J.n << J.p, stream));
-        if (J.codes) VGA_CHECK_CUDA(cudaMemsetAsync(J.win, 0, 4ull << J.p, stream));
+        if (J.codes) VGA_CHECK_CUDA(cudaMemsetAsync(J.win, 0, 8ull << J.p, stream));
         if (J.mode == 2) VGA_CHECK_CUDA(cudaMemsetAsync(J.tab_done, 0, 4ull * J.slices, stream));
     }
     if (!E.n_jobs) return VGA_OK;
@@ -750,24 +781,25 @@ int engine_start(const EngineArrays &A, const std::vector<JobDev> &jobs, const E
     std::vector<uint32_t> fj;
     std::vector<uint64_t> fs;
     struct Launch {
-        int p, n;
+        int p, n, groups;
         size_t job_off, start_off;
     };
     std::vector<Launch> launches;
-    for (int p = 4; p <= kFirstPassMaxP; p++) {
-        Launch L{p, 0, fj.size(), fs.size()};
-        uint64_t items = 0;
-        for (size_t k = 0; k < jobs.size(); k++) {
-            if (!jobs[k].first || jobs[k].p != p) continue;
-            fj.push_back((uint32_t)k);
+    for (int groups = 0; groups < 2; groups++)
+        for (int p = 4; p <= kFirstPassMaxP; p++) {
+            Launch L{p, 0, groups, fj.size(), fs.size()};
+            uint64_t items = 0;
+            for (size_t k = 0; k < jobs.size(); k++) {
+                if (!jobs[k].first || jobs[k].p != p || jobs[k].group_scatter != groups) continue;
+                fj.push_back((uint32_t)k);
+                fs.push_back(items);
+                items += groups ? jobs[k].uunits : jobs[k].units;
+                L.n++;
+            }
+            if (!L.n) continue;
             fs.push_back(items);
-            items += jobs[k].units;
-            L.n++;
+            launches.push_back(L);
         }
-        if (!L.n) continue;
-        fs.push_back(items);
-        launches.push_back(L);
-    }
     if (launches.empty()) return VGA_OK;
     VGA_CHECK_CUDA(cudaMemcpyAsync(A.fjobs, fj.data(), 4 * fj.size(), cudaMemcpyHostToDevice, stream));
     VGA_CHECK_CUDA(cudaMemcpyAsync(A.fstart, fs.data(), 8 * fs.size(), cudaMemcpyHostToDevice, stream));
@@ -780,12 +812,27 @@ int engine_start(const EngineArrays &A, const std::vector<JobDev> &jobs, const E
         if (attr_err == cudaSuccess)
             attr_err = cudaFuncSetAttribute(batch_first_pass_kernel<uint32_t>,
                                             cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (attr_err == cudaSuccess)
+            attr_err = cudaFuncSetAttribute(batch_first_groups_kernel<uint32_t>,
+                                            cudaFuncAttributeMaxDynamicSharedMemorySize, 8 << kFirstPassMaxP);
     });
     VGA_CHECK_CUDA(attr_err);
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     for (const Launch &L : launches) {
+        if (L.groups) {
+            const size_t smem = 8ull << L.p;
+            const unsigned grid = (unsigned)std::min<uint64_t>(std::max<uint64_t>(fs[L.start_off + L.n], 1), 1u << 30);
+            if (L.p <= kGroupKey16MaxP)
+                batch_first_groups_kernel<uint16_t><<<grid, kGroupScatterWarps * 32, smem, stream>>>(
+                    A.jobs, A.fjobs + L.job_off, A.fstart + L.start_off, L.n, L.p);
+            else
+                batch_first_groups_kernel<uint32_t><<<grid, kGroupScatterWarps * 32, smem, stream>>>(
+                    A.jobs, A.fjobs + L.job_off, A.fstart + L.start_off, L.n, L.p);
+            count_launch();
+            continue;
+        }
         const size_t smem = (size_t)kFirstPassWarps * ((1u << L.p) + 32u) * 4u;
         const bool k16 = L.p <= kKey16MaxP;
         int per_sm = 1;

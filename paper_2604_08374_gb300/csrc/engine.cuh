@@ -45,16 +45,17 @@ struct JobDev {
     int scheme;             // table scheme of the lookups (mode 2)
     // Codes (codes.cuh) from the second pass on, for run-aware jobs without split
     // hubs.  Everything lies in the table region, whose lower half holds the
-    // code tables: win (gmax, then the window's top and low words), full, list.
+    // code tables: win, full, list.
     int codes;
     int K;                  // bits per code of the pass in progress (0: the scattered first pass)
     int too_open;           // a one-bit pass left more than open_cap pieces open and was done again in 4 bits
-    uint32_t *win;
+    uint32_t *win;          // gmax, gbig, then the window's top and low words
     uint8_t *full;          // nodes whose registers have all reached the window's top
     uint2 *list;            // open pieces of the pass {node, 16-byte piece}, list_cap = all there are
     uint32_t list_cap, open_cap;
     uint32_t open;          // pieces the pass left open
     unsigned long long n_top;  // registers at the top, over every kTopSample-th node
+    int group_scatter;      // with `first`: for whole groups (first_pass.cuh)
     int first;              // 1: pass 1 is the scatter of the nodes' keys (engine_start; keys in tab)
     uint32_t changed, inc;  // flags of the pass in progress
     int t;                  // passes completed

@@ -52,9 +52,12 @@ namespace {
 
 // Alg. 1 initialisation; with `keys` given, each node's key for the first
 // pass's scatter as well (KeyFmt: 16-bit for p <= kKey16MaxP, else 32-bit);
-// with `gmax` given (zeroed), the largest rho inserted per register index.
+// with `gmax` given (zeroed), the largest rho inserted per register index;
+// with `gbig` given (zeroed), the rho from 16 on as well, and keys for
+// launch_first_pass_groups.
 __global__ void hb_init_kernel(uint8_t *__restrict__ regs, uint32_t n, int p, int S, uint64_t seed, int nib,
-                               uint32_t s0, uint32_t s1, void *__restrict__ keys, uint32_t *gmax = nullptr) {
+                               uint32_t s0, uint32_t s1, void *__restrict__ keys, uint32_t *gmax = nullptr,
+                               uint32_t *gbig = nullptr) {
     const uint64_t v = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= n) return;
     init_node(regs, n, p, S, seed, (uint32_t)v, nib != 0, s0, s1);
@@ -64,7 +67,15 @@ __global__ void hb_init_kernel(uint8_t *__restrict__ regs, uint32_t n, int p, in
         const uint32_t rho = key & 0xffu;
         if (*reinterpret_cast<volatile uint32_t *>(g) < rho) atomicMax(g, rho);
     }
-    if (keys) {
+    if (gbig) {
+        const uint32_t rho = key & 0xffu;
+        if (rho >= 16u) atomicOr(gbig + (key >> 8), 1u << min(rho - 16u, 31u));
+        const uint32_t k = (key >> 8) << 4 | (min(rho, 16u) - 1u);
+        if (p <= kGroupKey16MaxP)
+            static_cast<uint16_t *>(keys)[v] = (uint16_t)k;
+        else
+            static_cast<uint32_t *>(keys)[v] = k;
+    } else if (keys) {
         if (p <= kKey16MaxP)
             static_cast<uint16_t *>(keys)[v] = KeyFmt<uint16_t>::pack(key);
         else
@@ -705,8 +716,8 @@ static int make_plan(const vga_graph *g, int p, const vga_tuning *tune, Plan *P)
         o = align256(o + 4ull * (P->mode == kModeRuns ? table_rows(P->scheme) : 1) * P->n);
     }
     if (P->codes) {
-        P->off_win = o;  // gmax (u32 per register), then the window's top and low words
-        o = align256(o + 4ull * P->m + 2ull * P->node_bytes);
+        P->off_win = o;  // gmax and gbig (u32 per register each), then the window's top and low words
+        o = align256(o + 8ull * P->m + 2ull * P->node_bytes);
         P->off_full = o;
         o = align256(o + P->n);
         P->off_list = o;  // {node, 16-byte piece} of up to N open pieces
@@ -725,7 +736,7 @@ static int make_plan(const vga_graph *g, int p, const vga_tuning *tune, Plan *P)
 static void plan_csr_codes(Plan *P, uint64_t ws_bytes) {
     if (!P->csr_codes) return;
     uint64_t o = P->total;
-    P->off_win = o;   o = align256(o + 4ull * P->m + 2ull * P->node_bytes);
+    P->off_win = o;   o = align256(o + 8ull * P->m + 2ull * P->node_bytes);
     P->off_full = o;  o = align256(o + P->n);
     P->off_list = o;  o = align256(o + 8 * P->n);
     P->off_codes = o;
@@ -930,7 +941,7 @@ static int launch_codes(const Plan &P, const vga_graph *g, int K, uint8_t *base,
     const int node_codes = (int)(P.m * (uint32_t)K / 8u);
     C.S = std::min(P.S, node_codes);
     const uint32_t *gmax = reinterpret_cast<const uint32_t *>(base + P.off_win);
-    C.top = gmax + P.m;
+    C.top = gmax + 2 * P.m;
     C.low = C.top + P.node_bytes / 4;
     C.flags = flags;
     C.full = base + P.off_full;
@@ -998,7 +1009,7 @@ static int launch_codes_csr(const Plan &P, const vga_graph *g, int K, uint8_t *b
     C.nib = P.nib != 0;
     C.K = K;
     C.S = (int)std::min<uint32_t>(P.m * (uint32_t)K / 8u, 1024u);
-    C.top = reinterpret_cast<const uint32_t *>(base + P.off_win) + P.m;
+    C.top = reinterpret_cast<const uint32_t *>(base + P.off_win) + 2 * P.m;
     C.low = C.top + P.node_bytes / 4;
     C.flags = flags;
     C.full = base + P.off_full;
@@ -1035,10 +1046,11 @@ static int launch_codes_csr(const Plan &P, const vga_graph *g, int K, uint8_t *b
 }
 
 // First pass of a run (or of a register-range shard holding slices [s0, s1))
-// by the scatter of the nodes' keys; `keys` were written by hb_init_kernel.
+// by the scatter of the nodes' keys; `keys` were written by hb_init_kernel.  With
+// gmax (followed by gbig) given, for whole groups.
 static int launch_first_pass(const Plan &P, const vga_graph *g, const void *keys, uint8_t *nxt, uint32_t s0,
                              uint32_t s1, uint32_t *flags, cudaStream_t stream, std::vector<PendingTiming> *timings,
-                             uint8_t *chg = nullptr) {
+                             uint8_t *chg = nullptr, const uint32_t *gmax = nullptr, uint64_t seed = 0) {
     const size_t smem = (size_t)kFirstPassWarps * (P.m + 32u) * 4u;
     static std::once_flag attr_once;
     static cudaError_t attr_err = cudaSuccess;
@@ -1078,7 +1090,24 @@ static int launch_first_pass(const Plan &P, const vga_graph *g, const void *keys
     else                                                                                                            \
         hb_first_pass_csr_kernel<NIBV, KT><<<blocks, kFirstPassWarps * 32, smem, stream>>>(                        \
             g->d_offsets, g->d_bytes, static_cast<const KT *>(keys), n, P.p, s_log2, s0, s1, nxt, flags, chg)
-    if (blocks) {
+    if (gmax) {
+        FirstPassGroups F;
+        F.groups = &P.groups;
+        F.keys = keys;
+        F.n = n;
+        F.p = P.p;
+        F.scheme = P.scheme;
+        F.s_log2 = s_log2;
+        F.nib = P.nib != 0;
+        F.gmax = gmax;
+        F.gbig = gmax + P.m;
+        F.seed = seed;
+        F.nxt = nxt;
+        F.flags = flags;
+        F.chg = chg;
+        F.stream = stream;
+        VGA_TRY(launch_first_pass_groups(F));
+    } else if (blocks) {
         if (P.nib) {
             if (k16) VGA_FP(true, uint16_t);
             else VGA_FP(true, uint32_t);
@@ -1292,11 +1321,17 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
         if (P.items.hubs) VGA_CHECK_CUDA(cudaMemsetAsync(nxt, 0, P.n * P.node_bytes, stream));
         void *keys = P.first_scatter ? tab : nullptr;  // tab is unused in pass 1
         uint32_t *gmax = P.codes ? reinterpret_cast<uint32_t *>(base + P.off_win) : nullptr;
-        uint32_t *top = P.codes ? gmax + P.m : nullptr;
+        uint32_t *top = P.codes ? gmax + 2 * P.m : nullptr;
         uint8_t *full = P.codes ? base + P.off_full : nullptr;
-        if (gmax) VGA_CHECK_CUDA(cudaMemsetAsync(gmax, 0, 4ull * P.m, stream));
+        if (gmax) VGA_CHECK_CUDA(cudaMemsetAsync(gmax, 0, 8ull * P.m, stream));
+        // a CTA a group: two an SM at least (818 cells: 207 us an analysis by groups, 199 by nodes)
+        int sms = 1;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device);
+        const bool first_groups = keys && P.codes && P.mode == kModeRuns && P.n >> P.p <= kGroupScatterNodes &&
+                                  P.groups.count >= 2ull * (uint64_t)sms;
+        uint32_t *gbig = first_groups ? gmax + P.m : nullptr;
         hb_init_kernel<<<(unsigned)((P.n + 255) / 256), 256, 0, stream>>>(cur, (uint32_t)P.n, p, P.S, seed, P.nib, 0u,
-                                                                          (uint32_t)P.slices, keys, gmax);
+                                                                          (uint32_t)P.slices, keys, gmax, gbig);
         count_launch();
         VGA_CHECK_CUDA(cudaGetLastError());
         if (gmax) VGA_TRY(launch_code_window(gmax, P.node_bytes / 4, P.nib, top, top + P.node_bytes / 4, stream));
@@ -1343,7 +1378,7 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
                 VGA_TRY(launch_codes(P, g, K, base, cur, nxt, flags, stream, timed ? &timings : nullptr, tracked, chg));
             } else if (t == 1 && keys)
                 VGA_TRY(launch_first_pass(P, g, keys, nxt, 0u, (uint32_t)P.slices, flags, stream,
-                                          timed ? &timings : nullptr, chg));
+                                          timed ? &timings : nullptr, chg, first_groups ? gmax : nullptr, seed));
             else
                 VGA_TRY(launch_union(P, g, cur, nxt, tab, flags, stream, timed ? &timings : nullptr,
                                      tracked ? need : nullptr, chg));

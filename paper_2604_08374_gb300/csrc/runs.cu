@@ -54,48 +54,57 @@ __global__ void run_lookups_kernel(const uint64_t *__restrict__ off, const uint8
     }
 }
 
-// Merge key of a range lookup: (window start i, slot) from its row index
-// r = slot * n + i.  Within one node's list the window starts strictly
-// increase (the runs ascend and a run's windows start at a, a + w, ...,
-// a + L - w), so every list is sorted by this key.
-__device__ __forceinline__ uint64_t lookup_key(uint32_t r, uint32_t n) {
+// First id and width of a range lookup's window, from its row index r = slot *
+// n + i.  Within one node's list the windows' first ids strictly increase, and
+// so do their ends: the runs ascend with a gap between any two, and a run's
+// windows start at a, a + w, ..., a + L - w.
+__device__ __forceinline__ void lookup_window(uint32_t r, uint32_t n, int scheme, uint32_t &i, uint32_t &w) {
     uint32_t slot = 0;
 #pragma unroll
-    for (int k = 1; k < kMaxTableRows; k++) slot += (uint64_t)r >= (uint64_t)k * n ? 1u : 0u;
-    return ((uint64_t)(r - slot * n) << 3) | slot;
+    for (int k = 1; k < kMaxTableRows; k++) slot += r >= (uint32_t)k * n ? 1u : 0u;  // 5 n < 2^32 (kRunMaxNodes)
+    i = r - slot * n;
+    w = 1u << (scheme == 0 ? slot : 2u * slot);
 }
 
-// Entries of each list a merging lane loads at a time (independent loads).
-constexpr int kMergeWindow = 4;
-
-// First index of list[0 .. len) whose key is >= k (the list is sorted by key).
-__device__ __forceinline__ uint32_t key_lower_bound(const uint32_t *__restrict__ list, uint32_t len, uint64_t k,
-                                                    uint32_t n) {
+// First index of list[0 .. len) whose window starts at id x or later.
+__device__ __forceinline__ uint32_t start_lower_bound(const uint32_t *__restrict__ list, uint32_t len, uint32_t x,
+                                                      uint32_t n, int scheme) {
     uint32_t lo = 0, hi = len;
     while (lo < hi) {
         const uint32_t mid = (lo + hi) >> 1;
-        if (lookup_key(list[mid], n) < k) lo = mid + 1;
+        uint32_t i, w;
+        lookup_window(list[mid], n, scheme, i, w);
+        if (i < x) lo = mid + 1;
         else hi = mid;
     }
     return lo;
 }
 
-// One warp per group of up to NODES nodes: merge the group's lookup lists by
-// key; equal keys (the same row) become one entry whose class is the set of
-// lists holding it.  The key space is split among the lanes at 31 keys
-// sampled evenly from the group's longest list, and every lane merges its own
-// key range serially.  Without WRITE: count the group's entries of every class
-// into cc[group << NODES | class].  With WRITE: from those counts, write the
-// group's class descriptors (classes in decreasing mask order: the rows of all
-// nodes first, which the code passes cut short; empty ones left out) and its rows, sorted by class (within a class by key), at rows[b ...].
-// Shared memory: 2^NODES counters or write cursors per lane.
+// One warp per group of up to NODES nodes: the ids that the group's lists hold
+// are cut into segments of consecutive ids seen by the same nodes (the
+// segment's class), and each segment is covered by range lookups as a run is
+// (run_window).  The segments follow from the lists' runs, which are their
+// lookups' windows joined where they touch: a lane walks the runs of all lists
+// in step from one end of a run to the next.  The ids are split among the lanes
+// at run starts of the group's longest list.  Without WRITE: count the group's
+// rows of every class into cc[group << NODES | class].  With WRITE: from those
+// counts, write the group's class descriptors (classes in decreasing mask
+// order: the rows of all nodes first, which the code passes cut short; empty
+// ones left out) and its rows, sorted by class (within a class by id), at
+// rows[b ...].  Shared memory: 2^NODES counters or write cursors per lane.
+//
+// Rows of distinct lookups instead, which need no cutting, are 2 % more on the
+// city graph (1,688 a node against 1,657; 10 % on 42,700 cells) and cover ids
+// 2.5 times as often (15,100 a node against 6,087 ids), which is what the first
+// pass's scatter pays for.
 template <int NODES, bool WRITE>
 __global__ void group_merge_kernel(const GroupItem *__restrict__ items, uint64_t n_groups,
                                    const uint64_t *__restrict__ lk_off, const uint32_t *__restrict__ lk, uint32_t n,
-                                   uint32_t *__restrict__ cc, uint32_t *__restrict__ lane_cc,
+                                   int scheme, uint32_t *__restrict__ cc, uint32_t *__restrict__ lane_cc,
                                    uint32_t *__restrict__ rows, uint2 *__restrict__ cls) {
     extern __shared__ __align__(16) uint32_t s_cnt[];
     constexpr uint32_t C = 1u << NODES;
+    constexpr uint32_t kEnd = 0xffffffffu;  // past every id
     const int lane = threadIdx.x & 31;
     const uint64_t gid = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (gid >= n_groups) return;
@@ -117,54 +126,88 @@ __global__ void group_merge_kernel(const GroupItem *__restrict__ items, uint64_t
             longest = list[j];
         }
     }
-    // this lane's key range [k0, k1)
-    uint64_t k0 = lane == 0 || L == 0 ? 0ull : lookup_key(longest[(uint32_t)((uint64_t)L * lane / 32)], n);
-    uint64_t k1 = __shfl_down_sync(0xffffffffu, k0, 1);
-    if (lane == 31) k1 = ~0ull;
-    uint32_t p[NODES], p0[NODES], e[NODES];
-    uint64_t hk[NODES];
-    uint32_t win[NODES][kMergeWindow];  // the next entries of each list, loaded together
-    auto load_windows = [&]() {
-#pragma unroll
-        for (int j = 0; j < NODES; j++) {
-            p0[j] = p[j];
-#pragma unroll
-            for (int q = 0; q < kMergeWindow; q++) win[j][q] = p[j] + q < e[j] ? list[j][p[j] + q] : 0u;
-            hk[j] = p[j] < e[j] ? lookup_key(win[j][0], n) : ~0ull;
+    // this lane's ids [x0, x1): from the run start at or a few windows before its share of the longest list
+    uint32_t x0 = 0;
+    if (lane > 0 && L > 0) {
+        uint32_t q = (uint32_t)((uint64_t)L * lane / 32), w;
+        lookup_window(longest[q], n, scheme, x0, w);
+        for (int back = 0; back < 8 && q > 0; back++) {
+            uint32_t i, wi;
+            lookup_window(longest[q - 1], n, scheme, i, wi);
+            if (i + wi < x0) break;  // x0 starts a run
+            x0 = i;
+            q--;
+        }
+    }
+    uint32_t x1 = __shfl_down_sync(0xffffffffu, x0, 1);
+    if (lane == 31 || L == 0) x1 = kEnd;
+    // next lookup, its window, and the run [rs, re) that list j is at
+    uint32_t p[NODES], pi[NODES], pw[NODES], rs[NODES], re[NODES];
+    auto peek = [&](int j) {
+        pi[j] = kEnd;
+        pw[j] = 0;
+        if (p[j] < len[j]) lookup_window(__ldg(list[j] + p[j]), n, scheme, pi[j], pw[j]);
+    };
+    auto extend = [&](int j) {  // join the windows that touch the run, up to the lane's end
+        while (pi[j] <= re[j] && re[j] < x1) {
+            re[j] = pi[j] + pw[j];
+            p[j]++;
+            peek(j);
         }
     };
+    auto next_run = [&](int j) {
+        rs[j] = pi[j];
+        re[j] = kEnd;
+        if (pi[j] != kEnd) {
+            re[j] = pi[j] + pw[j];
+            p[j]++;
+            peek(j);
+            extend(j);
+        }
+    };
+    // the lane's segments, in id order: emit(mask, first id, ids)
+    auto walk = [&](auto emit) {
 #pragma unroll
-    for (int j = 0; j < NODES; j++) {
-        p[j] = k0 == 0 ? 0u : key_lower_bound(list[j], len[j], k0, n);
-        e[j] = k1 == ~0ull ? len[j] : key_lower_bound(list[j], len[j], k1, n);
-    }
-    load_windows();
+        for (int j = 0; j < NODES; j++) {
+            p[j] = x0 == 0 ? 0u : start_lower_bound(list[j], len[j], x0, n, scheme);
+            peek(j);
+            rs[j] = re[j] = kEnd;
+            if (p[j] > 0) {  // the run before may reach into the lane's ids
+                uint32_t i, w;
+                lookup_window(list[j][p[j] - 1], n, scheme, i, w);
+                if (i + w > x0) {
+                    rs[j] = x0;
+                    re[j] = i + w;
+                    extend(j);
+                }
+            }
+            if (rs[j] == kEnd) next_run(j);
+        }
+        uint32_t x = x0;
+        while (x < x1) {
+            uint32_t y = x1, mask = 0;
+#pragma unroll
+            for (int j = 0; j < NODES; j++) {
+                const bool in = rs[j] <= x;
+                mask |= in ? 1u << j : 0u;
+                y = min(y, in ? re[j] : rs[j]);
+            }
+            if (mask) emit(mask, x, y - x);
+            x = y;
+#pragma unroll
+            for (int j = 0; j < NODES; j++)
+                if (re[j] <= x && x != kEnd) next_run(j);
+        }
+    };
     uint32_t *mine = cc + (gid << NODES);
     for (uint32_t k = 0; k < C; k++) c[k * 32] = 0;
     uint32_t *my_lane_cc = lane_cc ? lane_cc + (gid << NODES) * 32 + lane : nullptr;  // [group][class][lane]
     if (WRITE && my_lane_cc) {
         for (uint32_t k = 0; k < C; k++) c[k * 32] = my_lane_cc[k * 32];
-    } else if (WRITE) {
-        // this lane's count in every class, found by a merge pass that only
-        // counts (when the count pass kept no per-lane counts)
-        for (;;) {
-            uint64_t best = ~0ull;
-#pragma unroll
-            for (int j = 0; j < NODES; j++) best = hk[j] < best ? hk[j] : best;
-            if (best == ~0ull) break;
-            uint32_t mask = 0;
-#pragma unroll
-            for (int j = 0; j < NODES; j++)
-                if (hk[j] == best) {
-                    mask |= 1u << j;
-                    p[j]++;
-                    hk[j] = p[j] < e[j] ? lookup_key(list[j][p[j]], n) : ~0ull;
-                }
-            c[mask * 32]++;
-        }
-#pragma unroll
-        for (int j = 0; j < NODES; j++) p[j] = k0 == 0 ? 0u : key_lower_bound(list[j], len[j], k0, n);
-        load_windows();
+    } else {
+        // this lane's count in every class (in the write pass, when the count
+        // pass kept no per-lane counts)
+        walk([&](uint32_t mask, uint32_t, uint32_t ids) { c[mask * 32] += run_lookup_count(ids, scheme); });
     }
     if (WRITE) {
         // this lane's cursor in class k: the class's base (classes in decreasing
@@ -185,36 +228,13 @@ __global__ void group_merge_kernel(const GroupItem *__restrict__ items, uint64_t
             ci++;
             base += total;
         }
-    }
-    uint32_t *row_base = WRITE ? rows + it.b : nullptr;
-    for (;;) {
-        uint64_t best = ~0ull;
-#pragma unroll
-        for (int j = 0; j < NODES; j++) best = hk[j] < best ? hk[j] : best;
-        if (best == ~0ull) break;
-        uint32_t mask = 0, r = 0;
-#pragma unroll
-        for (int j = 0; j < NODES; j++)
-            if (hk[j] == best) {
-                mask |= 1u << j;
-                r = win[j][0];
-                p[j]++;
-                // shift the look-ahead window; refill it with independent loads when empty
-#pragma unroll
-                for (int q = 0; q < kMergeWindow - 1; q++) win[j][q] = win[j][q + 1];
-                if (p[j] < e[j] && ((p[j] - p0[j]) % kMergeWindow) == 0) {
-#pragma unroll
-                    for (int q = 0; q < kMergeWindow; q++)
-                        win[j][q] = p[j] + q < e[j] ? list[j][p[j] + q] : 0u;
-                }
-                hk[j] = p[j] < e[j] ? lookup_key(win[j][0], n) : ~0ull;
-            }
-        if (WRITE)
-            row_base[c[mask * 32]++] = r;
-        else
-            c[mask * 32]++;
-    }
-    if (!WRITE) {
+        uint32_t *row_base = rows + it.b;
+        walk([&](uint32_t mask, uint32_t a, uint32_t ids) {
+            const uint32_t at = c[mask * 32];
+            run_lookup_write(a, ids, n, scheme, row_base + at);
+            c[mask * 32] = at + run_lookup_count(ids, scheme);
+        });
+    } else {
         __syncwarp();
         for (uint32_t k = 0; k < C; k++) {
             const uint32_t t = __reduce_add_sync(0xffffffffu, c[k * 32]);
@@ -450,11 +470,11 @@ int ensure_group_list(const vga_graph *g, int scheme, uint32_t hub_lookups, int 
 #define VGA_GM(NN)                                                                                                   \
     if (write)                                                                                                       \
         group_merge_kernel<NN, true><<<blocks, threads, smem, stream>>>(d_items.as<GroupItem>(), ng, L.d_off,       \
-                                                                        L.d_lk, g->n, d_cc.as<uint32_t>(),           \
+                                                                        L.d_lk, g->n, scheme, d_cc.as<uint32_t>(),   \
                                                                         d_lane_cc.as<uint32_t>(), rows, cls);        \
     else                                                                                                             \
         group_merge_kernel<NN, false><<<blocks, threads, smem, stream>>>(d_items.as<GroupItem>(), ng, L.d_off,      \
-                                                                         L.d_lk, g->n, d_cc.as<uint32_t>(),          \
+                                                                         L.d_lk, g->n, scheme, d_cc.as<uint32_t>(),  \
                                                                          d_lane_cc.as<uint32_t>(), rows, cls)
         if (nodes == 2) VGA_GM(2);
         else if (nodes == 4) VGA_GM(4);

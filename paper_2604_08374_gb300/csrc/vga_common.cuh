@@ -202,15 +202,14 @@ struct RunItemList {
 int ensure_run_items(const vga_graph *g, int scheme, uint32_t hub_lookups, cudaStream_t stream, RunItemList *out);
 
 // Grouped lookup lists of the run-aware union.  The non-hub nodes, in id
-// order, are cut into groups of up to kGroupMaxNodes consecutive ones;
-// adjacent cells see nearly the same runs, so their lookup lists share many
-// entries (about 40 % of a four-node group's at the city size).  Each group's
-// lists are merged once per graph into its distinct rows, each tagged with
-// its class -- the set of the group's nodes whose list holds it -- and sorted
-// by class.  The union then gathers every distinct row once and folds each
-// class into one accumulator, merged into the partial maxima of the class's
-// nodes when the class ends: the same registers, bit for bit (a max over a
-// union of sets), from fewer gathers and fewer folds.
+// order, are cut into groups of up to kGroupMaxNodes consecutive ones (with the
+// grid's geometry: blocks of cells); adjacent cells see nearly the same ids.
+// Once per graph, the ids that a group's lists hold are cut into segments seen
+// by the same nodes (the segment's class) and covered by range lookups, sorted
+// by class.  The union then gathers every row once and folds each class into
+// one accumulator, merged into the partial maxima of the class's nodes when the
+// class ends: the same registers, bit for bit (a max over a union of sets), from
+// fewer gathers and fewer folds.
 constexpr int kGroupMaxNodes = 8;
 struct GroupItem {
     uint32_t node[kGroupMaxNodes];  // the group's nodes (0xffffffff past its end)
@@ -271,6 +270,29 @@ int launch_code_open(const CodePass &C, const uint64_t *lk_off, const uint32_t *
 int launch_code_csr(const CodePass &C, uint32_t m, const uint64_t *off, const uint8_t *bytes, int sms);
 int launch_code_window(const uint32_t *gmax, uint32_t words, int nib, uint32_t *top, uint32_t *low,
                        cudaStream_t stream);
+
+// The first pass as a scatter for whole groups (first_pass.cuh).  A node's key
+// is j << 4 | level (level = min(rho, 16) - 1), 16 bits up to p = 12.  gbig[j]
+// has a bit for every rho from 16 on inserted with index j (bit rho - 16; bit
+// 31: 47 or more).
+constexpr int kGroupKey16MaxP = 12;
+// It is used while few indices can have several rho above 16 (such registers
+// are searched): up to this many nodes an index, where one index in 500 has.
+constexpr uint64_t kGroupScatterNodes = 2048;
+struct FirstPassGroups {
+    const GroupList *groups = nullptr;
+    const void *keys = nullptr;
+    uint32_t n = 0;
+    int p = 10, scheme = 0, s_log2 = 0;
+    bool nib = false;
+    const uint32_t *gmax = nullptr, *gbig = nullptr;
+    uint64_t seed = 0;
+    uint8_t *nxt = nullptr;
+    uint32_t *flags = nullptr;
+    uint8_t *chg = nullptr;
+    cudaStream_t stream = nullptr;
+};
+int launch_first_pass_groups(const FirstPassGroups &F);
 
 // Automatic hub threshold (lookups per work item): half of one warp's even
 // share of a slice's lookups when every SM holds 64 warps, and at least 2048,

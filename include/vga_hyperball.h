@@ -166,14 +166,17 @@ int vga_graph_set_cells(vga_graph *g, int W, int H, const uint64_t *cell_of_node
  * each end open or closed) is kept; a target is visible iff its slope lies in
  * one of them (the diagonal target also needs the cell beside it, whose
  * corner its segment touches, free).  The result equals the pairwise rule
- * above for every pair.  The lists go to a stage and from there to the CSR.
- * Device scratch besides the CSR: obstacle bitmaps (2 x W x H bits with
- * margins), a W*H node-id table and 12 bytes a node; per CTA a node bitmap
- * (in shared memory up to ~800k nodes) and, for sources whose interval lists
- * outgrow shared memory, global lists of max(W, H) + 2 entries per warp; and,
- * while it is to be had, a stage of about the CSR's size (at most 256 MB, or a
- * twentieth more than the sampled size), without which every source is swept
- * twice.
+ * above for every pair.  Half of each source's octants are swept into a bit
+ * matrix, which is joined with its transpose (visibility is symmetric) and
+ * encoded.
+ * Device scratch besides the CSR: the matrix (N^2 / 8 bytes, up to 16 GB),
+ * obstacle bitmaps (2 x W x H bits with margins), two W*H node-id tables and 28
+ * bytes a node; for sources whose interval lists outgrow shared memory, global
+ * lists of max(W, H) + 2 entries per warp.  Without room for the matrix, or
+ * above 370,000 nodes, all octants are swept instead, with a node bitmap per CTA
+ * (in shared memory up to ~800k nodes) and, while it is to be had, a stage of
+ * about the CSR's size (at most 256 MB, or a twentieth more than the sampled
+ * size), without which every source is swept twice.
  * Errors: VGA_EINVAL for bad sizes; VGA_ECORRUPT if the sweep's own checks
  * fail (a visible cell off the component, a list overflow past the proven
  * bound, a count/write mismatch).
@@ -185,8 +188,9 @@ int vga_visibility_build(int W, int H, const uint8_t *obst, uint64_t *cell_of_no
  * fallbacks: smem_list_cap (1..48, 0 = 48) caps the interval lists kept in
  * shared memory, so that more sources take the global-list retry, and (below
  * 48) the stage at 64 bytes a node, so that some lists are swept twice;
- * smem_bitmap_nodes > 0 keeps the node bitmap in global memory for graphs
- * with more nodes than that (0 = whenever shared memory is too small).
+ * smem_bitmap_nodes > 0 selects the way with a node bitmap per CTA, kept in
+ * global memory for graphs with more nodes than that (0 = the bit matrix; a CTA's
+ * bitmap in global memory whenever shared memory is too small).
  * Process-wide; both give the same graph as the defaults.
  */
 int vga_set_visibility_sweep_limits(int smem_list_cap, uint32_t smem_bitmap_nodes);

@@ -10,11 +10,14 @@
 // tan-space [0, 1] loses the ranges obstacles cover), with the gaps' ends kept
 // as exact integer fractions so that the result equals the pairwise rule above
 // for every pair.  Pipeline: (host) main component and numbering, obstacle
-// bitmaps; (device) per source, the octants swept into a node bitmap and its
-// list's LEB128 bytes written to a stage in the order the sources finish;
-// (host) prefix sum of the lists' sizes into offsets; (device) the lists copied
-// to their places; then the ordinary load path validates the stream and derives
-// degrees.
+// bitmaps; (device) per source, the four octants that see the cells after it in
+// raster order swept into its row of a bit matrix, and the matrix joined with
+// its transpose (visibility is symmetric); the bytes of every row's LEB128 list
+// counted; (host) prefix sum into offsets; (device) the lists written; then the
+// ordinary load path validates the stream and derives degrees.  Graphs whose
+// matrix would be too large (kMatrixBytes) have all eight octants of a source
+// swept into one CTA's node bitmap and its list written to a stage in the order
+// the sources finish, from where it is brought to its place.
 #include <algorithm>
 #include <utility>
 #include <vector>
@@ -115,10 +118,13 @@ constexpr int kSweepThreads = kSweepWarps * 32;
 constexpr int kSweepCap = 48;                      // intervals per list in shared memory
 constexpr int kPad = 64;                           // margin bits (obstacles) on both sides of a line
 constexpr uint32_t kNoSource = 0xffffffffu;
+// Largest bit matrix of the graph (N^2 / 8 bytes: up to 370,000 nodes).
+constexpr uint64_t kMatrixBytes = 16ull << 30;
 
 // Test hooks: a smaller shared-memory list capacity sends more sources down
 // the global-list retry (and makes the stage of the lists' bytes so small that
-// some are swept again); a node limit moves the node bitmap to global memory.
+// some are swept again); a node limit selects the builder with a bitmap per CTA and, above
+// it, moves the bitmap to global memory.
 int g_sweep_smem_cap = kSweepCap;
 uint32_t g_sweep_smem_bitmap_nodes = 0;   // 0: as many as shared memory allows
 
@@ -151,6 +157,9 @@ struct SweepArgs {
     const uint32_t *colbits;   // W lines of words_c words: bit y + kPad of line x = obstacle (x, y)
     int W, H, words_r, words_c;
     const int32_t *node_of_cell;   // W * H: node id, or -1 off the main component
+    const int32_t *node_of_cell_t; // the same by columns (rows kernel)
+    uint32_t *matrix;              // rows kernel: a row of `pitch` words per node
+    uint32_t pitch;
     const uint32_t *cells;         // n: raster cell of each node
     uint32_t n;
     const uint32_t *sources;       // the sources to sweep (nullptr: nodes 0 .. count - 1)
@@ -257,7 +266,10 @@ __device__ __forceinline__ uint32_t varint_len(uint32_t x) {
 }
 
 // One warp sweeps octant `oct` of source (sx, sy), setting the bits of the
-// visible nodes in bm.  Returns false when the interval list outgrew cap.
+// visible nodes in bm (ROWS: a row of the matrix in global memory; else the
+// CTA's bitmap, with the range of ids kept in id_lo and id_hi).  Returns false
+// when the interval list outgrew cap.
+template <bool ROWS>
 __device__ bool sweep_octant(const SweepArgs &A, int oct, int sx, int sy, uint32_t *bm, uint2 *la, uint2 *lb,
                              int cap, uint32_t *mask, uint32_t *obw, int *count, int &id_lo, int &id_hi) {
     const int lane = threadIdx.x & 31;
@@ -323,7 +335,33 @@ __device__ bool sweep_octant(const SweepArgs &A, int oct, int sx, int sy, uint32
                 const uint32_t m = mask[w];
                 uint32_t vis = m & ~obw[w];
                 if (diag_blocked && k >= w * 32 && k < w * 32 + 32) vis &= ~(1u << (k - w * 32));
-                if ((vis >> lane) & 1u) {
+                if (ROWS) {
+                    const int r = w * 32 + lane;
+                    const bool sees = (vis >> lane) & 1u;
+                    int id = -1;
+                    if (sees) {
+                        const int minor = min0 + smin * r;
+                        id = xmajor ? __ldg(A.node_of_cell_t + (size_t)maj * A.H + minor)
+                                    : __ldg(A.node_of_cell + (size_t)maj * A.W + minor);
+                        if (id < 0) atomicOr(A.err, 1);
+                    }
+                    // cells of a row have consecutive ids in raster order: the
+                    // lanes of up to two words join theirs into one atomic
+                    uint32_t left = __ballot_sync(0xffffffffu, id >= 0);
+                    if (!xmajor) {
+#pragma unroll
+                        for (int join = 0; join < 2; join++) {
+                            if (!left) break;
+                            const int lead = __ffs(left) - 1;
+                            const int word = __shfl_sync(0xffffffffu, id >> 5, lead);
+                            const bool same = ((left >> lane) & 1u) && (id >> 5) == word;
+                            const uint32_t bits = __reduce_or_sync(0xffffffffu, same ? 1u << (id & 31) : 0u);
+                            if (lane == lead) atomicOr(bm + word, bits);
+                            left &= ~__ballot_sync(0xffffffffu, same);
+                        }
+                    }
+                    if ((left >> lane) & 1u) atomicOr(bm + (id >> 5), 1u << (id & 31));
+                } else if ((vis >> lane) & 1u) {
                     const int r = w * 32 + lane;
                     const int x = xmajor ? maj : sx + smin * r;
                     const int y = xmajor ? sy + smin * r : maj;
@@ -421,7 +459,7 @@ __global__ void __launch_bounds__(kSweepThreads, 6) visibility_sweep_kernel(Swee
         const uint32_t cell = A.cells[u];
         const int sx = (int)(cell % (uint32_t)A.W), sy = (int)(cell / (uint32_t)A.W);
         int id_lo = 0x7fffffff, id_hi = -1;
-        if (!sweep_octant(A, warp, sx, sy, bm, la, lb, cap, mask, obw, &s_count[warp], id_lo, id_hi)) {
+        if (!sweep_octant<false>(A, warp, sx, sy, bm, la, lb, cap, mask, obw, &s_count[warp], id_lo, id_hi)) {
             if (lane == 0) s_overflow = 1;
             for (int w = lane; w < A.mask_words; w += 32) mask[w] = 0u;
         }
@@ -584,6 +622,205 @@ __global__ void __launch_bounds__(kSweepThreads, 6) visibility_sweep_kernel(Swee
     }
 }
 
+// The rows kernel: a warp takes (source, octant) pairs from a counter and sweeps
+// the octant into the source's row of the matrix.  Only the four octants that
+// hold the cells after the source in raster order (and the rest of its own row)
+// are swept; rows_join_kernel adds the other half.  No bitmap in shared memory
+// and no octant that waits for another's, so 48 warps an SM stay busy: bound by
+// the chain of steps from column to column.  City grid: 77 ms (with the joining
+// 5 and the encoding 20), where a CTA of eight octants with a bitmap in shared
+// memory took 229.
+constexpr int kRowsOctants = 4;
+template <bool GLOBAL_LISTS>
+__global__ void __launch_bounds__(kSweepThreads, 6) visibility_rows_kernel(SweepArgs A) {
+    extern __shared__ __align__(16) uint8_t smem[];
+    __shared__ int s_count[kSweepWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint8_t *p = smem;
+    uint2 *la, *lb;
+    int cap;
+    if (GLOBAL_LISTS) {
+        la = A.glists + ((size_t)blockIdx.x * kSweepWarps + warp) * 2 * A.glist_cap;
+        lb = la + A.glist_cap;
+        cap = A.glist_cap;
+    } else {
+        la = reinterpret_cast<uint2 *>(p) + (size_t)warp * 2 * kSweepCap;
+        lb = la + kSweepCap;
+        cap = A.smem_cap;
+        p += (size_t)kSweepWarps * 2 * kSweepCap * sizeof(uint2);
+    }
+    uint32_t *mask = reinterpret_cast<uint32_t *>(p) + (size_t)warp * A.mask_words;
+    uint32_t *obw = reinterpret_cast<uint32_t *>(p) + (size_t)(kSweepWarps + warp) * A.mask_words;
+    for (int w = lane; w < A.mask_words; w += 32) mask[w] = 0u;
+    __syncwarp();
+    for (;;) {
+        uint32_t i = 0;
+        if (lane == 0) i = atomicAdd(A.next, 1u);
+        i = __shfl_sync(0xffffffffu, i, 0);
+        if (i >= A.count) break;
+        const uint32_t item = A.sources ? A.sources[i] : i;
+        const uint32_t u = item / kRowsOctants, o = item % kRowsOctants;
+        const int oct = o < 2u ? (int)o : (int)(2u * o);  // 0, 1 (|dx| >= dy), 4, 6 (dy >= |dx|)
+        const uint32_t cell = A.cells[u];
+        int id_lo = 0, id_hi = 0;
+        if (!sweep_octant<true>(A, oct, (int)(cell % (uint32_t)A.W), (int)(cell / (uint32_t)A.W),
+                                A.matrix + (size_t)u * A.pitch, la, lb, cap, mask, obw, &s_count[warp], id_lo, id_hi)) {
+            if (lane == 0) {
+                if (GLOBAL_LISTS) atomicOr(A.err, 2);
+                else A.retry[atomicAdd(A.retry_count, 1u)] = item;
+            }
+            for (int w = lane; w < A.mask_words; w += 32) mask[w] = 0u;
+        }
+        __syncwarp();
+    }
+}
+
+// Transpose of the warp's 32 x 32 bits (lane = row, bit = column).
+__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
+    const uint32_t keep[5] = {0x0000ffffu, 0x00ff00ffu, 0x0f0f0f0fu, 0x33333333u, 0x55555555u};
+#pragma unroll
+    for (int s = 0; s < 5; s++) {
+        const int d = 16 >> s;
+        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, d);
+        x = (lane & d) ? (x & ~keep[s]) | ((y >> d) & keep[s]) : (x & keep[s]) | ((y << d) & ~keep[s]);
+    }
+    return x;
+}
+
+// matrix |= transpose(matrix), one CTA per pair of mirrored tiles of kTile x
+// kTile bits (blockIdx.x <= blockIdx.y), both in shared memory.  The matrix's
+// sides are multiples of kTile.  Bound: its bytes read and written once (14 GB
+// for the city).
+constexpr int kTile = 512, kTileWords = kTile / 32, kTilePitch = kTileWords + 1;
+constexpr size_t kJoinSmem = 2ull * kTile * kTilePitch * 4;
+__global__ void __launch_bounds__(256) rows_join_kernel(uint32_t *__restrict__ matrix, uint32_t pitch) {
+    extern __shared__ __align__(16) uint32_t s_bits[];
+    const uint32_t ti = blockIdx.x, tj = blockIdx.y;
+    if (ti > tj) return;
+    const bool diagonal = ti == tj;
+    uint32_t *a = s_bits, *b = diagonal ? s_bits : s_bits + kTile * kTilePitch;
+    auto tile = [&](uint32_t rt, uint32_t ct, int x) {  // 16 bytes x of tile (rt, ct)
+        return reinterpret_cast<uint4 *>(matrix + (size_t)(rt * kTile + x / (kTileWords / 4)) * pitch + ct * kTileWords) +
+               x % (kTileWords / 4);
+    };
+    constexpr int kChunks = kTile * kTileWords / 4;
+    for (int x = threadIdx.x; x < kChunks; x += blockDim.x) {
+        uint32_t *d = a + (x / (kTileWords / 4)) * kTilePitch + 4 * (x % (kTileWords / 4));
+        const uint4 v = *tile(ti, tj, x);
+        d[0] = v.x, d[1] = v.y, d[2] = v.z, d[3] = v.w;
+        if (!diagonal) {
+            uint32_t *e = d + (b - a);
+            const uint4 w = *tile(tj, ti, x);
+            e[0] = w.x, e[1] = w.y, e[2] = w.z, e[3] = w.w;
+        }
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    for (int q = threadIdx.x >> 5; q < kTileWords * kTileWords; q += blockDim.x >> 5) {
+        const int bi = q / kTileWords, bj = q % kTileWords;
+        if (diagonal && bi > bj) continue;
+        uint32_t &x = a[(bi * 32 + lane) * kTilePitch + bj], &y = b[(bj * 32 + lane) * kTilePitch + bi];
+        const uint32_t xv = x, yv = y;
+        const uint32_t xt = transpose32(xv, lane), yt = transpose32(yv, lane);
+        __syncwarp();
+        x = xv | yt;
+        if (!diagonal || bi != bj) y = yv | xt;
+    }
+    __syncthreads();
+    for (int x = threadIdx.x; x < kChunks; x += blockDim.x) {
+        const uint32_t *d = a + (x / (kTileWords / 4)) * kTilePitch + 4 * (x % (kTileWords / 4));
+        *tile(ti, tj, x) = make_uint4(d[0], d[1], d[2], d[3]);
+        if (!diagonal) {
+            const uint32_t *e = d + (b - a);
+            *tile(tj, ti, x) = make_uint4(e[0], e[1], e[2], e[3]);
+        }
+    }
+}
+
+// LEB128 delta lists of the matrix's rows, one warp per row, 32 words a step:
+// their sizes, or (WRITE) their bytes.  Within a word every delta is below 128,
+// so only a word's first id can take more than one byte.  A step's bytes (at
+// most 32 x 36) are put together in shared memory and stored 16 at a time.
+constexpr int kEncodeWarps = 8;
+template <bool WRITE>
+__global__ void __launch_bounds__(kEncodeWarps * 32) rows_encode_kernel(const uint32_t *__restrict__ matrix,
+                                                                       uint32_t pitch, uint32_t words, uint32_t n,
+                                                                       uint64_t *__restrict__ row_bytes,
+                                                                       const uint64_t *__restrict__ offsets,
+                                                                       uint8_t *__restrict__ out, int *err) {
+    __shared__ __align__(16) uint8_t s_buf[WRITE ? kEncodeWarps : 1][32 * 36 + 32];
+    const int lane = threadIdx.x & 31;
+    const uint64_t u = (uint64_t)blockIdx.x * kEncodeWarps + (threadIdx.x >> 5);
+    if (u >= n) return;
+    uint8_t *buf = s_buf[WRITE ? threadIdx.x >> 5 : 0];
+    const uint32_t *row = matrix + u * pitch;
+    int run = -1;  // last id so far
+    uint64_t pos = WRITE ? offsets[u] : 0;
+    const uint64_t end = WRITE ? offsets[u + 1] : 0;
+    uint32_t next = lane < (int)words ? __ldcs(row + lane) : 0u;
+    for (uint32_t c = 0; c < words; c += 32) {
+        const uint32_t wi = c + lane;
+        const uint32_t word = next;
+        next = wi + 32 < words ? __ldcs(row + wi + 32) : 0u;
+        if (!__any_sync(0xffffffffu, word != 0u)) continue;
+        int incl = word ? (int)(wi * 32 + 31 - __clz(word)) : -1;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o && t > incl) incl = t;
+        }
+        int excl = __shfl_up_sync(0xffffffffu, incl, 1);
+        if (lane == 0) excl = -1;
+        if (run > excl) excl = run;
+        uint32_t nb = 0;
+        if (word) {
+            const uint32_t wf = wi * 32 + (__ffs(word) - 1);
+            nb = (uint32_t)__popc(word) - 1u + varint_len(excl < 0 ? wf : wf - (uint32_t)excl);
+        }
+        run = max(run, __shfl_sync(0xffffffffu, incl, 31));
+        if (!WRITE) {
+            pos += __reduce_add_sync(0xffffffffu, nb);
+            continue;
+        }
+        uint32_t sc = nb;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, sc, o);
+            if (lane >= o) sc += t;
+        }
+        const uint32_t total = __shfl_sync(0xffffffffu, sc, 31);
+        const uint32_t head = (uint32_t)(pos & 15u);  // the buffer holds the bytes from pos - head on
+        uint32_t q = head + sc - nb, left = word;
+        int last = excl;
+        while (left) {
+            const uint32_t id = wi * 32 + (__ffs(left) - 1);
+            left &= left - 1u;
+            uint32_t x = last < 0 ? id : id - (uint32_t)last;
+            while (x > 0x7fu) {
+                buf[q++] = (uint8_t)(x | 0x80u);
+                x >>= 7;
+            }
+            buf[q++] = (uint8_t)x;
+            last = (int)id;
+        }
+        __syncwarp();
+        if (pos + total > end) {  // the count pass sized the list
+            if (lane == 0) atomicOr(err, 8);
+            break;
+        }
+        uint8_t *dst = out + (pos - head);
+        const uint32_t e = head + total, b0 = head ? 16u : 0u, b1 = e & ~15u;
+        if (head && lane >= (int)head && lane < 16 && lane < (int)e) dst[lane] = buf[lane];
+        for (uint32_t x = b0 + 16u * lane; x < b1; x += 512u)
+            *reinterpret_cast<uint4 *>(dst + x) = *reinterpret_cast<const uint4 *>(buf + x);
+        const uint32_t t0 = max(b1, b0) + lane;
+        if (t0 < e) dst[t0] = buf[t0];
+        pos += total;
+        __syncwarp();
+    }
+    if (!WRITE && lane == 0) row_bytes[u] = pos;
+}
+
 // Brings the staged lists to their places in the CSR, one warp per list: the
 // stage's lists start on 16-byte boundaries, the CSR's anywhere, so each lane
 // builds aligned 16-byte words of the destination from five words of the
@@ -678,6 +915,15 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
     const size_t mask_smem = (size_t)2 * kSweepWarps * mask_words * 4;   // row masks and staged obstacle words
     const size_t bitmap_smem = (size_t)((words_n + 3) & ~3u) * 4;
     // the node bitmap stays in shared memory while two CTAs fit an SM
+    const uint32_t pitch = (words_n + kTileWords - 1) / kTileWords * kTileWords;
+    const uint64_t matrix_bytes = 32ull * pitch * pitch * 4;
+    DeviceBuffer d_matrix;
+    bool by_rows = n && g_sweep_smem_bitmap_nodes == 0 && matrix_bytes <= kMatrixBytes;
+    if (by_rows && cudaMalloc(&d_matrix.ptr, matrix_bytes) != cudaSuccess) {
+        cudaGetLastError();
+        d_matrix.ptr = nullptr;
+        by_rows = false;
+    }
     const bool smem_bitmap = bitmap_smem + list_smem + mask_smem + 1024 <= (size_t)smem_optin / 2 &&
                              (g_sweep_smem_bitmap_nodes == 0 || n <= g_sweep_smem_bitmap_nodes);
     const int glist_cap = maxdim + 2;   // at most k + 1 intervals are alive at column k + 1
@@ -689,7 +935,7 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
     VGA_TRY(d_cells.alloc((size_t)std::max<uint32_t>(n, 1) * 4));
     VGA_TRY(d_rowbytes.alloc((size_t)std::max<uint32_t>(n, 1) * 8));
     VGA_TRY(d_counter.alloc(6 * sizeof(uint32_t)));
-    VGA_TRY(d_retry.alloc((size_t)std::max<uint32_t>(n, 1) * 4));
+    VGA_TRY(d_retry.alloc((size_t)std::max<uint32_t>(n, 1) * 4 * (by_rows ? kRowsOctants : 1)));
     VGA_TRY(d_err.alloc(sizeof(int)));
     cudaStream_t stream = 0;
     VGA_CHECK_CUDA(cudaMemcpyAsync(d_rowbits.ptr, rowbits.data(), rowbits.size() * 4, cudaMemcpyHostToDevice, stream));
@@ -795,7 +1041,56 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
         VGA_CHECK_CUDA(cudaStreamSynchronize(stream));
         return launch(mode, true, retry_list, n_retry, d_counter.as<uint32_t>() + 1);
     };
-    if (n) {
+    DeviceBuffer d_noc_t;
+    if (by_rows) {
+        std::vector<int32_t> noc_t((size_t)W * H);
+        for (int y = 0; y < H; y++)
+            for (int x = 0; x < W; x++) noc_t[(size_t)x * H + y] = node_of_cell[(size_t)y * W + x];
+        VGA_TRY(d_noc_t.alloc(noc_t.size() * 4));
+        VGA_CHECK_CUDA(cudaMemcpyAsync(d_noc_t.ptr, noc_t.data(), noc_t.size() * 4, cudaMemcpyHostToDevice, stream));
+        VGA_CHECK_CUDA(cudaMemsetAsync(d_matrix.ptr, 0, matrix_bytes, stream));
+        sa.node_of_cell_t = d_noc_t.as<int32_t>();
+        sa.matrix = d_matrix.as<uint32_t>();
+        sa.pitch = pitch;
+        auto sweep_rows = [&](bool global_lists, const uint32_t *sources, uint32_t count, uint32_t *counter) -> int {
+            if (!count) return VGA_OK;
+            auto fn = global_lists ? visibility_rows_kernel<true> : visibility_rows_kernel<false>;
+            const size_t smem = (global_lists ? 0 : list_smem) + mask_smem;
+            VGA_CHECK_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            int per_sm = 0;
+            VGA_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kSweepThreads, smem));
+            if (per_sm < 1) {
+                set_error("visibility sweep: %zu bytes of shared memory do not fit an SM", smem);
+                return VGA_EINVAL;
+            }
+            const uint32_t grid = (uint32_t)std::min<uint64_t>((uint64_t)sms * per_sm, (count + kSweepWarps - 1) / kSweepWarps);
+            if (global_lists) VGA_TRY(d_glists.alloc((size_t)grid * kSweepWarps * 2 * glist_cap * sizeof(uint2)));
+            SweepArgs a = sa;
+            a.sources = sources;
+            a.count = count;
+            a.next = counter;
+            a.glists = d_glists.as<uint2>();
+            fn<<<grid, kSweepThreads, smem, stream>>>(a);
+            count_launch();
+            VGA_CHECK_CUDA(cudaGetLastError());
+            return VGA_OK;
+        };
+        VGA_TRY(sweep_rows(false, nullptr, n * kRowsOctants, d_counter.as<uint32_t>()));
+        VGA_CHECK_CUDA(cudaMemcpyAsync(&n_retry, sa.retry_count, 4, cudaMemcpyDeviceToHost, stream));
+        VGA_CHECK_CUDA(cudaStreamSynchronize(stream));
+        VGA_TRY(sweep_rows(true, retry_list, n_retry, d_counter.as<uint32_t>() + 1));
+        VGA_CHECK_CUDA(cudaFuncSetAttribute(rows_join_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kJoinSmem));
+        const unsigned tiles = pitch / kTileWords;
+        rows_join_kernel<<<dim3(tiles, tiles), 256, kJoinSmem, stream>>>(sa.matrix, pitch);
+        count_launch();
+        rows_encode_kernel<false><<<(n + kEncodeWarps - 1) / kEncodeWarps, kEncodeWarps * 32, 0, stream>>>(
+            sa.matrix, pitch, words_n, n, sa.row_bytes, nullptr, nullptr, sa.err);
+        count_launch();
+        VGA_CHECK_CUDA(cudaGetLastError());
+        std::vector<uint64_t> rb;
+        VGA_TRY(read_row_bytes(rb));
+        for (uint32_t v = 0; v < n; v++) offsets[v + 1] = offsets[v] + rb[v];
+    } else if (n) {
         constexpr uint64_t kStageSmall = 256ull << 20;
         constexpr uint32_t kSampleStep = 128;
         std::vector<uint64_t> rb;
@@ -845,17 +1140,24 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
     DeviceBuffer d_off, d_bytes;
     VGA_TRY(d_off.alloc(((size_t)n + 1) * 8));
     if (d_bytes.alloc(n_bytes + kBytePad) != VGA_OK) {
-        if (!d_stage.ptr) return VGA_ENOMEM;
-        // no room beside the stage: every list is swept again
+        if (!d_stage.ptr && !d_matrix.ptr) return VGA_ENOMEM;
+        // no room beside the stage or the matrix: every list is swept again
         cudaGetLastError();
         clear_error();
         d_stage.reset();
+        d_matrix.reset();
         again.resize(n);
         for (uint32_t v = 0; v < n; v++) again[v] = v;
         VGA_TRY(d_bytes.alloc(n_bytes + kBytePad));
     }
     VGA_CHECK_CUDA(cudaMemcpyAsync(d_off.ptr, offsets.data(), ((size_t)n + 1) * 8, cudaMemcpyHostToDevice, stream));
     VGA_CHECK_CUDA(cudaMemsetAsync(d_bytes.as<uint8_t>() + n_bytes, 0, kBytePad, stream));
+    if (d_matrix.ptr) {
+        rows_encode_kernel<true><<<(n + kEncodeWarps - 1) / kEncodeWarps, kEncodeWarps * 32, 0, stream>>>(
+            sa.matrix, pitch, words_n, n, nullptr, d_off.as<uint64_t>(), d_bytes.as<uint8_t>(), sa.err);
+        count_launch();
+        VGA_CHECK_CUDA(cudaGetLastError());
+    }
     if (n && d_stage.ptr) {
         stage_gather_kernel<<<(n + 7) / 8, 256, 0, stream>>>(d_stage.as<uint8_t>(), d_stage_at.as<uint64_t>(),
                                                             d_off.as<uint64_t>(), n, d_bytes.as<uint8_t>());
@@ -871,16 +1173,16 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
         sa.out = d_bytes.as<uint8_t>();
         sa.retry = retry_list = d_again_retry.as<uint32_t>();
         VGA_TRY(sweep(kSweepWrite, d_again.as<uint32_t>(), (uint32_t)again.size()));
-        int err = 0;
-        VGA_CHECK_CUDA(cudaMemcpyAsync(&err, d_err.ptr, sizeof(int), cudaMemcpyDeviceToHost, stream));
-        VGA_CHECK_CUDA(cudaStreamSynchronize(stream));
-        if (err) {
-            set_error("visibility sweep failed its own checks (code %d)", err);
-            return VGA_ECORRUPT;
-        }
     }
+    int err = 0;
+    VGA_CHECK_CUDA(cudaMemcpyAsync(&err, d_err.ptr, sizeof(int), cudaMemcpyDeviceToHost, stream));
     VGA_CHECK_CUDA(cudaStreamSynchronize(stream));
+    if (err) {
+        set_error("visibility sweep failed its own checks (code %d)", err);
+        return VGA_ECORRUPT;
+    }
     d_stage.reset();
+    d_matrix.reset();
     uint64_t *po = d_off.as<uint64_t>();
     uint8_t *pb = d_bytes.as<uint8_t>();
     d_off.release();

@@ -327,6 +327,19 @@ int finish_graph_load(uint32_t n, uint64_t n_bytes, uint64_t *d_offsets, uint8_t
                       cudaStream_t stream, vga_graph **out, const uint64_t *h_offsets = nullptr,
                       const uint8_t *h_bytes = nullptr);
 
+// A graph whose builder knows its degrees (device), range lookups of table scheme
+// `scheme` (host) and edges.  Takes ownership of the device pointers and of
+// built.degree on success, and frees the pointers on failure.
+struct BuiltGraph {
+    DeviceBuffer degree;
+    std::vector<uint32_t> lookups;
+    int scheme = 0;
+    uint64_t edges = 0;
+    uint32_t max_degree = 0;
+};
+int make_built_graph(uint32_t n, uint64_t n_bytes, uint64_t *d_offsets, uint8_t *d_bytes, BuiltGraph &built,
+                     vga_graph **out);
+
 // ---------------------------------------------------------------------------
 // Warp LEB128 window decoder (Sec. 3.2 encoding; the paper decodes each list
 // with one thread into shared memory, here a whole warp decodes 32 bytes per

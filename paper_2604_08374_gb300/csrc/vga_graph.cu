@@ -145,6 +145,23 @@ int finish_graph_load(uint32_t n, uint64_t n_bytes, uint64_t *d_offsets, uint8_t
         set_error("malformed CSR: the byte range of node %u breaks the LEB128 delta format", bad);
         return VGA_ECORRUPT;
     }
+    BuiltGraph built;
+    built.degree.ptr = degree.release();
+    built.lookups.swap(h_cnt);
+    built.scheme = scheme;
+    built.edges = edges;
+    built.max_degree = maxdeg;
+    VGA_TRY(make_built_graph(n, n_bytes, static_cast<uint64_t *>(offsets.release()),
+                             static_cast<uint8_t *>(bytes.release()), built, out));
+    (*out)->d_comp = static_cast<uint32_t *>(comp.release());
+    return VGA_OK;
+}
+
+int make_built_graph(uint32_t n, uint64_t n_bytes, uint64_t *d_offsets, uint8_t *d_bytes, BuiltGraph &built,
+                     vga_graph **out) {
+    DeviceBuffer offsets, bytes;
+    offsets.ptr = d_offsets;
+    bytes.ptr = d_bytes;
     vga_graph *g = new (std::nothrow) vga_graph;
     if (!g) {
         set_error("out of host memory");
@@ -153,17 +170,16 @@ int finish_graph_load(uint32_t n, uint64_t n_bytes, uint64_t *d_offsets, uint8_t
     cudaGetDevice(&g->device);
     g->n = n;
     g->n_bytes = n_bytes;
-    g->n_edges = edges;
-    g->max_degree = maxdeg;
+    g->n_edges = built.edges;
+    g->max_degree = built.max_degree;
     g->d_offsets = static_cast<uint64_t *>(offsets.release());
     g->d_bytes = static_cast<uint8_t *>(bytes.release());
-    g->d_degree = static_cast<uint32_t *>(degree.release());
-    g->d_comp = static_cast<uint32_t *>(comp.release());
+    g->d_degree = static_cast<uint32_t *>(built.degree.release());
     // offsets of the run-aware union's lookups (the list itself is built on first use)
-    g->lk_scheme = scheme;
-    vga_graph::RunLookups &L = g->lk[scheme];
+    g->lk_scheme = built.scheme;
+    vga_graph::RunLookups &L = g->lk[built.scheme];
     L.h_off.assign((size_t)n + 1, 0);
-    for (uint32_t v = 0; v < n; v++) L.h_off[v + 1] = L.h_off[v] + h_cnt[v];
+    for (uint32_t v = 0; v < n; v++) L.h_off[v + 1] = L.h_off[v] + built.lookups[v];
     L.total = L.h_off[n];
     *out = g;
     return VGA_OK;

@@ -13,16 +13,17 @@
 // bitmaps; (device) per source, the four octants that see the cells after it in
 // raster order swept into its row of a bit matrix, and the matrix joined with
 // its transpose (visibility is symmetric); the bytes of every row's LEB128 list
-// counted; (host) prefix sum into offsets; (device) the lists written; then the
-// ordinary load path validates the stream and derives degrees.  Graphs whose
-// matrix would be too large (kMatrixBytes) have all eight octants of a source
-// swept into one CTA's node bitmap and its list written to a stage in the order
-// the sources finish, from where it is brought to its place.
+// counted, with the degrees and range lookups; (host) prefix sum into offsets;
+// (device) the lists written.  Graphs whose matrix would be too large
+// (kMatrixBytes) have all eight octants of a source swept into one CTA's node
+// bitmap and its list written to a stage in the order the sources finish, from
+// where it is brought to its place; the ordinary load path then validates the
+// stream and derives degrees.
 #include <algorithm>
 #include <utility>
 #include <vector>
 
-#include "vga_common.cuh"
+#include "runs.cuh"
 
 namespace vga {
 namespace {
@@ -737,26 +738,92 @@ __global__ void __launch_bounds__(256) rows_join_kernel(uint32_t *__restrict__ m
     }
 }
 
-// LEB128 delta lists of the matrix's rows, one warp per row, 32 words a step:
-// their sizes, or (WRITE) their bytes.  Within a word every delta is below 128,
-// so only a word's first id can take more than one byte.  A step's bytes (at
-// most 32 x 36) are put together in shared memory and stored 16 at a time.
+// What the graph object keeps of a row of the matrix: the node's degree, its
+// list's bytes and its range lookups (a run of L ids takes run_lookup_count(L)
+// of them), one warp per row, 32 words a step.  A run is counted where it ends;
+// its start follows from the last clear bit before it.
 constexpr int kEncodeWarps = 8;
-template <bool WRITE>
-__global__ void __launch_bounds__(kEncodeWarps * 32) rows_encode_kernel(const uint32_t *__restrict__ matrix,
-                                                                       uint32_t pitch, uint32_t words, uint32_t n,
-                                                                       uint64_t *__restrict__ row_bytes,
-                                                                       const uint64_t *__restrict__ offsets,
-                                                                       uint8_t *__restrict__ out, int *err) {
-    __shared__ __align__(16) uint8_t s_buf[WRITE ? kEncodeWarps : 1][32 * 36 + 32];
+__global__ void __launch_bounds__(kEncodeWarps * 32) rows_count_kernel(const uint32_t *__restrict__ matrix,
+                                                                      uint32_t pitch, uint32_t words, uint32_t n,
+                                                                      int scheme, uint64_t *__restrict__ row_bytes,
+                                                                      uint32_t *__restrict__ degree,
+                                                                      uint32_t *__restrict__ lookups) {
     const int lane = threadIdx.x & 31;
     const uint64_t u = (uint64_t)blockIdx.x * kEncodeWarps + (threadIdx.x >> 5);
     if (u >= n) return;
-    uint8_t *buf = s_buf[WRITE ? threadIdx.x >> 5 : 0];
+    const uint32_t *row = matrix + u * pitch;
+    int run = -1, clear = -1;  // last set and last clear id so far
+    uint32_t ids = 0, more = 0, lks = 0;
+    uint32_t next = lane < (int)words ? __ldcs(row + lane) : 0u;
+    for (uint32_t c = 0; c < words; c += 32) {
+        const uint32_t wi = c + lane;
+        const uint32_t word = next;
+        next = wi + 32 < words ? __ldcs(row + wi + 32) : 0u;
+        const int last_id = (int)(c * 32 + 1023);
+        if (!__any_sync(0xffffffffu, word != 0u)) {
+            clear = last_id;
+            continue;
+        }
+        int set = word ? (int)(wi * 32 + 31 - __clz(word)) : -1;
+        int zero = ~word ? (int)(wi * 32 + 31 - __clz(~word)) : -1;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, set, o), y = __shfl_up_sync(0xffffffffu, zero, o);
+            if (lane >= o) {
+                set = max(set, x);
+                zero = max(zero, y);
+            }
+        }
+        int set_before = __shfl_up_sync(0xffffffffu, set, 1), zero_before = __shfl_up_sync(0xffffffffu, zero, 1);
+        if (lane == 0) set_before = zero_before = -1;
+        set_before = max(set_before, run);
+        zero_before = max(zero_before, clear);
+        run = max(run, __shfl_sync(0xffffffffu, set, 31));
+        clear = max(clear, __shfl_sync(0xffffffffu, zero, 31));
+        uint32_t after = __shfl_down_sync(0xffffffffu, word, 1);
+        const uint32_t over = __shfl_sync(0xffffffffu, next, 0);
+        if (lane == 31) after = over;
+        if (word) {
+            const uint32_t wf = wi * 32 + (__ffs(word) - 1);
+            ids += __popc(word);
+            more += varint_len(set_before < 0 ? wf : wf - (uint32_t)set_before) - 1u;
+            for (uint32_t ends = word & ~(word >> 1 | after << 31); ends; ends &= ends - 1u) {
+                const int k = __ffs(ends) - 1;
+                const uint32_t z = ~word & ((1u << k) - 1u);
+                const int start = z ? (int)(wi * 32 + 32 - __clz(z)) : zero_before + 1;
+                lks += run_lookup_count(wi * 32 + k + 1u - (uint32_t)start, scheme);
+            }
+        }
+    }
+    ids = __reduce_add_sync(0xffffffffu, ids);
+    more = __reduce_add_sync(0xffffffffu, more);
+    lks = __reduce_add_sync(0xffffffffu, lks);
+    if (lane == 0) {
+        row_bytes[u] = (uint64_t)ids + more;
+        degree[u] = ids;
+        lookups[u] = lks;
+    }
+}
+
+// LEB128 delta lists of the matrix's rows, one warp per row, 32 words a step.
+// Within a word every delta is below 128, so only a word's first id can take
+// more than one byte.  Most bytes are the 1 of a consecutive id: a step's bytes
+// (at most 32 x 36) are filled with ones in shared memory, the lanes put in the
+// deltas where runs start, and the step is stored 16 bytes at a time.
+__global__ void __launch_bounds__(kEncodeWarps * 32) rows_encode_kernel(const uint32_t *__restrict__ matrix,
+                                                                       uint32_t pitch, uint32_t words, uint32_t n,
+                                                                       const uint64_t *__restrict__ offsets,
+                                                                       uint8_t *__restrict__ out, int *err) {
+    constexpr uint32_t kBuf = 32 * 36 + 32;
+    __shared__ __align__(16) uint8_t s_buf[kEncodeWarps][kBuf];
+    const int lane = threadIdx.x & 31;
+    const uint64_t u = (uint64_t)blockIdx.x * kEncodeWarps + (threadIdx.x >> 5);
+    if (u >= n) return;
+    uint8_t *buf = s_buf[threadIdx.x >> 5];
     const uint32_t *row = matrix + u * pitch;
     int run = -1;  // last id so far
-    uint64_t pos = WRITE ? offsets[u] : 0;
-    const uint64_t end = WRITE ? offsets[u + 1] : 0;
+    uint64_t pos = offsets[u];
+    const uint64_t end = offsets[u + 1];
     uint32_t next = lane < (int)words ? __ldcs(row + lane) : 0u;
     for (uint32_t c = 0; c < words; c += 32) {
         const uint32_t wi = c + lane;
@@ -772,16 +839,10 @@ __global__ void __launch_bounds__(kEncodeWarps * 32) rows_encode_kernel(const ui
         int excl = __shfl_up_sync(0xffffffffu, incl, 1);
         if (lane == 0) excl = -1;
         if (run > excl) excl = run;
-        uint32_t nb = 0;
-        if (word) {
-            const uint32_t wf = wi * 32 + (__ffs(word) - 1);
-            nb = (uint32_t)__popc(word) - 1u + varint_len(excl < 0 ? wf : wf - (uint32_t)excl);
-        }
+        const uint32_t wf = wi * 32 + (uint32_t)(word ? __ffs(word) - 1 : 0);
+        const uint32_t first = word ? varint_len(excl < 0 ? wf : wf - (uint32_t)excl) : 0u;  // bytes of the first id
+        const uint32_t nb = word ? (uint32_t)__popc(word) - 1u + first : 0u;
         run = max(run, __shfl_sync(0xffffffffu, incl, 31));
-        if (!WRITE) {
-            pos += __reduce_add_sync(0xffffffffu, nb);
-            continue;
-        }
         uint32_t sc = nb;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -790,26 +851,36 @@ __global__ void __launch_bounds__(kEncodeWarps * 32) rows_encode_kernel(const ui
         }
         const uint32_t total = __shfl_sync(0xffffffffu, sc, 31);
         const uint32_t head = (uint32_t)(pos & 15u);  // the buffer holds the bytes from pos - head on
-        uint32_t q = head + sc - nb, left = word;
-        int last = excl;
-        while (left) {
-            const uint32_t id = wi * 32 + (__ffs(left) - 1);
-            left &= left - 1u;
-            uint32_t x = last < 0 ? id : id - (uint32_t)last;
-            while (x > 0x7fu) {
-                buf[q++] = (uint8_t)(x | 0x80u);
-                x >>= 7;
-            }
-            buf[q++] = (uint8_t)x;
-            last = (int)id;
-        }
-        __syncwarp();
+        const uint32_t e = head + total;
         if (pos + total > end) {  // the count pass sized the list
             if (lane == 0) atomicOr(err, 8);
             break;
         }
+        for (uint32_t x = 16u * lane; x < e; x += 512u)
+            *reinterpret_cast<uint4 *>(buf + x) = make_uint4(0x01010101u, 0x01010101u, 0x01010101u, 0x01010101u);
+        __syncwarp();
+        if (word) {
+            const uint32_t q = head + sc - nb;
+            const bool goes_on = excl >= 0 && (uint32_t)excl + 1u == wi * 32;  // the id before the word is set
+            uint32_t starts = word & ~(word << 1 | (goes_on ? 1u : 0u));
+            if (starts & (word & (0u - word))) {  // the first id starts a run
+                uint32_t x = excl < 0 ? wf : wf - (uint32_t)excl, at = q;
+                starts &= starts - 1u;
+                while (x > 0x7fu) {
+                    buf[at++] = (uint8_t)(x | 0x80u);
+                    x >>= 7;
+                }
+                buf[at] = (uint8_t)x;
+            }
+            for (; starts; starts &= starts - 1u) {
+                const int k = __ffs(starts) - 1;
+                const uint32_t below = word & ((1u << k) - 1u);
+                buf[q + first - 1u + __popc(below)] = (uint8_t)(k - (31 - __clz(below)));
+            }
+        }
+        __syncwarp();
         uint8_t *dst = out + (pos - head);
-        const uint32_t e = head + total, b0 = head ? 16u : 0u, b1 = e & ~15u;
+        const uint32_t b0 = head ? 16u : 0u, b1 = e & ~15u;
         if (head && lane >= (int)head && lane < 16 && lane < (int)e) dst[lane] = buf[lane];
         for (uint32_t x = b0 + 16u * lane; x < b1; x += 512u)
             *reinterpret_cast<uint4 *>(dst + x) = *reinterpret_cast<const uint4 *>(buf + x);
@@ -818,7 +889,6 @@ __global__ void __launch_bounds__(kEncodeWarps * 32) rows_encode_kernel(const ui
         pos += total;
         __syncwarp();
     }
-    if (!WRITE && lane == 0) row_bytes[u] = pos;
 }
 
 // Brings the staged lists to their places in the CSR, one warp per list: the
@@ -1042,6 +1112,7 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
         return launch(mode, true, retry_list, n_retry, d_counter.as<uint32_t>() + 1);
     };
     DeviceBuffer d_noc_t;
+    BuiltGraph built;  // what the matrix tells of the graph (without it, the load path derives it)
     if (by_rows) {
         std::vector<int32_t> noc_t((size_t)W * H);
         for (int y = 0; y < H; y++)
@@ -1083,13 +1154,27 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
         const unsigned tiles = pitch / kTileWords;
         rows_join_kernel<<<dim3(tiles, tiles), 256, kJoinSmem, stream>>>(sa.matrix, pitch);
         count_launch();
-        rows_encode_kernel<false><<<(n + kEncodeWarps - 1) / kEncodeWarps, kEncodeWarps * 32, 0, stream>>>(
-            sa.matrix, pitch, words_n, n, sa.row_bytes, nullptr, nullptr, sa.err);
+        built.scheme = table_scheme_auto(n, dev);
+        VGA_TRY(built.degree.alloc((size_t)n * 4));
+        DeviceBuffer d_lookups;
+        VGA_TRY(d_lookups.alloc((size_t)n * 4));
+        rows_count_kernel<<<(n + kEncodeWarps - 1) / kEncodeWarps, kEncodeWarps * 32, 0, stream>>>(
+            sa.matrix, pitch, words_n, n, built.scheme, sa.row_bytes, built.degree.as<uint32_t>(),
+            d_lookups.as<uint32_t>());
         count_launch();
         VGA_CHECK_CUDA(cudaGetLastError());
+        std::vector<uint32_t> deg(n);
+        built.lookups.resize(n);
+        VGA_CHECK_CUDA(cudaMemcpyAsync(deg.data(), built.degree.ptr, (size_t)n * 4, cudaMemcpyDeviceToHost, stream));
+        VGA_CHECK_CUDA(cudaMemcpyAsync(built.lookups.data(), d_lookups.ptr, (size_t)n * 4, cudaMemcpyDeviceToHost,
+                                       stream));
         std::vector<uint64_t> rb;
         VGA_TRY(read_row_bytes(rb));
-        for (uint32_t v = 0; v < n; v++) offsets[v + 1] = offsets[v] + rb[v];
+        for (uint32_t v = 0; v < n; v++) {
+            offsets[v + 1] = offsets[v] + rb[v];
+            built.edges += deg[v];
+            built.max_degree = std::max(built.max_degree, deg[v]);
+        }
     } else if (n) {
         constexpr uint64_t kStageSmall = 256ull << 20;
         constexpr uint32_t kSampleStep = 128;
@@ -1153,8 +1238,8 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
     VGA_CHECK_CUDA(cudaMemcpyAsync(d_off.ptr, offsets.data(), ((size_t)n + 1) * 8, cudaMemcpyHostToDevice, stream));
     VGA_CHECK_CUDA(cudaMemsetAsync(d_bytes.as<uint8_t>() + n_bytes, 0, kBytePad, stream));
     if (d_matrix.ptr) {
-        rows_encode_kernel<true><<<(n + kEncodeWarps - 1) / kEncodeWarps, kEncodeWarps * 32, 0, stream>>>(
-            sa.matrix, pitch, words_n, n, nullptr, d_off.as<uint64_t>(), d_bytes.as<uint8_t>(), sa.err);
+        rows_encode_kernel<<<(n + kEncodeWarps - 1) / kEncodeWarps, kEncodeWarps * 32, 0, stream>>>(
+            sa.matrix, pitch, words_n, n, d_off.as<uint64_t>(), d_bytes.as<uint8_t>(), sa.err);
         count_launch();
         VGA_CHECK_CUDA(cudaGetLastError());
     }
@@ -1187,7 +1272,8 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
     uint8_t *pb = d_bytes.as<uint8_t>();
     d_off.release();
     d_bytes.release();
-    VGA_TRY(finish_graph_load(n, n_bytes, po, pb, nullptr, stream, out));
+    if (by_rows) VGA_TRY(make_built_graph(n, n_bytes, po, pb, built, out));
+    else VGA_TRY(finish_graph_load(n, n_bytes, po, pb, nullptr, stream, out));
     // the builder knows every node's cell: the grouped union groups 2 x 2 blocks
     (*out)->cells.swap(cells);
     (*out)->cells_W = W;

@@ -10,7 +10,7 @@
 //   codes     from the second pass on, jobs without split hubs gather register
 //             codes instead (codes.cuh): the same queue over code slices, then
 //             the pieces left open;
-//   estimate  one warp per node of every running job (estimator + Eq. sumD);
+//   estimate  warps over runs of nodes of every running job (estimator + Eq. sumD);
 //   step      one thread per job: pass count, stop rule, flags;
 //   finalize  mean depth and ball sizes of the jobs that just stopped.
 // The pass loop is either driven from the host (one flag read per pass) or
@@ -139,30 +139,30 @@ __global__ void __launch_bounds__(kGroupScatterWarps * 32) batch_first_groups_ke
 // The one-bit pass just run left too much open: it is done again in 4 bits.
 __device__ __forceinline__ bool pass_again(const JobDev &J) { return J.K == 1 && J.open > J.open_cap; }
 
-// Nodes that stand for all when the registers at the window's top are counted.
-constexpr uint32_t kTopSample = 8;
-
 // initial != 0: c_0 of every job; otherwise pass t = job.t + 1 of running jobs.
 __global__ void batch_estimate_kernel(JobDev *jobs, const uint64_t *__restrict__ node_start, int n_jobs,
                                       uint64_t total_nodes, int initial) {
     const int lane = threadIdx.x & 31;
     const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
-    for (uint64_t x = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); x < total_nodes; x += warps) {
+    const uint64_t per = (total_nodes + warps - 1) / warps;  // consecutive nodes: one search a job
+    uint64_t x = ((uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per;
+    const uint64_t x1 = min(x + per, total_nodes);
+    while (x < x1) {
         const int j = find_job(node_start, n_jobs, x);
         JobDev &J = jobs[j];
-        if (!initial && J.state != 0) continue;
-        if (!initial && pass_again(J)) continue;
+        const uint64_t start = node_start[j], stop = min((uint64_t)node_start[j + 1], x1);
+        if (!initial && (J.state != 0 || pass_again(J))) {
+            x = stop;
+            continue;
+        }
         const int t = initial ? 0 : J.t + 1;
         const double *c_prev = t ? J.c[(t - 1) & 1] : nullptr;
-        const uint32_t v = (uint32_t)(x - node_start[j]);
         const uint32_t *top = J.codes && !initial ? J.win + (2u << J.p) : nullptr;
-        uint32_t at_top = 0;
-        estimate_node(J.regs[t & 1], J.n, J.p, J.S, t, J.alpha_mm, J.lc, c_prev, J.c[t & 1], J.sum_d, &J.inc, v, lane,
-                      false, top, &at_top);
-        if (top && lane == 0) {
-            J.full[v] = at_top == (1u << J.p) ? 1u : 0u;
-            if (v % kTopSample == 0) atomicAdd(&J.n_top, (unsigned long long)at_top);
-        }
+        uint64_t at_top = 0;
+        estimate_nodes(J.regs[t & 1], J.n, J.p, J.S, t, J.alpha_mm, J.lc, c_prev, J.c[t & 1], J.sum_d, &J.inc,
+                       (uint32_t)(x - start), (uint32_t)(stop - start), lane, false, top, J.full, &at_top);
+        x = stop;
+        if (top && lane == 0) atomicAdd(&J.n_top, (unsigned long long)at_top);
     }
 }
 
@@ -291,7 +291,7 @@ constexpr size_t engine_code_smem() {
 // of a code slice, then blocks of kEngineBlock groups), with the tables packed
 // from the registers (code_table_item) and each group gathered and settled by
 // one warp (code_group, code_store).  A CTA that meets a job whose pass is of
-// another kind moves the queue past all of that job's items.  64 registers (4
+// another kind moves the queue past that job and the idle ones after it.  64 registers (4
 // CTAs of 8 warps an SM) as in the single-graph kernel's measurement.
 template <int S, int K>
 __global__ void __launch_bounds__(kEngineWarps * 32, 4) batch_code_kernel(JobDev *jobs,
@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(kEngineWarps * 32, 4) batch_code_kernel(JobDev
     extern __shared__ __align__(128) unsigned char s_dyn[];
     __shared__ unsigned long long s_item;
     __shared__ uint32_t s_next;
-    __shared__ int s_ok;
+    __shared__ int s_ok, s_skip;
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
     LkStage &st = reinterpret_cast<LkStage *>(s_dyn)[wib];
@@ -325,7 +325,19 @@ __global__ void __launch_bounds__(kEngineWarps * 32, 4) batch_code_kernel(JobDev
         const int k = find_job(item_start, n_jobs, item);
         JobDev &J = jobs[gjobs[k]];
         if (J.state != 0 || J.K != K) {
-            if (threadIdx.x == 0) atomicMax(counter, (unsigned long long)item_start[k + 1]);
+            // past this job and those after it that have nothing here either
+            const int next = k + 1 + (int)threadIdx.x;
+            bool idle = false;
+            if (next < n_jobs) {
+                const JobDev &N = jobs[gjobs[next]];
+                idle = N.state != 0 || N.K != K;
+            }
+            if (threadIdx.x == 0) s_skip = (int)blockDim.x;
+            __syncthreads();
+            if (!idle) atomicMin(&s_skip, (int)threadIdx.x);
+            __syncthreads();
+            if (threadIdx.x == 0)
+                atomicMax(counter, (unsigned long long)item_start[min(k + 1 + s_skip, n_jobs)]);
             continue;
         }
         const uint32_t n = J.n;
@@ -397,7 +409,7 @@ __global__ void __launch_bounds__(kEngineWarps * 32, 4) batch_code_kernel(JobDev
 
 // The pieces that this pass's code unions left open (code_open_piece),
 // kOpenCtas CTAs a job.
-constexpr unsigned kOpenCtas = 16;
+constexpr unsigned kOpenCtas = 64;
 __global__ void __launch_bounds__(256) batch_open_kernel(JobDev *jobs) {
     __shared__ uint4 s_max[8];
     JobDev &J = jobs[blockIdx.x / kOpenCtas];
@@ -432,8 +444,18 @@ __global__ void batch_step_kernel(JobDev *jobs, int n_jobs, unsigned long long *
                 bool stop = J.conv ? (J.inc == 0u) : (J.changed == 0u);
                 if (J.d > 0 && t >= J.d) stop = true;
                 if (stop) J.state = 1;
-                const double sampled = (double)((J.n + kTopSample - 1u) / kTopSample) * (double)(1u << J.p);
-                if (J.codes) J.K = (double)J.n_top >= kTopShare * sampled && !J.too_open ? 1 : 4;
+                const uint64_t regs = (uint64_t)J.n << J.p;
+                if (J.codes) J.K = (double)J.n_top >= kTopShare * (double)regs && !J.too_open ? 1 : 4;
+                // With every register at its maximum the next pass changes nothing
+                // and is the last: its estimates are these (in the other buffer's
+                // place), its distances gain 0.
+                if (J.codes && !stop && J.n_top == regs) {
+                    J.t = t + 1;
+                    double *c = J.c[0];
+                    J.c[0] = J.c[1];
+                    J.c[1] = c;
+                    J.state = 1;
+                }
             }
             J.changed = 0u;
             J.inc = 0u;

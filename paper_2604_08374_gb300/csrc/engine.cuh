@@ -54,7 +54,7 @@ struct JobDev {
     uint2 *list;            // open pieces of the pass {node, 16-byte piece}, list_cap = all there are
     uint32_t list_cap, open_cap;
     uint32_t open;          // pieces the pass left open
-    unsigned long long n_top;  // registers at the top, over every kTopSample-th node
+    unsigned long long n_top;  // registers at the top
     int group_scatter;      // with `first`: for whole groups (first_pass.cuh)
     int first;              // 1: pass 1 is the scatter of the nodes' keys (engine_start; keys in tab)
     uint32_t changed, inc;  // flags of the pass in progress

@@ -907,6 +907,21 @@ __device__ __forceinline__ void harmonic_partial(const uint8_t *__restrict__ reg
         }
         // A lane adds at most m / 32 terms of at most 2^(K-1) = 2^(64-p) each in
         // this loop, so its sum stays below 2^59: no carry into hi here.
+        if (!nib && !((x.x | x.y | x.z | x.w) & 0xE0E0E0E0u)) {
+            // every register is below 32: 2^(31-M) in 32 bits, a register of 0
+            // adding 2^31, which is taken off again
+            uint64_t sum = 0;
+            uint32_t none = 0;
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                none += __popc(__vcmpeq4(wv[i], 0u) & 0x01010101u);
+#pragma unroll
+                for (int b = 0; b < 4; b++) sum += 0x80000000u >> (uint32_t)__byte_perm(wv[i], 0u, 0x4440 + b);
+            }
+            zeros += none;
+            lo += (sum - ((uint64_t)none << 31)) << (K - 31);
+            continue;
+        }
 #pragma unroll
         for (int i = 0; i < 4; i++)
 #pragma unroll
@@ -961,20 +976,42 @@ __device__ __forceinline__ void estimate_finish(uint64_t lo, uint64_t hi, uint32
     c_cur[v] = c;
 }
 
-// Estimator and Eq. sumD for node v over all its registers (one warp; lane 0
-// writes the results).
-__device__ __forceinline__ void estimate_node(const uint8_t *__restrict__ regs, uint32_t n, int p, int S, int t,
-                                              double alpha_mm, const double *__restrict__ lc,
-                                              const double *__restrict__ c_prev, double *__restrict__ c_cur,
-                                              double *__restrict__ sum_d, uint32_t *__restrict__ inc_flag, uint32_t v,
-                                              int lane, bool nib = false, const uint32_t *__restrict__ top = nullptr,
-                                              uint32_t *at_top = nullptr) {
+// Estimator and Eq. sumD for nodes [v0, v1) over all their registers (one warp).
+// The warp sums one node after another and keeps 32 nodes' sums in its lanes,
+// which then finish together: FP64 issues at a small fraction of the other
+// rates, and a warp's instruction takes the pipe as long for one lane as for 32.
+// With top given (the window of a run that unions codes), full[v] records the
+// nodes whose registers all equal it and *at_top (every lane) their number of
+// registers that do.
+__device__ __forceinline__ void estimate_nodes(const uint8_t *__restrict__ regs, uint32_t n, int p, int S, int t,
+                                               double alpha_mm, const double *__restrict__ lc,
+                                               const double *__restrict__ c_prev, double *__restrict__ c_cur,
+                                               double *__restrict__ sum_d, uint32_t *__restrict__ inc_flag, uint32_t v0,
+                                               uint32_t v1, int lane, bool nib, const uint32_t *__restrict__ top,
+                                               uint8_t *__restrict__ full, uint64_t *at_top) {
     const uint32_t node_bytes = nib ? (1u << p) / 2u : (1u << p);  // 4-bit registers: two per byte
-    uint64_t lo, hi;
-    uint32_t zeros;
-    harmonic_partial(regs, n, p, S, 0u, node_bytes, v, lane, nib, lo, hi, zeros, top, at_top);
-    if (lane != 0) return;
-    estimate_finish(lo, hi, zeros, p, t, alpha_mm, lc, c_prev, c_cur, sum_d, inc_flag, v);
+    for (uint32_t base = v0; base < v1; base += 32u) {
+        const uint32_t cnt = min(v1 - base, 32u);
+        uint64_t my_lo = 0, my_hi = 0;
+        uint32_t my_zeros = 0, my_top = 0;
+        for (uint32_t i = 0; i < cnt; i++) {
+            uint64_t lo, hi;
+            uint32_t zeros, node_top = 0;
+            harmonic_partial(regs, n, p, S, 0u, node_bytes, base + i, lane, nib, lo, hi, zeros, top, &node_top);
+            if (lane == (int)i) {
+                my_lo = lo;
+                my_hi = hi;
+                my_zeros = zeros;
+                my_top = node_top;
+            }
+            *at_top += node_top;
+        }
+        if (lane < (int)cnt) {
+            estimate_finish(my_lo, my_hi, my_zeros, p, t, alpha_mm, lc, c_prev, c_cur, sum_d, inc_flag,
+                            base + (uint32_t)lane);
+            if (top) full[base + (uint32_t)lane] = my_top == (1u << p) ? 1u : 0u;
+        }
+    }
 }
 
 // MD(v) = sum_d[v] / (N_v - 1) (Sec. 3.3), NaN when N_v <= 1; ball = c_t.

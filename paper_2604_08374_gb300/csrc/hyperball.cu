@@ -428,28 +428,24 @@ __global__ void __launch_bounds__(512) stream_bench_kernel(const uint4 *__restri
     if ((threadIdx.x & 31) == 0) out[t0 >> 5] = acc;
 }
 
-// HLL estimate of every node, then Eq. sumD (estimate_node); flags[1]
-// records the paper's convergence test max_v(c_t - c_{t-1}) > 0.5.  With top
-// given (the window of a run that unions codes), full[v] records the nodes
-// whose registers all equal it, and the 64-bit count at flags[6] adds up the
-// registers that do.
+// HLL estimate of every node, then Eq. sumD (estimate_nodes), `per` nodes a
+// warp; flags[1] records the paper's convergence test max_v(c_t - c_{t-1}) >
+// 0.5.  With top given, the 64-bit count at flags[6] adds up the registers that
+// equal it.
 __global__ void hb_estimate_kernel(const uint8_t *__restrict__ regs, uint32_t n, int p, int S, int t,
                                    double alpha_mm, const double *__restrict__ lc, const double *__restrict__ c_prev,
                                    double *__restrict__ c_cur, double *__restrict__ sum_d,
                                    uint32_t *__restrict__ flags, int nib, const uint32_t *__restrict__ top,
-                                   uint8_t *__restrict__ full) {
-    __shared__ uint32_t s_top[32];
+                                   uint8_t *__restrict__ full, uint32_t per) {
+    __shared__ uint64_t s_top[32];
     const int lane = threadIdx.x & 31;
-    const uint64_t warp = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    uint32_t at_top = 0;
-    if (warp < n)
-        estimate_node(regs, n, p, S, t, alpha_mm, lc, c_prev, c_cur, sum_d, flags + 1, (uint32_t)warp, lane, nib != 0,
-                      top, &at_top);
+    const uint64_t v0 = ((uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per;
+    uint64_t at_top = 0;
+    if (v0 < n)
+        estimate_nodes(regs, n, p, S, t, alpha_mm, lc, c_prev, c_cur, sum_d, flags + 1, (uint32_t)v0,
+                       (uint32_t)(v0 + per < n ? v0 + per : n), lane, nib != 0, top, full, &at_top);
     if (!top) return;
-    if (lane == 0) {
-        if (warp < n) full[warp] = at_top == (1u << p) ? 1u : 0u;
-        s_top[threadIdx.x >> 5] = at_top;
-    }
+    if (lane == 0) s_top[threadIdx.x >> 5] = at_top;
     __syncthreads();
     if (threadIdx.x == 0) {
         unsigned long long sum = 0;
@@ -563,6 +559,14 @@ constexpr double kOpenShare = 0.2;
 // Hub threshold of the run-aware union (lookups per work item).
 static uint32_t hub_threshold(const vga_graph *g, int scheme, uint32_t requested) {
     return requested > 0 ? requested : hub_lookups_auto(g, scheme);
+}
+
+// Open pieces that the list of a code pass holds: one a node, or all there are
+// on small graphs, whose 4-bit passes (they leave next to none open) then need no
+// byte union behind them, two idle launches.
+static uint64_t list_entries(const Plan &P) {
+    const uint64_t pieces = P.n * P.node_bytes / 16;
+    return pieces <= (1u << 16) ? std::max<uint64_t>(P.n, pieces) : P.n;
 }
 
 static int make_plan(const vga_graph *g, int p, const vga_tuning *tune, Plan *P) {
@@ -720,8 +724,8 @@ static int make_plan(const vga_graph *g, int p, const vga_tuning *tune, Plan *P)
         o = align256(o + 8ull * P->m + 2ull * P->node_bytes);
         P->off_full = o;
         o = align256(o + P->n);
-        P->off_list = o;  // {node, 16-byte piece} of up to N open pieces
-        o = align256(o + 8 * P->n);
+        P->off_list = o;  // {node, 16-byte piece} of open pieces
+        o = align256(o + 8 * list_entries(*P));
     }
     P->total = o;
     // Per-neighbour mode: codes where a workspace happens to hold them past the
@@ -806,7 +810,7 @@ struct PendingTiming {
     int S, mode, rows;
     bool first;    // the first pass's scatter (hb_first_pass_kernel), not a union slice
     bool tracked;  // a union slice of a change-tracked pass (its work depends on the changes)
-    bool partial;  // the byte union of the pairs a code pass left open
+    bool partial;  // time without bytes: one-bit codes, or the byte union of the pairs a code pass left open
 };
 
 template <int SS, bool NIB>
@@ -947,7 +951,11 @@ static int launch_codes(const Plan &P, const vga_graph *g, int K, uint8_t *base,
     C.full = base + P.off_full;
     C.need = reinterpret_cast<uint32_t *>(base + P.off_need);
     C.list = reinterpret_cast<uint2 *>(base + P.off_list);
-    C.list_cap = (uint32_t)std::min((double)P.n, code_open_cap((double)P.groups.rows_used, P.node_bytes, g->n_edges, P.n));
+    const uint64_t pieces = P.n * P.node_bytes / 16;
+    const bool all_listed = K == 4 && list_entries(P) >= pieces;
+    C.list_cap = all_listed ? (uint32_t)pieces
+                            : (uint32_t)std::min((double)P.n, code_open_cap((double)P.groups.rows_used, P.node_bytes,
+                                                                            g->n_edges, P.n));
     // Warps per group: enough for twice the warps the GPU holds (about 40 an
     // SM), no more than leaves each about 32 rows.
     int dev = 0, sms = 1;
@@ -977,10 +985,12 @@ static int launch_codes(const Plan &P, const vga_graph *g, int K, uint8_t *base,
             pt.mode = P.mode;
             pt.rows = table_rows(P.scheme);
             pt.tracked = tracked;
+            pt.partial = K == 1;  // stops early: its bytes depend on the registers
             timings->push_back(pt);
         }
     }
     VGA_TRY(launch_code_open(C, g->lk[P.scheme].d_off, g->lk[P.scheme].d_lk, sms));
+    if (all_listed) return VGA_OK;
     // more of them: the byte union of their slices, asked for with a wait when
     // there are many slices, else launched for all (the kernels then return at
     // once; a wait costs about 12 us, an idle pair of launches 4)
@@ -1218,10 +1228,15 @@ static int launch_estimate(const Plan &P, const uint8_t *regs, int t, const doub
                            double *c_cur, double *sum_d, uint32_t *flags, cudaStream_t stream,
                            const uint32_t *top = nullptr, uint8_t *full = nullptr) {
     const int warps = 8;
-    const unsigned blocks = (unsigned)((P.n + warps - 1) / warps);
+    // nodes a warp: while the warps fill the GPU twice (about 48 an SM), up to 16
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const uint32_t per = (uint32_t)std::min<uint64_t>(16, std::max<uint64_t>(1, P.n / ((uint64_t)sms * 96)));
+    const unsigned blocks = (unsigned)((P.n + (uint64_t)warps * per - 1) / ((uint64_t)warps * per));
     const double alpha_mm = hll_alpha_host(P.p) * (double)P.m * (double)P.m;
     hb_estimate_kernel<<<blocks, warps * 32, 0, stream>>>(regs, (uint32_t)P.n, P.p, P.S, t, alpha_mm, lc, c_prev,
-                                                          c_cur, sum_d, flags, P.nib, top, full);
+                                                          c_cur, sum_d, flags, P.nib, top, full, per);
     count_launch();
     VGA_CHECK_CUDA(cudaGetLastError());
     return VGA_OK;
@@ -1382,8 +1397,10 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
             else
                 VGA_TRY(launch_union(P, g, cur, nxt, tab, flags, stream, timed ? &timings : nullptr,
                                      tracked ? need : nullptr, chg));
-            if (chg) VGA_TRY(launch_count(P, chg, flags, stream));
-            VGA_TRY(launch_estimate(P, nxt, t, lc, c_prev, c_cur, sum_d, flags, stream, top, full));
+            // what the next pass goes by is not needed of the last one
+            const bool last = d > 0 && t >= d;
+            if (chg && !last) VGA_TRY(launch_count(P, chg, flags, stream));
+            VGA_TRY(launch_estimate(P, nxt, t, lc, c_prev, c_cur, sum_d, flags, stream, last ? nullptr : top, full));
             if (t <= max_trace) VGA_TRY(copy_trace(P, nxt, c_cur, t, trace_regs, trace_c, stream));
             VGA_CHECK_CUDA(cudaMemcpyAsync(&h, flags, sizeof(h), cudaMemcpyDeviceToHost, stream));
             VGA_CHECK_CUDA(cudaStreamSynchronize(stream));
@@ -1397,6 +1414,13 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
             std::swap(c_prev, c_cur);
             const bool stop = (conv_mode == 1) ? (h.f[1] == 0) : (h.f[0] == 0);
             if (stop || (d > 0 && t >= d)) break;
+            // With every register at its maximum the next pass changes nothing:
+            // its estimates are these, its distances gain 0, and it stops.  (A
+            // profiled or traced run shows every pass.)
+            if (top && h.n_top == P.n * P.m && max_trace < 0 && !timed) {
+                t++;
+                break;
+            }
         }
         hb_finalize_kernel<<<(unsigned)((P.n + 255) / 256), 256, 0, stream>>>((uint32_t)P.n, g->d_comp, sum_d,
                                                                                c_prev, md_dev, ball_dev);

@@ -288,13 +288,13 @@ constexpr size_t engine_code_smem() {
 
 // Code union of the running jobs whose pass gathers K-bit codes, in code slices
 // of S bytes a node: the queue and the waits of batch_union_kernel (table items
-// of a code slice, then blocks of kEngineBlock groups), with the tables packed
+// of a code slice, then blocks of kCodeBlock groups), with the tables packed
 // from the registers (code_table_item) and each group gathered and settled by
 // one warp (code_group, code_store).  A CTA that meets a job whose pass is of
-// another kind moves the queue past that job and the idle ones after it.  64 registers (4
-// CTAs of 8 warps an SM) as in the single-graph kernel's measurement.
+// another kind moves the queue past that job and the idle ones after it.  Three CTAs of 8
+// warps an SM: 80 registers, so that little spills (kCodeBlock).
 template <int S, int K>
-__global__ void __launch_bounds__(kEngineWarps * 32, 4) batch_code_kernel(JobDev *jobs,
+__global__ void __launch_bounds__(kEngineWarps * 32, 3) batch_code_kernel(JobDev *jobs,
                                                                          const uint32_t *__restrict__ gjobs,
                                                                          const uint64_t *__restrict__ item_start,
                                                                          int n_jobs, uint64_t total_items,
@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(kEngineWarps * 32, 4) batch_code_kernel(JobDev
         }
         const uint32_t n = J.n;
         const uint32_t tblocks = (n + B - 1u) / B;
-        const uint64_t per_slice = (uint64_t)((J.uunits + kEngineBlock - 1) / kEngineBlock) + tblocks;
+        const uint64_t per_slice = (uint64_t)((J.uunits + kCodeBlock - 1) / kCodeBlock) + tblocks;
         const uint64_t r = item - item_start[k];
         const uint32_t s = (uint32_t)(r / per_slice);
         const uint64_t q = r % per_slice;
@@ -366,8 +366,8 @@ __global__ void __launch_bounds__(kEngineWarps * 32, 4) batch_code_kernel(JobDev
         }
         __syncthreads();
         if (!s_ok) continue;
-        const uint32_t u0 = (uint32_t)(q - tblocks) * kEngineBlock;
-        const uint32_t u1 = min(u0 + kEngineBlock, J.uunits);
+        const uint32_t u0 = (uint32_t)(q - tblocks) * kCodeBlock;
+        const uint32_t u1 = min(u0 + kCodeBlock, J.uunits);
         for (;;) {
             uint32_t x = 0;
             if (lane == 0) x = atomicAdd(&s_next, 1u);
@@ -752,7 +752,8 @@ int engine_upload(const EngineArrays &A, const std::vector<JobDev> &jobs, Engine
             gj.push_back(k);
             is.push_back(items);
             const JobDev &J = jobs[k];
-            const uint64_t ublocks = (J.uunits + kEngineBlock - 1) / kEngineBlock;
+            const uint32_t block = G.K ? kCodeBlock : kEngineBlock;
+            const uint64_t ublocks = (J.uunits + block - 1) / block;
             if (G.K) {
                 const uint64_t B = G.S >= 1024 ? 16 : 32;  // rows of a table item (TableShape)
                 items += ((1ull << J.p) * G.K / 8 / G.S) * (ublocks + (J.n + B - 1) / B);

@@ -11,6 +11,9 @@ namespace vga {
 constexpr int kEngineWarps = 8;
 constexpr int kEngineGroupNodes = 4;  // nodes per group of the grouped union in the engine
 constexpr uint32_t kEngineBlock = 16;  // work units (hub chunks, node groups) per union block of the queue
+// and in one of a code pass, whose groups differ more (they end early): 8 with 3
+// CTAs an SM 26.8 ms for 64 sites, 16 with 4 28.5, 48 36.4
+constexpr uint32_t kCodeBlock = 8;
 // union kernels: (per neighbour | per run | 4-bit codes | 1-bit codes) x slice
 // width 16..1024
 constexpr int kGroups = 28;

@@ -987,11 +987,13 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
     // the node bitmap stays in shared memory while two CTAs fit an SM
     const uint32_t pitch = (words_n + kTileWords - 1) / kTileWords * kTileWords;
     const uint64_t matrix_bytes = 32ull * pitch * pitch * 4;
-    DeviceBuffer d_matrix;
+    DeviceBuffer d_matrix, d_noc_t;
     bool by_rows = n && g_sweep_smem_bitmap_nodes == 0 && matrix_bytes <= kMatrixBytes;
-    if (by_rows && cudaMalloc(&d_matrix.ptr, matrix_bytes) != cudaSuccess) {
+    if (by_rows && (d_matrix.alloc(matrix_bytes) != VGA_OK || d_noc_t.alloc((size_t)W * H * 4) != VGA_OK)) {
         cudaGetLastError();
-        d_matrix.ptr = nullptr;
+        clear_error();
+        d_matrix.reset();
+        d_noc_t.reset();
         by_rows = false;
     }
     const bool smem_bitmap = bitmap_smem + list_smem + mask_smem + 1024 <= (size_t)smem_optin / 2 &&
@@ -1111,13 +1113,11 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
         VGA_CHECK_CUDA(cudaStreamSynchronize(stream));
         return launch(mode, true, retry_list, n_retry, d_counter.as<uint32_t>() + 1);
     };
-    DeviceBuffer d_noc_t;
     BuiltGraph built;  // what the matrix tells of the graph (without it, the load path derives it)
     if (by_rows) {
         std::vector<int32_t> noc_t((size_t)W * H);
         for (int y = 0; y < H; y++)
             for (int x = 0; x < W; x++) noc_t[(size_t)x * H + y] = node_of_cell[(size_t)y * W + x];
-        VGA_TRY(d_noc_t.alloc(noc_t.size() * 4));
         VGA_CHECK_CUDA(cudaMemcpyAsync(d_noc_t.ptr, noc_t.data(), noc_t.size() * 4, cudaMemcpyHostToDevice, stream));
         VGA_CHECK_CUDA(cudaMemsetAsync(d_matrix.ptr, 0, matrix_bytes, stream));
         sa.node_of_cell_t = d_noc_t.as<int32_t>();

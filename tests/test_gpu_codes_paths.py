@@ -81,3 +81,16 @@ def test_per_neighbour_codes(vga, name, p, d, conv, bits):
         assert st == 0, vga.lib().vga_last_error()
         _same(md.cpu().numpy(), ball.cpu().numpy(), it.value, ref)
         assert bool((ws[at + size:] == 0xA5).all())
+
+
+@pytest.mark.parametrize("name,p", [("tiny", 7), ("corridor", 8), ("rect60", 10), ("components", 9)])
+def test_per_neighbour_codes_of_4bit_registers(vga, name, p):
+    off, b, comp = graph(name)
+    ref = oracle.hyperball(off, b, p, 0, seed=4, reg_bits=4, comp_size=comp)
+    with vga.vga_graph_load(off, b, comp) as g:
+        n = g.n_nodes
+        md, ball = (torch.empty(n, dtype=torch.float64, device="cuda") for _ in range(2))
+        ws = torch.empty(8 << 20, dtype=torch.uint8, device="cuda")
+        assert ws.data_ptr() % 256 == 0
+        it = vga.hyperball_run_dev(g, p, 0, 4, md, ball, workspace=ws, union_mode=1, register_bits=4)
+        _same(md.cpu().numpy(), ball.cpu().numpy(), it, ref)

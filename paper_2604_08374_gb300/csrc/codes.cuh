@@ -20,8 +20,9 @@
 // Measured (GB300): the city graph's pass 2 takes four launches of 128-byte
 // K = 4 rows at 3.1 ms and pass 3 one of K = 1 rows at 0.5 ms (2.8 ms before
 // a class was cut short once all its bits were set, code_group), where the byte
-// union takes eight at 2.8 ms each; the d = 3 analysis 57.4 -> 24.3 ms, the
-// unlimited one at p = 12 342 -> 88 ms, medium d = 3 3.10 -> 1.94 ms.
+// union takes eight at 2.8 ms each; the d = 3 analysis (with pass 1 by
+// groups, first_pass.cuh) 57.4 -> 19.5 ms, the unlimited one at p = 12 343 -> 71
+// ms, medium d = 3 3.1 -> 1.5-1.7 ms.
 //
 // Layout: a 16-byte unit holds 32 registers as four bit planes (K = 4; word k =
 // bit k of the codes, bit i = register i) or 128 registers as one plane

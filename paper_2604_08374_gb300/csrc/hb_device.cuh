@@ -905,8 +905,9 @@ __device__ __forceinline__ void harmonic_partial(const uint8_t *__restrict__ reg
             for (int i = 0; i < 4; i++)
                 full += __popc(nib ? equal_bits<true>(wv[i], gv[i]) : equal_bits<false>(wv[i], gv[i]));
         }
-        // A lane adds at most m / 32 terms of at most 2^(K-1) = 2^(64-p) each in
-        // this loop, so its sum stays below 2^59: no carry into hi here.
+        // A lane adds max(16, m / 32) terms (32 of 4 bits) of at most 2^(K-1) =
+        // 2^(64-p) each: at most 2^64, which only a node whose 16 bytes of
+        // registers are all 1 reaches (p = 4, or p = 5 with 4-bit registers).
         if (!nib && !((x.x | x.y | x.z | x.w) & 0xE0E0E0E0u)) {
             // every register is below 32: 2^(31-M) in 32 bits, a register of 0
             // adding 2^31, which is taken off again
@@ -931,6 +932,8 @@ __device__ __forceinline__ void harmonic_partial(const uint8_t *__restrict__ reg
                 lo += M == 0u ? 0ull : 1ull << (K - (int)M);
             }
     }
+    // no register 0 and no sum: it is 2^64
+    if (lo == 0 && zeros == 0 && (uint32_t)lane * 16u < b1 - b0) hi = 1;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         zeros += __shfl_xor_sync(0xffffffffu, zeros, o);

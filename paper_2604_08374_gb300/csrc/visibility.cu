@@ -987,28 +987,21 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
     // the node bitmap stays in shared memory while two CTAs fit an SM
     const uint32_t pitch = (words_n + kTileWords - 1) / kTileWords * kTileWords;
     const uint64_t matrix_bytes = 32ull * pitch * pitch * 4;
-    DeviceBuffer d_matrix, d_noc_t;
     bool by_rows = n && g_sweep_smem_bitmap_nodes == 0 && matrix_bytes <= kMatrixBytes;
-    if (by_rows && (d_matrix.alloc(matrix_bytes) != VGA_OK || d_noc_t.alloc((size_t)W * H * 4) != VGA_OK)) {
-        cudaGetLastError();
-        clear_error();
-        d_matrix.reset();
-        d_noc_t.reset();
-        by_rows = false;
-    }
     const bool smem_bitmap = bitmap_smem + list_smem + mask_smem + 1024 <= (size_t)smem_optin / 2 &&
                              (g_sweep_smem_bitmap_nodes == 0 || n <= g_sweep_smem_bitmap_nodes);
     const int glist_cap = maxdim + 2;   // at most k + 1 intervals are alive at column k + 1
 
-    DeviceBuffer d_rowbits, d_colbits, d_noc, d_cells, d_rowbytes, d_counter, d_retry, d_err, d_gbitmap, d_glists;
+    DeviceBuffer d_rowbits, d_colbits, d_noc, d_cells, d_rowbytes, d_counter, d_retry, d_err, d_off, d_gbitmap, d_glists;
     VGA_TRY(d_rowbits.alloc(rowbits.size() * 4));
     VGA_TRY(d_colbits.alloc(colbits.size() * 4));
     VGA_TRY(d_noc.alloc(node_of_cell.size() * 4));
     VGA_TRY(d_cells.alloc((size_t)std::max<uint32_t>(n, 1) * 4));
     VGA_TRY(d_rowbytes.alloc((size_t)std::max<uint32_t>(n, 1) * 8));
     VGA_TRY(d_counter.alloc(6 * sizeof(uint32_t)));
-    VGA_TRY(d_retry.alloc((size_t)std::max<uint32_t>(n, 1) * 4 * (by_rows ? kRowsOctants : 1)));
+    VGA_TRY(d_retry.alloc((size_t)std::max<uint32_t>(n, 1) * 4));
     VGA_TRY(d_err.alloc(sizeof(int)));
+    VGA_TRY(d_off.alloc(((size_t)n + 1) * 8));
     cudaStream_t stream = 0;
     VGA_CHECK_CUDA(cudaMemcpyAsync(d_rowbits.ptr, rowbits.data(), rowbits.size() * 4, cudaMemcpyHostToDevice, stream));
     VGA_CHECK_CUDA(cudaMemcpyAsync(d_colbits.ptr, colbits.data(), colbits.size() * 4, cudaMemcpyHostToDevice, stream));
@@ -1082,7 +1075,7 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
         return VGA_OK;
     };
 
-    // The lists are swept once, into a stage of the size they are expected to
+    // Without the matrix the lists are swept once, into a stage of the size they are expected to
     // take: the bound of n - 1 varints a list (one more byte for every 128 ids
     // that a delta skips) while that is small, else what every kSampleStep-th
     // source's list takes, and a twentieth on top.  What a full stage leaves
@@ -1090,6 +1083,7 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
     // to its place in the CSR.
     std::vector<uint64_t> offsets((size_t)n + 1, 0);
     std::vector<uint32_t> again;   // sources to be swept again
+    bool all_again = false;        // every source
     uint32_t n_retry = 0;
     DeviceBuffer d_stage, d_stage_at;
     uint32_t *retry_list = d_retry.as<uint32_t>();
@@ -1114,7 +1108,15 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
         return launch(mode, true, retry_list, n_retry, d_counter.as<uint32_t>() + 1);
     };
     BuiltGraph built;  // what the matrix tells of the graph (without it, the load path derives it)
-    if (by_rows) {
+    DeviceBuffer d_matrix;
+    // The bit matrix and what it tells.  VGA_ENOMEM: no room for it and what goes with it.
+    auto build_rows = [&]() -> int {
+        DeviceBuffer d_noc_t, d_lookups, d_rows_retry;
+        VGA_TRY(d_noc_t.alloc((size_t)W * H * 4));
+        VGA_TRY(d_lookups.alloc((size_t)n * 4));
+        VGA_TRY(d_rows_retry.alloc((size_t)n * 4 * kRowsOctants));
+        VGA_TRY(built.degree.alloc((size_t)n * 4));
+        VGA_TRY(d_matrix.alloc(matrix_bytes));
         std::vector<int32_t> noc_t((size_t)W * H);
         for (int y = 0; y < H; y++)
             for (int x = 0; x < W; x++) noc_t[(size_t)x * H + y] = node_of_cell[(size_t)y * W + x];
@@ -1140,6 +1142,7 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
             a.sources = sources;
             a.count = count;
             a.next = counter;
+            a.retry = d_rows_retry.as<uint32_t>();
             a.glists = d_glists.as<uint2>();
             fn<<<grid, kSweepThreads, smem, stream>>>(a);
             count_launch();
@@ -1149,15 +1152,12 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
         VGA_TRY(sweep_rows(false, nullptr, n * kRowsOctants, d_counter.as<uint32_t>()));
         VGA_CHECK_CUDA(cudaMemcpyAsync(&n_retry, sa.retry_count, 4, cudaMemcpyDeviceToHost, stream));
         VGA_CHECK_CUDA(cudaStreamSynchronize(stream));
-        VGA_TRY(sweep_rows(true, retry_list, n_retry, d_counter.as<uint32_t>() + 1));
+        VGA_TRY(sweep_rows(true, d_rows_retry.as<uint32_t>(), n_retry, d_counter.as<uint32_t>() + 1));
         VGA_CHECK_CUDA(cudaFuncSetAttribute(rows_join_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kJoinSmem));
         const unsigned tiles = pitch / kTileWords;
         rows_join_kernel<<<dim3(tiles, tiles), 256, kJoinSmem, stream>>>(sa.matrix, pitch);
         count_launch();
         built.scheme = table_scheme_auto(n, dev);
-        VGA_TRY(built.degree.alloc((size_t)n * 4));
-        DeviceBuffer d_lookups;
-        VGA_TRY(d_lookups.alloc((size_t)n * 4));
         rows_count_kernel<<<(n + kEncodeWarps - 1) / kEncodeWarps, kEncodeWarps * 32, 0, stream>>>(
             sa.matrix, pitch, words_n, n, built.scheme, sa.row_bytes, built.degree.as<uint32_t>(),
             d_lookups.as<uint32_t>());
@@ -1175,12 +1175,30 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
             built.edges += deg[v];
             built.max_degree = std::max(built.max_degree, deg[v]);
         }
-    } else if (n) {
+        return VGA_OK;
+    };
+    // after a way that had no room: what it left behind, and its error
+    auto start_over = [&]() -> int {
+        cudaGetLastError();
+        clear_error();
+        d_matrix.reset();
+        built.degree.reset();
+        d_stage.reset();
+        d_stage_at.reset();
+        d_gbitmap.reset();
+        d_glists.reset();
+        std::fill(offsets.begin(), offsets.end(), 0);
+        VGA_CHECK_CUDA(cudaMemsetAsync(d_counter.ptr, 0, 6 * sizeof(uint32_t), stream));
+        VGA_CHECK_CUDA(cudaMemsetAsync(d_err.ptr, 0, sizeof(int), stream));
+        return VGA_OK;
+    };
+    // all octants of every source into CTAs' bitmaps, the lists counted and (kSweepStage) staged
+    auto build_sources = [&](SweepMode mode) -> int {
         constexpr uint64_t kStageSmall = 256ull << 20;
         constexpr uint32_t kSampleStep = 128;
         std::vector<uint64_t> rb;
         uint64_t cap = (uint64_t)n * ((uint64_t)n + n / 64 + 32);
-        if (cap > kStageSmall) {
+        if (mode == kSweepStage && cap > kStageSmall) {
             std::vector<uint32_t> sample;
             for (uint32_t v = kSampleStep / 2; v < n; v += kSampleStep) sample.push_back(v);
             DeviceBuffer d_sample;
@@ -1194,13 +1212,10 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
             cap = std::min<uint64_t>(cap, (uint64_t)((double)sum / sample.size() * n * 1.05) + 32ull * n);
         }
         if (sa.smem_cap < kSweepCap) cap = std::min<uint64_t>(cap, 64ull * n);   // the test hook fills the stage, too
-        SweepMode mode = kSweepStage;
-        if (cudaMalloc(&d_stage.ptr, cap + 16) != cudaSuccess) {
-            cudaGetLastError();
-            d_stage.ptr = nullptr;
-            mode = kSweepCount;
+        if (mode == kSweepStage) {
+            VGA_TRY(d_stage_at.alloc((size_t)n * 8));
+            VGA_TRY(d_stage.alloc(cap + 16));
         }
-        VGA_TRY(d_stage_at.alloc((size_t)n * 8));
         sa.out = d_stage.as<uint8_t>();
         sa.stage_used = reinterpret_cast<unsigned long long *>(d_counter.as<uint32_t>() + 4);
         sa.stage_cap = cap;
@@ -1212,27 +1227,43 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
         VGA_TRY(read_row_bytes(rb));
         for (uint32_t v = 0; v < n; v++) offsets[v + 1] = offsets[v] + rb[v];
         if (mode == kSweepCount) {
-            again.resize(n);
-            for (uint32_t v = 0; v < n; v++) again[v] = v;
+            all_again = true;
         } else if (used > cap) {
             std::vector<uint64_t> at(n);
             VGA_CHECK_CUDA(cudaMemcpy(at.data(), d_stage_at.ptr, (size_t)n * 8, cudaMemcpyDeviceToHost));
             for (uint32_t v = 0; v < n; v++)
                 if (at[v] == kNotStaged) again.push_back(v);
         }
+        return VGA_OK;
+    };
+    // each way needs less memory than the one before it
+    int rc = VGA_OK;
+    if (by_rows) {
+        rc = build_rows();
+        if (rc == VGA_ENOMEM) {
+            by_rows = false;
+            VGA_TRY(start_over());
+        }
     }
+    if (n && !by_rows) {
+        rc = build_sources(kSweepStage);
+        if (rc == VGA_ENOMEM) {
+            VGA_TRY(start_over());
+            rc = build_sources(kSweepCount);
+        }
+    }
+    VGA_TRY(rc);
     const uint64_t n_bytes = offsets[n];
-    DeviceBuffer d_off, d_bytes;
-    VGA_TRY(d_off.alloc(((size_t)n + 1) * 8));
+    DeviceBuffer d_bytes;
     if (d_bytes.alloc(n_bytes + kBytePad) != VGA_OK) {
         if (!d_stage.ptr && !d_matrix.ptr) return VGA_ENOMEM;
         // no room beside the stage or the matrix: every list is swept again
         cudaGetLastError();
         clear_error();
         d_stage.reset();
+        d_stage_at.reset();
         d_matrix.reset();
-        again.resize(n);
-        for (uint32_t v = 0; v < n; v++) again[v] = v;
+        all_again = true;
         VGA_TRY(d_bytes.alloc(n_bytes + kBytePad));
     }
     VGA_CHECK_CUDA(cudaMemcpyAsync(d_off.ptr, offsets.data(), ((size_t)n + 1) * 8, cudaMemcpyHostToDevice, stream));
@@ -1249,15 +1280,17 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
         count_launch();
         VGA_CHECK_CUDA(cudaGetLastError());
     }
-    if (!again.empty()) {
-        DeviceBuffer d_again, d_again_retry;
-        VGA_TRY(d_again.alloc(again.size() * 4));
-        VGA_TRY(d_again_retry.alloc(again.size() * 4));
-        VGA_CHECK_CUDA(cudaMemcpyAsync(d_again.ptr, again.data(), again.size() * 4, cudaMemcpyHostToDevice, stream));
+    d_stage.reset();
+    if (all_again || !again.empty()) {
+        DeviceBuffer d_again;
+        if (!all_again) {
+            VGA_TRY(d_again.alloc(again.size() * 4));
+            VGA_CHECK_CUDA(cudaMemcpyAsync(d_again.ptr, again.data(), again.size() * 4, cudaMemcpyHostToDevice,
+                                           stream));
+        }
         sa.offsets = d_off.as<uint64_t>();
         sa.out = d_bytes.as<uint8_t>();
-        sa.retry = retry_list = d_again_retry.as<uint32_t>();
-        VGA_TRY(sweep(kSweepWrite, d_again.as<uint32_t>(), (uint32_t)again.size()));
+        VGA_TRY(sweep(kSweepWrite, d_again.as<uint32_t>(), all_again ? n : (uint32_t)again.size()));
     }
     int err = 0;
     VGA_CHECK_CUDA(cudaMemcpyAsync(&err, d_err.ptr, sizeof(int), cudaMemcpyDeviceToHost, stream));
@@ -1266,7 +1299,6 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
         set_error("visibility sweep failed its own checks (code %d)", err);
         return VGA_ECORRUPT;
     }
-    d_stage.reset();
     d_matrix.reset();
     uint64_t *po = d_off.as<uint64_t>();
     uint8_t *pb = d_bytes.as<uint8_t>();

@@ -305,7 +305,10 @@ int vga_set_table_scheme_nodes(uint32_t nodes);
 int hyperball_run(const vga_graph *g, int p, int d, uint64_t seed, double *mean_depth, double *ball_size,
                   int *iterations);
 
-/* Bytes of device workspace hyperball_run_dev needs for this graph and p. */
+/* Bytes of device workspace hyperball_run_dev needs for this graph and p.  About
+ * 9 bytes a node of it (on graphs of at most 2^20 registers up to 512 KB) hold the arrays of the
+ * register-code passes, with which later passes gather a half or an eighth of
+ * the bytes; a workspace that lacks only those is accepted and runs without. */
 int hyperball_workspace_bytes(const vga_graph *g, int p, uint64_t *bytes);
 
 /*

@@ -536,7 +536,8 @@ struct Plan {
     uint64_t n = 0;
     // workspace layout (byte offsets, 256-aligned)
     uint64_t off_cur = 0, off_next = 0, off_c0 = 0, off_c1 = 0, off_sum = 0, off_lc = 0, off_flags = 0, off_tab = 0,
-             off_chg = 0, off_need = 0, off_ortab = 0, off_win = 0, off_full = 0, off_list = 0, off_codes = 0, chg_bytes = 0, total = 0;
+             off_chg = 0, off_need = 0, off_ortab = 0, off_win = 0, off_full = 0, off_list = 0, off_codes = 0, chg_bytes = 0, total = 0,
+             least = 0;  // what a run without codes takes of the total
 };
 
 static uint64_t align256(uint64_t x) { return (x + 255) & ~255ull; }
@@ -719,6 +720,7 @@ static int make_plan(const vga_graph *g, int p, const vga_tuning *tune, Plan *P)
         P->off_ortab = o;  // range-OR table (mode 2), or the per-node change masks (mode 1)
         o = align256(o + 4ull * (P->mode == kModeRuns ? table_rows(P->scheme) : 1) * P->n);
     }
+    P->least = P->track ? o : align256(P->off_flags + 64);
     if (P->codes) {
         P->off_win = o;  // gmax and gbig (u32 per register each), then the window's top and low words
         o = align256(o + 8ull * P->m + 2ull * P->node_bytes);
@@ -1287,10 +1289,20 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
     Plan P;
     VGA_TRY(make_plan(g, p, tune, &P));
     DeviceBuffer own_ws;
+    // a workspace without room for the codes' arrays (one sized for another
+    // graph, say) is enough for the byte union
+    if (ws && ws_bytes < P.total && ws_bytes >= P.least) P.codes = false;
     if (!ws) {
-        VGA_TRY(own_ws.alloc(P.total));
+        int rc = own_ws.alloc(P.total);
+        if (rc == VGA_ENOMEM && P.codes) {
+            cudaGetLastError();
+            clear_error();
+            P.codes = false;
+            rc = own_ws.alloc(P.least);
+        }
+        VGA_TRY(rc);
         ws = own_ws.ptr;
-    } else if (ws_bytes < P.total || (reinterpret_cast<uintptr_t>(ws) & 255u)) {
+    } else if (ws_bytes < P.least || (reinterpret_cast<uintptr_t>(ws) & 255u)) {
         set_error("workspace of %llu bytes at %p: need %llu bytes, 256-byte aligned", (unsigned long long)ws_bytes,
                   ws, (unsigned long long)P.total);
         return VGA_EINVAL;
@@ -1437,6 +1449,14 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
 // One run with the union launches timed (the autotuner's measurement):
 // outputs go to library-owned buffers, *union_ms gets the summed device time
 // of the union slices (sparse tables included).
+int workspace_sizes(const vga_graph *g, int p, uint64_t *total, uint64_t *least) {
+    Plan P;
+    VGA_TRY(make_plan(g, p, nullptr, &P));
+    *total = P.total;
+    *least = P.least;
+    return VGA_OK;
+}
+
 int run_timed(const vga_graph *g, int p, int d, uint64_t seed, const vga_tuning *tune, cudaStream_t stream,
               double *union_ms, int *iterations) {
     DeviceBuffer out;
@@ -1977,10 +1997,8 @@ int hyperball_workspace_bytes(const vga_graph *g, int p, uint64_t *bytes) {
         set_error("hyperball_workspace_bytes: null argument");
         return VGA_EINVAL;
     }
-    Plan P;
-    VGA_TRY(make_plan(g, p, nullptr, &P));
-    *bytes = P.total;
-    return VGA_OK;
+    uint64_t least = 0;
+    return workspace_sizes(g, p, bytes, &least);
 }
 
 int hyperball_run_dev(const vga_graph *g, int p, int d, uint64_t seed, int conv_mode, double *mean_depth_dev,

@@ -370,8 +370,9 @@ int vga_server_submit(vga_server *S, const vga_graph *g, int p, int d, uint64_t 
         r->L = job_layout(g->n, p, 0, S->l2_budget, 0, g->lk_scheme);
         r->bytes = request_bytes_batched(r->L, g->n);
     } else {
-        uint64_t ws = 0;
-        VGA_TRY(hyperball_workspace_bytes(g, p, &ws));
+        uint64_t ws = 0, least = 0;
+        VGA_TRY(workspace_sizes(g, p, &ws, &least));
+        if (align256(ws) + align256(16ull * g->n) > S->cfg.hbm_budget_bytes) ws = least;
         r->bytes = align256(ws) + align256(16ull * g->n);
     }
     if (r->bytes > S->cfg.hbm_budget_bytes) {

@@ -310,6 +310,9 @@ constexpr int kFirstPassWarps = 4;
 bool tune_table_lookup(const vga_graph *g, vga_tune_entry *out);
 
 // One run with the union launches timed (hyperball.cu), for the autotuner.
+// Workspace of a run with automatic tuning (hyperball_workspace_bytes), and
+// what one without codes takes of it, which run_impl accepts as well.
+int workspace_sizes(const vga_graph *g, int p, uint64_t *total, uint64_t *least);
 int run_timed(const vga_graph *g, int p, int d, uint64_t seed, const vga_tuning *tune, cudaStream_t stream,
               double *union_ms, int *iterations);
 

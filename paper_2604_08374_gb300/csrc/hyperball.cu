@@ -431,26 +431,48 @@ __global__ void __launch_bounds__(512) stream_bench_kernel(const uint4 *__restri
 // HLL estimate of every node, then Eq. sumD (estimate_nodes), `per` nodes a
 // warp; flags[1] records the paper's convergence test max_v(c_t - c_{t-1}) >
 // 0.5.  With top given, the 64-bit count at flags[6] adds up the registers that
-// equal it.
+// equal it, and (8-bit registers) the one at flags[10] the 16-byte pieces with a
+// register below the window (at most so many does a 4-bit pass leave open);
+// flags[12] counts a node's pieces whose low is not 0 throughout, flags[13] has
+// their slices (at most 32 with codes).
 __global__ void hb_estimate_kernel(const uint8_t *__restrict__ regs, uint32_t n, int p, int S, int t,
                                    double alpha_mm, const double *__restrict__ lc, const double *__restrict__ c_prev,
                                    double *__restrict__ c_cur, double *__restrict__ sum_d,
                                    uint32_t *__restrict__ flags, int nib, const uint32_t *__restrict__ top,
                                    uint8_t *__restrict__ full, uint32_t per) {
-    __shared__ uint64_t s_top[32];
+    __shared__ uint64_t s_top[32], s_low[32];
+    const uint32_t pieces = (nib ? 1u << p >> 1 : 1u << p) / 16u;  // of a node
     const int lane = threadIdx.x & 31;
     const uint64_t v0 = ((uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per;
-    uint64_t at_top = 0;
+    uint64_t at_top = 0, below = 0;
     if (v0 < n)
         estimate_nodes(regs, n, p, S, t, alpha_mm, lc, c_prev, c_cur, sum_d, flags + 1, (uint32_t)v0,
-                       (uint32_t)(v0 + per < n ? v0 + per : n), lane, nib != 0, top, full, &at_top);
+                       (uint32_t)(v0 + per < n ? v0 + per : n), lane, nib != 0, top, full, &at_top,
+                       top && !nib ? &below : nullptr);
     if (!top) return;
-    if (lane == 0) s_top[threadIdx.x >> 5] = at_top;
+    if (lane == 0) {
+        s_top[threadIdx.x >> 5] = at_top;
+        s_low[threadIdx.x >> 5] = below;
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
-        unsigned long long sum = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) sum += s_top[w];
+        unsigned long long sum = 0, low = 0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); w++) {
+            sum += s_top[w];
+            low += s_low[w];
+        }
         if (sum) atomicAdd(reinterpret_cast<unsigned long long *>(flags + 6), sum);
+        if (low) atomicAdd(reinterpret_cast<unsigned long long *>(flags + 10), low);
+    }
+    if (blockIdx.x == 0 && !nib) {
+        const uint4 *lows = reinterpret_cast<const uint4 *>(top) + pieces;
+        for (uint32_t k = threadIdx.x; k < pieces; k += blockDim.x) {
+            const uint4 l = __ldg(lows + k);
+            if (l.x | l.y | l.z | l.w) {
+                atomicAdd(flags + 12, 1u);
+                atomicOr(flags + 13, 1u << (16u * k / (uint32_t)S));
+            }
+        }
     }
 }
 
@@ -555,6 +577,11 @@ constexpr double kTrackBelow = 0.01;
 // A run goes back from one-bit codes (kTopShare) to four after a one-bit pass
 // that left more than this share of the 16-byte register pieces open.
 constexpr double kOpenShare = 0.2;
+// What a 4-bit pass saves of a byte pass where nearly all its work is rows
+// gathered (city: 3.1 ms for 256 registers a node against 5.6).  Beside the rows
+// a pass packs, reads and writes every node once, about three rows' worth: mazes
+// have as few rows a node and save a fifth.
+constexpr double kCodesSave = 0.45;
 
 
 // Hub threshold of the run-aware union (lookups per work item).
@@ -562,12 +589,21 @@ static uint32_t hub_threshold(const vga_graph *g, int scheme, uint32_t requested
     return requested > 0 ? requested : hub_lookups_auto(g, scheme);
 }
 
-// Open pieces that the list of a code pass holds: one a node, or all there are
-// on small graphs, whose 4-bit passes (they leave next to none open) then need no
-// byte union behind them, two idle launches.
+// Room for open pieces in the list of the code passes: one a node, or all there
+// are on small graphs.
 static uint64_t list_entries(const Plan &P) {
     const uint64_t pieces = P.n * P.node_bytes / 16;
     return pieces <= (1u << 16) ? std::max<uint64_t>(P.n, pieces) : P.n;
+}
+
+// Open pieces of a K-bit pass that are settled one by one (code_open_cap); more
+// of them leave a byte union to do after it.
+static uint32_t code_list_cap(const Plan &P, const vga_graph *g, int K) {
+    const uint64_t pieces = P.n * P.node_bytes / 16;
+    const bool csr = P.mode == kModePerEdge;
+    if (K == 4 && !csr && list_entries(P) >= pieces) return (uint32_t)pieces;
+    const double rows = csr ? (double)g->n_edges : (double)P.groups.rows_used;
+    return (uint32_t)std::min((double)P.n, code_open_cap(rows, P.node_bytes, g->n_edges, P.n));
 }
 
 static int make_plan(const vga_graph *g, int p, const vga_tuning *tune, Plan *P) {
@@ -732,7 +768,10 @@ static int make_plan(const vga_graph *g, int p, const vga_tuning *tune, Plan *P)
     P->total = o;
     // Per-neighbour mode: codes where a workspace happens to hold them past the
     // bytes that the mode asks for (plan_csr_codes).
+    // From 16 neighbours a node on: packing the codes takes as much as it saves
+    // with few (deg 5.6, 100,000 cells: 8.4 ms for 20 passes against 6.1; 20: 6.1 against 6.9).
     P->csr_codes = P->mode == kModePerEdge && P->track != 2 && P->m >= 128 && P->slices <= kTrackMaxSlices &&
+                   g->n_edges >= 16 * P->n &&
                    S >= (P->nib ? 16 : 32) && P->n > 0 && P->n * P->node_bytes / 16 < (1ull << 32);
     return VGA_OK;
 }
@@ -928,11 +967,12 @@ static int launch_union(const Plan &P, const vga_graph *g, const uint8_t *cur, u
     return VGA_OK;
 }
 
-// One pass of the union over register codes of K bits, then over the bytes of
-// the pairs it left open.
+// One pass of the union over register codes of K bits, then piece by piece or
+// over the bytes of the pairs what it left open.  sure: what it can leave open
+// is within code_list_cap.
 static int launch_codes(const Plan &P, const vga_graph *g, int K, uint8_t *base, const uint8_t *cur, uint8_t *nxt,
                         uint32_t *flags, cudaStream_t stream, std::vector<PendingTiming> *timings, bool tracked,
-                        uint8_t *chg) {
+                        uint8_t *chg, bool sure) {
     CodePass C;
     C.groups = &P.groups;
     C.cur = cur;
@@ -953,11 +993,7 @@ static int launch_codes(const Plan &P, const vga_graph *g, int K, uint8_t *base,
     C.full = base + P.off_full;
     C.need = reinterpret_cast<uint32_t *>(base + P.off_need);
     C.list = reinterpret_cast<uint2 *>(base + P.off_list);
-    const uint64_t pieces = P.n * P.node_bytes / 16;
-    const bool all_listed = K == 4 && list_entries(P) >= pieces;
-    C.list_cap = all_listed ? (uint32_t)pieces
-                            : (uint32_t)std::min((double)P.n, code_open_cap((double)P.groups.rows_used, P.node_bytes,
-                                                                            g->n_edges, P.n));
+    C.list_cap = code_list_cap(P, g, K);
     // Warps per group: enough for twice the warps the GPU holds (about 40 an
     // SM), no more than leaves each about 32 rows.
     int dev = 0, sms = 1;
@@ -992,7 +1028,7 @@ static int launch_codes(const Plan &P, const vga_graph *g, int K, uint8_t *base,
         }
     }
     VGA_TRY(launch_code_open(C, g->lk[P.scheme].d_off, g->lk[P.scheme].d_lk, sms));
-    if (all_listed) return VGA_OK;
+    if (sure) return VGA_OK;
     // more of them: the byte union of their slices, asked for with a wait when
     // there are many slices, else launched for all (the kernels then return at
     // once; a wait costs about 12 us, an idle pair of launches 4)
@@ -1009,9 +1045,10 @@ static int launch_codes(const Plan &P, const vga_graph *g, int K, uint8_t *base,
 
 // One pass of the per-neighbour union over register codes of K bits.  One that
 // leaves more pieces open than are worth settling one by one is done again over
-// the bytes.
+// the bytes (sure: none can, as in launch_codes).
 static int launch_codes_csr(const Plan &P, const vga_graph *g, int K, uint8_t *base, const uint8_t *cur, uint8_t *nxt,
-                            uint32_t *flags, cudaStream_t stream, std::vector<PendingTiming> *timings, uint8_t *chg) {
+                            uint32_t *flags, cudaStream_t stream, std::vector<PendingTiming> *timings, uint8_t *chg,
+                            bool sure) {
     CodePass C;
     C.cur = cur;
     C.nxt = nxt;
@@ -1026,7 +1063,7 @@ static int launch_codes_csr(const Plan &P, const vga_graph *g, int K, uint8_t *b
     C.flags = flags;
     C.full = base + P.off_full;
     C.list = reinterpret_cast<uint2 *>(base + P.off_list);
-    C.list_cap = (uint32_t)std::min((double)P.n, code_open_cap((double)g->n_edges, P.node_bytes, g->n_edges, P.n));
+    C.list_cap = code_list_cap(P, g, K);
     C.chg = chg;
     C.stream = stream;
     int dev = 0, sms = 1;
@@ -1049,6 +1086,7 @@ static int launch_codes_csr(const Plan &P, const vga_graph *g, int K, uint8_t *b
         pt.rows = 1;
         timings->push_back(pt);
     }
+    if (sure) return VGA_OK;
     uint32_t open = 0;
     VGA_CHECK_CUDA(cudaMemcpyAsync(&open, flags + 9, 4, cudaMemcpyDeviceToHost, stream));
     VGA_CHECK_CUDA(cudaStreamSynchronize(stream));
@@ -1369,6 +1407,9 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
             uint64_t n_changed;   // (node, slice) pairs changed by the pass (change tracking)
             uint64_t n_top;       // registers at the window's top (codes)
             uint32_t open[2];     // slices where a code pass left pieces open, and the pieces
+            uint64_t n_low;       // pieces with a register below the window (codes)
+            uint32_t window;      // pieces of a node where the window does not reach 0,
+            uint32_t win_slices;  // and the slices that have any
         } h{};
         VGA_CHECK_CUDA(cudaMemsetAsync(flags, 0, sizeof(h), stream));
         L2Window window;
@@ -1384,25 +1425,47 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
         uint32_t *ortab = P.track ? reinterpret_cast<uint32_t *>(base + P.off_ortab) : nullptr;
         uint64_t changed_prev = ~0ull;
         bool too_open = false;  // the last one-bit pass left too many pairs open
+        double low_prev = 0.0;  // n_low one pass earlier
         for (t = 1;; t++) {
             const bool tracked = chg && t >= 2 &&
                                  (P.track == 2 || (double)changed_prev < kTrackBelow * (double)P.n * P.slices);
             // Codes, from the second pass on: one bit a register once most have
-            // reached G, else four (or, after a pass that changed little, the
-            // change-tracked byte union, which then has less to recompute).
+            // reached G, else four, unless that pass would leave too many pieces
+            // open (or the one before changed little: the change-tracked byte
+            // union then has less to recompute).  A 4-bit pass can leave open what
+            // is below the window now; it is taken to leave the share of it that
+            // the pass before left.  Where that is more than the list holds, its
+            // byte union has to fit into what the codes save (kCodesSave; in mode 1
+            // it is a whole pass).  On graphs of small views (mazes,
+            // small rooms) nearly all stays open for many passes: 236,000 cells of
+            // maze at p = 8, 20 passes, took 33.6 ms with 4-bit passes, 15.6 over
+            // bytes alone, 12.3 by this rule.
             int K = 0;
+            bool sure = false;
             if (P.codes && t >= 2) {
                 const bool most = (double)h.n_top >= kTopShare * (double)P.n * P.m;
-                K = most && !too_open && P.m >= 128 ? 1 : tracked || P.code_bits < 4 ? 0 : 4;
+                const double low = (double)h.n_low, cap = (double)code_list_cap(P, g, 4);
+                if (t == 2) low_prev = (double)P.n * h.window;
+                const double left = low_prev > 0.0 ? low * low / low_prev : 0.0;
+                const double again = P.mode == kModePerEdge || low == 0.0 ? 1.0
+                                     : left / ((double)P.n * h.window) * __builtin_popcount(h.win_slices) / P.slices;
+                const double rows = (double)P.groups.rows_used;
+                const double saved = kCodesSave * rows / (rows + 3.0 * (double)P.n);
+                const bool fits = low <= cap || left <= cap || again <= saved;
+                low_prev = low;
+                K = most && !too_open && P.m >= 128 ? 1 : tracked || P.code_bits < 4 || !fits ? 0 : 4;
+                sure = K == 4 && low <= cap;
             }
             if (tracked && !K) VGA_TRY(launch_need(P, g, chg, ortab, need, stream, timed ? &timings : nullptr));
             const uint64_t clear = K && P.mode == kModeRuns ? P.off_need + 4 * P.n - P.off_flags
                                      : chg ? P.off_chg + P.chg_bytes - P.off_flags : sizeof(h);
             VGA_CHECK_CUDA(cudaMemsetAsync(flags, 0, clear, stream));
             if (K && P.mode == kModePerEdge) {
-                VGA_TRY(launch_codes_csr(P, g, K, base, cur, nxt, flags, stream, timed ? &timings : nullptr, chg));
+                VGA_TRY(launch_codes_csr(P, g, K, base, cur, nxt, flags, stream, timed ? &timings : nullptr, chg,
+                                         sure));
             } else if (K) {
-                VGA_TRY(launch_codes(P, g, K, base, cur, nxt, flags, stream, timed ? &timings : nullptr, tracked, chg));
+                VGA_TRY(launch_codes(P, g, K, base, cur, nxt, flags, stream, timed ? &timings : nullptr, tracked, chg,
+                                     sure));
             } else if (t == 1 && keys)
                 VGA_TRY(launch_first_pass(P, g, keys, nxt, 0u, (uint32_t)P.slices, flags, stream,
                                           timed ? &timings : nullptr, chg, first_groups ? gmax : nullptr, seed));

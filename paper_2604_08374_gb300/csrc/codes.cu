@@ -107,8 +107,8 @@ __global__ void __maxnreg__(56) hb_code_groups_kernel(
 }
 
 // The open pieces of a pass (node, 16-byte register piece), when there are at
-// most list_cap: one CTA per piece takes the maximum over the node's
-// neighbours straight from their registers, a thread per range lookup.
+// most list_cap: the maximum over the node's neighbours straight from their
+// registers (code_open_settle).
 // Reading deg(v) pieces costs a 32-byte sector each, far more per register
 // than the table's rows, but a handful of open pieces in every slice would
 // otherwise cost each slice a table and the whole walk of their groups'
@@ -120,16 +120,20 @@ __global__ void __launch_bounds__(256) hb_code_open_kernel(const uint2 *__restri
                                                            const uint8_t *__restrict__ cur, uint8_t *__restrict__ nxt,
                                                            uint32_t n, int s_log2, int scheme,
                                                            uint32_t *__restrict__ flags, uint8_t *__restrict__ chg) {
-    __shared__ uint4 s_max[8];
+    __shared__ OpenShared sh;
     const uint32_t count = flags[9];
     if (count > list_cap) return;
-    for (uint32_t e = blockIdx.x; e < count; e += gridDim.x) {
-        const uint32_t v = list[e].x, byte = 16u * list[e].y;
-        if (code_open_piece<NIB>(v, byte, lk_off[v], lk_off[v + 1], lk, cur, nxt, n, s_log2, scheme, s_max)) {
+    code_open_settle<NIB>(
+        list, count, blockIdx.x, gridDim.x,
+        [&](uint32_t v, uint64_t &b, uint64_t &e) {
+            b = lk_off[v];
+            e = lk_off[v + 1];
+        },
+        lk, cur, nxt, n, s_log2, scheme, sh,
+        [&](uint32_t v, uint32_t byte) {
             if (*reinterpret_cast<volatile uint32_t *>(flags) == 0u) atomicOr(flags, 1u);
             if (chg) chg[(uint64_t)(byte >> s_log2) * n + v] = 1u;
-        }
-    }
+        });
 }
 
 // Codes of every node, code slices of 2^cs_log2 bytes a node one after another.

@@ -160,28 +160,36 @@ __device__ __forceinline__ void code_store(uint4 code, const uint8_t *__restrict
 }
 
 // Open pieces of unit u of node v (open16: bit per 16 register bytes) to the
-// list, as far as it holds them; *count counts them all.
+// list, as far as it holds them; *count counts them all.  The lanes that get
+// here together raise it once: on graphs of small views every node has some.
 template <int K, bool NIB>
 __device__ __forceinline__ void code_push_open(uint32_t open16, uint32_t v, uint32_t u, uint2 *__restrict__ list,
                                                uint32_t list_cap, uint32_t *count) {
     constexpr uint32_t PIECES = kUnitRegs<K> / (NIB ? 2 : 1) / 16;
-    uint32_t at = atomicAdd(count, (uint32_t)__popc(open16));
+    const uint32_t mine = (uint32_t)__popc(open16), here = __activemask();
+    uint32_t at;
+    if (__all_sync(here, mine == 1u)) {
+        const int lead = __ffs(here) - 1;
+        const uint32_t lane = threadIdx.x & 31u;
+        if ((int)lane == lead) at = atomicAdd(count, (uint32_t)__popc(here));
+        at = __shfl_sync(here, at, lead) + __popc(here & ((1u << lane) - 1u));
+    } else {
+        at = atomicAdd(count, mine);
+    }
     for (uint32_t b = open16; b && at < list_cap; b &= b - 1u)
         list[at++] = make_uint2(v, u * PIECES + (uint32_t)__ffs(b) - 1u);
 }
 
-// next[v] for the open register piece at `byte`, from the registers of node v's
-// neighbours: the range lookups lk[b .. e), a thread each (CTAs of 256); thread
-// 0 gets whether it changed.
-template <bool NIB>
-__device__ __forceinline__ bool code_open_piece(uint32_t v, uint32_t byte, uint64_t b, uint64_t e,
-                                                const uint32_t *__restrict__ lk, const uint8_t *__restrict__ cur,
-                                                uint8_t *__restrict__ nxt, uint32_t n, int s_log2, int scheme,
-                                                uint4 *s_max) {
+// Maximum of the 16 register bytes at `base` + node * 2^s_log2 over the range
+// lookups lk[b .. e), lookups b + first, b + first + step, ... by this lane;
+// every lane of its group of G ends with the group's.
+template <bool NIB, int G>
+__device__ __forceinline__ uint4 code_open_fold(const uint8_t *__restrict__ base, const uint32_t *__restrict__ lk,
+                                                uint64_t b, uint64_t e, uint32_t first, uint32_t step, uint32_t n,
+                                                int s_log2, int scheme) {
     const int rows = table_rows(scheme);
-    const uint8_t *base = cur + ((uint64_t)(byte >> s_log2) * n << s_log2) + (byte & ((1u << s_log2) - 1u));
     uint4 acc = make_uint4(0, 0, 0, 0);
-    for (uint64_t k = b + threadIdx.x; k < e; k += blockDim.x) {
+    for (uint64_t k = b + first; k < e; k += step) {
         const uint32_t r = __ldg(lk + k);
         uint32_t slot = 0;
         for (int s = 1; s < rows; s++) slot += r >= (uint32_t)s * n ? 1u : 0u;
@@ -191,7 +199,7 @@ __device__ __forceinline__ bool code_open_piece(uint32_t v, uint32_t byte, uint6
             acc = RegFmt<NIB>::max4(acc, __ldg(reinterpret_cast<const uint4 *>(base + ((uint64_t)(i + j) << s_log2))));
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
+    for (int o = G / 2; o > 0; o >>= 1) {
         uint4 y;
         y.x = __shfl_xor_sync(0xffffffffu, acc.x, o);
         y.y = __shfl_xor_sync(0xffffffffu, acc.y, o);
@@ -199,19 +207,88 @@ __device__ __forceinline__ bool code_open_piece(uint32_t v, uint32_t byte, uint6
         y.w = __shfl_xor_sync(0xffffffffu, acc.w, o);
         acc = RegFmt<NIB>::max4(acc, y);
     }
-    if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    bool changed = false;
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < 8; w++) acc = RegFmt<NIB>::max4(acc, s_max[w]);
-        const uint64_t at = reg_at(n, s_log2, v, byte);
-        const uint4 own = *reinterpret_cast<const uint4 *>(cur + at);
-        acc = RegFmt<NIB>::max4(acc, own);
-        *reinterpret_cast<uint4 *>(nxt + at) = acc;
-        changed = ((acc.x ^ own.x) | (acc.y ^ own.y) | (acc.z ^ own.z) | (acc.w ^ own.w)) != 0u;
+    return acc;
+}
+
+// The larger of the folded registers and the node's own into nxt; whether that
+// changed them.
+template <bool NIB>
+__device__ __forceinline__ bool code_open_store(uint4 acc, const uint8_t *__restrict__ cur, uint8_t *__restrict__ nxt,
+                                                uint64_t at) {
+    const uint4 own = *reinterpret_cast<const uint4 *>(cur + at);
+    acc = RegFmt<NIB>::max4(acc, own);
+    *reinterpret_cast<uint4 *>(nxt + at) = acc;
+    return ((acc.x ^ own.x) | (acc.y ^ own.y) | (acc.z ^ own.z) | (acc.w ^ own.w)) != 0u;
+}
+
+struct OpenShared {
+    uint4 max[8];
+    uint32_t piece[32];
+};
+
+// next[v] for the open pieces list[0 .. count) ({node, 16-byte piece}), straight
+// from the registers of the nodes' neighbours: the lookups lk[b .. e) that
+// range(v, b, e) gives.  This CTA (of 256 threads) is `cta` of `ctas`.  G lanes
+// settle a piece whose node has up to 16 lookups a lane; the CTA does the others
+// one after another, a thread a lookup.  done(v, byte) is called by one thread
+// for every piece that changed.
+template <bool NIB, int G, class Range, class Done>
+__device__ __forceinline__ void code_open_pieces(const uint2 *__restrict__ list, uint32_t count, uint32_t cta,
+                                                 uint32_t ctas, const Range &range, const uint32_t *__restrict__ lk,
+                                                 const uint8_t *__restrict__ cur, uint8_t *__restrict__ nxt,
+                                                 uint32_t n, int s_log2, int scheme, OpenShared &sh,
+                                                 const Done &done) {
+    constexpr uint32_t GROUPS = 256 / G;
+    const uint32_t sub = threadIdx.x % G, group = threadIdx.x / G;
+    auto base_of = [&](uint32_t byte) {
+        return cur + ((uint64_t)(byte >> s_log2) * n << s_log2) + (byte & ((1u << s_log2) - 1u));
+    };
+    for (uint64_t first = cta; first < count; first += (uint64_t)GROUPS * ctas) {
+        const uint64_t x = first + (uint64_t)group * ctas;
+        uint32_t v = 0, byte = 0;
+        uint64_t b = 0, e = 0;
+        if (x < count) {
+            v = list[x].x;
+            byte = 16u * list[x].y;
+            range(v, b, e);
+        }
+        const bool whole = e - b > 16u * G, mine = x < count && !whole;
+        const uint4 acc = code_open_fold<NIB, G>(base_of(byte), lk, b, whole ? b : e, sub, G, n, s_log2, scheme);
+        if (mine && sub == 0 && code_open_store<NIB>(acc, cur, nxt, reg_at(n, s_log2, v, byte))) done(v, byte);
+        if (sub == 0) sh.piece[group] = whole ? (uint32_t)x : 0xffffffffu;
+        __syncthreads();
+        for (uint32_t q = 0; q < GROUPS; q++) {
+            const uint32_t y = sh.piece[q];
+            if (y == 0xffffffffu) continue;
+            v = list[y].x;
+            byte = 16u * list[y].y;
+            range(v, b, e);
+            uint4 all = code_open_fold<NIB, 32>(base_of(byte), lk, b, e, threadIdx.x, 256u, n, s_log2, scheme);
+            if (threadIdx.x % 32u == 0) sh.max[threadIdx.x / 32u] = all;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                for (int w = 1; w < 8; w++) all = RegFmt<NIB>::max4(all, sh.max[w]);
+                if (code_open_store<NIB>(all, cur, nxt, reg_at(n, s_log2, v, byte))) done(v, byte);
+            }
+            __syncthreads();
+        }
+        __syncthreads();
     }
-    __syncthreads();
-    return changed;
+}
+
+// Where nodes see little, most have a piece open: with 8 lanes a piece a CTA
+// takes 32 at a time (a CTA a piece: 160 us a pass for the 100,000 of a maze
+// of as many cells).  Few pieces, up to two a CTA, go faster by whole warps.
+template <bool NIB, class Range, class Done>
+__device__ __forceinline__ void code_open_settle(const uint2 *__restrict__ list, uint32_t count, uint32_t cta,
+                                                 uint32_t ctas, const Range &range, const uint32_t *__restrict__ lk,
+                                                 const uint8_t *__restrict__ cur, uint8_t *__restrict__ nxt,
+                                                 uint32_t n, int s_log2, int scheme, OpenShared &sh,
+                                                 const Done &done) {
+    if (count > 2u * ctas)
+        code_open_pieces<NIB, 8>(list, count, cta, ctas, range, lk, cur, nxt, n, s_log2, scheme, sh, done);
+    else
+        code_open_pieces<NIB, 32>(list, count, cta, ctas, range, lk, cur, nxt, n, s_log2, scheme, sh, done);
 }
 
 // Word k of the window of a run (CodeWindow) from the largest rho inserted per

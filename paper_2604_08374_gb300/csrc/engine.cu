@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(kGroupScatterWarps * 32) batch_first_groups_ke
 __device__ __forceinline__ bool pass_again(const JobDev &J) { return J.K == 1 && J.open > J.open_cap; }
 
 // initial != 0: c_0 of every job; otherwise pass t = job.t + 1 of running jobs.
-__global__ void batch_estimate_kernel(JobDev *jobs, const uint64_t *__restrict__ node_start, int n_jobs,
+__global__ void __launch_bounds__(256, 4) batch_estimate_kernel(JobDev *jobs, const uint64_t *__restrict__ node_start, int n_jobs,
                                       uint64_t total_nodes, int initial) {
     const int lane = threadIdx.x & 31;
     const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
@@ -407,22 +407,25 @@ __global__ void __launch_bounds__(kEngineWarps * 32, 3) batch_code_kernel(JobDev
     }
 }
 
-// The pieces that this pass's code unions left open (code_open_piece),
-// kOpenCtas CTAs a job.
-constexpr unsigned kOpenCtas = 64;
-__global__ void __launch_bounds__(256) batch_open_kernel(JobDev *jobs) {
-    __shared__ uint4 s_max[8];
-    JobDev &J = jobs[blockIdx.x / kOpenCtas];
+// The pieces that this pass's code unions left open (code_open_settle), `ctas`
+// CTAs a job: eight an SM over all jobs, 64 a job at least.
+__global__ void __launch_bounds__(256) batch_open_kernel(JobDev *jobs, uint32_t ctas) {
+    __shared__ OpenShared sh;
+    JobDev &J = jobs[blockIdx.x / ctas];
     if (J.state != 0 || !J.K || pass_again(J)) return;
     const int t = J.t + 1;
     const uint32_t count = min(J.open, J.list_cap);
-    for (uint32_t e = blockIdx.x % kOpenCtas; e < count; e += kOpenCtas) {
-        const uint32_t v = J.list[e].x, byte = 16u * J.list[e].y;
-        const RunItem &it = J.items[v];  // no split hubs: one item per node, in id order
-        if (code_open_piece<false>(v, byte, it.b, it.b + it.cnt, J.lk, J.regs[(t - 1) & 1], J.regs[t & 1], J.n,
-                                   __ffs(J.S) - 1, J.scheme, s_max))
-            atomicOr(&J.changed, 1u);
-    }
+    code_open_settle<false>(
+        J.list, count, blockIdx.x % ctas, ctas,
+        [&](uint32_t v, uint64_t &b, uint64_t &e) {
+            const RunItem &it = J.items[v];  // no split hubs: one item per node, in id order
+            b = it.b;
+            e = it.b + it.cnt;
+        },
+        J.lk, J.regs[(t - 1) & 1], J.regs[t & 1], J.n, __ffs(J.S) - 1, J.scheme, sh,
+        [&](uint32_t, uint32_t) {
+            if (*reinterpret_cast<volatile uint32_t *>(&J.changed) == 0u) atomicOr(&J.changed, 1u);
+        });
 }
 
 // One thread per job: close the pass (or leave it to be done again), apply the
@@ -778,6 +781,7 @@ int engine_upload(const EngineArrays &A, const std::vector<JobDev> &jobs, Engine
     E->n_jobs = nj;
     E->total_nodes = ns[nj];
     E->grid_nodes = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((E->total_nodes + 255) / 256, (uint64_t)sms * 32));
+    E->open_ctas = (unsigned)std::max(64, sms * 8 / std::max(nj, 1));
     E->grid_warps = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((E->total_nodes + 7) / 8, (uint64_t)sms * 64));
     return VGA_OK;
 }
@@ -949,7 +953,7 @@ int engine_pass(const EngineArrays &A, const EngineSet &E, cudaStream_t stream, 
     bool codes = false;
     for (const EngineGroup &G : E.groups) codes |= G.K != 0;
     if (codes) {
-        batch_open_kernel<<<(unsigned)E.n_jobs * kOpenCtas, 256, 0, stream>>>(A.jobs);
+        batch_open_kernel<<<(unsigned)E.n_jobs * E.open_ctas, 256, 0, stream>>>(A.jobs, E.open_ctas);
         count_launch();
     }
     batch_estimate_kernel<<<E.grid_warps, 256, 0, stream>>>(A.jobs, A.node_start, E.n_jobs, E.total_nodes, 0);

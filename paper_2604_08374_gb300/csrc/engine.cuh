@@ -100,6 +100,7 @@ struct EngineSet {
     int n_jobs = 0;
     uint64_t total_nodes = 0;
     unsigned grid_nodes = 1, grid_warps = 1;
+    unsigned open_ctas = 64;  // CTAs a job of the open-piece kernel
     std::vector<EngineGroup> groups;
 };
 

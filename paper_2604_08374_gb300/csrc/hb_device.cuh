@@ -879,10 +879,11 @@ __device__ __forceinline__ double u128_to_double(uint64_t hi, uint64_t lo) {
 // every node): lo/hi accumulate sum of 2^(K - M) over the registers M >= 1,
 // zeros counts M = 0 (K = 65 - p).  Warp-cooperative; every lane ends with the
 // warp's totals.  With top given (the node's register words of a window's
-// top), *at_top gets the number of registers equal to it, and the lane's *below
-// is raised by its 16-byte pieces with a register under the window's low words,
+// top), *at_top gets the number of registers equal to it; with BELOW the lane's
+// *below is raised by its 16-byte pieces with a register under the window's low words,
 // which follow the top words; has: bit i % 32 is set if the lane's i-th piece can
 // have one (low is not 0 throughout).
+template <bool BELOW = false>
 __device__ __forceinline__ void harmonic_partial(const uint8_t *__restrict__ regs, uint32_t n, int p, int S,
                                                  uint32_t b0, uint32_t b1, uint32_t v, int lane, bool nib,
                                                  uint64_t &lo, uint64_t &hi, uint32_t &zeros,
@@ -907,7 +908,7 @@ __device__ __forceinline__ void harmonic_partial(const uint8_t *__restrict__ reg
 #pragma unroll
             for (int i = 0; i < 4; i++)
                 full += __popc(nib ? equal_bits<true>(wv[i], gv[i]) : equal_bits<false>(wv[i], gv[i]));
-            if ((has >> ((rel / 512u) & 31u)) & 1u) {
+            if (BELOW && ((has >> ((rel / 512u) & 31u)) & 1u)) {
                 const uint4 l = __ldg(reinterpret_cast<const uint4 *>(top + (b1 - b0) / 4u) + r0 / 16u);
                 *below += (__vcmpltu4(x.x, l.x) | __vcmpltu4(x.y, l.y) | __vcmpltu4(x.z, l.z) |
                            __vcmpltu4(x.w, l.w)) != 0u;
@@ -993,9 +994,10 @@ __device__ __forceinline__ void estimate_finish(uint64_t lo, uint64_t hi, uint32
 // rates, and a warp's instruction takes the pipe as long for one lane as for 32.
 // With top given (the window of a run that unions codes), full[v] records the
 // nodes whose registers all equal it and *at_top (every lane) their number of
-// registers that do; with below given, *below (every lane) gets their pieces
+// registers that do; with BELOW, *below (every lane) gets their pieces
 // under the window (harmonic_partial; few pieces of a node can be, so which is
 // found once).
+template <bool BELOW = false>
 __device__ __forceinline__ void estimate_nodes(const uint8_t *__restrict__ regs, uint32_t n, int p, int S, int t,
                                                double alpha_mm, const double *__restrict__ lc,
                                                const double *__restrict__ c_prev, double *__restrict__ c_cur,
@@ -1005,7 +1007,7 @@ __device__ __forceinline__ void estimate_nodes(const uint8_t *__restrict__ regs,
                                                uint64_t *below = nullptr) {
     const uint32_t node_bytes = nib ? (1u << p) / 2u : (1u << p);  // 4-bit registers: two per byte
     uint32_t has = 0, under = 0;
-    if (below)
+    if (BELOW)
         for (uint32_t k = 0, r0 = (uint32_t)lane * 16u; r0 < node_bytes; r0 += 512u, k++) {
             const uint4 l = __ldg(reinterpret_cast<const uint4 *>(top + node_bytes / 4u) + r0 / 16u);
             if (l.x | l.y | l.z | l.w) has |= 1u << (k & 31u);
@@ -1017,8 +1019,8 @@ __device__ __forceinline__ void estimate_nodes(const uint8_t *__restrict__ regs,
         for (uint32_t i = 0; i < cnt; i++) {
             uint64_t lo, hi;
             uint32_t zeros, node_top = 0;
-            harmonic_partial(regs, n, p, S, 0u, node_bytes, base + i, lane, nib, lo, hi, zeros, top, &node_top,
-                             has, &under);
+            harmonic_partial<BELOW>(regs, n, p, S, 0u, node_bytes, base + i, lane, nib, lo, hi, zeros, top, &node_top,
+                                    has, &under);
             if (lane == (int)i) {
                 my_lo = lo;
                 my_hi = hi;
@@ -1033,7 +1035,7 @@ __device__ __forceinline__ void estimate_nodes(const uint8_t *__restrict__ regs,
             if (top) full[base + (uint32_t)lane] = my_top == (1u << p) ? 1u : 0u;
         }
     }
-    if (below) *below = __reduce_add_sync(0xffffffffu, under);
+    if (BELOW) *below = __reduce_add_sync(0xffffffffu, under);
 }
 
 // MD(v) = sum_d[v] / (N_v - 1) (Sec. 3.3), NaN when N_v <= 1; ball = c_t.

@@ -445,10 +445,15 @@ __global__ void hb_estimate_kernel(const uint8_t *__restrict__ regs, uint32_t n,
     const int lane = threadIdx.x & 31;
     const uint64_t v0 = ((uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per;
     uint64_t at_top = 0, below = 0;
-    if (v0 < n)
-        estimate_nodes(regs, n, p, S, t, alpha_mm, lc, c_prev, c_cur, sum_d, flags + 1, (uint32_t)v0,
-                       (uint32_t)(v0 + per < n ? v0 + per : n), lane, nib != 0, top, full, &at_top,
-                       top && !nib ? &below : nullptr);
+    const uint32_t v1 = (uint32_t)(v0 + per < n ? v0 + per : n);
+    if (v0 < n) {
+        if (top && !nib)
+            estimate_nodes<true>(regs, n, p, S, t, alpha_mm, lc, c_prev, c_cur, sum_d, flags + 1, (uint32_t)v0, v1,
+                                 lane, false, top, full, &at_top, &below);
+        else
+            estimate_nodes(regs, n, p, S, t, alpha_mm, lc, c_prev, c_cur, sum_d, flags + 1, (uint32_t)v0, v1, lane,
+                           nib != 0, top, full, &at_top);
+    }
     if (!top) return;
     if (lane == 0) {
         s_top[threadIdx.x >> 5] = at_top;

@@ -28,6 +28,23 @@ def _band(reach=1, hub=None, hub_reach=0):
     return oracle.csr_encode(row_ptr, np.concatenate(lists))
 
 
+def _spokes(n, hub, hub_reach):
+    """A band of `n` nodes; nodes 100, 101, ... also see every 3rd, 15th, 16th, 120th, ... id (up to 1,334
+    runs), and `hub` and the first hub_reach each other."""
+    sees = [set(range(max(0, v - 1), min(n, v + 2))) for v in range(n)]
+    for k, step in enumerate((3, 15, 16, 17, 120, 130, 140)):
+        for u in range(0, n, step):
+            sees[100 + k].add(u)
+            sees[u].add(100 + k)
+    for u in range(hub_reach):
+        sees[hub].add(u)
+        sees[u].add(hub)
+    lists = [np.array(sorted(s - {v}), np.uint32) for v, s in enumerate(sees)]
+    row_ptr = np.zeros(n + 1, np.uint64)
+    row_ptr[1:] = np.cumsum([len(x) for x in lists])
+    return oracle.csr_encode(row_ptr, np.concatenate(lists))
+
+
 def _large(seed):
     """The nodes and register indices with a rho of 16 or more."""
     return np.nonzero(oracle.hll_init(N, P, seed) >= 16)
@@ -83,3 +100,22 @@ def test_pass_that_leaves_more_open_than_foreseen(vga):  # noqa: F811
     with vga.vga_graph_load(off, b) as g:
         # as above, and the byte union of the open pairs behind them
         assert _launches(vga, g, seed, 2) == _launches(vga, g, seed, 2, slice_bytes=1 << P) + 4
+
+
+@pytest.mark.parametrize("hub_reach", [0, 3500], ids=["many", "few"])
+@pytest.mark.parametrize("levels", [5, 3])
+def test_settling_of_open_pieces(vga, levels, hub_reach):  # noqa: F811
+    # all pieces fit the list of a graph this small: 4-bit passes leave up to 4,000
+    # open, of nodes with 1 to 1,335 range lookups
+    n = 4000
+    seed, hub, _ = _one_large()
+    off, b = _spokes(n, hub, hub_reach)
+    check(vga, off, b, None, P, 5, seed, 8, table_levels=levels)
+    ref = oracle.hyperball(off, b, P, 5, seed=seed)
+    with vga.vga_graph_load(off, b) as g:
+        out = [[torch.empty(n, dtype=torch.float64, device="cuda") for _ in range(2)] for _ in range(3)]
+        jobs = [dict(graph=g, p=P, d=5, seed=seed, mean_depth=md, ball=ball) for md, ball in out]
+        assert vga.hyperball_run_batch(jobs) == [ref["iterations"]] * 3
+        for md, ball in out:
+            assert np.array_equal(md.cpu().numpy(), ref["mean_depth"])
+            assert np.array_equal(ball.cpu().numpy(), ref["ball"])

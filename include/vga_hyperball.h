@@ -540,7 +540,7 @@ typedef struct vga_profile {
     int union_mode;               /* union variant of the last timed launch (1 or 2)      */
     int table_rows;               /* rows per node it gathered from: the table scheme's
                                      (mode 2) or 1 (mode 1)                               */
-    int reserved;
+    int first_pass_grouped;       /* first passes (below) that took whole groups of nodes */
     uint64_t first_pass_launches; /* first passes computed by the scatter (vga_tuning.
                                      first_pass), timed apart from the union slices       */
     double first_pass_ms;         /* their summed device time                             */

@@ -56,7 +56,8 @@ class VgaServerStats(C.Structure):
 class VgaProfile(C.Structure):
     _fields_ = [("kernel_launches", C.c_uint64), ("union_launches", C.c_uint64), ("union_ms", C.c_double),
                 ("union_edges", C.c_uint64), ("union_gather_bytes", C.c_uint64), ("union_hbm_bytes", C.c_uint64),
-                ("slice_bytes", C.c_int), ("union_mode", C.c_int), ("table_rows", C.c_int), ("reserved", C.c_int),
+                ("slice_bytes", C.c_int), ("union_mode", C.c_int), ("table_rows", C.c_int),
+                ("first_pass_grouped", C.c_int),
                 ("first_pass_launches", C.c_uint64), ("first_pass_ms", C.c_double),
                 ("first_pass_edges", C.c_uint64), ("tracked_launches", C.c_uint64), ("tracked_ms", C.c_double)]
 
@@ -498,7 +499,7 @@ def vga_profile_reset():
 def vga_profile_read() -> dict:
     p = VgaProfile()
     _check(lib().vga_profile_read(C.byref(p)))
-    return {name: getattr(p, name) for name, _ in VgaProfile._fields_ if name != "reserved"}
+    return {name: getattr(p, name) for name, _ in VgaProfile._fields_}
 
 
 def vga_bench_gather(resident_bytes: int, chunk_bytes: int, gathers: int, consumer: int = 1, stream=None) -> float:

@@ -577,8 +577,7 @@ int make_jobdev(const vga_graph *g, int p, int d, uint64_t seed, int conv, const
         const uint64_t off_list = q;  q += 8 * pieces;
         J.codes = J.first && J.hub_units == 0 && J.groups && m >= 128 && L.S >= 32 && q <= tab_bytes &&
                   pieces < (1ull << 32);
-        // whole groups while few indices can have several rho above 16 (run_impl)
-        J.group_scatter = J.codes && n >> p <= kGroupScatterNodes;
+        J.group_scatter = J.codes && group_scatter_pays(n, g->n_edges, p);
         if (J.codes) {
             J.win = reinterpret_cast<uint32_t *>(J.tab + off_win);
             J.full = J.tab + off_full;

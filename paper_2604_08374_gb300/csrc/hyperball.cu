@@ -855,6 +855,7 @@ struct PendingTiming {
     uint64_t edges, gather_bytes, hbm_bytes;
     int S, mode, rows;
     bool first;    // the first pass's scatter (hb_first_pass_kernel), not a union slice
+    bool grouped;  // and that by whole groups
     bool tracked;  // a union slice of a change-tracked pass (its work depends on the changes)
     bool partial;  // time without bytes: one-bit codes, or the byte union of the pairs a code pass left open
 };
@@ -1180,6 +1181,7 @@ static int launch_first_pass(const Plan &P, const vga_graph *g, const void *keys
         pt.S = P.S;
         pt.mode = P.mode;
         pt.first = true;
+        pt.grouped = gmax != nullptr;
         timings->push_back(pt);
     }
     return VGA_OK;
@@ -1246,6 +1248,7 @@ static void settle_timings(std::vector<PendingTiming> &timings, bool to_profile,
         if (sum_ms && ok && *sum_ms >= 0.0) *sum_ms += ms;
         if (to_profile && ok && pt.first) {
             ps.acc.first_pass_launches++;
+            ps.acc.first_pass_grouped += pt.grouped;
             ps.acc.first_pass_ms += ms;
             ps.acc.first_pass_edges += pt.edges;
         } else if (to_profile && ok && pt.tracked) {
@@ -1397,7 +1400,7 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
         // a CTA a group: two an SM at least (818 cells: 207 us an analysis by groups, 199 by nodes)
         int sms = 1;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device);
-        const bool first_groups = keys && P.codes && P.mode == kModeRuns && P.n >> P.p <= kGroupScatterNodes &&
+        const bool first_groups = keys && P.codes && P.mode == kModeRuns && group_scatter_pays(P.n, g->n_edges, P.p) &&
                                   P.groups.count >= 2ull * (uint64_t)sms;
         uint32_t *gbig = first_groups ? gmax + P.m : nullptr;
         hb_init_kernel<<<(unsigned)((P.n + 255) / 256), 256, 0, stream>>>(cur, (uint32_t)P.n, p, P.S, seed, P.nib, 0u,

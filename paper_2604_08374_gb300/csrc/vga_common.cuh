@@ -279,6 +279,14 @@ constexpr int kGroupKey16MaxP = 12;
 // It is used while few indices can have several rho above 16 (such registers
 // are searched): up to this many nodes an index, where one index in 500 has.
 constexpr uint64_t kGroupScatterNodes = 2048;
+// And from this mean degree on, 768 + m / 4: a CTA clears and reads its cells
+// whatever the group sees, and the visits that it saves grow with the degree.
+// Time by groups over time by nodes, p = 8 / 10 / 12: degree 6 3.5 / 3.5 / 3.2, 176
+// 1.5 / 1.7 / 1.6, 628 1.0 / 1.2 / 1.4, 967 0.93 / 1.2 / 1.2, 1,087 0.86 / 1.0 / 1.2,
+// 1,947 0.69 / 0.80 / 0.94, 4,698 0.51 / 0.58 / 0.58, 22,900 0.52 / 0.53 / 0.75.
+inline bool group_scatter_pays(uint64_t n, uint64_t edges, int p) {
+    return n >> p <= kGroupScatterNodes && edges >= n * (768 + (1ull << p) / 4);
+}
 struct FirstPassGroups {
     const GroupList *groups = nullptr;
     const void *keys = nullptr;

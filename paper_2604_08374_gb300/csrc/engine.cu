@@ -576,7 +576,7 @@ int make_jobdev(const vga_graph *g, int p, int d, uint64_t seed, int conv, const
         const uint64_t off_full = q;  q = align256(q + n);
         const uint64_t off_list = q;  q += 8 * pieces;
         J.codes = J.first && J.hub_units == 0 && J.groups && m >= 128 && L.S >= 32 && q <= tab_bytes &&
-                  pieces < (1ull << 32);
+                  pieces < (1ull << 32) && code_rows_pay(n, rows_used, (uint32_t)m, L.slices);
         J.group_scatter = J.codes && group_scatter_pays(n, g->n_edges, p);
         if (J.codes) {
             J.win = reinterpret_cast<uint32_t *>(J.tab + off_win);

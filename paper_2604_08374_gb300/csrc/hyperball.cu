@@ -583,9 +583,10 @@ constexpr double kTrackBelow = 0.01;
 // that left more than this share of the 16-byte register pieces open.
 constexpr double kOpenShare = 0.2;
 // What a 4-bit pass saves of a byte pass where nearly all its work is rows
-// gathered (city: 3.1 ms for 256 registers a node against 5.6).  Beside the rows
-// a pass packs, reads and writes every node once, about three rows' worth: mazes
-// have as few rows a node and save a fifth.
+// gathered (city: 3.1 ms for 256 registers a node against 5.6).  Beside its rows
+// a pass builds the table and reads and writes every node once, about eight rows'
+// worth, of which codes save little: mazes have three rows a node and save a
+// sixth, rooms of 400 cells (25 rows) a third.
 constexpr double kCodesSave = 0.45;
 
 
@@ -1455,13 +1456,15 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
                 const double low = (double)h.n_low, cap = (double)code_list_cap(P, g, 4);
                 if (t == 2) low_prev = (double)P.n * h.window;
                 const double left = low_prev > 0.0 ? low * low / low_prev : 0.0;
+                const double rows = (double)P.groups.rows_used / (double)P.n;
                 const double again = P.mode == kModePerEdge || low == 0.0 ? 1.0
-                                     : left / ((double)P.n * h.window) * __builtin_popcount(h.win_slices) / P.slices;
-                const double rows = (double)P.groups.rows_used;
-                const double saved = kCodesSave * rows / (rows + 3.0 * (double)P.n);
+                                     : (left / ((double)P.n * h.window) * rows + 6.0) / (rows + 8.0) *
+                                           __builtin_popcount(h.win_slices) / P.slices;
+                const double saved = kCodesSave * rows / (rows + 6.0);
                 const bool fits = low <= cap || left <= cap || again <= saved;
                 low_prev = low;
-                K = most && !too_open && P.m >= 128 ? 1 : tracked || P.code_bits < 4 || !fits ? 0 : 4;
+                const bool wide = P.mode == kModePerEdge || code_rows_pay(P.n, P.groups.rows_used, P.m, P.slices);
+                K = most && !too_open && P.m >= 128 ? 1 : tracked || P.code_bits < 4 || !fits || !wide ? 0 : 4;
                 sure = K == 4 && low <= cap;
             }
             if (tracked && !K) VGA_TRY(launch_need(P, g, chg, ortab, need, stream, timed ? &timings : nullptr));

@@ -238,11 +238,21 @@ constexpr int kCodeNodes = 4;  // nodes per group of the code kernels
 // maximum.
 constexpr double kTopShare = 0.75;
 // Open pieces of a code pass that are settled one by one: while their
-// neighbours' 32-byte sectors stay below an eighth of the bytes (node_bytes a
-// row) that a union of the groups' rows gathers.
+// neighbours' 32-byte sectors, and six more for what a piece takes of its own,
+// stay below an eighth of the bytes (node_bytes a row) that a union of the
+// groups' rows gathers.  (Without the six, a maze of 30,000 cells at p = 9 settled
+// 30,000 pieces a pass: 1.64 ms for 12 passes against 1.21 over bytes.)
 inline double code_open_cap(double rows_used, uint32_t node_bytes, uint64_t edges, uint64_t n) {
-    const double piece = 32.0 * (double)edges / (double)n;
-    return rows_used * node_bytes / 8.0 / (piece > 1.0 ? piece : 1.0);
+    return rows_used * node_bytes / 8.0 / (32.0 * ((double)edges / (double)n + 6.0));
+}
+// 4-bit rows of less than 512 bytes (in one slice) are worth it from 32 rows a
+// node on: a warp folds 2,048 bytes of rows at a time, more than a class of a
+// group has where nodes see little.  28,600 cells of rooms (19 rows a node), 12
+// passes: p = 8 1.60 ms with 4-bit passes, 1.40 without, p = 9 1.78 and 1.60; with 33
+// rows 1.23 and 1.23, 1.40 and 1.47; 83 rows 0.22 and 0.30, 0.23 and 0.35 (4,800
+// cells).  Smaller graphs are bound by launches either way.
+inline bool code_rows_pay(uint64_t n, uint64_t rows_used, uint32_t m, int slices) {
+    return n < 8192 || m >= 1024 || slices > 1 || rows_used >= 32 * n;
 }
 struct CodePass {
     const GroupList *groups = nullptr;

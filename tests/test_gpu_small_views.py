@@ -119,3 +119,33 @@ def test_settling_of_open_pieces(vga, levels, hub_reach):  # noqa: F811
         for md, ball in out:
             assert np.array_equal(md.cpu().numpy(), ref["mean_depth"])
             assert np.array_equal(ball.cpu().numpy(), ref["ball"])
+
+
+def test_narrow_rows_of_few_go_over_bytes(vga):  # noqa: F811
+    # 9,000 nodes of a handful of rows each: no 4-bit pass at p = 9, one at p = 10
+    n = 9000
+    row_ptr = np.zeros(n + 1, np.uint64)
+    lists = [np.array([u for u in range(max(0, v - 9), min(n, v + 10)) if u != v], np.uint32) for v in range(n)]
+    row_ptr[1:] = np.cumsum([len(x) for x in lists])
+    off, b = oracle.csr_encode(row_ptr, np.concatenate(lists))
+    seed = next(s for s in range(0, 1 << 20, 1 << 14)
+                if max(oracle.hll_init(n, p, s).max() for p in (9, 10)) < 16)  # the window reaches 0
+    with vga.vga_graph_load(off, b) as g:
+        md, ball = (torch.empty(n, dtype=torch.float64, device="cuda") for _ in range(2))
+
+        def launches(p, **kw):
+            for _ in range(2):
+                vga.vga_profile_reset()
+                it = vga.hyperball_run_dev(g, p, 2, seed, md, ball, track_changes=1, **kw)
+            ref = oracle.hyperball(off, b, p, 2, seed=seed)
+            assert it == 2 and np.array_equal(md.cpu().numpy(), ref["mean_depth"])
+            return vga.vga_profile_read()["kernel_launches"]
+
+        assert launches(9) == launches(9, slice_bytes=512) + 1   # the window
+        assert launches(10) == launches(10, slice_bytes=1024) + 2  # and the (no) open pieces
+        jobs = [dict(graph=g, p=p, d=3, seed=seed, mean_depth=torch.empty(n, dtype=torch.float64, device="cuda"),
+                     ball=torch.empty(n, dtype=torch.float64, device="cuda")) for p in (9, 10)]
+        vga.hyperball_run_batch(jobs)
+        for job in jobs:
+            ref = oracle.hyperball(off, b, job["p"], 3, seed=seed)
+            assert np.array_equal(job["mean_depth"].cpu().numpy(), ref["mean_depth"])

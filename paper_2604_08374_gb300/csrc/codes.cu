@@ -114,7 +114,7 @@ __global__ void __maxnreg__(56) hb_code_groups_kernel(
 // otherwise cost each slice a table and the whole walk of their groups'
 // rows by single warps (city pass 3: 2.4 ms for 0.28 % of the pairs, now 0.1).
 template <bool NIB>
-__global__ void __launch_bounds__(256) hb_code_open_kernel(const uint2 *__restrict__ list, uint32_t list_cap,
+__global__ void __launch_bounds__(256, 8) hb_code_open_kernel(const uint2 *__restrict__ list, uint32_t list_cap,
                                                            const uint64_t *__restrict__ lk_off,
                                                            const uint32_t *__restrict__ lk,
                                                            const uint8_t *__restrict__ cur, uint8_t *__restrict__ nxt,

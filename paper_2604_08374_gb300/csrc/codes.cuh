@@ -229,10 +229,10 @@ struct OpenShared {
 // next[v] for the open pieces list[0 .. count) ({node, 16-byte piece}), straight
 // from the registers of the nodes' neighbours: the lookups lk[b .. e) that
 // range(v, b, e) gives.  This CTA (of 256 threads) is `cta` of `ctas`.  G lanes
-// settle a piece whose node has up to 16 lookups a lane; the CTA does the others
-// one after another, a thread a lookup.  done(v, byte) is called by one thread
-// for every piece that changed.
-template <bool NIB, int G, class Range, class Done>
+// settle a piece whose node has up to MOST lookups and a warp one of up to
+// BY_WARP; the CTA does the others one after another, a thread a lookup.
+// done(v, byte) is called by one thread for every piece that changed.
+template <bool NIB, int G, int MOST, int BY_WARP, class Range, class Done>
 __device__ __forceinline__ void code_open_pieces(const uint2 *__restrict__ list, uint32_t count, uint32_t cta,
                                                  uint32_t ctas, const Range &range, const uint32_t *__restrict__ lk,
                                                  const uint8_t *__restrict__ cur, uint8_t *__restrict__ nxt,
@@ -252,11 +252,29 @@ __device__ __forceinline__ void code_open_pieces(const uint2 *__restrict__ list,
             byte = 16u * list[x].y;
             range(v, b, e);
         }
-        const bool whole = e - b > 16u * G, mine = x < count && !whole;
+        const bool whole = e - b > (uint64_t)MOST, mine = x < count && !whole;
         const uint4 acc = code_open_fold<NIB, G>(base_of(byte), lk, b, whole ? b : e, sub, G, n, s_log2, scheme);
         if (mine && sub == 0 && code_open_store<NIB>(acc, cur, nxt, reg_at(n, s_log2, v, byte))) done(v, byte);
         if (sub == 0) sh.piece[group] = whole ? (uint32_t)x : 0xffffffffu;
         __syncthreads();
+        if (BY_WARP > MOST) {
+            for (uint32_t q = threadIdx.x / 32u; q < GROUPS; q += 8u) {
+                const uint32_t y = sh.piece[q];
+                if (y == 0xffffffffu) continue;
+                v = list[y].x;
+                byte = 16u * list[y].y;
+                range(v, b, e);
+                if (e - b > (uint64_t)BY_WARP) continue;
+                const uint4 w = code_open_fold<NIB, 32>(base_of(byte), lk, b, e, threadIdx.x % 32u, 32u, n, s_log2,
+                                                        scheme);
+                if (threadIdx.x % 32u == 0) {
+                    if (code_open_store<NIB>(w, cur, nxt, reg_at(n, s_log2, v, byte))) done(v, byte);
+                    sh.piece[q] = 0xffffffffu;
+                }
+                __syncwarp();
+            }
+            __syncthreads();
+        }
         for (uint32_t q = 0; q < GROUPS; q++) {
             const uint32_t y = sh.piece[q];
             if (y == 0xffffffffu) continue;
@@ -278,7 +296,8 @@ __device__ __forceinline__ void code_open_pieces(const uint2 *__restrict__ list,
 
 // Where nodes see little, most have a piece open: with 8 lanes a piece a CTA
 // takes 32 at a time (a CTA a piece: 160 us a pass for the 100,000 of a maze
-// of as many cells).  Few pieces, up to two a CTA, go faster by whole warps.
+// of as many cells).  Few pieces, up to two a CTA, go faster by a warp or the
+// CTA each (12,000 cells, 400 lookups a node, at p = 12: 1.00 ms, by warps 1.08).
 template <bool NIB, class Range, class Done>
 __device__ __forceinline__ void code_open_settle(const uint2 *__restrict__ list, uint32_t count, uint32_t cta,
                                                  uint32_t ctas, const Range &range, const uint32_t *__restrict__ lk,
@@ -286,9 +305,9 @@ __device__ __forceinline__ void code_open_settle(const uint2 *__restrict__ list,
                                                  uint32_t n, int s_log2, int scheme, OpenShared &sh,
                                                  const Done &done) {
     if (count > 2u * ctas)
-        code_open_pieces<NIB, 8>(list, count, cta, ctas, range, lk, cur, nxt, n, s_log2, scheme, sh, done);
+        code_open_pieces<NIB, 8, 32, 128>(list, count, cta, ctas, range, lk, cur, nxt, n, s_log2, scheme, sh, done);
     else
-        code_open_pieces<NIB, 32>(list, count, cta, ctas, range, lk, cur, nxt, n, s_log2, scheme, sh, done);
+        code_open_pieces<NIB, 32, 32, 0>(list, count, cta, ctas, range, lk, cur, nxt, n, s_log2, scheme, sh, done);
 }
 
 // Word k of the window of a run (CodeWindow) from the largest rho inserted per

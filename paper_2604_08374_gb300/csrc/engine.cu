@@ -78,11 +78,16 @@ __global__ void batch_init_kernel(JobDev *jobs, const uint64_t *__restrict__ nod
 
 // The windows of the jobs that gather codes, one CTA per job.
 __global__ void batch_window_kernel(JobDev *jobs) {
-    const JobDev &J = jobs[blockIdx.x];
+    JobDev &J = jobs[blockIdx.x];
     if (!J.codes) return;
     const uint32_t m = 1u << J.p;
-    for (uint32_t k = threadIdx.x; k < m / 4u; k += blockDim.x)
+    uint32_t idle = 0;
+    for (uint32_t k = threadIdx.x; k < m / 4u; k += blockDim.x) {
         window_word(J.win, k, false, J.win + 2 * m, J.win + 2 * m + m / 4u);
+        idle += __popc(equal_bits<false>(J.win[2 * m + k], 0u));
+    }
+    idle = __reduce_add_sync(0xffffffffu, idle);
+    if ((threadIdx.x & 31) == 0 && idle) atomicAdd(&J.idle, idle);
 }
 
 // Pass 1 of the jobs in fjobs[0 .. n) (all of precision p, all fresh) as the
@@ -409,7 +414,7 @@ __global__ void __launch_bounds__(kEngineWarps * 32, 3) batch_code_kernel(JobDev
 
 // The pieces that this pass's code unions left open (code_open_settle), `ctas`
 // CTAs a job: eight an SM over all jobs, 64 a job at least.
-__global__ void __launch_bounds__(256) batch_open_kernel(JobDev *jobs, uint32_t ctas) {
+__global__ void __launch_bounds__(256, 8) batch_open_kernel(JobDev *jobs, uint32_t ctas) {
     __shared__ OpenShared sh;
     JobDev &J = jobs[blockIdx.x / ctas];
     if (J.state != 0 || !J.K || pass_again(J)) return;
@@ -448,7 +453,7 @@ __global__ void batch_step_kernel(JobDev *jobs, int n_jobs, unsigned long long *
                 if (J.d > 0 && t >= J.d) stop = true;
                 if (stop) J.state = 1;
                 const uint64_t regs = (uint64_t)J.n << J.p;
-                if (J.codes) J.K = (double)J.n_top >= kTopShare * (double)regs && !J.too_open ? 1 : 4;
+                if (J.codes) J.K = mostly_at_top(J.n, 1u << J.p, J.idle, J.n_top) && !J.too_open ? 1 : 4;
                 // With every register at its maximum the next pass changes nothing
                 // and is the last: its estimates are these (in the other buffer's
                 // place), its distances gain 0.

@@ -51,6 +51,7 @@ struct JobDev {
     // code tables: win, full, list.
     int codes;
     int K;                  // bits per code of the pass in progress (0: the scattered first pass)
+    uint32_t idle;          // registers whose top is 0
     int too_open;           // a one-bit pass left more than open_cap pieces open and was done again in 4 bits
     uint32_t *win;          // gmax, gbig, then the window's top and low words
     uint8_t *full;          // nodes whose registers have all reached the window's top

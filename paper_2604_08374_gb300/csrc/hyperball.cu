@@ -434,7 +434,8 @@ __global__ void __launch_bounds__(512) stream_bench_kernel(const uint4 *__restri
 // equal it, and (8-bit registers) the one at flags[10] the 16-byte pieces with a
 // register below the window (at most so many does a 4-bit pass leave open);
 // flags[12] counts a node's pieces whose low is not 0 throughout, flags[13] has
-// their slices (at most 32 with codes).
+// their slices (at most 32 with codes), flags[14] counts the registers whose top
+// is 0.
 __global__ void hb_estimate_kernel(const uint8_t *__restrict__ regs, uint32_t n, int p, int S, int t,
                                    double alpha_mm, const double *__restrict__ lc, const double *__restrict__ c_prev,
                                    double *__restrict__ c_cur, double *__restrict__ sum_d,
@@ -468,6 +469,13 @@ __global__ void hb_estimate_kernel(const uint8_t *__restrict__ regs, uint32_t n,
         }
         if (sum) atomicAdd(reinterpret_cast<unsigned long long *>(flags + 6), sum);
         if (low) atomicAdd(reinterpret_cast<unsigned long long *>(flags + 10), low);
+    }
+    if (blockIdx.x == 0) {
+        uint32_t idle = 0;
+        for (uint32_t k = threadIdx.x; k < 4u * pieces; k += blockDim.x)
+            idle += __popc(nib ? equal_bits<true>(__ldg(top + k), 0u) : equal_bits<false>(__ldg(top + k), 0u));
+        idle = __reduce_add_sync(0xffffffffu, idle);
+        if (lane == 0 && idle) atomicAdd(flags + 14, idle);
     }
     if (blockIdx.x == 0 && !nib) {
         const uint4 *lows = reinterpret_cast<const uint4 *>(top) + pieces;
@@ -580,8 +588,10 @@ constexpr int kTrackMaxSlices = 32;
 // nearly every node has a changed neighbour in every slice.
 constexpr double kTrackBelow = 0.01;
 // A run goes back from one-bit codes (kTopShare) to four after a one-bit pass
-// that left more than this share of the 16-byte register pieces open.
-constexpr double kOpenShare = 0.2;
+// that left more 16-byte pieces open than this share of the (node, slice) pairs:
+// a pair's byte union is all its rows however few of its pieces are open, and the
+// share, with the eighth that one-bit codes take, is what a 4-bit pass takes.
+constexpr double kOpenShare = 0.4;
 // What a 4-bit pass saves of a byte pass where nearly all its work is rows
 // gathered (city: 3.1 ms for 256 registers a node against 5.6).  Beside its rows
 // a pass builds the table and reads and writes every node once, about eight rows'
@@ -609,7 +619,8 @@ static uint32_t code_list_cap(const Plan &P, const vga_graph *g, int K) {
     const bool csr = P.mode == kModePerEdge;
     if (K == 4 && !csr && list_entries(P) >= pieces) return (uint32_t)pieces;
     const double rows = csr ? (double)g->n_edges : (double)P.groups.rows_used;
-    return (uint32_t)std::min((double)P.n, code_open_cap(rows, P.node_bytes, g->n_edges, P.n));
+    const double room = csr ? (double)P.n : (double)list_entries(P);
+    return (uint32_t)std::min(room, code_open_cap(rows, P.node_bytes, g->n_edges, P.n));
 }
 
 static int make_plan(const vga_graph *g, int p, const vga_tuning *tune, Plan *P) {
@@ -1370,6 +1381,7 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
         VGA_TRY(ensure_run_items(g, P.scheme, P.hub, stream, &P.items));
         if (P.group) VGA_TRY(ensure_group_list(g, P.scheme, P.hub, P.group, stream, &P.groups));
         if (P.items.hubs) P.codes = false;  // split hubs merge bytes
+        if (!code_rows_pay(P.n, P.groups.rows_used, P.m, P.slices)) P.codes = false;
     }
 
     bool profiling;
@@ -1419,6 +1431,8 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
             uint64_t n_low;       // pieces with a register below the window (codes)
             uint32_t window;      // pieces of a node where the window does not reach 0,
             uint32_t win_slices;  // and the slices that have any
+            uint32_t idle;        // registers whose top is 0
+            uint32_t unused;
         } h{};
         VGA_CHECK_CUDA(cudaMemsetAsync(flags, 0, sizeof(h), stream));
         L2Window window;
@@ -1452,7 +1466,7 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
             int K = 0;
             bool sure = false;
             if (P.codes && t >= 2) {
-                const bool most = (double)h.n_top >= kTopShare * (double)P.n * P.m;
+                const bool most = mostly_at_top(P.n, P.m, h.idle, h.n_top);
                 const double low = (double)h.n_low, cap = (double)code_list_cap(P, g, 4);
                 if (t == 2) low_prev = (double)P.n * h.window;
                 const double left = low_prev > 0.0 ? low * low / low_prev : 0.0;
@@ -1463,8 +1477,7 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
                 const double saved = kCodesSave * rows / (rows + 6.0);
                 const bool fits = low <= cap || left <= cap || again <= saved;
                 low_prev = low;
-                const bool wide = P.mode == kModePerEdge || code_rows_pay(P.n, P.groups.rows_used, P.m, P.slices);
-                K = most && !too_open && P.m >= 128 ? 1 : tracked || P.code_bits < 4 || !fits || !wide ? 0 : 4;
+                K = most && !too_open && P.m >= 128 ? 1 : tracked || P.code_bits < 4 || !fits ? 0 : 4;
                 sure = K == 4 && low <= cap;
             }
             if (tracked && !K) VGA_TRY(launch_need(P, g, chg, ortab, need, stream, timed ? &timings : nullptr));
@@ -1495,7 +1508,7 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
                 return VGA_ETIMEOUT;
             }
             changed_prev = h.n_changed;
-            if (K == 1) too_open = (double)h.open[1] > kOpenShare * (double)P.n * (P.node_bytes / 16.0);
+            if (K == 1) too_open = (double)h.open[1] > kOpenShare * (double)P.n * P.slices;
             std::swap(cur, nxt);
             std::swap(c_prev, c_cur);
             const bool stop = (conv_mode == 1) ? (h.f[1] == 0) : (h.f[0] == 0);

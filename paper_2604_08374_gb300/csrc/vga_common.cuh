@@ -234,18 +234,26 @@ int ensure_group_list(const vga_graph *g, int scheme, uint32_t hub_lookups, int 
 // One pass of the grouped union over register codes (codes.cu): table and
 // union of one code slice of S bytes a node at a time.
 constexpr int kCodeNodes = 4;  // nodes per group of the code kernels
-// A pass gathers one-bit codes once this share of the registers has reached its
-// maximum.
+// A pass gathers one-bit codes once this share of the registers that any node
+// raises has reached its maximum.  (Those that none does are at it from the
+// start: counted as well, 690 nodes at p = 12 took one-bit passes at once, and the
+// byte union after them: 338 us for d = 2 against 270.)
 constexpr double kTopShare = 0.75;
+__host__ __device__ inline bool mostly_at_top(uint64_t n, uint32_t m, uint32_t idle, uint64_t at_top) {
+    return (double)(n * m - at_top) <= (1.0 - kTopShare) * (double)n * (double)(m - idle);
+}
 // Open pieces of a code pass that are settled one by one: while their
 // neighbours' 32-byte sectors, and six more for what a piece takes of its own,
 // stay below an eighth of the bytes (node_bytes a row) that a union of the
 // groups' rows gathers.  (Without the six, a maze of 30,000 cells at p = 9 settled
-// 30,000 pieces a pass: 1.64 ms for 12 passes against 1.21 over bytes.)
+// 30,000 pieces a pass: 1.64 ms for 12 passes against 1.21 over bytes.)  And
+// always as many as its kernel has CTAs, which take them side by side (690 cells
+// at p = 8: cap 55, a byte union of 25 us after a one-bit pass).
 inline double code_open_cap(double rows_used, uint32_t node_bytes, uint64_t edges, uint64_t n) {
-    return rows_used * node_bytes / 8.0 / (32.0 * ((double)edges / (double)n + 6.0));
+    const double cap = rows_used * node_bytes / 8.0 / (32.0 * ((double)edges / (double)n + 6.0));
+    return cap > 1024.0 ? cap : 1024.0;
 }
-// 4-bit rows of less than 512 bytes (in one slice) are worth it from 32 rows a
+// Codes with 4-bit rows of less than 512 bytes (in one slice) are worth it from 32 rows a
 // node on: a warp folds 2,048 bytes of rows at a time, more than a class of a
 // group has where nodes see little.  28,600 cells of rooms (19 rows a node), 12
 // passes: p = 8 1.60 ms with 4-bit passes, 1.40 without, p = 9 1.78 and 1.60; with 33

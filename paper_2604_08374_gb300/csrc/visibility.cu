@@ -15,7 +15,7 @@
 // its transpose (visibility is symmetric); the bytes of every row's LEB128 list
 // counted, with the degrees and range lookups; (host) prefix sum into offsets;
 // (device) the lists written.  Graphs whose matrix would be too large
-// (kMatrixBytes) have all eight octants of a source swept into one CTA's node
+// (kMatrixBytes) or too empty (kMatrixView) have all eight octants of a source swept into one CTA's node
 // bitmap and its list written to a stage in the order the sources finish, from
 // where it is brought to its place; the ordinary load path then validates the
 // stream and derives degrees.
@@ -29,6 +29,25 @@ namespace vga {
 namespace {
 
 constexpr int kMaxSide = 16384;
+
+// Mean length of the row and column of free main-component cells that a node's
+// cell lies in, over 256 nodes.
+double mean_view(int W, int H, const std::vector<uint32_t> &cells, const std::vector<int32_t> &node_of_cell) {
+    const size_t n = cells.size(), step = std::max<size_t>(n / 256, 1);
+    double sum = 0.0;
+    size_t count = 0;
+    for (size_t v = step / 2; v < n; v += step, count++) {
+        const size_t c = cells[v];
+        const int x = (int)(c % (size_t)W), y = (int)(c / (size_t)W);
+        int seen = 2;
+        for (int k = 1; k <= x && node_of_cell[c - k] >= 0; k++) seen++;
+        for (int k = 1; x + k < W && node_of_cell[c + k] >= 0; k++) seen++;
+        for (int k = 1; k <= y && node_of_cell[c - (size_t)k * W] >= 0; k++) seen++;
+        for (int k = 1; y + k < H && node_of_cell[c + (size_t)k * W] >= 0; k++) seen++;
+        sum += 0.5 * seen;
+    }
+    return count ? sum / (double)count : 0.0;
+}
 
 // Largest 4-connected free component (ties: lowest raster index), numbered in
 // raster order.  Returns the raster cell of every node.
@@ -121,6 +140,14 @@ constexpr int kPad = 64;                           // margin bits (obstacles) on
 constexpr uint32_t kNoSource = 0xffffffffu;
 // Largest bit matrix of the graph (N^2 / 8 bytes: up to 370,000 nodes).
 constexpr uint64_t kMatrixBytes = 16ull << 30;
+// From kMatrixNodes nodes on, the matrix is used where the nodes' mean view along
+// a row or column is at least N / kMatrixView cells.  Its passes take time with
+// N^2, and what it saves of the sweep grows with how far the nodes see.  Build
+// with the matrix against without, ms: N = 236,000: views of 4 cells (a maze) 27.1
+// and 12.5, 12 (rooms) 26.5 and 18.5, 30 30.4 and 32.9, 60 39.2 and 62.0; N = 100,000: 4
+// 7.8 and 5.5, 9 8.1 and 7.8, 12 7.5 and 7.8, 30 10.5 and 15.0; N = 46,000: 5 3.3 and 3.4,
+// 9 3.4 and 3.9; N = 360,000: 12 55 and 34, 30 61 and 67, 60 76 and 127.
+constexpr uint32_t kMatrixNodes = 32768, kMatrixView = 10000;
 
 // Test hooks: a smaller shared-memory list capacity sends more sources down
 // the global-list retry (and makes the stage of the lists' bytes so small that
@@ -1001,7 +1028,8 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
     // the node bitmap stays in shared memory while two CTAs fit an SM
     const uint32_t pitch = (words_n + kTileWords - 1) / kTileWords * kTileWords;
     const uint64_t matrix_bytes = 32ull * pitch * pitch * 4;
-    bool by_rows = n && g_sweep_smem_bitmap_nodes == 0 && matrix_bytes <= kMatrixBytes;
+    bool by_rows = n && g_sweep_smem_bitmap_nodes == 0 && matrix_bytes <= kMatrixBytes &&
+                   (n < kMatrixNodes || mean_view(W, H, cells, node_of_cell) * kMatrixView >= (double)n);
     const bool smem_bitmap = bitmap_smem + list_smem + mask_smem + 1024 <= (size_t)smem_optin / 2 &&
                              (g_sweep_smem_bitmap_nodes == 0 || n <= g_sweep_smem_bitmap_nodes);
     const int glist_cap = maxdim + 2;   // at most k + 1 intervals are alive at column k + 1

@@ -498,8 +498,11 @@ def run_ours(args, dist: Dist):
     l2_stream = vga.vga_bench_gather(stream_bytes, S, 64_000_000_000 // S, consumer=2, stream=stream)
     achieved = gather_per_launch / (avg_ms / 1e3) / 1e9
     grouped = mode == 2 and args.group_nodes != 1
-    kernel_name = (f"hb_union_groups_kernel<{S}>" if grouped else f"hb_union_runs_kernel<{S}>") if mode == 2 \
-        else f"hb_union_kernel<{S}>"
+    # launches over 4-bit register codes do not cover a node's register bytes in a pass
+    per_pass = prof["union_launches"] / max(passes - args.steps, 1)
+    codes = grouped and per_pass * S < (1 << args.p) // (2 if args.register_bits == 4 else 1)
+    kernel_name = (f"hb_code_groups_kernel<{S}, 4>" if codes else f"hb_union_groups_kernel<{S}>" if grouped
+                   else f"hb_union_runs_kernel<{S}>") if mode == 2 else f"hb_union_kernel<{S}>"
     traffic, traffic_note = recorded_traffic(kernel_name, args.config)
     peaks = measured_peaks()
     hbm_peak = peaks.get("hbm_gbs")
@@ -533,9 +536,11 @@ def run_ours(args, dist: Dist):
                                "what": "same microbenchmark folding with the union's bytewise max (no decode)"},
         "algorithmic_bytes_per_launch": gather_per_launch,
         "algorithmic_bytes_definition": (
-            ("distinct table rows of the grouped lookup lists (groups of "
-             f"{args.group_nodes or 4} consecutive nodes, each shared row gathered once) plus the split hubs' "
-             "lookups, x slice_bytes, per slice launch (table build included in the timed launch)") if grouped else
+            ("rows covering the ids that groups of "
+             f"{args.group_nodes or 4} nodes see (each row gathered once a group) plus the split hubs' "
+             "lookups, x slice_bytes, per slice launch (table build included in the timed launch"
+             + (f"; a row holds the 4-bit codes of {2 * S} registers; the 1-bit code passes that follow are not "
+                "among the timed launches)" if codes else ")")) if grouped else
             "range lookups x slice_bytes register-row gathers per slice launch (sparse-table build included in the "
             "timed launch); a lookup covers a run of consecutive neighbour ids" if mode == 2 else
             "E x slice_bytes neighbour-register gathers per slice launch"),
@@ -565,11 +570,13 @@ def run_ours(args, dist: Dist):
         # pass 1 by the scatter of the nodes' hashes (one launch for all slices)
         fp_ms = prof["first_pass_ms"] / prof["first_pass_launches"]
         roofline["first_pass"] = {
-            "kernel": "hb_first_pass_kernel", "launches_timed": prof["first_pass_launches"], "avg_launch_ms": fp_ms,
+            "kernel": "hb_first_pass_groups_kernel" if prof["first_pass_grouped"] else "hb_first_pass_kernel",
+            "launches_timed": prof["first_pass_launches"], "avg_launch_ms": fp_ms,
             "share_of_step": prof["first_pass_ms"] / (sec * 1e3) if sec > 0 else None,
             "edge_unions_per_s": E / (fp_ms / 1e3) / 1e9, "unit": "GEdge-unions/s",
             "what": "pass 1 of Eq. hll-union as a scatter: every counter holds only its own node, so each "
                     "neighbour's (register index, rho) is max-folded into shared-memory cells; no rows gathered"}
+    # without the 1-bit code passes, which are not timed launch by launch
     union_share = (prof["union_ms"] + prof["first_pass_ms"]) / (sec * 1e3) if sec > 0 else None
 
     extras = {}
@@ -649,8 +656,8 @@ def run_ours(args, dist: Dist):
                     entry["union"] = {"slice_bytes": p4["slice_bytes"], "launches_timed": p4["union_launches"],
                                       "avg_launch_ms": ms4, "achieved_gbs": ach4,
                                       "frac_vs_l2_stream": ach4 / l2_stream, "frac_vs_gather_shape": ach4 / l2_peak,
-                                      "what": "distinct table rows x slice bytes per launch over the launch time "
-                                              "(a 128-byte row holds 256 packed registers)"}
+                                      "what": "group rows x row bytes per launch over the launch time (a "
+                                              "128-byte row holds 256 packed registers or their 4-bit codes)"}
             sweep.append(entry)
         # register shards (the multi-GPU split) run in lockstep on this one GPU: the same
         # union work as one run plus the per-pass partial sums and their estimate, so the
@@ -691,10 +698,10 @@ def run_ours(args, dist: Dist):
         # the GPU visibility builder (run once before the timed region) beside the oracle's
         extras["builder"] = {"gpu_seconds": build_s, "pair_tests": N * (N - 1) // 2,
                              "pair_tests_per_s": N * (N - 1) / 2 / build_s,
-                             "what": "vga_visibility_build: main component on the host, then each source's "
-                                     "8 octants swept column by column on the device with exact slope intervals, "
-                                     "lists counted and LEB128-encoded in two passes; pair_tests = the N(N-1)/2 "
-                                     "pairs it decides"}
+                             "what": "vga_visibility_build: main component on the host, then half of each source's "
+                                     "octants swept column by column on the device with exact slope intervals into a "
+                                     "bit matrix, joined with its transpose, the lists counted and LEB128-encoded "
+                                     "from it; pair_tests = the N(N-1)/2 pairs it decides"}
         if "cpu_baseline" in extras:
             cb = extras["cpu_baseline"]["builder"]
             extras["builder"]["cpu_oracle_pair_tests_per_s"] = cb["pair_tests_per_s"]

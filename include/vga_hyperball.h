@@ -529,14 +529,18 @@ int vga_metrics(const vga_graph *g, const double *mean_depth_dev, double *out_de
 typedef struct vga_profile {
     uint64_t kernel_launches;     /* library kernels launched since the last reset        */
     uint64_t union_launches;      /* union slices timed (one union kernel, plus the
-                                     sparse-table build in mode 2)                        */
+                                     sparse-table build in mode 2), over registers or
+                                     4-bit register codes.  Passes of 1-bit codes and the
+                                     byte union of what a code pass left open are not among
+                                     them: their work depends on the registers            */
     double union_ms;              /* their summed device time                             */
     uint64_t union_edges;         /* neighbour unions they performed (E per slice)        */
-    uint64_t union_gather_bytes;  /* register rows gathered x slice bytes, summed: E x S
+    uint64_t union_gather_bytes;  /* register (or code) rows gathered x slice bytes, summed: E x S
                                      in mode 1, lookups x S in mode 2                     */
     uint64_t union_hbm_bytes;     /* streamed list bytes (CSR, or 4 x lookups) + 8(N+1)
                                      + 2 x N x slice bytes, summed                        */
-    int slice_bytes;              /* slice width of the last timed launch                 */
+    int slice_bytes;              /* slice width (of registers or codes) of the last timed
+                                     launch                                               */
     int union_mode;               /* union variant of the last timed launch (1 or 2)      */
     int table_rows;               /* rows per node it gathered from: the table scheme's
                                      (mode 2) or 1 (mode 1)                               */

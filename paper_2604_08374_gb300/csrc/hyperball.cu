@@ -869,7 +869,7 @@ struct PendingTiming {
     bool first;    // the first pass's scatter (hb_first_pass_kernel), not a union slice
     bool grouped;  // and that by whole groups
     bool tracked;  // a union slice of a change-tracked pass (its work depends on the changes)
-    bool partial;  // time without bytes: one-bit codes, or the byte union of the pairs a code pass left open
+    bool partial;  // one-bit codes, or the byte union of the pairs a code pass left open: no fixed bytes, not profiled
 };
 
 template <int SS, bool NIB>
@@ -1266,9 +1266,7 @@ static void settle_timings(std::vector<PendingTiming> &timings, bool to_profile,
         } else if (to_profile && ok && pt.tracked) {
             ps.acc.tracked_launches++;
             ps.acc.tracked_ms += ms;
-        } else if (to_profile && ok && pt.partial) {
-            ps.acc.union_ms += ms;
-        } else if (to_profile && ok) {
+        } else if (to_profile && ok && !pt.partial) {
             ps.acc.union_launches++;
             ps.acc.union_ms += ms;
             ps.acc.union_edges += pt.edges;

@@ -149,3 +149,13 @@ def test_narrow_rows_of_few_go_over_bytes(vga):  # noqa: F811
         for job in jobs:
             ref = oracle.hyperball(off, b, job["p"], 3, seed=seed)
             assert np.array_equal(job["mean_depth"].cpu().numpy(), ref["mean_depth"])
+
+
+def test_open_slices_after_a_pass_over_many(vga):  # noqa: F811
+    # as above with 8 slices of 32 registers: the byte union of the one slice with open pairs
+    seed, hub, j = _one_large()
+    off, b = _band(6, hub, 2600)
+    check(vga, off, b, None, P, 4, seed, 8, track_changes=1, l2_budget_mb=1)
+    with vga.vga_graph_load(off, b) as g:
+        # bytes: 8 tables and unions; codes: 4 and 4, the window, the open pieces, a table and a union
+        assert _launches(vga, g, seed, 2, l2_budget_mb=1) == _launches(vga, g, seed, 2, slice_bytes=32) - 16 + 12

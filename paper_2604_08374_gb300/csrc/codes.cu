@@ -24,8 +24,9 @@ __global__ void __launch_bounds__(256) hb_code_table_kernel(const uint8_t *__res
 // 16-byte register pieces go to the list (the first list_cap of them) and, by
 // register slice, to the need masks; flags: [0] a register changed, [2] a
 // bounded wait ran out, [8] slices with open pieces, [9] open pieces.
-// Bound: the L2 bytes of the rows and the ALU pipe (K = 4: 3.2 ms a city launch,
-// 8 logic operations a 16-byte unit; K = 1: 0.56 ms, 2.8 with every row).  One warp
+// Bound: the L2 bytes of the rows and the ALU pipe (K = 4: 3.1 ms a city launch
+// beside 0.05 of its table, 8 logic operations a 16-byte unit; K = 1: 0.5 ms beside
+// 0.1, 2.8 with every row).  One warp
 // per group until the groups fill the GPU twice; below that several, which
 // took 42,680 cells from 2.19 to 1.85 ms and 4,997 cells at p = 12 from 0.86 to
 // 0.74 ms an analysis.  56 registers: measured 25.4 ms on the city against 25.9
@@ -93,7 +94,7 @@ __global__ void __maxnreg__(56) hb_code_groups_kernel(
         }
         if (mine) {
             atomicOr(need + v, mine);
-            code_push_open<K, NIB>(open16, v, u, list, list_cap, flags + 9);
+            code_push_open<K, NIB, true>(open16, v, u, list, list_cap, flags + 9);
         }
         open_slices |= mine;
     }
@@ -218,7 +219,7 @@ __global__ void __launch_bounds__(256) hb_code_csr_kernel(const uint64_t *__rest
                 for (int h = 0; h < UNIT_BYTES / 16; h++)
                     if ((chg16 >> h) & 1u) chg[(uint64_t)((u * UNIT_BYTES + 16u * h) >> s_log2) * n + v] = 1u;
             }
-            if (open16) code_push_open<K, NIB>(open16, v, u, list, list_cap, flags + 9);
+            if (open16) code_push_open<K, NIB, true>(open16, v, u, list, list_cap, flags + 9);
         }
     }
     if (__any_sync(0xffffffffu, changed) && lane == 0) {
@@ -278,13 +279,26 @@ __global__ void __launch_bounds__(256) hb_code_open_csr_kernel(const uint2 *__re
     }
 }
 
-// The window of a run from the largest rho inserted per register index: one
-// word of registers a thread.
-__global__ void hb_window_kernel(const uint32_t *__restrict__ gmax, uint32_t words, int nib, uint32_t *__restrict__ top,
-                                 uint32_t *__restrict__ low) {
-    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= words) return;
-    window_word(gmax, k, nib != 0, top, low);
+// The window of a run from the largest rho inserted per register index, and its
+// counts (launch_code_window): one word of registers a thread.
+__global__ void hb_window_kernel(const uint32_t *__restrict__ gmax, uint32_t words, int nib, int s_log2,
+                                 uint32_t *__restrict__ top, uint32_t *__restrict__ low,
+                                 uint32_t *__restrict__ flags) {
+    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31u;
+    uint32_t idle = 0;
+    bool above = false;
+    if (k < words) {
+        window_word(gmax, k, nib != 0, top, low);
+        idle = __popc(nib ? equal_bits<true>(top[k], 0u) : equal_bits<false>(top[k], 0u));
+        above = low[k] != 0u;
+    }
+    const uint32_t any = __ballot_sync(0xffffffffu, above);
+    if (lane % 4u == 0u && ((any >> lane) & 0xFu)) {
+        atomicAdd(flags + 12, 1u);
+        atomicOr(flags + 13, 1u << (((4u * k) >> s_log2) & 31u));
+    }
+    idle = __reduce_add_sync(0xffffffffu, idle);
+    if (lane == 0u && idle) atomicAdd(flags + 14, idle);
 }
 
 template <int S, int K, bool NIB>
@@ -376,9 +390,9 @@ int launch_code_open(const CodePass &C, const uint64_t *lk_off, const uint32_t *
     return VGA_OK;
 }
 
-int launch_code_window(const uint32_t *gmax, uint32_t words, int nib, uint32_t *top, uint32_t *low,
-                       cudaStream_t stream) {
-    hb_window_kernel<<<(words + 255) / 256, 256, 0, stream>>>(gmax, words, nib, top, low);
+int launch_code_window(const uint32_t *gmax, uint32_t words, int nib, int s_log2, uint32_t *top, uint32_t *low,
+                       uint32_t *flags, cudaStream_t stream) {
+    hb_window_kernel<<<(words + 255) / 256, 256, 0, stream>>>(gmax, words, nib, s_log2, top, low, flags);
     count_launch();
     VGA_CHECK_CUDA(cudaGetLastError());
     return VGA_OK;

@@ -18,11 +18,13 @@
 // pass 3 all but 1e-5 of the city's.
 //
 // Measured (GB300): the city graph's pass 2 takes four launches of 128-byte
-// K = 4 rows at 3.1 ms and pass 3 one of K = 1 rows at 0.5 ms (2.8 ms before
-// a class was cut short once all its bits were set, code_group), where the byte
-// union takes eight at 2.8 ms each; the d = 3 analysis (with pass 1 by
-// groups, first_pass.cuh) 57.4 -> 19.5 ms, the unlimited one at p = 12 343 -> 71
-// ms, medium d = 3 3.1 -> 1.5-1.7 ms.
+// K = 4 rows at 3.16 ms, table included, and pass 3 one of K = 1 rows at 0.6 ms (2.8
+// before a class was cut short once all its bits were set, code_group), where the
+// byte union takes eight at 2.8 ms each; the d = 3 analysis (with pass 1 by
+// groups, first_pass.cuh) 57.4 -> 19.6 ms, the unlimited one at p = 12 343 -> 70
+// ms, medium d = 3 3.1 -> 1.5-1.7 ms.  Graphs of small views have to be told apart
+// (run_impl, code_rows_pay): there many registers stay below the window, and rows
+// are too few to save on.
 //
 // Layout: a 16-byte unit holds 32 registers as four bit planes (K = 4; word k =
 // bit k of the codes, bit i = register i) or 128 registers as one plane
@@ -160,15 +162,17 @@ __device__ __forceinline__ void code_store(uint4 code, const uint8_t *__restrict
 }
 
 // Open pieces of unit u of node v (open16: bit per 16 register bytes) to the
-// list, as far as it holds them; *count counts them all.  The lanes that get
-// here together raise it once: on graphs of small views every node has some.
-template <int K, bool NIB>
+// list, as far as it holds them; *count counts them all.  With JOIN the lanes
+// that get here together raise it once: on graphs of small views every node has
+// some.  (Not in the engine: its kernel for 512-byte rows then took 25 % longer,
+// 5.0 ms against 4.0 in the second pass of 64 sites.)
+template <int K, bool NIB, bool JOIN>
 __device__ __forceinline__ void code_push_open(uint32_t open16, uint32_t v, uint32_t u, uint2 *__restrict__ list,
                                                uint32_t list_cap, uint32_t *count) {
     constexpr uint32_t PIECES = kUnitRegs<K> / (NIB ? 2 : 1) / 16;
-    const uint32_t mine = (uint32_t)__popc(open16), here = __activemask();
+    const uint32_t mine = (uint32_t)__popc(open16), here = JOIN ? __activemask() : 0u;
     uint32_t at;
-    if (__all_sync(here, mine == 1u)) {
+    if (JOIN && __all_sync(here, mine == 1u)) {
         const int lead = __ffs(here) - 1;
         const uint32_t lane = threadIdx.x & 31u;
         if ((int)lane == lead) at = atomicAdd(count, (uint32_t)__popc(here));

@@ -14,7 +14,7 @@
 //   step      one thread per job: pass count, stop rule, flags;
 //   finalize  mean depth and ball sizes of the jobs that just stopped.
 // The pass loop is either driven from the host (one flag read per pass) or
-// captured once as a CUDA graph whose WHILE conditional node repeats the four
+// captured once as a CUDA graph whose WHILE conditional node repeats the pass's
 // launches until no job is running, with no host round trip at all.
 //
 // Every job's registers, estimates and outputs are bit-identical to a
@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(kEngineWarps * 32, 3) batch_code_kernel(JobDev
                 uint32_t chg16, open16;
                 code_store<K, false>(part[w], cur, nxt, n, s_log2, v, u, win, chg16, open16);
                 changed |= chg16 != 0u;
-                if (open16) code_push_open<K, false>(open16, v, u, J.list, J.list_cap, &J.open);
+                if (open16) code_push_open<K, false, false>(open16, v, u, J.list, J.list_cap, &J.open);
             }
             if (__any_sync(0xffffffffu, changed) && lane == 0) {
                 if (*reinterpret_cast<volatile uint32_t *>(&J.changed) == 0u) atomicOr(&J.changed, 1u);

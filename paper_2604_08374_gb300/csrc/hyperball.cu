@@ -431,24 +431,21 @@ __global__ void __launch_bounds__(512) stream_bench_kernel(const uint4 *__restri
 // HLL estimate of every node, then Eq. sumD (estimate_nodes), `per` nodes a
 // warp; flags[1] records the paper's convergence test max_v(c_t - c_{t-1}) >
 // 0.5.  With top given, the 64-bit count at flags[6] adds up the registers that
-// equal it, and (8-bit registers) the one at flags[10] the 16-byte pieces with a
-// register below the window (at most so many does a 4-bit pass leave open);
-// flags[12] counts a node's pieces whose low is not 0 throughout, flags[13] has
-// their slices (at most 32 with codes), flags[14] counts the registers whose top
-// is 0.
+// equal it, and with count_low (8-bit registers) the one at flags[10] the 16-byte
+// pieces with a register below the window: at most so many does a 4-bit pass
+// leave open.
 __global__ void hb_estimate_kernel(const uint8_t *__restrict__ regs, uint32_t n, int p, int S, int t,
                                    double alpha_mm, const double *__restrict__ lc, const double *__restrict__ c_prev,
                                    double *__restrict__ c_cur, double *__restrict__ sum_d,
                                    uint32_t *__restrict__ flags, int nib, const uint32_t *__restrict__ top,
-                                   uint8_t *__restrict__ full, uint32_t per) {
+                                   uint8_t *__restrict__ full, int count_low, uint32_t per) {
     __shared__ uint64_t s_top[32], s_low[32];
-    const uint32_t pieces = (nib ? 1u << p >> 1 : 1u << p) / 16u;  // of a node
     const int lane = threadIdx.x & 31;
     const uint64_t v0 = ((uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per;
     uint64_t at_top = 0, below = 0;
     const uint32_t v1 = (uint32_t)(v0 + per < n ? v0 + per : n);
     if (v0 < n) {
-        if (top && !nib)
+        if (count_low)
             estimate_nodes<true>(regs, n, p, S, t, alpha_mm, lc, c_prev, c_cur, sum_d, flags + 1, (uint32_t)v0, v1,
                                  lane, false, top, full, &at_top, &below);
         else
@@ -469,23 +466,6 @@ __global__ void hb_estimate_kernel(const uint8_t *__restrict__ regs, uint32_t n,
         }
         if (sum) atomicAdd(reinterpret_cast<unsigned long long *>(flags + 6), sum);
         if (low) atomicAdd(reinterpret_cast<unsigned long long *>(flags + 10), low);
-    }
-    if (blockIdx.x == 0) {
-        uint32_t idle = 0;
-        for (uint32_t k = threadIdx.x; k < 4u * pieces; k += blockDim.x)
-            idle += __popc(nib ? equal_bits<true>(__ldg(top + k), 0u) : equal_bits<false>(__ldg(top + k), 0u));
-        idle = __reduce_add_sync(0xffffffffu, idle);
-        if (lane == 0 && idle) atomicAdd(flags + 14, idle);
-    }
-    if (blockIdx.x == 0 && !nib) {
-        const uint4 *lows = reinterpret_cast<const uint4 *>(top) + pieces;
-        for (uint32_t k = threadIdx.x; k < pieces; k += blockDim.x) {
-            const uint4 l = __ldg(lows + k);
-            if (l.x | l.y | l.z | l.w) {
-                atomicAdd(flags + 12, 1u);
-                atomicOr(flags + 13, 1u << (16u * k / (uint32_t)S));
-            }
-        }
     }
 }
 
@@ -591,6 +571,7 @@ constexpr double kTrackBelow = 0.01;
 // that left more 16-byte pieces open than this share of the (node, slice) pairs:
 // a pair's byte union is all its rows however few of its pieces are open, and the
 // share, with the eighth that one-bit codes take, is what a 4-bit pass takes.
+// (Medium workload, unlimited: 2.83 ms at 0.2 against 2.27; 0.8 changes nothing.)
 constexpr double kOpenShare = 0.4;
 // What a 4-bit pass saves of a byte pass where nearly all its work is rows
 // gathered (city: 3.1 ms for 256 registers a node against 5.6).  Beside its rows
@@ -612,12 +593,14 @@ static uint64_t list_entries(const Plan &P) {
     return pieces <= (1u << 16) ? std::max<uint64_t>(P.n, pieces) : P.n;
 }
 
+static bool all_listed(const Plan &P) { return list_entries(P) >= P.n * P.node_bytes / 16; }
+
 // Open pieces of a K-bit pass that are settled one by one (code_open_cap); more
 // of them leave a byte union to do after it.
 static uint32_t code_list_cap(const Plan &P, const vga_graph *g, int K) {
     const uint64_t pieces = P.n * P.node_bytes / 16;
     const bool csr = P.mode == kModePerEdge;
-    if (K == 4 && !csr && list_entries(P) >= pieces) return (uint32_t)pieces;
+    if (K == 4 && !csr && all_listed(P)) return (uint32_t)pieces;
     const double rows = csr ? (double)g->n_edges : (double)P.groups.rows_used;
     const double room = csr ? (double)P.n : (double)list_entries(P);
     return (uint32_t)std::min(room, code_open_cap(rows, P.node_bytes, g->n_edges, P.n));
@@ -1293,8 +1276,10 @@ static int launch_estimate(const Plan &P, const uint8_t *regs, int t, const doub
     const uint32_t per = (uint32_t)std::min<uint64_t>(16, std::max<uint64_t>(1, P.n / ((uint64_t)sms * 96)));
     const unsigned blocks = (unsigned)((P.n + (uint64_t)warps * per - 1) / ((uint64_t)warps * per));
     const double alpha_mm = hll_alpha_host(P.p) * (double)P.m * (double)P.m;
+    // where the list holds every piece the count decides nothing (code_list_cap)
+    const int count_low = top && !P.nib && (P.mode == kModePerEdge || !all_listed(P));
     hb_estimate_kernel<<<blocks, warps * 32, 0, stream>>>(regs, (uint32_t)P.n, P.p, P.S, t, alpha_mm, lc, c_prev,
-                                                          c_cur, sum_d, flags, P.nib, top, full, per);
+                                                          c_cur, sum_d, flags, P.nib, top, full, count_low, per);
     count_launch();
     VGA_CHECK_CUDA(cudaGetLastError());
     return VGA_OK;
@@ -1418,7 +1403,6 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
                                                                           (uint32_t)P.slices, keys, gmax, gbig);
         count_launch();
         VGA_CHECK_CUDA(cudaGetLastError());
-        if (gmax) VGA_TRY(launch_code_window(gmax, P.node_bytes / 4, P.nib, top, top + P.node_bytes / 4, stream));
         VGA_TRY(launch_estimate(P, cur, 0, lc, nullptr, c_prev, sum_d, flags, stream));  // c_0
         if (max_trace >= 0) VGA_TRY(copy_trace(P, cur, c_prev, 0, trace_regs, trace_c, stream));
         struct {
@@ -1427,11 +1411,12 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
             uint64_t n_top;       // registers at the window's top (codes)
             uint32_t open[2];     // slices where a code pass left pieces open, and the pieces
             uint64_t n_low;       // pieces with a register below the window (codes)
-            uint32_t window;      // pieces of a node where the window does not reach 0,
-            uint32_t win_slices;  // and the slices that have any
-            uint32_t idle;        // registers whose top is 0
-            uint32_t unused;
+            struct {              // of the first pass only (launch_code_window)
+                uint32_t pieces, slices, idle, unused;
+            } win;
         } h{};
+        static_assert(sizeof(h) == 64, "the flags' 64 bytes");
+        decltype(h.win) win{};
         VGA_CHECK_CUDA(cudaMemsetAsync(flags, 0, sizeof(h), stream));
         L2Window window;
         if (tune && tune->l2_window) {
@@ -1464,17 +1449,20 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
             int K = 0;
             bool sure = false;
             if (P.codes && t >= 2) {
-                const bool most = mostly_at_top(P.n, P.m, h.idle, h.n_top);
                 const double low = (double)h.n_low, cap = (double)code_list_cap(P, g, 4);
-                if (t == 2) low_prev = (double)P.n * h.window;
+                if (t == 2) {
+                    win = h.win;
+                    low_prev = (double)P.n * win.pieces;
+                }
                 const double left = low_prev > 0.0 ? low * low / low_prev : 0.0;
                 const double rows = (double)P.groups.rows_used / (double)P.n;
                 const double again = P.mode == kModePerEdge || low == 0.0 ? 1.0
-                                     : (left / ((double)P.n * h.window) * rows + 6.0) / (rows + 8.0) *
-                                           __builtin_popcount(h.win_slices) / P.slices;
+                                     : (left / ((double)P.n * win.pieces) * rows + 6.0) / (rows + 8.0) *
+                                           __builtin_popcount(win.slices) / P.slices;
                 const double saved = kCodesSave * rows / (rows + 6.0);
                 const bool fits = low <= cap || left <= cap || again <= saved;
                 low_prev = low;
+                const bool most = mostly_at_top(P.n, P.m, win.idle, h.n_top);
                 K = most && !too_open && P.m >= 128 ? 1 : tracked || P.code_bits < 4 || !fits ? 0 : 4;
                 sure = K == 4 && low <= cap;
             }
@@ -1482,6 +1470,9 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
             const uint64_t clear = K && P.mode == kModeRuns ? P.off_need + 4 * P.n - P.off_flags
                                      : chg ? P.off_chg + P.chg_bytes - P.off_flags : sizeof(h);
             VGA_CHECK_CUDA(cudaMemsetAsync(flags, 0, clear, stream));
+            if (t == 1 && gmax)
+                VGA_TRY(launch_code_window(gmax, P.node_bytes / 4, P.nib, __builtin_ctz((unsigned)P.S), top,
+                                           top + P.node_bytes / 4, flags, stream));
             if (K && P.mode == kModePerEdge) {
                 VGA_TRY(launch_codes_csr(P, g, K, base, cur, nxt, flags, stream, timed ? &timings : nullptr, chg,
                                          sure));

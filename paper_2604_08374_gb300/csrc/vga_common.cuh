@@ -237,7 +237,10 @@ constexpr int kCodeNodes = 4;  // nodes per group of the code kernels
 // A pass gathers one-bit codes once this share of the registers that any node
 // raises has reached its maximum.  (Those that none does are at it from the
 // start: counted as well, 690 nodes at p = 12 took one-bit passes at once, and the
-// byte union after them: 338 us for d = 2 against 270.)
+// byte union after them: 338 us for d = 2 against 270.)  At 0.5, one-bit passes
+// come too early: 5,003 cells at p = 12, unlimited, 0.93 ms against 0.53, 232,000
+// cells of rooms, 12 passes, 22.3 against 20.0; 0.9 is between 6 % faster and 5 %
+// slower.
 constexpr double kTopShare = 0.75;
 __host__ __device__ inline bool mostly_at_top(uint64_t n, uint32_t m, uint32_t idle, uint64_t at_top) {
     return (double)(n * m - at_top) <= (1.0 - kTopShare) * (double)n * (double)(m - idle);
@@ -245,7 +248,9 @@ __host__ __device__ inline bool mostly_at_top(uint64_t n, uint32_t m, uint32_t i
 // Open pieces of a code pass that are settled one by one: while their
 // neighbours' 32-byte sectors, and six more for what a piece takes of its own,
 // stay below an eighth of the bytes (node_bytes a row) that a union of the
-// groups' rows gathers.  (Without the six, a maze of 30,000 cells at p = 9 settled
+// groups' rows gathers.  (At a sixteenth, 100,000 cells of maze took 6.8 ms for 12
+// passes against 5.7, of noise 5.8 against 5.1; a quarter is as an eighth but for
+// the medium workload at p = 12, 6.1 against 7.3.  Without the six, a maze of 30,000 cells at p = 9 settled
 // 30,000 pieces a pass: 1.64 ms for 12 passes against 1.21 over bytes.)  And
 // always as many as its kernel has CTAs, which take them side by side (690 cells
 // at p = 8: cap 55, a byte union of 25 us after a one-bit pass).
@@ -286,8 +291,11 @@ int launch_code_open(const CodePass &C, const uint64_t *lk_off, const uint32_t *
 // The same over neighbour lists instead of groups, for a caller without range
 // lookups: `tab` takes the codes of all slices (N * m * K / 8 bytes).
 int launch_code_csr(const CodePass &C, uint32_t m, const uint64_t *off, const uint8_t *bytes, int sms);
-int launch_code_window(const uint32_t *gmax, uint32_t words, int nib, uint32_t *top, uint32_t *low,
-                       cudaStream_t stream);
+// The window of a run in register words, with its counts in flags[12 .. 14]
+// (zeroed): a node's 16-byte pieces whose low is not 0 throughout, their slices of
+// 2^s_log2 bytes (bit i % 32), and the registers whose top is 0.
+int launch_code_window(const uint32_t *gmax, uint32_t words, int nib, int s_log2, uint32_t *top, uint32_t *low,
+                       uint32_t *flags, cudaStream_t stream);
 
 // The first pass as a scatter for whole groups (first_pass.cuh).  A node's key
 // is j << 4 | level (level = min(rho, 16) - 1), 16 bits up to p = 12.  gbig[j]

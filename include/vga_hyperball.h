@@ -214,7 +214,12 @@ int vga_visibility_count(int W, int H, const uint8_t *obst, uint32_t *n_nodes);
 /* HyperBall (Sec. 3.3, Algorithm 1, Sec. 3.4)                             */
 /* ---------------------------------------------------------------------- */
 
-/* Tuning knobs (all 0 = choose automatically). */
+/* Tuning knobs (all 0 = choose automatically).  Automatic runs gather 4-bit or
+ * 1-bit codes of the registers from the second pass on, a half or an eighth of the
+ * bytes, with the same results.  An explicit slice_bytes, group_nodes other than 4,
+ * track_changes = 2, more than 32 slices and a split hub (hub_lookups) each keep
+ * every pass over the register bytes, about three times as long on city graphs;
+ * so does a width from an installed tuning table. */
 typedef struct vga_tuning {
     int slice_bytes;     /* registers per union slice: power of two in [16, min(m, 1024)] */
     int warps_per_cta;   /* union kernel CTA size in warps: 1..16 (0: 4 in mode 2, 8 in 1) */
@@ -322,10 +327,16 @@ int hyperball_workspace_bytes(const vga_graph *g, int p, uint64_t *bytes);
  *   iterations      host out or NULL.
  *   workspace_dev   device scratch of at least hyperball_workspace_bytes(),
  *                   256-byte aligned, or NULL to let the library allocate and
- *                   free its own.
+ *                   free its own.  With union_mode 1 all workspace_bytes are
+ *                   used: past what the mode asks for, room for N m / 2 bytes
+ *                   (or N m / 8) of register codes and about 10 (m + N) more
+ *                   makes later passes gather those, on graphs of at least 16
+ *                   neighbours a node; a workspace of the library's own has none.
  *   stream          cudaStream_t to run on (NULL = legacy default stream).  The
  *                   call returns after the last pass; it synchronises on the
- *                   stream once per pass to read the stop flag.
+ *                   stream once per pass to read the stop flag, and once more in
+ *                   a pass over register codes that may leave something to the
+ *                   byte union behind it.
  *   tuning          NULL or knobs.
  */
 int hyperball_run_dev(const vga_graph *g, int p, int d, uint64_t seed, int conv_mode, double *mean_depth_dev,
@@ -687,6 +698,10 @@ typedef struct vga_tune_entry {
  * Each candidate runs two union passes (d = 2) twice and
  * keeps its faster run; a run of each variant first builds any lookup list.
  * Every candidate computes the same registers (they differ only in launch shape).
+ * The candidates have explicit widths, and so has every entry: they are timed, and
+ * later run, over register bytes.  The automatic choice, whose later passes
+ * gather register codes (vga_tuning), is not among them and is faster on most
+ * graphs: install a table where that has been compared.
  */
 int vga_autotune(const vga_graph *const *graphs, int n_graphs, int p, void *stream, vga_tune_entry *out,
                  int max_out, int *n_out, int install);

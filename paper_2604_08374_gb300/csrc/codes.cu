@@ -25,8 +25,8 @@ __global__ void __launch_bounds__(256) hb_code_table_kernel(const uint8_t *__res
 // register slice, to the need masks; flags: [0] a register changed, [2] a
 // bounded wait ran out, [8] slices with open pieces, [9] open pieces.
 // Bound: the L2 bytes of the rows and the ALU pipe (K = 4: 3.1 ms a city launch
-// beside 0.05 of its table, 8 logic operations a 16-byte unit; K = 1: 0.5 ms beside
-// 0.1, 2.8 with every row).  One warp
+// beside 0.05 of its table, 8 logic operations a 16-byte unit; K = 1: 0.55 ms beside
+// 0.17, 2.8 with every row).  One warp
 // per group until the groups fill the GPU twice; below that several, which
 // took 42,680 cells from 2.19 to 1.85 ms and 4,997 cells at p = 12 from 0.86 to
 // 0.74 ms an analysis.  56 registers: measured 25.4 ms on the city against 25.9

@@ -18,7 +18,7 @@
 // pass 3 all but 1e-5 of the city's.
 //
 // Measured (GB300): the city graph's pass 2 takes four launches of 128-byte
-// K = 4 rows at 3.16 ms, table included, and pass 3 one of K = 1 rows at 0.6 ms (2.8
+// K = 4 rows at 3.16 ms, table included, and pass 3 one of K = 1 rows at 0.73 ms (2.8
 // before a class was cut short once all its bits were set, code_group), where the
 // byte union takes eight at 2.8 ms each; the d = 3 analysis (with pass 1 by
 // groups, first_pass.cuh) 57.4 -> 19.6 ms, the unlimited one at p = 12 343 -> 70

@@ -657,7 +657,7 @@ __global__ void __launch_bounds__(kSweepThreads, 6) visibility_sweep_kernel(Swee
 // hold the cells after the source in raster order (and the rest of its own row)
 // are swept; rows_join_kernel adds the other half.  No bitmap in shared memory
 // and no octant that waits for another's, so 48 warps an SM stay busy: bound by
-// the chain of steps from column to column.  City grid: 77 ms, with the joining 5,
+// the chain of steps from column to column.  City grid: 75 ms, with the joining 5,
 // the counting 7 and the encoding 10, where a CTA of eight octants with a bitmap in
 // shared memory took 229.
 constexpr int kRowsOctants = 4;

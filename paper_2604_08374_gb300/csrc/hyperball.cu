@@ -1267,7 +1267,7 @@ static void settle_timings(std::vector<PendingTiming> &timings, bool to_profile,
 
 static int launch_estimate(const Plan &P, const uint8_t *regs, int t, const double *lc, const double *c_prev,
                            double *c_cur, double *sum_d, uint32_t *flags, cudaStream_t stream,
-                           const uint32_t *top = nullptr, uint8_t *full = nullptr) {
+                           const uint32_t *top = nullptr, uint8_t *full = nullptr, bool low = false) {
     const int warps = 8;
     // nodes a warp: while the warps fill the GPU twice (about 48 an SM), up to 16
     int dev = 0, sms = 1;
@@ -1277,7 +1277,7 @@ static int launch_estimate(const Plan &P, const uint8_t *regs, int t, const doub
     const unsigned blocks = (unsigned)((P.n + (uint64_t)warps * per - 1) / ((uint64_t)warps * per));
     const double alpha_mm = hll_alpha_host(P.p) * (double)P.m * (double)P.m;
     // where the list holds every piece the count decides nothing (code_list_cap)
-    const int count_low = top && !P.nib && (P.mode == kModePerEdge || !all_listed(P));
+    const int count_low = low && top && !P.nib && (P.mode == kModePerEdge || !all_listed(P));
     hb_estimate_kernel<<<blocks, warps * 32, 0, stream>>>(regs, (uint32_t)P.n, P.p, P.S, t, alpha_mm, lc, c_prev,
                                                           c_cur, sum_d, flags, P.nib, top, full, count_low, per);
     count_launch();
@@ -1488,7 +1488,8 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
             // what the next pass goes by is not needed of the last one
             const bool last = d > 0 && t >= d;
             if (chg && !last) VGA_TRY(launch_count(P, chg, flags, stream));
-            VGA_TRY(launch_estimate(P, nxt, t, lc, c_prev, c_cur, sum_d, flags, stream, last ? nullptr : top, full));
+            VGA_TRY(launch_estimate(P, nxt, t, lc, c_prev, c_cur, sum_d, flags, stream, last ? nullptr : top, full,
+                                    K != 4));
             if (t <= max_trace) VGA_TRY(copy_trace(P, nxt, c_cur, t, trace_regs, trace_c, stream));
             VGA_CHECK_CUDA(cudaMemcpyAsync(&h, flags, sizeof(h), cudaMemcpyDeviceToHost, stream));
             VGA_CHECK_CUDA(cudaStreamSynchronize(stream));
@@ -1497,6 +1498,7 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
                 return VGA_ETIMEOUT;
             }
             changed_prev = h.n_changed;
+            if (K == 4) h.n_low = h.open[1];  // what a 4-bit pass settles is in the window
             if (K == 1) too_open = (double)h.open[1] > kOpenShare * (double)P.n * P.slices;
             std::swap(cur, nxt);
             std::swap(c_prev, c_cur);

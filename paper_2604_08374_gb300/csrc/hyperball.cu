@@ -1444,8 +1444,8 @@ static int run_impl(const vga_graph *g, int p, int d, uint64_t seed, int conv_mo
             // byte union has to fit into what the codes save (kCodesSave; in mode 1
             // it is a whole pass).  On graphs of small views (mazes,
             // small rooms) nearly all stays open for many passes: 236,000 cells of
-            // maze at p = 8, 20 passes, took 33.6 ms with 4-bit passes, 15.6 over
-            // bytes alone, 12.3 by this rule.
+            // maze at p = 8, 20 passes, took 33.7 ms with 4-bit passes, 15.6 over
+            // bytes alone, 11.9 by this rule.
             int K = 0;
             bool sure = false;
             if (P.codes && t >= 2) {

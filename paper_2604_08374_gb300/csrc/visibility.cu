@@ -1043,7 +1043,12 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
     VGA_TRY(d_cells.alloc((size_t)std::max<uint32_t>(n, 1) * 4));
     VGA_TRY(d_rowbytes.alloc((size_t)std::max<uint32_t>(n, 1) * 8));
     VGA_TRY(d_counter.alloc(6 * sizeof(uint32_t)));
-    VGA_TRY(d_retry.alloc((size_t)std::max<uint32_t>(n, 1) * 4));
+    if (by_rows && d_retry.alloc((size_t)n * 4 * kRowsOctants) != VGA_OK) {
+        cudaGetLastError();
+        clear_error();
+        by_rows = false;
+    }
+    if (!by_rows) VGA_TRY(d_retry.alloc((size_t)std::max<uint32_t>(n, 1) * 4));
     VGA_TRY(d_err.alloc(sizeof(int)));
     VGA_TRY(d_off.alloc(((size_t)n + 1) * 8));
     cudaStream_t stream = 0;
@@ -1155,10 +1160,9 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
     DeviceBuffer d_matrix;
     // The bit matrix and what it tells.  VGA_ENOMEM: no room for it and what goes with it.
     auto build_rows = [&]() -> int {
-        DeviceBuffer d_noc_t, d_lookups, d_rows_retry;
+        DeviceBuffer d_noc_t, d_lookups;
         VGA_TRY(d_noc_t.alloc((size_t)W * H * 4));
         VGA_TRY(d_lookups.alloc((size_t)n * 4));
-        VGA_TRY(d_rows_retry.alloc((size_t)n * 4 * kRowsOctants));
         VGA_TRY(built.degree.alloc((size_t)n * 4));
         VGA_TRY(d_matrix.alloc(matrix_bytes));
         cells_transpose_kernel<<<dim3((W + 31) / 32, (H + 31) / 32), 256, 0, stream>>>(sa.node_of_cell, W, H,
@@ -1186,7 +1190,6 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
             a.sources = sources;
             a.count = count;
             a.next = counter;
-            a.retry = d_rows_retry.as<uint32_t>();
             a.glists = d_glists.as<uint2>();
             fn<<<grid, kSweepThreads, smem, stream>>>(a);
             count_launch();
@@ -1196,7 +1199,7 @@ int vga_visibility_build_ordered(int W, int H, const uint8_t *obst, int order, u
         VGA_TRY(sweep_rows(false, nullptr, n * kRowsOctants, d_counter.as<uint32_t>()));
         VGA_CHECK_CUDA(cudaMemcpyAsync(&n_retry, sa.retry_count, 4, cudaMemcpyDeviceToHost, stream));
         VGA_CHECK_CUDA(cudaStreamSynchronize(stream));
-        VGA_TRY(sweep_rows(true, d_rows_retry.as<uint32_t>(), n_retry, d_counter.as<uint32_t>() + 1));
+        VGA_TRY(sweep_rows(true, retry_list, n_retry, d_counter.as<uint32_t>() + 1));
         VGA_CHECK_CUDA(cudaFuncSetAttribute(rows_join_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kJoinSmem));
         const unsigned tiles = pitch / kTileWords;
         rows_join_kernel<<<dim3(tiles, tiles), 256, kJoinSmem, stream>>>(sa.matrix, pitch);

@@ -173,7 +173,8 @@ int vga_graph_set_cells(vga_graph *g, int W, int H, const uint64_t *cell_of_node
  * obstacle bitmaps (2 x W x H bits with margins), two W*H node-id tables and 28
  * bytes a node; for sources whose interval lists outgrow shared memory, global
  * lists of max(W, H) + 2 entries per warp.  Without room for the matrix,
- * above 370,000 nodes, or where N is large against how far the nodes see, all octants are swept instead, with a node bitmap per CTA
+ * above 370,000 nodes, or where N is large against how far the nodes see, all
+ * octants are swept instead, with a node bitmap per CTA
  * (in shared memory up to ~800k nodes) and, while it is to be had, a stage of
  * about the CSR's size (at most 256 MB, or a twentieth more than the sampled
  * size), without which every source is swept twice.

@@ -888,7 +888,8 @@ __device__ __forceinline__ void harmonic_partial(const uint8_t *__restrict__ reg
                                                  uint32_t b0, uint32_t b1, uint32_t v, int lane, bool nib,
                                                  uint64_t &lo, uint64_t &hi, uint32_t &zeros,
                                                  const uint32_t *__restrict__ top = nullptr,
-                                                 uint32_t *at_top = nullptr, uint32_t has = 0, uint32_t *below = nullptr) {
+                                                 uint32_t *at_top = nullptr, uint32_t has = 0,
+                                                 uint32_t *below = nullptr) {
     const int K = 65 - p;
     lo = 0;
     hi = 0;

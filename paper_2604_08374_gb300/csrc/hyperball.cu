@@ -551,8 +551,8 @@ struct Plan {
     uint64_t n = 0;
     // workspace layout (byte offsets, 256-aligned)
     uint64_t off_cur = 0, off_next = 0, off_c0 = 0, off_c1 = 0, off_sum = 0, off_lc = 0, off_flags = 0, off_tab = 0,
-             off_chg = 0, off_need = 0, off_ortab = 0, off_win = 0, off_full = 0, off_list = 0, off_codes = 0, chg_bytes = 0, total = 0,
-             least = 0;  // what a run without codes takes of the total
+             off_chg = 0, off_need = 0, off_ortab = 0, off_win = 0, off_full = 0, off_list = 0, off_codes = 0,
+             chg_bytes = 0, total = 0, least = 0;  // what a run without codes takes of the total
 };
 
 static uint64_t align256(uint64_t x) { return (x + 255) & ~255ull; }

@@ -250,16 +250,17 @@ __host__ __device__ inline bool mostly_at_top(uint64_t n, uint32_t m, uint32_t i
 // stay below an eighth of the bytes (node_bytes a row) that a union of the
 // groups' rows gathers.  (At a sixteenth, 100,000 cells of maze took 6.8 ms for 12
 // passes against 5.7, of noise 5.8 against 5.1; a quarter is as an eighth but for
-// the medium workload at p = 12, 6.1 against 7.3.  Without the six, a maze of 30,000 cells at p = 9 settled
-// 30,000 pieces a pass: 1.64 ms for 12 passes against 1.21 over bytes.)  And
+// the medium workload at p = 12, 6.1 against 7.3.  Without the six, a maze of
+// 30,000 cells at p = 9 settled 30,000 pieces a pass: 1.64 ms for 12 passes
+// against 1.21 over bytes.)  And
 // always as many as its kernel has CTAs, which take them side by side (690 cells
 // at p = 8: cap 55, a byte union of 25 us after a one-bit pass).
 inline double code_open_cap(double rows_used, uint32_t node_bytes, uint64_t edges, uint64_t n) {
     const double cap = rows_used * node_bytes / 8.0 / (32.0 * ((double)edges / (double)n + 6.0));
     return cap > 1024.0 ? cap : 1024.0;
 }
-// Codes with 4-bit rows of less than 512 bytes (in one slice) are worth it from 32 rows a
-// node on: a warp folds 2,048 bytes of rows at a time, more than a class of a
+// Codes with 4-bit rows of less than 512 bytes (in one slice) are worth it from
+// 32 rows a node on: a warp folds 2,048 bytes of rows at a time, more than a class of a
 // group has where nodes see little.  28,600 cells of rooms (19 rows a node), 12
 // passes: p = 8 1.60 ms with 4-bit passes, 1.40 without, p = 9 1.78 and 1.60; with 33
 // rows 1.23 and 1.23, 1.40 and 1.47; 83 rows 0.22 and 0.30, 0.23 and 0.35 (4,800
